@@ -360,9 +360,14 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   SvdScratchLayout JL;
   {
     std::vector<int> sm, sn;
+    std::vector<char> exact;   // reduced-precision products round Y in its own basis: keep its phases
     for (int u = 0; u < nreq; ++u)
-      for (auto& e : W[u].plan.sectors) { sm.push_back(e.rows); sn.push_back(e.cols); }
-    svd_layout((int)sm.size(), sm.data(), sn.data(), JL);
+      for (auto& e : W[u].plan.sectors) {
+        sm.push_back(e.rows);
+        sn.push_back(e.cols);
+        exact.push_back(reqs[u].h->precision != MPS_FP64);
+      }
+    svd_layout((int)sm.size(), sm.data(), sn.data(), JL, -1, exact.data());
   }
   const int64_t jac_base = ws;
   ws = a256(ws + JL.total);

@@ -22,6 +22,12 @@
 // Storage: M is kept row-major with an odd leading dimension ld >= n, so the QR
 // rank-1 updates are coalesced (32 consecutive columns per warp) and, once R's
 // rows are conjugated in place, they are the contiguous columns of R^dag.
+// Sectors from min(m, n) = 48 (but those of reduced-precision updates) do not run these FP64 sweeps:
+// svd_front_kernel does an unpivoted QR and FP32 sweeps, and k_refine.cu finishes them with exact
+// tensor-core products; the kernels below take what that leaves.  A layer of 16 updates at chi = 512
+// (Bose-Hubbard, L = 32) takes 95 ms with it, 272 ms with the FP64 sweeps; three layers at chi = 128
+// (L = 24) 19 and 60 ms.
+//
 // GB300 runs FP64 at 2 FMA/clk/SM, so one SM per large sector would leave a
 // layer waiting on its largest sectors.  Three kernels share the work:
 //   jacobi_cta_kernel:           one CTA per sector, all of it in shared memory,
@@ -64,6 +70,9 @@ constexpr int kMaxCached = 16;          // rows cached in registers per lane (n 
 constexpr int kMaxCluster = 16;
 constexpr int kMaxWarps = 16;
 constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps per CTA, 2 CTAs per SM
+// smallest min(m, n) of a refined sector: below it the one-CTA kernel's few sweeps cost less than
+// the dozen launches of the refinement (chi = 64 layers of 31-35 columns, 1.4 ms)
+constexpr int kRefineMinK = 48;
 constexpr int kMaxStaged = 16;          // block pairs staged at once by one block-Jacobi CTA
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1022,6 +1031,278 @@ __device__ void mixed_precondition(const SvdSector& S, const Work& w, const doub
   *nsel_out = ns;
 }
 
+// ---------------------------------------------------------------------------------------
+// Front of the refined SVD of a sector (one cluster): M's columns in order of decreasing norm,
+// Householder QR, J = R^dag, FP32 one-sided Jacobi on J accumulating the rotations V.  The
+// refinement of k_refine.cu then makes J V orthogonal to FP64 rounding on the tensor cores.
+//
+// QR: the columns are sorted once and not pivoted again; on the lambda-graded sectors that costs
+// at most one more FP32 sweep than pivoting at every step (7 -> 8 on evolved and synthetic
+// sectors of 51-197 columns), and a column step needs one cluster barrier instead of five: the
+// warp that owns column k + 1 applies reflector k to it first and forms reflector k + 1 before
+// it goes on with its other columns.
+// ---------------------------------------------------------------------------------------
+
+// Column-major Householder QR of K reflectors over ncol columns (column j at A + pos(j) * ld) by all
+// warps of the cluster; a column belongs to one warp.  u_k stays in rows k.. of column k, R_kk goes
+// to rkk[k], 2 / u^dag u to tau[k].  ush: the CTA's copy of u_k (rows complex).
+template <typename T2> struct RealOf;
+template <> struct RealOf<double2> { using type = double; };
+template <> struct RealOf<float2> { using type = float; };
+__device__ __forceinline__ double real_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ float real_sqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ double warp_sum_t(double v) { return warp_sum(v); }
+__device__ __forceinline__ float warp_sum_t(float v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+template <typename T2, class Pos, class Sync>
+__device__ void qr_columns(T2* A, int64_t ld, int rows, int ncol, int K, T2* rkk, typename RealOf<T2>::type* tau,
+                           Pos pos, T2* ush, int rank, int nctas, Sync sync) {
+  using T = typename RealOf<T2>::type;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int worker = rank * nwarps + warp, workers = nctas * nwarps;
+  auto reflector = [&](int k) {      // one warp: column k is final above row k
+    T2* x = A + (int64_t)pos(k) * ld;
+    T s0 = 0, s1 = 0;
+    for (int i = k + lane; i < rows; i += 32) {
+      const T2 v = x[i];
+      s0 = fma(v.x, v.x, s0);
+      s1 = fma(v.y, v.y, s1);
+    }
+    const T x2 = warp_sum_t(s0 + s1);
+    const T xn = real_sqrt(x2);
+    const T2 x0 = x[k];
+    const T a0 = real_sqrt(x0.x * x0.x + x0.y * x0.y);
+    T2 beta;
+    if (a0 > 0) {
+      const T f = -xn / a0;
+      beta.x = x0.x * f;
+      beta.y = x0.y * f;
+    } else {
+      beta.x = -xn;
+      beta.y = 0;
+    }
+    const T uu = 2 * x2 + 2 * xn * a0;
+    __syncwarp();
+    if (lane == 0) {
+      T2 u0;
+      u0.x = x0.x - beta.x;
+      u0.y = x0.y - beta.y;
+      x[k] = u0;
+      __stcg(rkk + k, beta);
+      __stcg(tau + k, uu > 0 ? 2 / uu : 0);
+    }
+    __syncwarp();
+  };
+  if (worker == 0) reflector(0);
+  for (int k = 0; k < K; ++k) {
+    sync();
+    const T2* xk = A + (int64_t)pos(k) * ld;
+    const T tk = __ldcg(tau + k);
+    for (int i = k + tid; i < rows; i += blockDim.x) ush[i] = __ldcg(xk + i);
+    __syncthreads();
+    // columns j = worker (mod workers) beyond k, the next one first
+    int j0 = worker + (k + 1 - worker + workers - 1) / workers * workers;
+    if (k + 1 <= worker) j0 = worker;
+    for (int j = j0; j < ncol; j += 2 * workers) {
+      const bool two = j + workers < ncol;
+      T2* xa = A + (int64_t)pos(j) * ld;
+      T2* xb = A + (int64_t)pos(two ? j + workers : j) * ld;
+      T pa = 0, qa = 0, pb = 0, qb = 0, ra = 0, sa = 0, rb = 0, sb = 0;
+      for (int i = k + lane; i < rows; i += 32) {
+        const T2 u = ush[i], a = xa[i], b = xb[i];
+        pa = fma(u.x, a.x, pa);
+        ra = fma(u.y, a.y, ra);
+        qa = fma(u.x, a.y, qa);
+        sa = fma(-u.y, a.x, sa);
+        pb = fma(u.x, b.x, pb);
+        rb = fma(u.y, b.y, rb);
+        qb = fma(u.x, b.y, qb);
+        sb = fma(-u.y, b.x, sb);
+      }
+      pa += ra;
+      qa += sa;
+      pb += rb;
+      qb += sb;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        pa += __shfl_xor_sync(0xffffffffu, pa, o);
+        qa += __shfl_xor_sync(0xffffffffu, qa, o);
+        pb += __shfl_xor_sync(0xffffffffu, pb, o);
+        qb += __shfl_xor_sync(0xffffffffu, qb, o);
+      }
+      pa *= tk;
+      qa *= tk;
+      pb *= tk;
+      qb *= tk;
+      for (int i = k + lane; i < rows; i += 32) {
+        const T2 u = ush[i];
+        T2 a = xa[i];
+        a.x = fma(-u.x, pa, fma(u.y, qa, a.x));
+        a.y = fma(-u.x, qa, fma(-u.y, pa, a.y));
+        xa[i] = a;
+        if (two) {
+          T2 b = xb[i];
+          b.x = fma(-u.x, pb, fma(u.y, qb, b.x));
+          b.y = fma(-u.x, qb, fma(-u.y, pb, b.y));
+          xb[i] = b;
+        }
+      }
+      __syncwarp();
+      if (j == k + 1 && k + 1 < K) reflector(k + 1);
+    }
+  }
+  sync();
+}
+
+template <class Sync>
+__device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas, Sync sync, int max_sweeps,
+                          const JacobiBlocks32& j32, unsigned char* smem) {
+  const int m = S.m, n = S.n, K = min(m, n);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int tid_all = rank * blockDim.x + tid, threads_all = nctas * blockDim.x;
+  const int worker = rank * nwarps + warp, workers = nctas * nwarps;
+  double2* W = w.W;            // column-major, m rows
+  // ---- M = diag(lambda) Theta', transposed to columns: a warp moves 4 rows x 8 columns ----
+  {
+    const int tr = (m + 3) / 4, tc = (n + 7) / 8;
+    for (int64_t t = worker; t < (int64_t)tr * tc; t += workers) {
+      const int i = (int)(t / tc) * 4 + (lane >> 3), j = (int)(t % tc) * 8 + (lane & 7);
+      if (i < m && j < n) {
+        const double s = S.rowscale ? S.rowscale[i] : 1.0;
+        const double2 x = S.theta[(int64_t)i * n + j];
+        __stcg(W + (int64_t)j * m + i, make_double2(s * x.x, s * x.y));
+      }
+    }
+  }
+  if (tid_all < 16) __stcg(S.rstate + tid_all, 0);
+  sync();
+  for (int j = worker; j < n; j += workers) {
+    double a0 = 0.0, a1 = 0.0;
+    for (int i = lane; i < m; i += 32) {
+      const double2 x = __ldcg(W + (int64_t)j * m + i);
+      a0 = fma(x.x, x.x, a0);
+      a1 = fma(x.y, x.y, a1);
+    }
+    a0 = warp_sum(a0 + a1);
+    if (lane == 0) __stcg(w.nu + j, a0);
+  }
+  sync();
+  // descending order of the column norms (NaN last: the order stays a permutation), |M|_F^2
+  double fro2 = 0.0;
+  for (int j = lane; j < n; j += 32) fro2 += __ldcg(w.nu + j);
+  fro2 = warp_sum(fro2);
+  for (int j = tid_all; j < n; j += threads_all) {
+    const double vj = __ldcg(w.nu + j), v = isnan(vj) ? -1.0 : vj;
+    int rk = 0;
+    for (int q = 0; q < n; ++q) {
+      const double wq = __ldcg(w.nu + q), x = isnan(wq) ? -1.0 : wq;
+      rk += (x > v) || (x == v && q < j);
+    }
+    __stcg(w.perm + rk, j);
+  }
+  if (!(fro2 > 1e-270 && fro2 < 1e270)) {      // zero, not finite, or squares out of range
+    if (tid_all == 0) __stcg(S.rstate + 1, 1);
+    return;
+  }
+  const int sc = -(ilogb(fro2) / 2);            // J is scaled so that |J|_F is about 1 (exactly, by 2^sc)
+  const double scale = scalbn(1.0, sc);
+  const double frel = fmax(32.0 * kEps, S.floor_rel);
+  const double floor2 = fmax(frel * frel * fro2, S.floor_abs * S.floor_abs) * scale * scale;
+  if (tid_all == 0) {
+    S.rfloor2[0] = floor2;
+    S.rfloor2[1] = scalbn(1.0, -sc);
+  }
+  sync();
+  const int* perm = w.perm;
+  qr_columns(W, (int64_t)m, m, n, K, w.u, w.nu0, [&](int j) { return __ldcg(perm + j); },
+             reinterpret_cast<double2*>(smem), rank, nctas, sync);
+
+  // ---- J = R^dag: column i (n long) is the conjugate of row i of R, in sorted column order ----
+  double2* J = S.J;
+  const bool wide = S.wide;
+  const int jlen = wide ? K : n;
+  const int Rr = jlen + K, fld = (Rr + 1) & ~1;   // even: columns 16-byte aligned for bulk copies
+  float2* F = S.F;
+  float2* F1 = wide ? reinterpret_cast<float2*>(S.A1) : F;     // FP32 J: n x K for the second QR, or in place
+  const int64_t ld1 = wide ? n : fld;
+  {
+    const int tr = (K + 3) / 4, tc = (n + 7) / 8;
+    for (int64_t t = worker; t < (int64_t)tr * tc; t += workers) {
+      const int i = (int)(t / tc) * 4 + (lane & 3), j = (int)(t % tc) * 8 + (lane >> 2);
+      if (i < K && j < n) {
+        double2 x = make_double2(0.0, 0.0);
+        if (i == j) x = __ldcg(w.u + i);
+        else if (i < j) x = __ldcg(W + (int64_t)__ldcg(perm + j) * m + i);
+        x.x *= scale;
+        x.y *= -scale;
+        J[(int64_t)i * n + j] = x;
+        __stcg(F1 + (int64_t)i * ld1 + j, make_float2((float)x.x, (float)x.y));
+      }
+    }
+  }
+  for (int s = tid_all; s <= max_sweeps; s += threads_all) L2Mem::st(w.flags + s, 0);
+  if (wide) {      // FP32 QR of J: the sweeps rotate the K x K factor, the rotations are the same
+    sync();
+    float2* rk = reinterpret_cast<float2*>(w.u);      // m >= K entries
+    float* tk = reinterpret_cast<float*>(w.nu0);
+    qr_columns(F1, (int64_t)n, n, K, K, rk, tk, [](int j) { return j; }, reinterpret_cast<float2*>(smem), rank, nctas,
+               sync);
+    for (int64_t e = tid_all; e < (int64_t)K * K; e += threads_all) {
+      const int c = (int)(e / K), i = (int)(e % K);
+      float2 v = make_float2(0.f, 0.f);
+      if (i == c) v = __ldcg(rk + c);
+      else if (i < c) v = __ldcg(F1 + (int64_t)c * n + i);
+      __stcg(F + (int64_t)c * fld + i, v);
+    }
+  }
+  for (int64_t e = tid_all; e < (int64_t)K * (fld - jlen); e += threads_all) {   // V = I below
+    const int c = (int)(e / (fld - jlen)), i = (int)(e % (fld - jlen));
+    __stcg(F + (int64_t)c * fld + jlen + i, make_float2(i == c ? 1.f : 0.f, 0.f));
+  }
+  sync();
+  // ---- FP32 sweeps to FP32 convergence; the floor is a tenth of the FP64 one -------------------
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the staging area held reflectors
+  __syncthreads();
+  const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
+  const float fl32 = (float)(0.01 * floor2);
+  bool conv32 = false;
+  j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps + 6), conv32);
+  for (int j = worker; j < K; j += workers) {   // final FP32 norms
+    const float2* a = F + (int64_t)j * fld;
+    float acc = 0.f;
+    for (int i = lane; i < jlen; i += 32) {
+      const float2 x = __ldcg(a + i);
+      acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
+    }
+    acc = warp_sum_f(acc);
+    if (lane == 0) __stcg(S.nrm32 + j, acc);
+  }
+  sync();
+  if (tid_all < 32) {   // the kept columns, in column order
+    int ns = 0;
+    for (int c0 = 0; c0 < K; c0 += 32) {
+      const bool keep = c0 + lane < K && __ldcg(S.nrm32 + c0 + lane) > fl32;
+      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      if (keep) __stcg(S.sel + ns + __popc(mask & ((1u << lane) - 1)), c0 + lane);
+      ns += __popc(mask);
+    }
+    if (lane == 0) {
+      __stcg(S.rstate, ns);
+      if (ns == 0) __stcg(S.rstate + 1, 1);
+    }
+  }
+  sync();
+  const int ns = __ldcg(S.rstate);
+  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) {
+    const int t = (int)(e / K), k = (int)(e % K);
+    const float2 v = __ldcg(F + (int64_t)__ldcg(S.sel + t) * fld + jlen + k);
+    S.V0[e] = make_double2((double)v.x, (double)v.y);
+  }
+}
+
 template <class Mem, class Sync, class Jacobi, class J32 = NoJacobi32>
 __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int nctas, Sync sync, int max_sweeps,
                            Jacobi jacobi, J32 j32 = J32()) {
@@ -1496,7 +1777,24 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(
   j32.bsmax = jb.bsmax;
   j32.sm = reinterpret_cast<float2*>(smem_raw);
   j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * jb.gs * jb.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
+  if (S.F && S.rstate[1] == 0 && S.rstate[2] > 0) return;   // settled by the refinement
   svd_sector<L2Mem>(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, jb, j32);
+}
+
+__global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSector* __restrict__ secs, int cluster,
+                                                                     int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rank = (int)cluster_rank();
+  const SvdSector S = secs[blockIdx.x / cluster];
+  const int K = min(S.m, S.n);
+  // FP32 columns of jlen + K <= 2 jlen complex values in the staging area sized for FP64 ones
+  JacobiBlocks32 j32;
+  j32.g = S.groups;
+  j32.gs = S.staged;
+  j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
+  j32.sm = reinterpret_cast<float2*>(smem_raw);
+  j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
+  svd_front(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, j32, smem_raw);
 }
 
 
@@ -1536,13 +1834,16 @@ cudaError_t set_attrs(int* big_out) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBlockSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
   if (e != cudaSuccess) return e;
   // clusters of 16 CTAs are non-portable: use them only where the device can place them
   int big = 8;
   if (cudaFuncSetAttribute(jacobi_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
           cudaSuccess &&
       cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-          cudaSuccess) {
+          cudaSuccess &&
+      cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(16);
     cfg.blockDim = dim3(kBlockThreads);
@@ -1564,7 +1865,9 @@ cudaError_t set_attrs(int* big_out) {
   return cudaSuccess;
 }
 
-cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_sweeps, cudaStream_t st) {
+// fallback: the FP64 sweeps of a refined group, for the sectors the refinement left
+cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_sweeps, cudaStream_t st,
+                         bool fallback = false) {
   if (g.count <= 0) return cudaSuccess;
   const SvdSector* d = d_secs + g.first;
   count_launch();
@@ -1574,7 +1877,7 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g.count * g.cl);
-  cfg.blockDim = dim3(g.kind == kSvdClusterBlock ? kBlockThreads : kSvdThreads);
+  cfg.blockDim = dim3(g.kind == kSvdCluster ? kSvdThreads : kBlockThreads);
   cfg.dynamicSmemBytes = g.smem;
   cfg.stream = st;
   cudaLaunchAttribute at;
@@ -1584,7 +1887,8 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  if (g.kind == kSvdClusterBlock) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, g.cl, max_sweeps);
+  if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps);
+  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, g.cl, max_sweeps);
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
 }
 
@@ -1639,13 +1943,16 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
       }
     }
     if (std::min(S.m, S.n) >= tune.rr_min_k) pick_cl = 0;
+    if (16LL * std::max(S.m, S.n) > kBlockSmemMax) secs[k].F = nullptr;   // no room for a reflector
     if (pick_cl) {
-      key[k] = {kSvdClusterBlock, pick_cl};
-      smem[k] = block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs);
+      key[k] = {secs[k].F ? kSvdRefine : kSvdClusterBlock, pick_cl};
+      smem[k] = std::max<int64_t>(block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs),
+                                  secs[k].F ? 16LL * std::max(S.m, S.n) : 0);      // the QR's copy of a reflector
       secs[k].groups = pick_g;
       secs[k].staged = pick_gs;
     } else {
       key[k] = {kSvdCluster, big_cluster};
+      secs[k].F = nullptr;        // the round-robin kernel runs in FP64 alone
     }
   }
   // group by (kind, cluster size); the most expensive sectors first inside a group
@@ -1671,10 +1978,13 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
       g.smem = 0;
       g.first = (int)out.size();
       g.count = 0;
+      g.max_k = g.max_n = 0;
       groups.push_back(g);
     }
     groups.back().count++;
     groups.back().smem = std::max<int>(groups.back().smem, (int)smem[k]);
+    groups.back().max_k = std::max(groups.back().max_k, std::min(secs[k].m, secs[k].n));
+    groups.back().max_n = std::max(groups.back().max_n, secs[k].n);
     out.push_back(secs[k]);
   }
   secs.swap(out);
@@ -1699,16 +2009,31 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
     cudaStream_t s = (fan && g > 0) ? side[g - 1] : st;
     if ((e = launch_group(d_secs, groups[g], max_sweeps, s)) != cudaSuccess) return e;
   }
-  if (fan) {
-    for (int g = 1; g < ng; ++g) {
-      if ((e = cudaEventRecord(join[g - 1], side[g - 1])) != cudaSuccess) return e;
-      if ((e = cudaStreamWaitEvent(st, join[g - 1], 0)) != cudaSuccess) return e;
-    }
+  auto joined = [&](int g) -> cudaError_t {
+    cudaError_t e2 = cudaEventRecord(join[g - 1], side[g - 1]);
+    return e2 == cudaSuccess ? cudaStreamWaitEvent(st, join[g - 1], 0) : e2;
+  };
+  // the refined groups come first (group 0 on st): refine them together once their fronts are done,
+  // while the other groups go on
+  int nr = 0, count = 0, max_k = 0, max_n = 0;
+  for (; nr < ng && groups[nr].kind == kSvdRefine; ++nr) {
+    count += groups[nr].count;
+    max_k = std::max(max_k, groups[nr].max_k);
+    max_n = std::max(max_n, groups[nr].max_n);
+    if (fan && nr > 0 && (e = joined(nr)) != cudaSuccess) return e;
   }
+  if (nr > 0) {
+    if ((e = launch_refine(d_secs + groups[0].first, count, max_k, max_n, st)) != cudaSuccess) return e;
+    for (int g = 0; g < nr; ++g)
+      if ((e = launch_group(d_secs, groups[g], max_sweeps, st, true)) != cudaSuccess) return e;
+  }
+  if (fan)
+    for (int g = std::max(nr, 1); g < ng; ++g)
+      if ((e = joined(g)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
-bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k) {
+bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k, const char* exact) {
   if (cluster_min_k < 0) cluster_min_k = svd_cluster_min_k();
   L.mode.assign(ns, kSvdSmem);
   L.work_off.assign(ns, -1);
@@ -1718,17 +2043,21 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
   L.flag_off.assign(ns, -1);
   L.piv_off.assign(ns, -1);
   L.wide.assign(ns, 0);
+  L.exact.assign(ns, 0);
   L.w2_off.assign(ns, -1);
   L.yt_off.assign(ns, -1);
-  for (auto* v : {&L.f32_off, &L.n32_off, &L.vd_off, &L.gm_off, &L.a1_off, &L.sel_off}) v->assign(ns, -1);
+  for (auto* v : {&L.f32_off, &L.n32_off, &L.vd_off, &L.gm_off, &L.a1_off, &L.sel_off, &L.j_off, &L.v_off2, &L.misc_off})
+    v->assign(ns, -1);
   L.smem = 0;
-  const int mix_k = svd_mixed_min_k();
+  const int set_k = svd_mixed_min_k(), own_k = std::min(set_k, kRefineMinK);   // 0: off
   int64_t off = 0;
   auto a256 = [](int64_t x) { return (x + 255) & ~int64_t(255); };
   for (int k = 0; k < ns; ++k) {
     if (m[k] < 1 || n[k] < 1) return false;
     const int64_t need = svd_smem_need(m[k], n[k]);
-    if (need <= kSvdSmemMax && std::min(m[k], n[k]) < cluster_min_k) {
+    L.exact[k] = exact && exact[k];
+    const bool refine = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) >= own_k;
+    if (need <= kSvdSmemMax && std::min(m[k], n[k]) < cluster_min_k && !refine) {
       L.smem = std::max<int>(L.smem, (int)need);
       continue;
     }
@@ -1740,19 +2069,32 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     L.ord_off[k] = off;  off = a256(off + 4 * (N + Kk));                // perm, ord
     L.flag_off[k] = off; off = a256(off + 4 * (kJacobiMaxSweeps + 1 + kMaxCluster));   // flags, pivot index
     L.piv_off[k] = off;  off = a256(off + 8 * (kMaxCluster + 2));       // pivot value, scalars
-    if (4LL * n[k] >= 5LL * m[k]) {   // wide: the Jacobi sweeps run on the K x K factor R2
-      L.wide[k] = 1;
-      L.w2_off[k] = off; off = a256(off + 16 * Kk * odd_ld((int)Kk));     // R2 / Jacobi matrix
-      L.yt_off[k] = off; off = a256(off + 16 * N * Kk);                   // Q2 applied to its columns
-    }
-    if (mix_k > 0 && Kk >= mix_k) {   // FP32 sweeps first (see mixed_precondition)
-      const int64_t jlen = L.wide[k] ? Kk : N, jld = L.wide[k] ? odd_ld((int)Kk) : odd_ld(n[k]);
-      L.f32_off[k] = off; off = a256(off + 8 * (jlen + Kk + 2) * Kk);
-      L.n32_off[k] = off; off = a256(off + 4 * Kk);
-      L.vd_off[k] = off;  off = a256(off + 16 * Kk * Kk);
-      L.gm_off[k] = off;  off = a256(off + 16 * Kk * Kk);
-      L.a1_off[k] = off;  off = a256(off + 16 * jld * Kk);
-      L.sel_off[k] = off; off = a256(off + 4 * (Kk + 1));
+    const bool wide = 4LL * n[k] >= 5LL * m[k];   // the Jacobi sweeps run on the K x K factor R2
+    L.wide[k] = wide;
+    if (refine) {   // FP32 start and refinement (svd_front, k_refine.cu); the FP64 sweeps that may
+                    // follow use A1 and V's space for their second QR
+      const int64_t jlen = wide ? Kk : N;
+      L.j_off[k] = off;    off = a256(off + 16 * N * Kk);
+      L.a1_off[k] = off;   off = a256(off + 16 * N * Kk);
+      L.v_off2[k] = off;   off = a256(off + 2 * 16 * Kk * odd_ld((int)Kk));
+      L.misc_off[k] = off; off = a256(off + 64 + 16 + 8 * Kk + 4 * (4 * Kk + 1) + 16);
+      off = a256(off + 8 * (jlen + Kk + 2) * Kk);      // F, behind the small arrays
+      L.w2_off[k] = L.v_off2[k];
+      L.yt_off[k] = L.a1_off[k];
+    } else {
+      if (wide) {
+        L.w2_off[k] = off; off = a256(off + 16 * Kk * odd_ld((int)Kk));     // R2 / Jacobi matrix
+        L.yt_off[k] = off; off = a256(off + 16 * N * Kk);                   // Q2 applied to its columns
+      }
+      if (set_k > 0 && Kk >= set_k) {   // FP32 sweeps first (see mixed_precondition)
+        const int64_t jlen = wide ? Kk : N, jld = wide ? odd_ld((int)Kk) : odd_ld(n[k]);
+        L.f32_off[k] = off; off = a256(off + 8 * (jlen + Kk + 2) * Kk);
+        L.n32_off[k] = off; off = a256(off + 4 * Kk);
+        L.vd_off[k] = off;  off = a256(off + 16 * Kk * Kk);
+        L.gm_off[k] = off;  off = a256(off + 16 * Kk * Kk);
+        L.a1_off[k] = off;  off = a256(off + 16 * jld * Kk);
+        L.sel_off[k] = off; off = a256(off + 4 * (Kk + 1));
+      }
     }
   }
   L.total = off;
@@ -1775,6 +2117,7 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
   }
   S.f32 = nullptr;
   S.fp32_sweeps = svd_mixed_sweeps();
+  S.F = nullptr;
   if (L.f32_off[k] >= 0) {
     S.f32 = reinterpret_cast<float2*>(base + L.f32_off[k]);
     S.nrm32 = reinterpret_cast<float*>(base + L.n32_off[k]);
@@ -1782,6 +2125,24 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
     S.gm = reinterpret_cast<double2*>(base + L.gm_off[k]);
     S.a1 = reinterpret_cast<double2*>(base + L.a1_off[k]);
     S.sel = reinterpret_cast<int*>(base + L.sel_off[k]);
+  }
+  if (L.misc_off[k] >= 0) {
+    const int64_t K = std::min(S.m, S.n);
+    S.J = reinterpret_cast<double2*>(base + L.j_off[k]);
+    S.A0 = S.work;
+    S.A1 = reinterpret_cast<double2*>(base + L.a1_off[k]);
+    S.V0 = reinterpret_cast<double2*>(base + L.v_off2[k]);
+    S.V1 = S.V0 + K * odd_ld((int)K);
+    char* p = base + L.misc_off[k];
+    S.rstate = reinterpret_cast<int*>(p);          p += 64;
+    S.rfloor2 = reinterpret_cast<double*>(p);      p += 16;
+    S.rnorm = reinterpret_cast<double*>(p);        p += 8 * K;
+    S.cexp = reinterpret_cast<int*>(p);            p += 4 * K;
+    S.rdiag = reinterpret_cast<int*>(p);           p += 4 * K;
+    S.nrm32 = reinterpret_cast<float*>(p);         p += 4 * K;
+    S.sel = reinterpret_cast<int*>(p);             p += 4 * (K + 1);
+    S.F = reinterpret_cast<float2*>(base + ((p - base + 255) & ~int64_t(255)));
+    S.E = S.F;
   }
 }
 
@@ -1899,6 +2260,10 @@ extern "C" int mps_svd_sectors_noalloc(int n_sectors, const int* m, const int* n
   SvdScratchLayout L;
   if (!svd_layout(n_sectors, m, n, L)) return MPS_EINVAL;
   const int64_t desc = ((int64_t)sizeof(SvdSector) * n_sectors + 255) / 256 * 256;
+  if (desc + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) {   // the FP64 sweeps need less scratch
+    const std::vector<char> plain(n_sectors, 1);
+    if (!svd_layout(n_sectors, m, n, L, -1, plain.data())) return MPS_EINVAL;
+  }
   if (desc + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) return MPS_ENOMEM;   // over the fixed scratch
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return MPS_ECUDA;

@@ -11,7 +11,7 @@
 
 namespace mps {
 
-constexpr int kSvdSideStreams = 4;      // side streams for concurrent SVD kernel groups
+constexpr int kSvdSideStreams = 8;      // side streams for concurrent SVD kernel groups
 
 // ---------------------------------------------------------------------------
 // Charge arithmetic.  U(1) (zn = 0, Sec. II): block (l, m) of a site carries the physical
@@ -202,6 +202,7 @@ struct TileRef { int task; int ti; int tj; };
 
 constexpr int kSvdSmem = 0;          // one CTA, the whole sector in shared memory
 constexpr int kSvdCluster = 1;       // a thread-block cluster, data in L2, round-robin Jacobi
+constexpr int kSvdRefine = 3;        // QR and FP32 Jacobi on a cluster, then tensor-core refinement
 constexpr int kSvdClusterBlock = 2;  // a thread-block cluster, data in L2, block Jacobi staged in shared memory
 
 struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
@@ -233,6 +234,16 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   double2* gm;                // K x K: their Gram matrix, then its Cholesky factor
   double2* a1;                // jld x K: the Jacobi matrix times V, the start of the FP64 sweeps
   int* sel;                   // K + 1: selected columns, then their count
+  // FP32 start and tensor-core refinement (cluster mode, F == nullptr: not refined):
+  float2* F;                  // the Jacobi matrix in FP32 stacked on V (identity), (jlen + K, even) x K
+  double2 *J, *A0, *A1;       // n x K column-major: R^dag, and J V of even / odd refinement steps (A0 overlays work)
+  double2 *V0, *V1;           // K x K: the rotations of even / odd steps
+  float2* E;                  // K x K: the scaled correction of a step (overlays F)
+  double* rnorm;              // K squared column norms of the current A
+  double* rfloor2;            // [0] the floor in the scale of J, [1] the power of two that undoes that scale
+  int* cexp;                  // K scale exponents of the columns of J or A
+  int* rdiag;                 // K: 1 - cosine of the large angles of a step, in units of 2^-30
+  int* rstate;                // [0] columns kept, [1] left to the FP64 sweeps, [2] steps when settled, [4 + step] size of E
   int fp32_sweeps;            // limit of the FP32 sweeps
 };
 
@@ -241,14 +252,19 @@ struct SvdScratchLayout {
   std::vector<int> mode;
   std::vector<int64_t> work_off, v_off, norm_off, ord_off, flag_off, piv_off, w2_off, yt_off;
   std::vector<int64_t> f32_off, n32_off, vd_off, gm_off, a1_off, sel_off;   // mixed precision (-1: off)
+  std::vector<int64_t> j_off, v_off2, misc_off;       // refinement (-1: off)
   std::vector<int> wide;
+  std::vector<char> exact;
   int smem = 0;               // dynamic shared memory of the one-CTA kernel
   int64_t total = 0;
 };
 // Sectors that fit in shared memory run on the one-CTA kernel unless min(m, n) >= cluster_min_k
 // (a cluster kernel then spreads them over several SMs; -1: the process setting
 // mps_svd_cluster_min_k, off by default).
-bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k = -1);
+// exact (or nullptr): per sector, whether the phases of Y's columns are part of the result; such a
+// sector is not refined (its pivoted QR and the order of its sweeps fix the phases).
+bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k = -1,
+                const char* exact = nullptr);
 int svd_cluster_min_k();
 // Cluster sectors with min(m, n) >= this run FP32 Jacobi sweeps first and finish in FP64
 // (0: every sector FP64 only); mps_svd_mixed_min_k sets it.
@@ -375,7 +391,7 @@ namespace mps {
 // Kernel launchers (defined in the .cu files).
 cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
-struct SvdGroup { int kind, cl, smem, first, count; };
+struct SvdGroup { int kind, cl, smem, first, count, max_k, max_n; };
 // Tile shape of the cluster SVD: target column-block width of the block-Jacobi kernel, the
 // smallest cluster size tried, and the sector size (min(m, n)) from which a sector gets a
 // cluster of 16 CTAs (the largest sectors of a layer set its critical path), and the sector
@@ -408,6 +424,11 @@ bool svd_forced_tune(SvdTune& t);
 cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGroup>& groups, cudaStream_t st,
                               const cudaStream_t* side, int n_side, cudaEvent_t fork, const cudaEvent_t* join,
                               int max_sweeps = 40);
+
+// The refinement of sectors that svd_front_kernel has prepared (k_refine.cu): J V, at most
+// kRefineSteps corrections, and the outputs of the sectors that have settled.
+constexpr int kRefineSteps = 5;
+cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max_n, cudaStream_t st);
 
 cudaError_t launch_select(const SelectSector* d_secs, const SelectTask* d_tasks, int n_tasks,
                           int* d_kept, SelectResult* d_res, cudaStream_t st);
