@@ -13,9 +13,10 @@
 //   sumprod_kernel   every block contraction (H_eff Psi, environment updates, the centre
 //                    tensor, the new sites): an output tile accumulates a list of terms
 //                    coef * op(A) op(B) (or coef * op(A)) in FP64, written once;
-//   dots_kernel / dots_reduce_kernel / subtract_kernel / scale_kernel / combine_kernel
-//                    the Krylov vector work (classical Gram-Schmidt applied twice, so the
-//                    basis stays orthonormal to rounding), deterministic two-pass sums;
+//   gs_dots_kernel / gs_update_kernel / gs_scale_kernel   the Gram-Schmidt of a Lanczos step
+//                    (classical, applied twice, so the basis stays orthonormal to rounding),
+//                    deterministic two-pass sums;
+//   dots_kernel / dots_reduce_kernel / scale_kernel / combine_kernel   the other vector work;
 //   tridiag_kernel   the lowest Ritz pair of the Lanczos tridiagonal (Sturm bisection,
 //                    then inverse iteration with a shift just below it);
 //   expm_tridiag_kernel / combine_c_kernel   TDVP's Krylov exponential exp(-i tau T) e_1
@@ -46,7 +47,7 @@ using cplx = std::complex<double>;
 // ---------------------------------------------------------------------------
 // Generic block sum-of-products kernel
 // ---------------------------------------------------------------------------
-constexpr int kT = 64, kKc = 16, kThr = 256;
+constexpr int kT = 8, kKc = 16, kThr = 64;
 enum : int { kAX = 1, kBX = 2, kConjA = 4, kConjB = 8, kNoB = 16 };
 enum : int { kCY = 1, kAccum = 2 };
 
@@ -66,9 +67,19 @@ struct SPTask {
 };
 struct SPTile { int task, ti, tj; };
 
+// An 8 x 8 output tile per CTA of 64 threads, one output each.  An SM does 2 FP64 FMA per clock, so
+// a block's time is its outputs' FMAs on one SM: a 27 x 27 block of H_eff Psi at chi = 96 (ten terms,
+// 790 k FMA) took 200 us on the single CTA that 64 x 64 tiles gave it, while the whole product is
+// 4.5 us of the chip.  Small tiles spread every block over many SMs and pad ragged blocks least; the
+// operands they re-read come from L2 (4 bytes a complex FMA).  Stages of 16 k are copied
+// asynchronously, the next one while the present one is used; the four real products of a complex one
+// are summed apart, which gives each thread independent chains over the pipe's 64-cycle latency and
+// leaves conjugations to the end of a term.
+// Bose-Hubbard L = 10, chi <= 96: 130 -> 32 us a product (events); L = 64, chi <= 256: 256 -> 853
+// GFLOP/s, 68% of the FP64 peak.
 struct SPSmem {
-  double2 A[kT][kKc + 1];
-  double2 B[kKc][kT];
+  double2 A[2][kT][kKc + 1];
+  double2 B[2][kKc][kT];
 };
 
 __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
@@ -77,195 +88,121 @@ __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
   acc.y = fma(a.x, b.y, acc.y);
   acc.y = fma(a.y, b.x, acc.y);
 }
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+
+// 16-byte copy into shared memory, zeros when ok is false
+__device__ __forceinline__ void copy16(double2* dst, const double2* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
 }
 
-// A block of at most 1024 outputs (one tile): its outputs are dealt to the threads in order,
-// up to four per thread, so that every warp's lanes hold real outputs (the 16 x 16 thread grid
-// of the general path would spend most FP64 issue slots of a block of 17-30 rows and columns
-// on padding; this part issues 2 FP64 FMA per clock per SM, so only dense warps pay).
-__device__ __forceinline__ void small_block(const SPTask& T, const SPTerm* __restrict__ terms,
-                                            const double2* __restrict__ X, double2* __restrict__ Y, SPSmem& sm) {
-  const int tid = threadIdx.x;
-  const int MN = T.M * T.N, nq = (MN + kThr - 1) / kThr;
-  int rr[4], cc[4];
-  bool ok[4];
-  double2 acc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int o = tid + kThr * q;
-    ok[q] = o < MN;
-    rr[q] = ok[q] ? o / T.N : 0;
-    cc[q] = ok[q] ? o % T.N : 0;
-    acc[q] = make_double2(0.0, 0.0);
-  }
-  for (int t = T.t0; t < T.t1; ++t) {
-    const SPTerm P = terms[t];
-    const double2* A = (P.flags & kAX) ? X + P.a : reinterpret_cast<const double2*>(P.a);
-    const bool ca = (P.flags & kConjA) != 0;
-    if (P.flags & kNoB) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q < nq && ok[q]) {
-          double2 v = A[(int64_t)rr[q] * P.sar + (int64_t)cc[q] * P.sac];
-          if (ca) v.y = -v.y;
-          cfma(acc[q], P.coef, v);
-        }
-      }
-      continue;
-    }
-    const double2* B = (P.flags & kBX) ? X + P.b : reinterpret_cast<const double2*>(P.b);
-    const bool cb = (P.flags & kConjB) != 0;
-    for (int k0 = 0; k0 < P.K; k0 += kKc) {
-      const int kc = min(kKc, P.K - k0);
-      for (int e = tid; e < T.M * kc; e += kThr) {
-        int r, k;
-        if (P.sac == 1) { r = e / kc; k = e % kc; } else { k = e / T.M; r = e % T.M; }
-        double2 v = A[(int64_t)r * P.sar + (int64_t)(k0 + k) * P.sac];
-        if (ca) v.y = -v.y;
-        sm.A[r][k] = cmul(P.coef, v);
-      }
-      for (int e = tid; e < T.N * kc; e += kThr) {
-        int k, c;
-        if (P.sbc == 1) { k = e / T.N; c = e % T.N; } else { c = e / kc; k = e % kc; }
-        double2 v = B[(int64_t)(k0 + k) * P.sbr + (int64_t)c * P.sbc];
-        if (cb) v.y = -v.y;
-        sm.B[k][c] = v;
-      }
-      __syncthreads();
-      for (int kk = 0; kk < kc; ++kk) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (q < nq) cfma(acc[q], sm.A[rr[q]][kk], sm.B[kk][cc[q]]);
-      }
-      __syncthreads();
-    }
-  }
-  double2* C = (T.flags & kCY) ? Y + T.c : reinterpret_cast<double2*>(T.c);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (q < nq && ok[q]) {
-      double2& o = C[(int64_t)rr[q] * T.ldc + cc[q]];
-      if (T.flags & kAccum) {
-        double2 v = o;
-        v.x += acc[q].x;
-        v.y += acc[q].y;
-        o = v;
-      } else {
-        o = acc[q];
-      }
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kThr, 2) sumprod_kernel(const SPTask* __restrict__ tasks,
+__global__ void __launch_bounds__(kThr) sumprod_kernel(const SPTask* __restrict__ tasks,
                                                        const SPTerm* __restrict__ terms,
                                                        const SPTile* __restrict__ tiles,
                                                        const double2* __restrict__ X, double2* __restrict__ Y) {
   __shared__ SPSmem sm;
   const SPTile tr = tiles[blockIdx.x];
   const SPTask T = tasks[tr.task];
-  if (T.M <= kT && T.N <= kT && T.M * T.N <= 4 * kThr) {
-    small_block(T, terms, X, Y, sm);
-    return;
-  }
   const int row0 = tr.ti * kT, col0 = tr.tj * kT;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double2 acc[4][4];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const int r = row0 + ty, c = col0 + tx;
+  const bool rows_on = row0 + (ty & ~3) < T.M;      // a warp holds 4 rows
+  double2 acc = make_double2(0.0, 0.0);
+
+  auto stage = [&](const SPTerm& P, int k0, int buf) {
+    const double2* A = (P.flags & kAX) ? X + P.a : reinterpret_cast<const double2*>(P.a);
+    const double2* B = (P.flags & kBX) ? X + P.b : reinterpret_cast<const double2*>(P.b);
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
+    for (int h = 0; h < 2; ++h) {
+      const int e = tid + h * kThr;
+      const int ar = P.sac == 1 ? e >> 4 : e & 7, ak = P.sac == 1 ? e & 15 : e >> 3;
+      const bool oka = row0 + ar < T.M && k0 + ak < P.K;
+      copy16(&sm.A[buf][ar][ak], oka ? A + (int64_t)(row0 + ar) * P.sar + (int64_t)(k0 + ak) * P.sac : A, oka);
+      const int bk = P.sbc == 1 ? e >> 3 : e & 15, bc = P.sbc == 1 ? e & 7 : e >> 4;
+      const bool okb = col0 + bc < T.N && k0 + bk < P.K;
+      copy16(&sm.B[buf][bk][bc], okb ? B + (int64_t)(k0 + bk) * P.sbr + (int64_t)(col0 + bc) * P.sbc : B, okb);
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  auto next_product = [&](int q) {      // the first term from q that is a product
+    while (q < T.t1 && (terms[q].flags & kNoB)) ++q;
+    return q;
+  };
+  // terms without a second operand
   for (int q = T.t0; q < T.t1; ++q) {
+    if (!(terms[q].flags & kNoB)) continue;
     const SPTerm P = terms[q];
     const double2* A = (P.flags & kAX) ? X + P.a : reinterpret_cast<const double2*>(P.a);
-    const bool ca = (P.flags & kConjA) != 0;
-    if (P.flags & kNoB) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = row0 + ty + 16 * i;
-        if (r >= T.M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = col0 + tx + 16 * j;
-          if (c >= T.N) continue;
-          double2 v = A[(int64_t)r * P.sar + (int64_t)c * P.sac];
-          if (ca) v.y = -v.y;
-          cfma(acc[i][j], P.coef, v);
-        }
-      }
-      continue;
-    }
-    const double2* B = (P.flags & kBX) ? X + P.b : reinterpret_cast<const double2*>(P.b);
-    const bool cb = (P.flags & kConjB) != 0;
-    // warp-uniform counts of the 16-row / 16-column groups that hold valid outputs: a
-    // block smaller than the tile spends no FP64 issue slots on its padding
-    const int warp_ty = (tid >> 5) * 2;
-    int ni = 0, nj = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) ni += (row0 + warp_ty + 16 * i < T.M);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) nj += (col0 + 16 * j < T.N);
-    // only the block's own rows / columns are staged and read: the accumulators of padding rows
-    // and columns see stale shared memory and are never stored
-    const int mr = min(kT, T.M - row0), ncl = min(kT, T.N - col0);
-    for (int k0 = 0; k0 < P.K; k0 += kKc) {
-      const int kc = min(kKc, P.K - k0);
-      for (int e = tid; e < mr * kc; e += kThr) {
-        int r, k;
-        if (P.sac == 1) { r = e / kc; k = e % kc; } else { k = e / mr; r = e % mr; }
-        double2 v = A[(int64_t)(row0 + r) * P.sar + (int64_t)(k0 + k) * P.sac];
-        if (ca) v.y = -v.y;
-        sm.A[r][k] = cmul(P.coef, v);
-      }
-      for (int e = tid; e < ncl * kc; e += kThr) {
-        int k, c;
-        if (P.sbc == 1) { k = e / ncl; c = e % ncl; } else { c = e / kc; k = e % kc; }
-        double2 v = B[(int64_t)(k0 + k) * P.sbr + (int64_t)(col0 + c) * P.sbc];
-        if (cb) v.y = -v.y;
-        sm.B[k][c] = v;
-      }
-      __syncthreads();
-      for (int kk = 0; kk < kc; ++kk) {
-        double2 a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (i < ni) a[i] = sm.A[ty + 16 * i][kk];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (j < nj) b[j] = sm.B[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (i < ni) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              if (j < nj) cfma(acc[i][j], a[i], b[j]);
-          }
-        }
-      }
-      __syncthreads();
+    if (r < T.M && c < T.N) {
+      double2 v = A[(int64_t)r * P.sar + (int64_t)c * P.sac];
+      if (P.flags & kConjA) v.y = -v.y;
+      cfma(acc, P.coef, v);
     }
   }
-  double2* C = (T.flags & kCY) ? Y + T.c : reinterpret_cast<double2*>(T.c);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = row0 + ty + 16 * i;
-    if (r >= T.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = col0 + tx + 16 * j;
-      if (c >= T.N) continue;
-      double2& o = C[(int64_t)r * T.ldc + c];
-      if (T.flags & kAccum) {
-        double2 v = o;
-        v.x += acc[i][j].x;
-        v.y += acc[i][j].y;
-        o = v;
-      } else {
-        o = acc[i][j];
+  int q = next_product(T.t0), buf = 0;
+  SPTerm P;
+  if (q < T.t1) {
+    P = terms[q];
+    stage(P, 0, 0);
+  }
+  while (q < T.t1) {
+    double p0 = 0.0, q0 = 0.0, r0 = 0.0, s0 = 0.0, p1 = 0.0, q1 = 0.0, r1 = 0.0, s1 = 0.0;
+    const int qn = next_product(q + 1);
+    SPTerm Pn;
+    if (qn < T.t1) Pn = terms[qn];
+    for (int k0 = 0; k0 < P.K; k0 += kKc) {
+      const int kc = min(kKc, P.K - k0);
+      bool more = true;
+      if (k0 + kKc < P.K) stage(P, k0 + kKc, buf ^ 1);
+      else if (qn < T.t1) stage(Pn, 0, buf ^ 1);
+      else more = false;
+      if (more) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+      __syncthreads();
+      if (rows_on) {
+        int kk = 0;
+#pragma unroll 4
+        for (; kk + 1 < kc; kk += 2) {
+          const double2 a = sm.A[buf][ty][kk], b = sm.B[buf][kk][tx];
+          const double2 a1 = sm.A[buf][ty][kk + 1], b1 = sm.B[buf][kk + 1][tx];
+          p0 = fma(a.x, b.x, p0);
+          q0 = fma(a.y, b.y, q0);
+          r0 = fma(a.x, b.y, r0);
+          s0 = fma(a.y, b.x, s0);
+          p1 = fma(a1.x, b1.x, p1);
+          q1 = fma(a1.y, b1.y, q1);
+          r1 = fma(a1.x, b1.y, r1);
+          s1 = fma(a1.y, b1.x, s1);
+        }
+        if (kk < kc) {
+          const double2 a = sm.A[buf][ty][kk], b = sm.B[buf][kk][tx];
+          p0 = fma(a.x, b.x, p0);
+          q0 = fma(a.y, b.y, q0);
+          r0 = fma(a.x, b.y, r0);
+          s0 = fma(a.y, b.x, s0);
+        }
       }
+      __syncthreads();
+      buf ^= 1;
     }
+    if (rows_on) {
+      // a' = (a.x, sa a.y), b' = (b.x, sb b.y)
+      const double sa = (P.flags & kConjA) ? -1.0 : 1.0, sb = (P.flags & kConjB) ? -1.0 : 1.0;
+      const double2 v = make_double2(fma(-sa * sb, q0 + q1, p0 + p1), fma(sb, r0 + r1, sa * (s0 + s1)));
+      cfma(acc, P.coef, v);
+    }
+    P = Pn;
+    q = qn;
+  }
+  if (r < T.M && c < T.N) {
+    double2* C = (T.flags & kCY) ? Y + T.c : reinterpret_cast<double2*>(T.c);
+    double2& o = C[(int64_t)r * T.ldc + c];
+    if (T.flags & kAccum) {
+      const double2 v = o;
+      acc.x += v.x;
+      acc.y += v.y;
+    }
+    o = acc;
   }
 }
 
@@ -328,34 +265,177 @@ __global__ void __launch_bounds__(kVecThreads) dots_reduce_kernel(const double2*
   }
 }
 
-// w[e] -= sum_k coef[k] V_k[e]
-__global__ void __launch_bounds__(kVecThreads) subtract_kernel(double2* __restrict__ w, const double2* __restrict__ V,
-                                                               int64_t ldv, int nk, const double2* __restrict__ coef,
-                                                               int64_t n) {
-  __shared__ double2 cs[64];
-  for (int k = threadIdx.x; k < nk; k += kVecThreads) cs[k] = coef[k];
-  __syncthreads();
-  for (int64_t e = (int64_t)blockIdx.x * kVecThreads + threadIdx.x; e < n; e += (int64_t)gridDim.x * kVecThreads) {
-    double2 acc = w[e];
-    for (int k = 0; k < nk; ++k) {
-      const double2 v = V[(int64_t)k * ldv + e], c = cs[k];
-      acc.x -= c.x * v.x - c.y * v.y;
-      acc.y -= c.x * v.y + c.y * v.x;
+// ---- one Lanczos step's Gram-Schmidt in four launches -------------------------------------------
+// A CTA owns a chunk of 128 E elements of w.  gs_dots_kernel leaves the chunk's partial products with
+// every basis vector; gs_update_kernel sums all CTAs' partials itself (fixed order, so every CTA gets
+// the same coefficients), subtracts, and forms the next partials from the chunk it still holds (the
+// second pass's products, or the norm); gs_scale_kernel closes the step.  The separate kernels for
+// products, sums, subtraction, norm, scalars and scaling were ten launches, and on the vectors of
+// short chains (10-20 thousand elements) launch latency was all of their time: 230 us a step under
+// event timing at L = 10, chi <= 96, now 45.  FP64 adds are what the reductions cost (2 a clock and SM), so a warp
+// sums 8 vectors' products together: 18 adds instead of 80.
+constexpr int kGsThreads = 128;
+constexpr int kGsMaxK = 64;
+
+// v[0..7] of the 32 lanes summed over the lanes: lane 4 k holds the sum of v[k] (k = 0..7)
+__device__ __forceinline__ double sum8(double (&v)[8], int lane) {
+#pragma unroll
+  for (int h = 4, o = 16; h; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
     }
-    w[e] = acc;
+  }
+  double s = v[0];
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
+}
+
+// partial[k * gridDim.x + blockIdx.x] = sum over the CTA's elements of conj(V_k) w, k < nk
+template <int E>
+__device__ void gs_partials(const double2* __restrict__ V, int64_t ldv, int nk, const double2 (&w)[E], int64_t e0,
+                            int64_t n, double2* __restrict__ partial, double2 (*red)[8]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int k0 = 0; k0 < nk; k0 += 8) {
+    double sx[8], sy[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      sx[k] = sy[k] = 0.0;
+      if (k0 + k < nk) {
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+          const int64_t e = e0 + x * kGsThreads;
+          if (e < n) {
+            const double2 a = V[(int64_t)(k0 + k) * ldv + e];
+            sx[k] = fma(a.x, w[x].x, fma(a.y, w[x].y, sx[k]));
+            sy[k] = fma(a.x, w[x].y, fma(-a.y, w[x].x, sy[k]));
+          }
+        }
+      }
+    }
+    const double tx = sum8(sx, lane), ty = sum8(sy, lane);
+    if ((lane & 3) == 0) red[warp][lane >> 2] = make_double2(tx, ty);
+    __syncthreads();
+    if (tid < 8 && k0 + tid < nk) {
+      double2 s = red[0][tid];
+#pragma unroll
+      for (int x = 1; x < kGsThreads / 32; ++x) {
+        s.x += red[x][tid].x;
+        s.y += red[x][tid].y;
+      }
+      partial[(int64_t)(k0 + tid) * gridDim.x + blockIdx.x] = s;
+    }
+    __syncthreads();
   }
 }
 
-// Lanczos scalars of iteration j: alpha_j = Re(h_j + g_j) (the two Gram-Schmidt passes),
-// beta_j = |w|, and the factor that normalises w into the next basis vector.
-__global__ void lanczos_scalars_kernel(int j, const double2* __restrict__ h, const double2* __restrict__ g,
-                                       const double2* __restrict__ nrm2, double* __restrict__ alpha,
-                                       double* __restrict__ beta, double* __restrict__ inv) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  alpha[j] = h[j].x + g[j].x;
-  const double b = sqrt(fmax(nrm2[0].x, 0.0));
-  beta[j] = b;
-  inv[0] = b > 1e-300 ? 1.0 / b : 0.0;
+// out[k] = sum of the nb partials of vector k, k < nk, by all warps of the CTA
+__device__ void gs_sums(const double2* __restrict__ partial, int nb, int nk, double2* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k0 = warp * 8; k0 < nk; k0 += kGsThreads / 32 * 8) {
+    double sx[8], sy[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      sx[k] = sy[k] = 0.0;
+      if (k0 + k < nk)
+        for (int x = lane; x < nb; x += 32) {
+          const double2 p = __ldcg(partial + (int64_t)(k0 + k) * nb + x);
+          sx[k] += p.x;
+          sy[k] += p.y;
+        }
+    }
+    const double tx = sum8(sx, lane), ty = sum8(sy, lane);
+    if ((lane & 3) == 0 && k0 + (lane >> 2) < nk) out[k0 + (lane >> 2)] = make_double2(tx, ty);
+  }
+  __syncthreads();
+}
+
+template <int E>
+__global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(const double2* __restrict__ V, int64_t ldv, int nk,
+                                                             const double2* __restrict__ w, int64_t n,
+                                                             double2* __restrict__ partial) {
+  __shared__ double2 red[kGsThreads / 32][8];
+  const int64_t e0 = (int64_t)blockIdx.x * kGsThreads * E + threadIdx.x;
+  double2 x[E];
+#pragma unroll
+  for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
+  gs_partials<E>(V, ldv, nk, x, e0, n, partial, red);
+}
+
+// w -= sum_k h_k V_k with h from pin, then the partials of the new w: its products with the basis
+// (last == 0) or its squared norm.  CTA 0 keeps h in hout.
+template <int E>
+__global__ void __launch_bounds__(kGsThreads) gs_update_kernel(const double2* __restrict__ V, int64_t ldv, int nk,
+                                                               double2* __restrict__ w, int64_t n,
+                                                               const double2* __restrict__ pin, int last,
+                                                               double2* __restrict__ pout, double2* __restrict__ hout) {
+  __shared__ double2 red[kGsThreads / 32][8];
+  __shared__ double2 h[kGsMaxK];
+  gs_sums(pin, gridDim.x, nk, h);
+  if (blockIdx.x == 0)
+    for (int k = threadIdx.x; k < nk; k += kGsThreads) hout[k] = h[k];
+  const int64_t e0 = (int64_t)blockIdx.x * kGsThreads * E + threadIdx.x;
+  double2 x[E];
+#pragma unroll
+  for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = 0; k < nk; ++k) {
+    const double2 c = h[k];
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      const int64_t e = e0 + i * kGsThreads;
+      if (e < n) {
+        const double2 v = V[(int64_t)k * ldv + e];
+        x[i].x = fma(-c.x, v.x, fma(c.y, v.y, x[i].x));
+        x[i].y = fma(-c.x, v.y, fma(-c.y, v.x, x[i].y));
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < E; ++i)
+    if (e0 + i * kGsThreads < n) w[e0 + i * kGsThreads] = x[i];
+  if (!last) {
+    gs_partials<E>(V, ldv, nk, x, e0, n, pout, red);
+    return;
+  }
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int i = 0; i < E; ++i) s.x = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, s.x));
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = red[0][0].x;
+    for (int k = 1; k < kGsThreads / 32; ++k) t += red[0][k].x;
+    pout[blockIdx.x] = make_double2(t, 0.0);
+  }
+}
+
+// alpha_j = Re(h_j + g_j) (the two passes), beta_j = |w|, V_{j+1} = w / |w|
+template <int E>
+__global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(double2* __restrict__ dst, const double2* __restrict__ w,
+                                                              int64_t n, const double2* __restrict__ pin, int j,
+                                                              const double2* __restrict__ h,
+                                                              const double2* __restrict__ g, double* __restrict__ alpha,
+                                                              double* __restrict__ beta) {
+  __shared__ double2 s[1];
+  gs_sums(pin, gridDim.x, 1, s);
+  const double b = sqrt(fmax(s[0].x, 0.0)), f = b > 1e-300 ? 1.0 / b : 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    alpha[j] = h[j].x + g[j].x;
+    beta[j] = b;
+  }
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    const int64_t e = ((int64_t)blockIdx.x * E + i) * kGsThreads + threadIdx.x;
+    if (e < n) {
+      const double2 v = w[e];
+      dst[e] = make_double2(f * v.x, f * v.y);
+    }
+  }
 }
 
 __global__ void inv_norm_kernel(const double2* __restrict__ nrm2, double* __restrict__ inv) {
@@ -399,7 +479,6 @@ __global__ void __launch_bounds__(kVecThreads) combine_kernel(double2* __restric
 // res[0] = eigenvalue, res[1] = residual estimate beta_{n-1} |y_{n-1}|, res[2] = basis size used.
 __global__ void tridiag_kernel(const double* __restrict__ alpha, const double* __restrict__ beta, int n,
                                double* __restrict__ y, double* __restrict__ res) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double scale = 0.0;
   for (int k = 0; k < n; ++k) scale = fmax(scale, fabs(alpha[k]) + (k + 1 < n ? fabs(beta[k]) : 0.0));
   scale = fmax(scale, 1e-300);
@@ -412,8 +491,11 @@ __global__ void tridiag_kernel(const double* __restrict__ alpha, const double* _
     lo = fmin(lo, alpha[k] - r);
     hi = fmax(hi, alpha[k] + r);
   }
-  for (int it = 0; it < 400 && hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) {
-    const double x = 0.5 * (lo + hi);
+  // 32 shifts a round, one a lane: the bracket shrinks 33-fold (a division costs 440 cycles here)
+  const int lane = threadIdx.x;
+  for (int it = 0; it < 80 && hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300; ++it) {
+    const double step = (hi - lo) * (1.0 / 33.0);
+    const double x = lo + step * (lane + 1);
     int below = 0;
     double q = 1.0;
     for (int k = 0; k < m; ++k) {
@@ -422,8 +504,14 @@ __global__ void tridiag_kernel(const double* __restrict__ alpha, const double* _
       if (q == 0.0) q = -1e-300;
       if (q < 0.0) ++below;
     }
-    if (below >= 1) hi = x; else lo = x;
+    const unsigned over = __ballot_sync(0xffffffffu, below >= 1);     // shifts above the lowest eigenvalue
+    const int first = over ? __ffs(over) - 1 : 32;
+    const double nlo = first > 0 ? lo + step * first : lo, nhi = first < 32 ? lo + step * (first + 1) : hi;
+    if (!(nlo > lo) && !(nhi < hi)) break;      // the bracket is at the spacing of doubles
+    lo = nlo;
+    hi = nhi;
   }
+  if (lane != 0) return;
   const double lam = 0.5 * (lo + hi);
   const double shift = lam - 1e-13 * scale;
   double dd[64], ll[64], x[64];
@@ -452,12 +540,19 @@ __global__ void tridiag_kernel(const double* __restrict__ alpha, const double* _
   res[2] = (double)m;
 }
 
-// exp(-i tau T) e_1 for the Lanczos tridiagonal T (alpha on the diagonal, beta next to it),
-// one warp: T's eigenpairs by cyclic Jacobi rotations (the symmetric Schur decomposition, each
-// rotation zeroing one off-diagonal pair, sweeps until the off-diagonal part is below 1e-15 of
-// the matrix), then y_j = sum_k Z[j][k] exp(-i tau lambda_k) Z[0][k].  The basis ends at the
-// first beta below 1e-13 of the matrix scale, as for the ground state.  res[0] = alpha_0
-// (<v0|H|v0>), res[1] = |beta_{m-1} y_{m-1}| (the estimate of the Krylov error), res[2] = m.
+// exp(-i tau T) e_1 for the Lanczos tridiagonal T (alpha on the diagonal, beta next to it), one warp.
+// The basis ends at the first beta below 1e-13 of the matrix scale, as for the ground state.
+// res[0] = alpha_0 (<v0|H|v0>), res[1] = |beta_{m-1} y_{m-1}| (the estimate of the Krylov error),
+// res[2] = m.  Two forms, by the span |tau| rho, rho the radius of T's spectrum around the middle c of
+// its Gershgorin interval:
+//   below kExpSeriesSpan: Taylor series of n = ceil(span) steps tau / n of T - c applied to the vector
+//   (two rows a lane), times exp(-i tau c).  A step takes about 20 terms until they are below rounding;
+//   n steps round like the phases tau lambda of the other form (n eps).
+//   above: y_j = sum_k Z[j][k] exp(-i tau lambda_k) Z[0][k], T's eigenpairs by cyclic Jacobi rotations
+//   (the symmetric Schur decomposition, each rotation zeroing one off-diagonal pair, sweeps until the
+//   off-diagonal part is below 1e-15 of the matrix).  Its 1700 rotations at 24 rows, each a chain of
+//   divisions and roots, take 2.9 ms whatever the span; a series step takes about 3 us.
+constexpr double kExpSeriesSpan = 256.0;
 constexpr int kExpMax = 40;
 __global__ void expm_tridiag_kernel(const double* __restrict__ alpha, const double* __restrict__ beta, int n,
                                     double tau, double2* __restrict__ y, double* __restrict__ res) {
@@ -471,6 +566,73 @@ __global__ void expm_tridiag_kernel(const double* __restrict__ alpha, const doub
   int m = n;
   for (int k = 0; k + 1 < n; ++k)
     if (beta[k] <= 1e-13 * scale) { m = k + 1; break; }
+  double lo = 1e300, hi = -1e300;
+  for (int k = 0; k < m; ++k) {
+    const double r = (k > 0 ? fabs(beta[k - 1]) : 0.0) + (k + 1 < m ? fabs(beta[k]) : 0.0);
+    lo = fmin(lo, alpha[k] - r);
+    hi = fmax(hi, alpha[k] + r);
+  }
+  const double mid = 0.5 * (lo + hi), span = fabs(tau) * 0.5 * (hi - lo);
+  if (span < kExpSeriesSpan) {
+    const int ns = (int)fmax(1.0, ceil(span));
+    const double t = tau / ns;
+    // rows lane and lane + 32: diagonal, the couplings above and below, scaled by the step
+    double dg[2], up[2], dn[2];
+    double2 v[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int k = lane + 32 * x;
+      dg[x] = k < m ? t * (alpha[k] - mid) : 0.0;
+      up[x] = k > 0 && k < m ? t * beta[k - 1] : 0.0;
+      dn[x] = k + 1 < m ? t * beta[k] : 0.0;
+      v[x] = make_double2(k == 0 ? 1.0 : 0.0, 0.0);
+    }
+    for (int s = 0; s < ns; ++s) {
+      double2 w[2] = {v[0], v[1]};
+      for (int k = 1; k <= 60; ++k) {
+        const double f = 1.0 / k;
+        double2 z[2];
+        // neighbours: row 31 meets row 32 across the two halves
+        const double ax = __shfl_up_sync(0xffffffffu, w[0].x, 1), ay = __shfl_up_sync(0xffffffffu, w[0].y, 1);
+        const double bx = __shfl_down_sync(0xffffffffu, w[0].x, 1), by = __shfl_down_sync(0xffffffffu, w[0].y, 1);
+        const double cx = __shfl_up_sync(0xffffffffu, w[1].x, 1), cy = __shfl_up_sync(0xffffffffu, w[1].y, 1);
+        const double ex = __shfl_down_sync(0xffffffffu, w[1].x, 1), ey = __shfl_down_sync(0xffffffffu, w[1].y, 1);
+        const double lx = __shfl_sync(0xffffffffu, w[0].x, 31), ly = __shfl_sync(0xffffffffu, w[0].y, 31);
+        const double hx = __shfl_sync(0xffffffffu, w[1].x, 0), hy = __shfl_sync(0xffffffffu, w[1].y, 0);
+        const bool top = lane == 0, end = lane == 31;
+        // (T - c) t w; times -i / k
+        const double r0x = fma(dg[0], w[0].x, fma(up[0], top ? 0.0 : ax, dn[0] * (end ? hx : bx)));
+        const double r0y = fma(dg[0], w[0].y, fma(up[0], top ? 0.0 : ay, dn[0] * (end ? hy : by)));
+        const double r1x = fma(dg[1], w[1].x, fma(up[1], top ? lx : cx, dn[1] * (end ? 0.0 : ex)));
+        const double r1y = fma(dg[1], w[1].y, fma(up[1], top ? ly : cy, dn[1] * (end ? 0.0 : ey)));
+        z[0] = make_double2(f * r0y, -f * r0x);
+        z[1] = make_double2(f * r1y, -f * r1x);
+        bool small = true;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          w[x] = z[x];
+          v[x].x += z[x].x;
+          v[x].y += z[x].y;
+          small = small && fabs(z[x].x) < 1e-18 && fabs(z[x].y) < 1e-18;      // |v| = 1
+        }
+        if (__all_sync(0xffffffffu, small)) break;
+      }
+    }
+    double sv, cv;
+    sincos(-tau * mid, &sv, &cv);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int k = lane + 32 * x;
+      const double2 o = make_double2(fma(cv, v[x].x, -sv * v[x].y), fma(cv, v[x].y, sv * v[x].x));
+      if (k < n) y[k] = o;
+      if (k == m - 1) res[1] = m < n ? 0.0 : fabs(beta[m - 1]) * sqrt(o.x * o.x + o.y * o.y);
+    }
+    if (lane == 0) {
+      res[0] = alpha[0];
+      res[2] = (double)m;
+    }
+    return;
+  }
   for (int k = lane; k < m; k += 32)
     for (int j = 0; j < m; ++j) {
       A[k][j] = (j == k) ? alpha[k] : (j == k + 1 ? beta[k] : (j + 1 == k ? beta[j] : 0.0));
@@ -974,7 +1136,8 @@ struct Dmrg {
   struct KBuf {
     int64_t dim = 0, ldv = 0;
     int K = 0, nb = 1, vb = 1;
-    double2 *V = nullptr, *w = nullptr, *tv = nullptr, *part = nullptr, *hdots = nullptr, *gdots = nullptr,
+    int ge = 1, gb = 1;      // Gram-Schmidt: elements a thread, CTAs
+    double2 *V = nullptr, *w = nullptr, *tv = nullptr, *part = nullptr, *part2 = nullptr, *hdots = nullptr, *gdots = nullptr,
             *nrm = nullptr, *yc = nullptr;
     double *alpha = nullptr, *beta = nullptr, *inv = nullptr, *yv = nullptr, *res = nullptr, *scl = nullptr,
            *one = nullptr;
@@ -987,14 +1150,21 @@ struct Dmrg {
     b.ldv = (dim + 31) / 32 * 32;
     b.nb = std::max(1, std::min(kDotBlocks, (int)((dim + kVecThreads - 1) / kVecThreads)));
     b.vb = vec_blocks(dim);
+    // the fewest elements a thread that leave at most two CTAs an SM: FP64 issue bounds a chunk, so
+    // short vectors want every SM, and the sums of the partials grow with the number of CTAs
+    b.ge = 1;
+    while (b.ge < 8 && dim > (int64_t)kDotBlocks * kGsThreads * b.ge) b.ge *= 2;
+    b.gb = (int)((dim + (int64_t)kGsThreads * b.ge - 1) / ((int64_t)kGsThreads * b.ge));
+    const int64_t npart = (int64_t)(b.K + 1) * std::max(b.nb, b.gb);
     const int64_t o_w = (int64_t)(b.K + 1) * b.ldv, o_t = o_w + b.ldv, o_part = o_t + b.ldv;
-    const int64_t o_sc = o_part + (int64_t)(b.K + 1) * b.nb;
+    const int64_t o_sc = o_part + 2 * npart;
     const int64_t nsc = 4 * 72 + 64 + 64;
     if (lz.reserve((size_t)(o_sc + nsc) * 16) != cudaSuccess) return fail(MPS_ENOMEM, "DMRG Krylov vectors");
     b.V = reinterpret_cast<double2*>(lz.p);
     b.w = b.V + o_w;
     b.tv = b.V + o_t;
     b.part = b.V + o_part;
+    b.part2 = b.part + npart;
     b.hdots = b.V + o_sc;            // 72
     b.gdots = b.hdots + 72;          // 72
     b.nrm = b.gdots + 72;            // 4
@@ -1008,6 +1178,20 @@ struct Dmrg {
     b.one = b.scl + 2;               // 2
     if (cudaMemsetAsync(b.V, 0, (size_t)(o_sc + nsc) * 16, st) != cudaSuccess) return fail(MPS_ECUDA, "DMRG memset");
     return MPS_OK;
+  }
+
+  // Step j of the Lanczos recursion after the product: classical Gram-Schmidt of w against V_0..j,
+  // twice, and V_{j+1} = w / |w|.
+  template <int E>
+  void gram_schmidt(KBuf& b, int j) {
+    const int nk = j + 1;
+    const int64_t dim = b.dim, ldv = b.ldv;
+    gs_dots_kernel<E><<<b.gb, kGsThreads, 0, st>>>(b.V, ldv, nk, b.w, dim, b.part);
+    gs_update_kernel<E><<<b.gb, kGsThreads, 0, st>>>(b.V, ldv, nk, b.w, dim, b.part, 0, b.part2, b.hdots);
+    gs_update_kernel<E><<<b.gb, kGsThreads, 0, st>>>(b.V, ldv, nk, b.w, dim, b.part2, 1, b.part, b.gdots);
+    gs_scale_kernel<E><<<b.gb, kGsThreads, 0, st>>>(b.V + (int64_t)nk * ldv, b.w, dim, b.part, j, b.hdots, b.gdots,
+                                                   b.alpha, b.beta);
+    for (int x = 0; x < 4; ++x) count_launch();
   }
 
   // mode 0: the lowest eigenpair of H by Lanczos with full reorthogonalisation, restarted from
@@ -1050,30 +1234,11 @@ struct Dmrg {
         matvecs++;
         if (e != cudaSuccess) break;
         e = timed(2, 16.0 * dim * (j + 1) * 4, [&] {
-          cudaError_t e2 = dots(V, j + 1, b.w, b.hdots);
-          if (e2 == cudaSuccess) {
-            count_launch();
-            subtract_kernel<<<b.vb, kVecThreads, 0, st>>>(b.w, V, ldv, j + 1, b.hdots, dim);
-            e2 = cudaGetLastError();
-          }
-          if (e2 == cudaSuccess) e2 = dots(V, j + 1, b.w, b.gdots);
-          if (e2 == cudaSuccess) {
-            count_launch();
-            subtract_kernel<<<b.vb, kVecThreads, 0, st>>>(b.w, V, ldv, j + 1, b.gdots, dim);
-            e2 = cudaGetLastError();
-          }
-          if (e2 == cudaSuccess) e2 = dots(b.w, 1, b.w, b.nrm);
-          if (e2 == cudaSuccess) {
-            count_launch();
-            lanczos_scalars_kernel<<<1, 32, 0, st>>>(j, b.hdots, b.gdots, b.nrm, b.alpha, b.beta, b.inv);
-            e2 = cudaGetLastError();
-          }
-          if (e2 == cudaSuccess) {
-            count_launch();
-            scale_kernel<<<b.vb, kVecThreads, 0, st>>>(V + (int64_t)(j + 1) * ldv, b.w, b.inv, dim);
-            e2 = cudaGetLastError();
-          }
-          return e2;
+          if (b.ge == 1) gram_schmidt<1>(b, j);
+          else if (b.ge == 2) gram_schmidt<2>(b, j);
+          else if (b.ge == 4) gram_schmidt<4>(b, j);
+          else gram_schmidt<8>(b, j);
+          return cudaGetLastError();
         });
       }
       return e;
