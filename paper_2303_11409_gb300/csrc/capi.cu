@@ -356,7 +356,9 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
         gemm_tiles_bound += (int64_t)((Dl + kTile - 1) / kTile) * ((k + kTile - 1) / kTile);
       }
     }
-  // Jacobi scratch: one-CTA sectors live in shared memory, cluster sectors in L2
+  // Jacobi scratch: one-CTA sectors live in shared memory, cluster sectors in L2.  Teams of CTAs wait for
+  // one another across launches of other streams, which a captured phase cannot express.
+  const bool teams = !owner->graphs;
   SvdScratchLayout JL;
   {
     std::vector<int> sm, sn;
@@ -367,7 +369,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
         sn.push_back(e.cols);
         exact.push_back(reqs[u].h->precision != MPS_FP64);
       }
-    svd_layout((int)sm.size(), sm.data(), sn.data(), JL, -1, exact.data());
+    svd_layout((int)sm.size(), sm.data(), sn.data(), JL, -1, exact.data(), teams);
   }
   const int64_t jac_base = ws;
   ws = a256(ws + JL.total);
@@ -713,7 +715,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   std::vector<std::vector<SvdGroup>> svd_groups(n_cand);
   for (int c = 0; c < n_cand; ++c) {
     const SvdTune tune = n_cand > 1 ? svd_tune_candidate(c) : (chosen >= 0 ? svd_tune_candidate(chosen) : SvdTune());
-    CUDA_OR_FAIL(owner, svd_group(svd_sorted[c], svd_groups[c], tune));
+    CUDA_OR_FAIL(owner, svd_group(svd_sorted[c], svd_groups[c], tune, teams));
   }
 
   // ---- descriptors into the staging buffer (uploaded in one copy) ---------------------
@@ -919,7 +921,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       std::vector<SvdGroup> sub_groups;
       // the tile shape the first run used for these sectors
       const SvdTune tune = n_cand > 1 ? svd_tune_candidate(c_used) : (chosen >= 0 ? svd_tune_candidate(chosen) : SvdTune());
-      CUDA_OR_FAIL(owner, svd_group(sub, sub_groups, tune));
+      CUDA_OR_FAIL(owner, svd_group(sub, sub_groups, tune, teams));
       // the phase-1 SVD descriptors are no longer read (the stream is synchronised): reuse them
       char* hsrc = (char*)owner->pin_in.p + o_svd[c_used];
       std::memcpy(hsrc, sub.data(), sizeof(SvdSector) * sub.size());
@@ -956,6 +958,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     int bmax = 0;
     int64_t bsum = 0;
     for (int k = 0; k < n_sec_total; ++k) {
+      if (sstat[k] < -1) return fail(owner, MPS_ETIMEOUT, "a bounded wait inside the sector SVD expired");
       bmax = std::max(bmax, sstat[k]);
       bsum += std::max(sstat[k], 0);
     }

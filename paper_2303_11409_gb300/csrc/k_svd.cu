@@ -55,6 +55,7 @@
 // test; at most two rsqrt, one sqrt and one division per rotation; column norms tracked through the
 // exact 2x2 relations within a sweep).
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <atomic>
 #include <mutex>
@@ -68,11 +69,16 @@ namespace {
 constexpr double kEps = 2.220446049250313e-16;
 constexpr int kMaxCached = 16;          // rows cached in registers per lane (n <= 512)
 constexpr int kMaxCluster = 16;
+constexpr int kMaxTeam = 304;           // CTAs of a team: 2 on each of 152 SMs
+constexpr int kSvdTeamExpired = -2;     // a sector's status when a team's wait ran out
 constexpr int kMaxWarps = 16;
 constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps per CTA, 2 CTAs per SM
 // smallest min(m, n) of a refined sector: below it the one-CTA kernel's few sweeps cost less than
 // the dozen launches of the refinement (chi = 64 layers of 31-35 columns, 1.4 ms)
 constexpr int kRefineMinK = 48;
+// rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
+// a row's dependent FMAs 128)
+constexpr int kAhead = 8;
 constexpr int kMaxStaged = 16;          // block pairs staged at once by one block-Jacobi CTA
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -526,8 +532,14 @@ struct JacobiBlocks {
   double2* sm;   // 2 * gs * bsmax columns of n complex (shared memory)
   double* smn;   // 2 * gs * bsmax norms (shared memory)
   int bsmax;
-  int g;         // block pairs per CTA and round
+  int g;         // a round has cl0 * g block pairs; CTA `rank` takes the pairs rank, rank + nctas, ...
   int gs;        // block pairs staged at once
+  int cl0;       // the cluster size that fixes the block ordering (nctas itself on a cluster)
+  // how many block pairs a cluster's CTA stages together with pair p
+  __device__ int staged_with(int p) const {
+    const int q = p / cl0;
+    return min(gs, g - q / gs * gs);
+  }
   template <class Sync>
   __device__ int operator()(double2* W, int n, int ld, int K, const Work& w, int rank, int nctas, Sync sync,
                             double tol2, double floor2, int max_sweeps, bool& converged) const {
@@ -542,7 +554,8 @@ struct JacobiBlocks {
     __shared__ int s_len[2 * kMaxStaged];   // its width (0: slot unused)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int worker = rank * nwarps + warp, workers = nctas * nwarps;
-    const int nb = 2 * nctas * g;
+    const int nb = 2 * cl0 * g, own = (cl0 * g - rank + nctas - 1) / nctas;
+    const bool team = nctas != cl0;   // one pair at a time, in the lane groups the cluster would use
     int sweep = 0;
     converged = K < 2;
     for (; !converged && sweep < max_sweeps; ++sweep) {
@@ -562,8 +575,9 @@ struct JacobiBlocks {
       if (tid == 0) s_rot = 0;
       bool rot = false;
       for (int r = 0; r < nb - 1; ++r) {
-        for (int c0 = 0; c0 < g; c0 += gs) {        // chunks of gs block pairs of this CTA
-          const int ns = min(gs, g - c0);
+        for (int c0 = 0; c0 < own; c0 += team ? 1 : gs) {        // chunks of gs block pairs of this CTA
+          const int ns = team ? 1 : min(gs, g - c0);
+          const int ns_ref = team ? staged_with(rank + c0 * nctas) : ns;
           if (tid < 2 * gs) {
             const int j = tid >> 1;
             int col = 0, len = 0;
@@ -598,7 +612,7 @@ struct JacobiBlocks {
           if (r == 0) {   // pairs inside each staged block, round-robin within the block
             const int mpb = bsmax + (bsmax & 1);
             const int P = 2 * ns * (mpb / 2);
-            const int G = group_width_mw(P, n, nwarps), slots = group_slots(G, nwarps), slot = group_slot(G);
+            const int G = group_width_mw(2 * ns_ref * (mpb / 2), n, nwarps), slots = group_slots(G, nwarps), slot = group_slot(G);
             for (int rr = 0; rr < mpb - 1; ++rr) {
               for (int base = 0; base < P; base += slots) {
                 const int k = base + slot, j = k / (mpb / 2);
@@ -620,7 +634,7 @@ struct JacobiBlocks {
           }
           {   // cross pairs: block slots 2j and 2j + 1, the smaller block shifted against the larger
             const int P = ns * bsmax;
-            const int G = group_width_mw(P, n, nwarps), slots = group_slots(G, nwarps), slot = group_slot(G);
+            const int G = group_width_mw(ns_ref * bsmax, n, nwarps), slots = group_slots(G, nwarps), slot = group_slot(G);
             for (int t = 0; t < bsmax; ++t) {
               for (int base = 0; base < P; base += slots) {
                 const int k = base + slot, j = k / bsmax, i = k % bsmax;
@@ -755,7 +769,11 @@ __device__ __forceinline__ int group_width32(int P, int R, int nwarps) {
 struct JacobiBlocks32 {
   float2* sm;
   float* smn;
-  int bsmax, g, gs;
+  int bsmax, g, gs, cl0;      // as in JacobiBlocks
+  __device__ int staged_with(int p) const {
+    const int q = p / cl0;
+    return min(gs, g - q / gs * gs);
+  }
   template <class Sync>
   __device__ int operator()(float2* F, int R, int Rr, int ld, int K, float* nrm, int* flags, int rank, int nctas,
                             Sync sync, float tol, float floor2, int max_sweeps, bool& converged) const {
@@ -768,7 +786,8 @@ struct JacobiBlocks32 {
     __syncthreads();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int worker = rank * nwarps + warp, workers = nctas * nwarps;
-    const int nb = 2 * nctas * g;
+    const int nb = 2 * cl0 * g, own = (cl0 * g - rank + nctas - 1) / nctas;
+    const bool team = nctas != cl0;
     int sweep = 0;
     converged = K < 2;
     for (; !converged && sweep < max_sweeps; ++sweep) {
@@ -786,8 +805,9 @@ struct JacobiBlocks32 {
       if (tid == 0) s_rot32 = 0;
       bool rot = false;
       for (int r = 0; r < nb - 1; ++r) {
-        for (int c0 = 0; c0 < g; c0 += gs) {
-          const int ns = min(gs, g - c0);
+        for (int c0 = 0; c0 < own; c0 += team ? 1 : gs) {
+          const int ns = team ? 1 : min(gs, g - c0);
+          const int ns_ref = team ? staged_with(rank + c0 * nctas) : ns;
           if (tid < 2 * gs) {
             const int j = tid >> 1;
             int col = 0, len = 0;
@@ -822,7 +842,7 @@ struct JacobiBlocks32 {
           if (r == 0) {
             const int mpb = bsmax + (bsmax & 1);
             const int P = 2 * ns * (mpb / 2);
-            const int G = group_width32(P, R, nwarps), per = 32 / G, slot = warp * per + lane / G;
+            const int G = group_width32(2 * ns_ref * (mpb / 2), R, nwarps), per = 32 / G, slot = warp * per + lane / G;
             for (int rr = 0; rr < mpb - 1; ++rr) {
               for (int base = 0; base < P; base += nwarps * per) {
                 const int k = base + slot, j = k / (mpb / 2);
@@ -840,7 +860,7 @@ struct JacobiBlocks32 {
           }
           {
             const int P = ns * bsmax;
-            const int G = group_width32(P, R, nwarps), per = 32 / G, slot = warp * per + lane / G;
+            const int G = group_width32(ns_ref * bsmax, R, nwarps), per = 32 / G, slot = warp * per + lane / G;
             for (int t = 0; t < bsmax; ++t) {
               for (int base = 0; base < P; base += nwarps * per) {
                 const int k = base + slot, j = k / bsmax, i = k % bsmax;
@@ -1368,12 +1388,28 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
       Mem::st(w.pi + rank, bi);
     }
     sync();
-    bv = Mem::ld(w.pv);
-    bi = Mem::ld(w.pi);
-    for (int x = 1; x < nctas; ++x) {
-      const double v = Mem::ld(w.pv + x);
-      const int ix = Mem::ld(w.pi + x);
-      if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+    if (nctas <= kMaxCluster) {
+      bv = Mem::ld(w.pv);
+      bi = Mem::ld(w.pi);
+      for (int x = 1; x < nctas; ++x) {
+        const double v = Mem::ld(w.pv + x);
+        const int ix = Mem::ld(w.pi + x);
+        if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+      }
+    } else {
+      bv = -1.0;
+      bi = n;
+      for (int x = lane; x < nctas; x += 32) {
+        const double v = Mem::ld(w.pv + x);
+        const int ix = Mem::ld(w.pi + x);
+        if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+      }
     }
     const int p = (bi < n) ? bi : k;
     if (p != k) {
@@ -1417,45 +1453,64 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
       if (lane == 0) Mem::st(w.scal, uu > 0.0 ? 2.0 / uu : 0.0);
     }
     sync();
-    // trailing update W[k:, j] -= (2/u^dag u) u (u^dag W[k:, j]) for j > k, 32 columns x 8 row chunks per CTA
+    // trailing update W[k:, j] -= (2/u^dag u) u (u^dag W[k:, j]) for j > k: a CTA takes tiles of tc columns,
+    // each column's dot product in nwarps interleaved row chunks (summed in order whatever the tile
+    // width).  32 columns fill the CTA's warps; with more CTAs than such tiles narrower ones put the
+    // chunks of several columns into a warp, so that every CTA has FP64 work.
+    constexpr int ahead = Mem::kCache ? kAhead : 1;      // shared memory answers at once
     const double sc = Mem::ld(w.scal);
     const int ncols = n - k - 1;
-    const int ntiles = (ncols + 31) / 32;
+    int tc = 32;
+    if constexpr (Mem::kCache)
+      while (nctas > kMaxCluster && tc > 8 && (ncols + tc / 2 - 1) / (tc / 2) <= nctas) tc >>= 1;
+    const int ntiles = (ncols + tc - 1) / tc;
+    const int tcol = tid % tc, chunk = tid / tc;      // chunks beyond nwarps have no rows in the dot product
     if (sc != 0.0) {
       for (int tile = rank; tile < ntiles; tile += nctas) {
-        const int j = k + 1 + tile * 32 + lane;
+        const int j = k + 1 + tile * tc + tcol;
         double pr = 0.0, pim = 0.0;
-        if (j < n) {
-          for (int i = k + warp; i < m; i += nwarps) {
+        if (j < n && chunk < nwarps) {
+#pragma unroll ahead
+          for (int i = k + chunk; i < m; i += nwarps) {
             const double2 ui = Mem::ld(w.u + i);
             const double2 x = Mem::ld(W + (int64_t)i * ld + j);
             pr = fma(ui.x, x.x, fma(ui.y, x.y, pr));      // conj(u_i) x
             pim = fma(ui.x, x.y, fma(-ui.y, x.x, pim));
           }
         }
-        red_d[warp][lane] = pr;
+        if (chunk < nwarps) red_d[chunk][tcol] = pr;
         __syncthreads();
         double wr = 0.0;
-        for (int x = 0; x < nwarps; ++x) wr += red_d[x][lane];
+        for (int x = 0; x < nwarps; ++x) wr += red_d[x][tcol];
         __syncthreads();
-        red_d[warp][lane] = pim;
+        if (chunk < nwarps) red_d[chunk][tcol] = pim;
         __syncthreads();
         double wi = 0.0;
-        for (int x = 0; x < nwarps; ++x) wi += red_d[x][lane];
+        for (int x = 0; x < nwarps; ++x) wi += red_d[x][tcol];
         __syncthreads();
         wr *= sc;
         wi *= sc;
         if (j < n) {
-          for (int i = k + warp; i < m; i += nwarps) {
-            const double2 ui = Mem::ld(w.u + i);
-            double2 x = Mem::ld(W + (int64_t)i * ld + j);
-            x.x -= ui.x * wr - ui.y * wi;
-            x.y -= ui.x * wi + ui.y * wr;
-            Mem::st(W + (int64_t)i * ld + j, x);
+          const int step = (int)blockDim.x / tc;
+          for (int i0 = k + chunk; i0 < m; i0 += ahead * step) {
+            double2 ui[ahead], x[ahead];
+#pragma unroll
+            for (int a = 0; a < ahead; ++a)
+              if (i0 + a * step < m) {
+                ui[a] = Mem::ld(w.u + i0 + a * step);
+                x[a] = Mem::ld(W + (int64_t)(i0 + a * step) * ld + j);
+              }
+#pragma unroll
+            for (int a = 0; a < ahead; ++a)
+              if (i0 + a * step < m) {
+                x[a].x -= ui[a].x * wr - ui[a].y * wi;
+                x[a].y -= ui[a].x * wi + ui[a].y * wr;
+                Mem::st(W + (int64_t)(i0 + a * step) * ld + j, x[a]);
+              }
           }
         }
         __syncthreads();
-        if (warp == 0 && j < n) {       // downdate the partial norm, recompute on cancellation
+        if (chunk == 0 && j < n) {       // downdate the partial norm, recompute on cancellation
           const double2 r = Mem::ld(W + (int64_t)k * ld + j);
           double v = Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y);
           if (v <= 1.4901161193847656e-8 * Mem::ld(w.nu0 + j)) {
@@ -1471,8 +1526,8 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
       }
     } else {
       for (int tile = rank; tile < ntiles; tile += nctas) {
-        const int j = k + 1 + tile * 32 + lane;
-        if (warp == 0 && j < n) {
+        const int j = k + 1 + tile * tc + tcol;
+        if (chunk == 0 && j < n) {
           const double2 r = Mem::ld(W + (int64_t)k * ld + j);
           Mem::st(w.nu + j, fmax(Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y), 0.0));
         }
@@ -1690,6 +1745,41 @@ struct ClusterSync {
   __device__ void operator()() const { cluster_sync_all(); }
 };
 
+// The barrier of a team: CTAs of one cooperative launch (all resident) that share a sector.  bar[0] counts
+// arrivals, zero at the launch.  The wait is bounded (about 20 s): a CTA whose wait expires marks the
+// sector and leaves; no bulk copy is in flight at a barrier, so nothing outlives it.
+struct TeamSync {
+  unsigned* bar;
+  int* status;
+  unsigned size;
+  unsigned* target;      // shared memory, thread 0's: arrivals that complete the present barrier
+  __device__ void operator()() const {
+    __shared__ int s_expired;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int expired = 0;
+      *target += size;
+      asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
+      atomicAdd(bar, 1u);
+      const long long t0 = clock64();
+      for (;;) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(bar) : "memory");
+        if ((int)(v - *target) >= 0) break;
+        if (clock64() - t0 > 40000000000LL) {
+          expired = 1;
+          break;
+        }
+      }
+      asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
+      s_expired = expired;
+      if (expired) *status = kSvdTeamExpired;
+    }
+    __syncthreads();
+    if (s_expired) asm volatile("exit;\n");
+  }
+};
+
 // shared-memory layout of the one-CTA kernel (offsets in bytes)
 struct SmemLayout {
   int64_t W, u, nu, nu0, perm, nrm, ord, flags, pv, pi, scal, total;
@@ -1746,7 +1836,7 @@ __device__ __forceinline__ Work cluster_work(const SvdSector& S) {
   w.flags = S.flags;
   w.pv = S.pivv;
   w.pi = S.flags + kJacobiMaxSweeps + 1;
-  w.scal = S.pivv + kMaxCluster;
+  w.scal = S.pivv + (S.teambar ? kMaxTeam : kMaxCluster);
   return w;
 }
 
@@ -1757,28 +1847,54 @@ __global__ void __launch_bounds__(kSvdThreads) jacobi_cluster_kernel(const SvdSe
   svd_sector<L2Mem>(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, JacobiRoundRobin<L2Mem>{});
 }
 
-__global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(const SvdSector* __restrict__ secs,
-                                                                                int cluster, int max_sweeps) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int rank = (int)cluster_rank();
-  const SvdSector S = secs[blockIdx.x / cluster];
+// The block-Jacobi SVD of one sector by nctas CTAs in the ordering of a cluster of cl0.
+template <class Sync>
+__device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* smem, int rank, int nctas, int cl0,
+                                           Sync sync, int max_sweeps) {
   const int K = min(S.m, S.n);
   JacobiBlocks jb;
   jb.g = S.groups;
   jb.gs = S.staged;
-  jb.bsmax = (K + 2 * cluster * jb.g - 1) / (2 * cluster * jb.g);
-  jb.sm = reinterpret_cast<double2*>(smem_raw);
-  jb.smn = reinterpret_cast<double*>(smem_raw + 16LL * 2 * jb.gs * jb.bsmax * (S.wide ? K : S.n));
+  jb.cl0 = cl0;
+  jb.bsmax = (K + 2 * cl0 * jb.g - 1) / (2 * cl0 * jb.g);
+  jb.sm = reinterpret_cast<double2*>(smem);
+  jb.smn = reinterpret_cast<double*>(smem + 16LL * 2 * jb.gs * jb.bsmax * (S.wide ? K : S.n));
   // the FP32 sweeps of a mixed-precision sector stage columns of jlen + K <= 2 jlen FP32
   // complex values in the same area
   JacobiBlocks32 j32;
   j32.g = jb.g;
   j32.gs = jb.gs;
+  j32.cl0 = cl0;
   j32.bsmax = jb.bsmax;
-  j32.sm = reinterpret_cast<float2*>(smem_raw);
-  j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * jb.gs * jb.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
+  j32.sm = reinterpret_cast<float2*>(smem);
+  j32.smn = reinterpret_cast<float*>(smem + 8LL * 2 * jb.gs * jb.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
+  svd_sector<L2Mem>(S, cluster_work(S), rank, nctas, sync, max_sweeps, jb, j32);
+}
+
+__global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(const SvdSector* __restrict__ secs,
+                                                                                int cluster, int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const SvdSector S = secs[blockIdx.x / cluster];
   if (S.F && S.rstate[1] == 0 && S.rstate[2] > 0) return;   // settled by the refinement
-  svd_sector<L2Mem>(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, jb, j32);
+  svd_blocks(S, smem_raw, (int)cluster_rank(), cluster, cluster, ClusterSync{}, max_sweeps);
+}
+
+// The same for batches with few large sectors: one cooperative launch, in which a sector has a team
+// of S.team_size CTAs (those from S.team_first) instead of a cluster of at most 8.  The block ordering and
+// every sum stay those of the cluster, so the results are the same bits; only more SMs share a
+// round's block pairs, a column's trailing update and the products.  A chi = 2048 update whose 796 x 796
+// sector kept 8 SMs busy for 1.23 s takes 165 ms (a team of 104), three updates at chi = 1024 297 -> 125 ms;
+// there the FP64 pipes of the whole chip are the bound.
+__global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const SvdSector* __restrict__ secs, int count,
+                                                                       int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int k = 0;
+  while (k + 1 < count && (int)blockIdx.x >= secs[k + 1].team_first) ++k;
+  const SvdSector S = secs[k];
+  __shared__ unsigned s_target;
+  if (threadIdx.x == 0) s_target = 0;
+  svd_blocks(S, smem_raw, (int)blockIdx.x - S.team_first, S.team_size, S.team_cl0,
+             TeamSync{S.teambar, S.status, (unsigned)S.team_size, &s_target}, max_sweeps);
 }
 
 __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSector* __restrict__ secs, int cluster,
@@ -1791,6 +1907,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSe
   JacobiBlocks32 j32;
   j32.g = S.groups;
   j32.gs = S.staged;
+  j32.cl0 = cluster;
   j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
   j32.sm = reinterpret_cast<float2*>(smem_raw);
   j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
@@ -1836,6 +1953,8 @@ cudaError_t set_attrs(int* big_out) {
                              kBlockSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(jacobi_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
   if (e != cudaSuccess) return e;
   // clusters of 16 CTAs are non-portable: use them only where the device can place them
   int big = 8;
@@ -1865,6 +1984,35 @@ cudaError_t set_attrs(int* big_out) {
   return cudaSuccess;
 }
 
+// One cooperative launch of a group of teams.  Two such launches on different streams must not share
+// the chip (each could hold SMs that the other's missing CTAs wait for), so every one waits for the
+// previous one of its device.
+cudaError_t launch_teams(const SvdSector* d, const SvdGroup& g, int max_sweeps, cudaStream_t st) {
+  static std::mutex mu;
+  static cudaEvent_t last[kMaxDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!last[dev]) e = cudaEventCreateWithFlags(&last[dev], cudaEventDisableTiming);
+  else e = cudaStreamWaitEvent(st, last[dev], 0);
+  if (e == cudaSuccess) e = cudaMemsetAsync(g.bar0, 0, (char*)g.bar1 - (char*)g.bar0 + 64, st);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.ctas);
+  cfg.blockDim = dim3(kBlockThreads);
+  cfg.dynamicSmemBytes = g.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, jacobi_team_kernel, d, g.count, max_sweeps);
+  return e == cudaSuccess ? cudaEventRecord(last[dev], st) : e;
+}
+
 // fallback: the FP64 sweeps of a refined group, for the sectors the refinement left
 cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_sweeps, cudaStream_t st,
                          bool fallback = false) {
@@ -1887,6 +2035,7 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
+  if (g.kind == kSvdTeam) return launch_teams(d, g, max_sweeps, st);
   if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps);
   if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, g.cl, max_sweeps);
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
@@ -1894,7 +2043,69 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
 
 }  // namespace
 
-cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& groups, const SvdTune& tune) {
+// Teams instead of clusters for the block-Jacobi sectors of a batch whose largest sectors would
+// run on long after the others.  A sector's work in CTA-seconds, fitted to measured sectors from
+// 1551 x 47 to 796 x 796: 13.5 K^3 + 6 m n K, 9.2 m n K when wide (units of 1e-9).  Clusters end after the
+// largest work / cluster size; teams are sized so that all sectors end together, at most one CTA per
+// block pair of a round.  They are formed when that is less than 2/3 of the clusters' time: teams pay for
+// barriers across the chip (2 us), and with hundreds of large sectors the clusters keep every SM busy.
+cudaError_t form_teams(std::vector<SvdSector>& secs, std::vector<std::pair<int, int>>& key,
+                       const std::vector<int64_t>& smem) {
+  std::vector<size_t> who;
+  int64_t need = 0;
+  double total = 0.0, longest = 0.0;
+  std::vector<double> work(secs.size(), 0.0);
+  for (size_t k = 0; k < secs.size(); ++k) {
+    if (key[k].first != kSvdClusterBlock || secs[k].F || !secs[k].teambar) continue;
+    const double m = secs[k].m, n = secs[k].n, K = std::min(m, n);
+    work[k] = 13.5 * K * K * K + (secs[k].wide ? 9.2 : 6.0) * m * n * K;
+    who.push_back(k);
+    need = std::max(need, smem[k]);
+    total += work[k];
+    longest = std::max(longest, work[k] / key[k].second);
+  }
+  if (who.empty()) return cudaSuccess;
+  int dev = 0, sms = 0, coop = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_team_kernel, kBlockThreads, (size_t)need);
+  if (e != cudaSuccess) return e;
+  const int cap = std::min(kMaxTeam, sms * per_sm);
+  if (!coop || (int)who.size() > cap) return cudaSuccess;
+  // the fewest CTAs that end sector k by time T (or one per block pair): the pairs of a round are dealt
+  // out in whole turns, so only sizes that change the number of turns count
+  auto size_for = [&](size_t k, double T) {
+    const int pairs = key[k].second * secs[k].groups;
+    const int turns = (int)std::max(1.0, std::min((double)pairs, std::floor(T * pairs / work[k])));
+    return std::min(kMaxTeam, (pairs + turns - 1) / turns);
+  };
+  auto ctas = [&](double T) {
+    int64_t s = 0;
+    for (size_t k : who) s += size_for(k, T);
+    return s;
+  };
+  double lo = total / cap, hi = total;
+  while (ctas(lo) > cap && hi > 1.02 * lo) {
+    const double T = 0.5 * (lo + hi);
+    if (hi < 1.04 * lo) break;
+    if (ctas(T) > cap) lo = T; else hi = T;
+  }
+  const double T = ctas(lo) <= cap ? lo : hi;
+  if (ctas(T) > cap) return cudaSuccess;
+  double ends = 0.0;
+  for (size_t k : who) ends = std::max(ends, work[k] / size_for(k, T));
+  if (ends > 2.0 / 3.0 * longest) return cudaSuccess;
+  for (size_t k : who) {
+    secs[k].team_size = size_for(k, T);
+    secs[k].team_cl0 = key[k].second;
+    key[k] = {kSvdTeam, 1};
+  }
+  return cudaSuccess;
+}
+
+cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& groups, const SvdTune& tune, bool team) {
   int big_cluster = 0;
   cudaError_t e = set_attrs(&big_cluster);
   if (e != cudaSuccess) return e;
@@ -1955,6 +2166,7 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
       secs[k].F = nullptr;        // the round-robin kernel runs in FP64 alone
     }
   }
+  if (team && (e = form_teams(secs, key, smem)) != cudaSuccess) return e;
   // group by (kind, cluster size); the most expensive sectors first inside a group
   std::vector<size_t> idx(secs.size());
   for (size_t k = 0; k < idx.size(); ++k) idx[k] = k;
@@ -1972,7 +2184,7 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
   for (size_t t = 0; t < idx.size(); ++t) {
     const size_t k = idx[t];
     if (groups.empty() || groups.back().kind != key[k].first || groups.back().cl != key[k].second) {
-      SvdGroup g;
+      SvdGroup g = {};
       g.kind = key[k].first;
       g.cl = key[k].second;
       g.smem = 0;
@@ -1985,6 +2197,13 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
     groups.back().smem = std::max<int>(groups.back().smem, (int)smem[k]);
     groups.back().max_k = std::max(groups.back().max_k, std::min(secs[k].m, secs[k].n));
     groups.back().max_n = std::max(groups.back().max_n, secs[k].n);
+    if (key[k].first == kSvdTeam) {
+      SvdGroup& g = groups.back();
+      secs[k].team_first = g.ctas;
+      g.ctas += secs[k].team_size;
+      if (!g.bar0 || secs[k].teambar < g.bar0) g.bar0 = secs[k].teambar;
+      if (!g.bar1 || secs[k].teambar > g.bar1) g.bar1 = secs[k].teambar;
+    }
     out.push_back(secs[k]);
   }
   secs.swap(out);
@@ -2033,7 +2252,8 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
   return cudaSuccess;
 }
 
-bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k, const char* exact) {
+bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k, const char* exact,
+                bool team) {
   if (cluster_min_k < 0) cluster_min_k = svd_cluster_min_k();
   L.mode.assign(ns, kSvdSmem);
   L.work_off.assign(ns, -1);
@@ -2044,6 +2264,8 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
   L.piv_off.assign(ns, -1);
   L.wide.assign(ns, 0);
   L.exact.assign(ns, 0);
+  L.bar_off = -1;
+  const int members = team ? kMaxTeam : kMaxCluster;
   L.w2_off.assign(ns, -1);
   L.yt_off.assign(ns, -1);
   for (auto* v : {&L.f32_off, &L.n32_off, &L.vd_off, &L.gm_off, &L.a1_off, &L.sel_off, &L.j_off, &L.v_off2, &L.misc_off})
@@ -2067,8 +2289,8 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     L.v_off[k] = off;    off = a256(off + 16 * M);                      // Householder vector
     L.norm_off[k] = off; off = a256(off + 8 * (2 * N + Kk));            // nu, nu0, nrm
     L.ord_off[k] = off;  off = a256(off + 4 * (N + Kk));                // perm, ord
-    L.flag_off[k] = off; off = a256(off + 4 * (kJacobiMaxSweeps + 1 + kMaxCluster));   // flags, pivot index
-    L.piv_off[k] = off;  off = a256(off + 8 * (kMaxCluster + 2));       // pivot value, scalars
+    L.flag_off[k] = off; off = a256(off + 4 * (kJacobiMaxSweeps + 1 + members));       // flags, pivot index
+    L.piv_off[k] = off;  off = a256(off + 8 * (members + 2));           // pivot value, scalars
     const bool wide = 4LL * n[k] >= 5LL * m[k];   // the Jacobi sweeps run on the K x K factor R2
     L.wide[k] = wide;
     if (refine) {   // FP32 start and refinement (svd_front, k_refine.cu); the FP64 sweeps that may
@@ -2097,6 +2319,10 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
       }
     }
   }
+  if (team) {   // one 64-byte line a sector for the barrier of its team
+    L.bar_off = off;
+    off = a256(off + 64LL * ns);
+  }
   L.total = off;
   return true;
 }
@@ -2118,6 +2344,7 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
   S.f32 = nullptr;
   S.fp32_sweeps = svd_mixed_sweeps();
   S.F = nullptr;
+  S.teambar = L.bar_off >= 0 ? reinterpret_cast<unsigned*>(base + L.bar_off + 64LL * k) : nullptr;
   if (L.f32_off[k] >= 0) {
     S.f32 = reinterpret_cast<float2*>(base + L.f32_off[k]);
     S.nrm32 = reinterpret_cast<float*>(base + L.n32_off[k]);

@@ -202,7 +202,8 @@ struct TileRef { int task; int ti; int tj; };
 
 constexpr int kSvdSmem = 0;          // one CTA, the whole sector in shared memory
 constexpr int kSvdCluster = 1;       // a thread-block cluster, data in L2, round-robin Jacobi
-constexpr int kSvdRefine = 3;        // QR and FP32 Jacobi on a cluster, then tensor-core refinement
+constexpr int kSvdTeam = 3;          // block Jacobi by teams of CTAs in one cooperative launch
+constexpr int kSvdRefine = 4;        // QR and FP32 Jacobi on a cluster, then tensor-core refinement
 constexpr int kSvdClusterBlock = 2;  // a thread-block cluster, data in L2, block Jacobi staged in shared memory
 
 struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
@@ -245,6 +246,9 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   int* rdiag;                 // K: 1 - cosine of the large angles of a step, in units of 2^-30
   int* rstate;                // [0] columns kept, [1] left to the FP64 sweeps, [2] steps when settled, [4 + step] size of E
   int fp32_sweeps;            // limit of the FP32 sweeps
+  unsigned* teambar;          // barrier of the sector's team (nullptr: no teams in this batch)
+  int team_first, team_size;  // the team's CTAs in its launch
+  int team_cl0;               // the cluster size whose block ordering the team keeps
 };
 
 // Scratch layout of a batch of sector SVDs (cluster-mode sectors only need global scratch).
@@ -255,6 +259,7 @@ struct SvdScratchLayout {
   std::vector<int64_t> j_off, v_off2, misc_off;       // refinement (-1: off)
   std::vector<int> wide;
   std::vector<char> exact;
+  int64_t bar_off = -1;       // barriers of teams, 64 bytes a sector
   int smem = 0;               // dynamic shared memory of the one-CTA kernel
   int64_t total = 0;
 };
@@ -262,9 +267,10 @@ struct SvdScratchLayout {
 // (a cluster kernel then spreads them over several SMs; -1: the process setting
 // mps_svd_cluster_min_k, off by default).
 // exact (or nullptr): per sector, whether the phases of Y's columns are part of the result; such a
-// sector is not refined (its pivoted QR and the order of its sweeps fix the phases).
+// sector is not refined (its pivoted QR and the order of its sweeps fix the phases).  team: with room
+// for teams of CTAs (svd_group's team).
 bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k = -1,
-                const char* exact = nullptr);
+                const char* exact = nullptr, bool team = false);
 int svd_cluster_min_k();
 // Cluster sectors with min(m, n) >= this run FP32 Jacobi sweeps first and finish in FP64
 // (0: every sector FP64 only); mps_svd_mixed_min_k sets it.
@@ -391,7 +397,11 @@ namespace mps {
 // Kernel launchers (defined in the .cu files).
 cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
-struct SvdGroup { int kind, cl, smem, first, count, max_k, max_n; };
+struct SvdGroup {
+  int kind, cl, smem, first, count, max_k, max_n;
+  int ctas;                    // kSvdTeam: CTAs of all teams, and the range of their barriers
+  unsigned *bar0, *bar1;
+};
 // Tile shape of the cluster SVD: target column-block width of the block-Jacobi kernel, the
 // smallest cluster size tried, and the sector size (min(m, n)) from which a sector gets a
 // cluster of 16 CTAs (the largest sectors of a layer set its critical path), and the sector
@@ -417,7 +427,7 @@ inline SvdTune svd_tune_candidate(int k) {
 }
 // Orders `secs` into groups (costliest first inside each) and fills `groups`.
 cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& groups,
-                      const SvdTune& tune = SvdTune());
+                      const SvdTune& tune = SvdTune(), bool team = false);
 // The candidate mps_autotune_force set (true), or false when none is forced.
 bool svd_forced_tune(SvdTune& t);
 // Group 0 on st, group g > 0 on side[g-1] when n_side >= groups - 1; st then waits for all.

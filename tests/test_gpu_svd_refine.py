@@ -72,3 +72,27 @@ def test_refined_sectors_do_not_depend_on_their_batch(gpu_lib):
     for A, (s, y, _) in zip(mats, every):
         s1, y1, _ = m.svd_sectors([A])[0]
         assert np.array_equal(s, s1) and np.array_equal(y, y1)
+
+
+@pytest.mark.parametrize("L,chi", [(10, 300), (12, 700)])
+def test_teams_give_the_bits_of_the_clusters(gpu_lib, L, chi):
+    """A TF32 update whose few large sectors run on teams of CTAs equals, bit for bit, the same update
+    with captured phases (which keep the cluster kernels)."""
+    import torch
+    from oracle import gates
+    from tests.helpers import load_state, random_state
+    m = gpu_lib
+    st = random_state(L, 5, L, chi, seed=chi)
+    stream = torch.cuda.Stream()
+    out = []
+    for graphs in (False, True):
+        g = m.MPS(5, [1] * L, chi, precision=m.MPS_TF32, stream=stream.cuda_stream)
+        load_state(g, st)
+        g.set_graphs(graphs)
+        for s in (L // 2 - 1, L // 2, L // 2 - 1):
+            g.apply_gate2(s, gates.bh_gate(L, s, 5, 1.0, 2.0, 0.3), chi, 1e-10)
+        out.append([g.bond(b) for b in range(L + 1)] + [g.site(s) for s in range(L)])
+        g.close()
+    for a, b in zip(*out):
+        assert a.keys() == b.keys()
+        assert all(np.array_equal(a[k], b[k]) for k in a)
