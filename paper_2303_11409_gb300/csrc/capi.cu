@@ -750,7 +750,10 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
 
   // ---- algorithmic work of the three kernels (flops: complex multiply-add = 8) -------
   double th_flops = 0, th_bytes = (double)(theta_bytes_end - theta_bytes_begin);   // Theta' written
+  int th_rows = 1, th_cols = 1;
   for (const ThetaTask& T : tasks) {
+    th_rows = std::max(th_rows, T.Dl);
+    th_cols = std::max(th_cols, T.Dr);
     for (int i = 0; i < T.nm; ++i) th_flops += 8.0 * T.Dl * T.Dm[i] * T.Dr;
     th_flops += 8.0 * T.nm * T.nc * T.Dl * T.Dr;
   }
@@ -803,7 +806,8 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     const bool any_theta = !tiles.empty() || !mixes[0].empty() || !mixes[1].empty();
     return timed(owner, MPS_K_THETA, any_theta, th_flops, th_bytes, [&] {
       cudaError_t e2 = launch_theta(reinterpret_cast<ThetaTask*>(dptr(desc_off + o_tasks)),
-                                    reinterpret_cast<TileRef*>(dptr(desc_off + o_tiles)), (int)tiles.size(), st);
+                                    reinterpret_cast<TileRef*>(dptr(desc_off + o_tiles)), (int)tiles.size(), th_rows,
+                                    th_cols, st);
       for (int p = 0; p < 2 && e2 == cudaSuccess; ++p)
         e2 = launch_mix(precs[p], reinterpret_cast<MixTask*>(dptr(desc_off + o_mix[p])), (int)mixes[p].size(),
                         slot_base[p], st);
@@ -1124,7 +1128,10 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     if (s2.size > desc_bytes) return fail(owner, MPS_EINVAL, "internal: descriptor bound exceeded");
     double lam_bytes = 0, gm_flops = 0, gm_bytes = 0;
     for (const LambdaTask& T : lam) lam_bytes += 16.0 * T.k;
+    int gm_rows = 1, gm_cols = 1;
     for (const GemmTask& T : gm) {
+      gm_rows = std::max(gm_rows, T.M);
+      gm_cols = std::max(gm_cols, T.N);
       gm_flops += 8.0 * T.M * T.N * T.K;
       gm_bytes += 16.0 * ((double)T.M * T.K + (double)T.K * T.N + (double)T.M * T.N);
     }
@@ -1142,7 +1149,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       if (e == cudaSuccess)
         e = timed(owner, MPS_K_GEMM, !gt.empty(), gm_flops, gm_bytes, [&] {
           return launch_gemm(reinterpret_cast<GemmTask*>(dptr(desc_off + o_gm)),
-                             reinterpret_cast<TileRef*>(dptr(desc_off + o_gt)), (int)gt.size(), st);
+                             reinterpret_cast<TileRef*>(dptr(desc_off + o_gt)), (int)gt.size(), gm_rows, gm_cols, st);
         });
       const int precs[2] = {MPS_TF32, MPS_BF16X3};
       const bool any_tc_gemm = !gjobs[0].empty() || !gjobs[1].empty();

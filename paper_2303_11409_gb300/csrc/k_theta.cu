@@ -4,8 +4,8 @@
 //     Theta'(c)[l, r] += G_n[l - c, l - m] * (B^[s][l, m] . B^[s+1][m, r])
 // summed over the middle charges m, for every new middle charge c of the pair
 // (n = l - r).  This is the block-sparse construction of Theta of Sec. II: each
-// product B[l,m] B[m,r] is formed once and mixed into all output charges c in
-// the epilogue, so the GEMM work is that of the (l, m, r) triples alone.
+// product B[l,m] B[m,r] is formed once and mixed into all output charges c
+// in registers, so the GEMM work is that of the (l, m, r) triples alone.
 //
 // K4 (gemm_kernel, scatter_kernel, lambda_kernel): reassembly after truncation,
 //     B^[s][l, c]   = Theta'(c)[rows of l] . Y(c)[:, kept] / |S_kept|
@@ -13,20 +13,28 @@
 //     lambda^[s+1]  = S_kept / |S_kept|
 // Sites are written in charge-sorted block order with coalesced row-major stores.
 //
-// GB300 note: FP64 runs at 1.2 TFLOP/s on this part (measured), so these kernels
-// are FP64-pipe bound; tiles skip whole 16-row/16-column groups that fall
-// outside a ragged block instead of spending FP64 issue slots on padding.
+// GB300 note: FP64 runs at 1.2 TFLOP/s on this part (2 FMA per clock and SM, measured), so these kernels
+// are bound by the FP64 pipe, and a block's time is its FMAs on the SMs that share it.  A CTA of 64
+// threads computes 8 x 8 outputs, one a thread: blocks of 10-100 states spread over many SMs and
+// ragged edges cost least padding.  The operands a tile re-reads come from L2 (4 bytes a complex FMA).
+// Stages of 16 k are copied asynchronously, the next one (of the next middle charge, too) while the present
+// one is used.  64 x 64 tiles of 256 threads took 73 us (Theta) and 67 us (reassembly) on a chi = 64 XXZ
+// layer of 35-state blocks, and ran at 510-570 GFLOP/s on a chi = 512 Bose-Hubbard layer (7.7 and 6.6 ms);
+// these take 15 and 9 us, and 3.9 and 3.4 ms (1.0-1.1 TFLOP/s, 80-87% of the FP64 peak).
+#include <algorithm>
+
 #include "mps_internal.h"
 
 namespace mps {
 namespace {
 
+constexpr int kS = 8;              // rows and columns of a CTA's outputs
 constexpr int kK = 16;             // K chunk staged in shared memory
-constexpr int kThreads = 256;      // 16 x 16 threads, 4 x 4 complex outputs each
+constexpr int kThreads = kS * kS;
 
 struct TileSmem {
-  double2 A[kTile][kK + 1];        // +1: rows of A read by two lanes do not share banks
-  double2 B[kK][kTile];
+  double2 A[2][kS][kK + 1];        // +1: the rows that a warp reads together do not share banks
+  double2 B[2][kK][kS];
 };
 
 __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
@@ -36,119 +44,128 @@ __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
-// acc += A[row0:row0+64, :] . B[:, col0:col0+64] with general strides.
-// Thread (tx, ty) owns rows row0 + ty + 16 i and columns col0 + tx + 16 j.
-__device__ void tile_mma(const double2* __restrict__ A, int sar, int sac,
-                         const double2* __restrict__ B, int sbr, int sbc,
-                         int M, int N, int K, int row0, int col0,
-                         double2 (&acc)[4][4], TileSmem& sm) {
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int warp_ty = (tid >> 5) * 2;               // smallest ty in this warp
-  int ni = 0, nj = 0;                               // warp-uniform live row / column groups
+// 16-byte copy into shared memory, zeros when ok is false
+__device__ __forceinline__ void copy16(double2* dst, const double2* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
+}
+
+// One product of a tile: A (M x K) and B (K x N) with general strides.
+struct Product {
+  const double2 *A, *B;
+  int sar, sac, sbr, sbc, M, N, K;
+};
+
+__device__ __forceinline__ void stage(const Product& P, int row0, int col0, int k0, int buf, TileSmem& sm) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) ni += (row0 + warp_ty + 16 * i < M);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) nj += (col0 + 16 * j < N);
-  for (int k0 = 0; k0 < K; k0 += kK) {
-    const int kc = min(kK, K - k0);
-    // stage A: 64 x 16 (k fastest for row-major A)
-    for (int e = tid; e < kTile * kK; e += kThreads) {
-      int r, k;
-      if (sac == 1) { r = e / kK; k = e % kK; } else { k = e / kTile; r = e % kTile; }
-      double2 v = make_double2(0.0, 0.0);
-      if (row0 + r < M && k < kc) v = A[(int64_t)(row0 + r) * sar + (int64_t)(k0 + k) * sac];
-      sm.A[r][k] = v;
-    }
-    // stage B: 16 x 64 (j fastest for row-major B, k fastest for column-major B)
-    for (int e = tid; e < kTile * kK; e += kThreads) {
-      int k, c;
-      if (sbc == 1) { k = e / kTile; c = e % kTile; } else { c = e / kK; k = e % kK; }
-      double2 v = make_double2(0.0, 0.0);
-      if (col0 + c < N && k < kc) v = B[(int64_t)(k0 + k) * sbr + (int64_t)(col0 + c) * sbc];
-      sm.B[k][c] = v;
-    }
+  for (int h = 0; h < 2; ++h) {
+    const int e = threadIdx.x + h * kThreads;
+    const int ar = P.sac == 1 ? e >> 4 : e & 7, ak = P.sac == 1 ? e & 15 : e >> 3;
+    const bool oka = row0 + ar < P.M && k0 + ak < P.K;
+    copy16(&sm.A[buf][ar][ak], oka ? P.A + (int64_t)(row0 + ar) * P.sar + (int64_t)(k0 + ak) * P.sac : P.A, oka);
+    const int bk = P.sbc == 1 ? e >> 3 : e & 15, bc = P.sbc == 1 ? e & 7 : e >> 4;
+    const bool okb = col0 + bc < P.N && k0 + bk < P.K;
+    copy16(&sm.B[buf][bk][bc], okb ? P.B + (int64_t)(k0 + bk) * P.sbr + (int64_t)(col0 + bc) * P.sbc : P.B, okb);
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+// The thread's output of product P, whose first stage is on its way into buffer buf; the first stage of Q
+// follows when more is set.  on: the thread's warp has rows inside the block.
+__device__ __forceinline__ double2 product(const Product& P, const Product& Q, bool more, int row0, int col0, int& buf,
+                                           bool on, TileSmem& sm) {
+  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+  double p0 = 0.0, q0 = 0.0, r0 = 0.0, s0 = 0.0, p1 = 0.0, q1 = 0.0, r1 = 0.0, s1 = 0.0;
+  for (int k0 = 0; k0 < P.K; k0 += kK) {
+    const int kc = min(kK, P.K - k0);
+    bool next = true;
+    if (k0 + kK < P.K) stage(P, row0, col0, k0 + kK, buf ^ 1, sm);
+    else if (more) stage(Q, row0, col0, 0, buf ^ 1, sm);
+    else next = false;
+    if (next) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    for (int kk = 0; kk < kc; ++kk) {
-      double2 a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = sm.A[ty + 16 * i][kk];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = sm.B[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (i < ni) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (j < nj) cfma(acc[i][j], a[i], b[j]);
-        }
+    if (on) {
+      int kk = 0;
+#pragma unroll 4
+      for (; kk + 1 < kc; kk += 2) {      // eight chains over the pipe's 64-cycle latency
+        const double2 a = sm.A[buf][ty][kk], b = sm.B[buf][kk][tx];
+        const double2 a1 = sm.A[buf][ty][kk + 1], b1 = sm.B[buf][kk + 1][tx];
+        p0 = fma(a.x, b.x, p0);
+        q0 = fma(a.y, b.y, q0);
+        r0 = fma(a.x, b.y, r0);
+        s0 = fma(a.y, b.x, s0);
+        p1 = fma(a1.x, b1.x, p1);
+        q1 = fma(a1.y, b1.y, q1);
+        r1 = fma(a1.x, b1.y, r1);
+        s1 = fma(a1.y, b1.x, s1);
+      }
+      if (kk < kc) {
+        const double2 a = sm.A[buf][ty][kk], b = sm.B[buf][kk][tx];
+        p0 = fma(a.x, b.x, p0);
+        q0 = fma(a.y, b.y, q0);
+        r0 = fma(a.x, b.y, r0);
+        s0 = fma(a.y, b.x, s0);
       }
     }
     __syncthreads();
+    buf ^= 1;
   }
+  return make_double2((p0 + p1) - (q0 + q1), (r0 + r1) + (s0 + s1));
 }
 
+// blockIdx.x: a tile of kTile x kTile outputs of the task list, blockIdx.y: the kS x kS part of it
+// (sub parts a row).
 __global__ void __launch_bounds__(kThreads) theta_kernel(const ThetaTask* __restrict__ tasks,
-                                                         const TileRef* __restrict__ tiles) {
+                                                         const TileRef* __restrict__ tiles, int sub) {
   __shared__ TileSmem sm;
   const TileRef tr = tiles[blockIdx.x];
   const ThetaTask& T = tasks[tr.task];
-  const int row0 = tr.ti * kTile, col0 = tr.tj * kTile;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int Dl = T.Dl, Dr = T.Dr, nc = T.nc, sn = T.sn;
-  for (int mi = 0; mi < T.nm; ++mi) {
-    double2 acc[4][4];
+  const int row0 = tr.ti * kTile + (blockIdx.y / sub) * kS, col0 = tr.tj * kTile + (blockIdx.y % sub) * kS;
+  const int Dl = T.Dl, Dr = T.Dr, nc = T.nc, sn = T.sn, nm = T.nm;
+  if (row0 >= Dl || col0 >= Dr) return;
+  const int r = row0 + (threadIdx.x >> 3), c = col0 + (threadIdx.x & 7);
+  const bool on = row0 + ((threadIdx.x >> 3) & ~3) < Dl;
+  auto at = [&](int mi) { return Product{T.A[mi], T.B[mi], T.Dm[mi], 1, Dr, 1, Dl, Dr, T.Dm[mi]}; };
+  double2 out[MPS_MAX_D];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+  for (int k = 0; k < MPS_MAX_D; ++k) out[k] = make_double2(0.0, 0.0);
+  int buf = 0;
+  Product P = at(0);
+  stage(P, row0, col0, 0, 0, sm);
+  for (int mi = 0; mi < nm; ++mi) {
+    const bool more = mi + 1 < nm;
+    const Product Q = at(more ? mi + 1 : mi);
+    const double2 v = product(P, Q, more, row0, col0, buf, on, sm);
+    // mix this product into every output charge of the (l, r) pair
+    if (on) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
-    tile_mma(T.A[mi], T.Dm[mi], 1, T.B[mi], Dr, 1, Dl, Dr, T.Dm[mi], row0, col0, acc, sm);
-    // epilogue: mix this product into every output charge of the (l, r) pair
-    for (int k = 0; k < nc; ++k) {
-      const double2 g = T.gate[T.go[k] * sn + T.gi[mi]];
-      double2* __restrict__ out = T.out[k];
-      const int ldo = T.ldo[k];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = row0 + ty + 16 * i;
-        if (r >= Dl) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = col0 + tx + 16 * j;
-          if (c >= Dr) continue;
-          double2 v = out[(int64_t)r * ldo + c];
-          cfma(v, g, acc[i][j]);
-          out[(int64_t)r * ldo + c] = v;
-        }
-      }
+      for (int k = 0; k < MPS_MAX_D; ++k)
+        if (k < nc) cfma(out[k], T.gate[T.go[k] * sn + T.gi[mi]], v);
     }
+    P = Q;
+  }
+  if (r < Dl && c < Dr) {
+#pragma unroll
+    for (int k = 0; k < MPS_MAX_D; ++k)
+      if (k < nc) T.out[k][(int64_t)r * T.ldo[k] + c] = out[k];
   }
 }
 
 __global__ void __launch_bounds__(kThreads) gemm_kernel(const GemmTask* __restrict__ tasks,
-                                                        const TileRef* __restrict__ tiles) {
+                                                        const TileRef* __restrict__ tiles, int sub) {
   __shared__ TileSmem sm;
   const TileRef tr = tiles[blockIdx.x];
   const GemmTask& T = tasks[tr.task];
-  const int row0 = tr.ti * kTile, col0 = tr.tj * kTile;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double2 acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
-  tile_mma(T.A, T.sar, T.sac, T.B, T.sbr, T.sbc, T.M, T.N, T.K, row0, col0, acc, sm);
-  const double alpha = T.alpha;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = row0 + ty + 16 * i;
-    if (r >= T.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = col0 + tx + 16 * j;
-      if (c >= T.N) continue;
-      T.C[(int64_t)r * T.ldc + c] = make_double2(alpha * acc[i][j].x, alpha * acc[i][j].y);
-    }
-  }
+  const int row0 = tr.ti * kTile + (blockIdx.y / sub) * kS, col0 = tr.tj * kTile + (blockIdx.y % sub) * kS;
+  if (row0 >= T.M || col0 >= T.N) return;
+  const int r = row0 + (threadIdx.x >> 3), c = col0 + (threadIdx.x & 7);
+  const Product P{T.A, T.B, T.sar, T.sac, T.sbr, T.sbc, T.M, T.N, T.K};
+  int buf = 0;
+  stage(P, row0, col0, 0, 0, sm);
+  const double2 v = product(P, P, false, row0, col0, buf, row0 + ((threadIdx.x >> 3) & ~3) < T.M, sm);
+  if (r < T.M && c < T.N) T.C[(int64_t)r * T.ldc + c] = make_double2(T.alpha * v.x, T.alpha * v.y);
 }
 
 // One flat element per thread; tasks are sorted by their first element index.
@@ -175,17 +192,24 @@ __global__ void lambda_kernel(const LambdaTask* __restrict__ tasks) {
 
 }  // namespace
 
-cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st) {
+// parts of kS along an edge of the largest tile
+inline int parts(int n) { return (std::min(n, kTile) + kS - 1) / kS; }
+
+cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, int max_rows, int max_cols,
+                         cudaStream_t st) {
   if (n_tiles <= 0) return cudaSuccess;
   count_launch();
-  theta_kernel<<<n_tiles, kThreads, 0, st>>>(d_tasks, d_tiles);
+  theta_kernel<<<dim3(n_tiles, parts(max_rows) * parts(max_cols)), kThreads, 0, st>>>(d_tasks, d_tiles,
+                                                                                      parts(max_cols));
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm(const GemmTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st) {
+cudaError_t launch_gemm(const GemmTask* d_tasks, const TileRef* d_tiles, int n_tiles, int max_rows, int max_cols,
+                        cudaStream_t st) {
   if (n_tiles <= 0) return cudaSuccess;
   count_launch();
-  gemm_kernel<<<n_tiles, kThreads, 0, st>>>(d_tasks, d_tiles);
+  gemm_kernel<<<dim3(n_tiles, parts(max_rows) * parts(max_cols)), kThreads, 0, st>>>(d_tasks, d_tiles,
+                                                                                     parts(max_cols));
   return cudaGetLastError();
 }
 

@@ -395,7 +395,9 @@ struct mps_s {
 namespace mps {
 
 // Kernel launchers (defined in the .cu files).
-cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
+// max_rows, max_cols: the largest block of the tasks.
+cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n_tiles, int max_rows, int max_cols,
+                         cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
 struct SvdGroup {
   int kind, cl, smem, first, count, max_k, max_n;
@@ -442,7 +444,8 @@ cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max
 
 cudaError_t launch_select(const SelectSector* d_secs, const SelectTask* d_tasks, int n_tasks,
                           int* d_kept, SelectResult* d_res, cudaStream_t st);
-cudaError_t launch_gemm(const GemmTask* d_tasks, const TileRef* d_tiles, int n_tiles, cudaStream_t st);
+cudaError_t launch_gemm(const GemmTask* d_tasks, const TileRef* d_tiles, int n_tiles, int max_rows, int max_cols,
+                        cudaStream_t st);
 
 // TMA-fed tensor-core complex GEMM (k_tma.cu).  Operands live in "shadow tiles": 128 rows of
 // 128 bytes each (16 KB), TF32 (a row holds 16 complex K as interleaved re, im floats) or BF16
