@@ -5,7 +5,7 @@
 // rotations V of an FP32 one-sided Jacobi run on it, so that A = J V has columns orthogonal to
 // about 1e-5 and V^dag V = I to about 1e-6.  What remains is to make both exact:
 //     R = I - V^dag V,  S = A^dag A,
-//     E_pq = (S_pq + lambda_q R_pq) / (lambda_q - lambda_p),  E_pp = R_pp / 2,
+//     E_pq = (S_pq + lambda_q R_pq) / (lambda_q - lambda_p),  E_pp = (R_pp - sum_k |E_kp|^2) / 2,
 //     V <- V + V E,  A <- A + A E,
 // which squares the error in every step (the symmetric-eigenvalue refinement of Ogita and Aishima,
 // "Iterative refinement for symmetric eigenvalue decomposition", 2018, applied to the Gram matrix
@@ -26,6 +26,7 @@
 #include <climits>
 
 #include "mps_internal.h"
+#include "refine_pair.cuh"
 
 namespace mps {
 namespace {
@@ -34,6 +35,7 @@ constexpr int kOzSlices = 7;
 constexpr int kOzM = 64, kOzN = 32, kOzK = 32;      // complex rows, columns and contraction of a stage
 constexpr int kOzThreads = 256;                     // 4 x 2 warps of 16 x 16 complex outputs
 constexpr int kOzABytes = kOzM * 128, kOzBBytes = kOzN * 128;   // one slice: 32 complex BF16 pairs a row
+constexpr int kOzAhead = 4;                         // operand loads in flight ahead of their conversion
 constexpr int kOzSmem = kOzSlices * (kOzABytes + kOzBBytes);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -101,12 +103,13 @@ struct OzSum {
   long long hi[2][2][4], lo[2][2][4];      // [re / im][h][x]
 };
 
-// One stage in shared memory: the MMAs of its 4 k-steps into acc[slice sum][re/im * 2 + h][4].
+// One stage in shared memory: the MMAs of its k-steps (8 complex each, at most 4) into acc[slice sum][re/im * 2 + h][4].
 template <int NS>
-__device__ __forceinline__ void oz_stage(float (&acc)[NS][4][4], uint32_t sA, uint32_t sB, int wr, int wc, int lane) {
+__device__ __forceinline__ void oz_stage(float (&acc)[NS][4][4], uint32_t sA, uint32_t sB, int wr, int wc, int lane,
+                                         int steps) {
   const int arow = wr * 16 + (lane & 15), brow = wc * 16 + (lane & 7) + ((lane >> 4) << 3);
 #pragma unroll 1
-  for (int s = 0; s < 4; ++s) {
+  for (int s = 0; s < steps; ++s) {
     uint32_t a[NS][4];
     const int ac = (2 * s + (lane >> 4)) ^ (arow & 7), bc = (2 * s + ((lane >> 3) & 1)) ^ (brow & 7);
 #pragma unroll
@@ -148,9 +151,10 @@ __device__ __forceinline__ void oz_flush(float (&acc)[NS][4][4], OzSum& t) {
 }
 
 // t = sum over k < kt of (the A tile)(row, k)^* (the B tile)(col, k); load_a(k0) and load_b(k0) put the
-// slices of stage [k0, k0 + 32) into shared memory (zero beyond the operands).
+// slices of stage [k0, k0 + 32) into shared memory (zero beyond kt up to a k-step).  A warp whose
+// outputs are not wanted (on == false) only helps to load.
 template <int NS, class LA, class LB>
-__device__ void oz_product(OzSum& t, char* smem, int kt, LA load_a, LB load_b) {
+__device__ void oz_product(OzSum& t, char* smem, int kt, bool on, LA load_a, LB load_b) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wr = warp & 3, wc = warp >> 2;
   const uint32_t sA = smem_u32(smem), sB = sA + kOzSlices * kOzABytes;
   float acc[NS][4][4];
@@ -172,7 +176,8 @@ __device__ void oz_product(OzSum& t, char* smem, int kt, LA load_a, LB load_b) {
     load_a(k0);
     load_b(k0);
     __syncthreads();
-    oz_stage<NS>(acc, sA, sB, wr, wc, lane);
+    if (!on) continue;
+    oz_stage<NS>(acc, sA, sB, wr, wc, lane, (min(kOzK, kt - k0) + 7) / 8);
     if (++held == 2) {      // 64 complex k: the FP32 sums are still exact
       oz_flush<NS>(acc, t);
       held = 0;
@@ -199,13 +204,24 @@ template <int NS, int ROWS, typename T2>
 __device__ __forceinline__ void load_cols(char* dst, int slice_bytes, const T2* X, int64_t ld, int c0, int ncol, int k0,
                                           int kn, const int* e_sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane >= (min(kOzK, kn - k0) + 7) / 8 * 8) return;
+  const int rows = min(ROWS, ncol - c0);
 #pragma unroll 1
-  for (int r = warp; r < ROWS; r += kOzThreads / 32) {
-    T2 v;
-    v.x = 0;
-    v.y = 0;
-    if (c0 + r < ncol && k0 + lane < kn) v = X[(int64_t)(c0 + r) * ld + k0 + lane];
-    oz_store<NS>(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2), slice_bytes, v, e_sh[r], 0u);
+  for (int r0 = warp; r0 < rows; r0 += kOzAhead * kOzThreads / 32) {
+    T2 v[kOzAhead];
+#pragma unroll
+    for (int a = 0; a < kOzAhead; ++a) {
+      const int r = r0 + a * kOzThreads / 32;
+      v[a].x = 0;
+      v[a].y = 0;
+      if (r < rows && k0 + lane < kn) v[a] = X[(int64_t)(c0 + r) * ld + k0 + lane];
+    }
+#pragma unroll
+    for (int a = 0; a < kOzAhead; ++a) {
+      const int r = r0 + a * kOzThreads / 32;
+      if (r < rows)
+        oz_store<NS>(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2), slice_bytes, v[a], e_sh[r], 0u);
+    }
   }
 }
 // The left operand of X W: rows r0.. of X (column-major), contraction over its columns k with the
@@ -214,29 +230,49 @@ template <int NS>
 __device__ __forceinline__ void load_rows(char* dst, const double2* X, int64_t ld, int r0, int nrow, int k0, int kn,
                                           const int* e) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nr = (min(kOzM, nrow - r0) + 7) / 8, nb = (min(kOzK, kn - k0) + 7) / 8 * 2;      // 8 rows x 4 k each
 #pragma unroll 1
-  for (int t = warp; t < (kOzM / 8) * (kOzK / 4); t += kOzThreads / 32) {
-    const int r = (t & 7) * 8 + (lane & 7), b = t >> 3, k = 4 * b + (lane >> 3);
-    double2 v = make_double2(0.0, 0.0);
-    int ek = 0;
-    if (k0 + k < kn) {
-      ek = e ? e[k0 + k] : 1;
-      if (r0 + r < nrow) v = X[(int64_t)(k0 + k) * ld + r0 + r];
+  for (int t0 = warp; t0 < nr * nb; t0 += kOzAhead * kOzThreads / 32) {
+    double2 v[kOzAhead];
+    int ek[kOzAhead];
+#pragma unroll
+    for (int a = 0; a < kOzAhead; ++a) {
+      const int t = t0 + a * kOzThreads / 32;
+      const int r = (t % nr) * 8 + (lane & 7), k = 4 * (t / nr) + (lane >> 3);
+      v[a] = make_double2(0.0, 0.0);
+      ek[a] = 0;
+      if (t < nr * nb && k0 + k < kn) {
+        ek[a] = e[k0 + k];
+        if (r0 + r < nrow) v[a] = X[(int64_t)(k0 + k) * ld + r0 + r];
+      }
     }
-    oz_store<NS>(dst + r * 128 + ((b ^ (r & 7)) << 4) + ((lane >> 3) << 2), kOzABytes, v, ek, 0x80000000u);
+#pragma unroll
+    for (int a = 0; a < kOzAhead; ++a) {
+      const int t = t0 + a * kOzThreads / 32, r = (t % nr) * 8 + (lane & 7), b = t / nr;
+      if (t < nr * nb)
+        oz_store<NS>(dst + r * 128 + ((b ^ (r & 7)) << 4) + ((lane >> 3) << 2), kOzABytes, v[a], ek[a], 0x80000000u);
+    }
   }
 }
 
+constexpr int kLeftAt = 100;       // rstate[1] when step it leaves the sector: kLeftAt + it
 __device__ __forceinline__ int ns_of(const SvdSector& S) { return __ldg(S.rstate); }
 __device__ __forceinline__ bool skip(const SvdSector& S) { return S.rstate[1] != 0 || S.rstate[2] != 0; }
 
-// Squared norm (FP64) and scale exponent of every column of the current A (which == 0: of J), one
-// warp a column; the last step's decision whether the sector has settled is taken here too.
+// Squared norm (FP64) and scale exponent of every column of the current A (which == 0: of J), and the scale
+// exponent of V's, one warp a column; and whether step `it` has settled the sector or does not contract.  The words it writes for
+// that hold `it`, so that CTAs of the same launch that see them go on with their norms.
 __global__ void __launch_bounds__(256) refine_norm_kernel(const SvdSector* __restrict__ secs, int which, int it) {
   const SvdSector S = secs[blockIdx.y];
-  if (skip(S)) return;
+  const int left = S.rstate[1], done = S.rstate[2];
+  if ((left != 0 && left != kLeftAt + it) || (done != 0 && done != it)) return;
   const int K = min(S.m, S.n), n = S.n, lane = threadIdx.x & 31;
   const int ncol = which == 0 ? K : ns_of(S);
+  if (it > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+    const float th = __int_as_float(S.rstate[4 + it - 1]);
+    if (refine_fails(th, it - 1)) S.rstate[1] = kLeftAt + it;
+    else if (refine_settles(th, ncol, n)) S.rstate[2] = it;
+  }
   const double2* X = which == 0 ? S.J : ((it & 1) ? S.A1 : S.A0);
   for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < ncol; c += gridDim.x * 8) {
     const double2* a = X + (int64_t)c * n;
@@ -250,32 +286,24 @@ __global__ void __launch_bounds__(256) refine_norm_kernel(const SvdSector* __res
                          (unsigned)(__double_as_longlong(x.y) >> 52) & 0x7ffu));
     }
     s0 += s1;
+    unsigned vtop = 0;
+    if (which == 1) {
+      const double2* v = ((it & 1) ? S.V1 : S.V0) + (int64_t)c * K;
+      for (int k = lane; k < K; k += 32)
+        vtop = max(vtop, max((unsigned)(__double_as_longlong(v[k].x) >> 52) & 0x7ffu,
+                             (unsigned)(__double_as_longlong(v[k].y) >> 52) & 0x7ffu));
+    }
     for (int o = 16; o; o >>= 1) {
       s0 += __shfl_xor_sync(0xffffffffu, s0, o);
       top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+      vtop = max(vtop, __shfl_xor_sync(0xffffffffu, vtop, o));
     }
     if (lane == 0) {
+      S.vexp[c] = max((int)vtop - 1022, -200);
       S.rnorm[c] = s0;
       S.cexp[c] = max((int)top - 1022, -900);
-      S.rdiag[c] = 0;
-      if (!(s0 < 1e300)) S.rstate[1] = 1;      // infinities and NaN go to the FP64 sweeps
+      if (!(s0 < 1e300)) S.rstate[1] = kLeftAt + it;      // infinities and NaN go to the FP64 sweeps
     }
-  }
-}
-
-// Settled when the last step's largest relative entry theta leaves a second-order error K theta^2
-// below half the orthogonality threshold eps max(n, 32) of the FP64 sweeps.
-__global__ void refine_check_kernel(const SvdSector* __restrict__ secs, int count, int it) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= count) return;
-  const SvdSector S = secs[k];
-  if (skip(S)) return;
-  const float th = __int_as_float(S.rstate[4 + it - 1]);
-  const int K = S.rstate[0];
-  const double tol = 2.220446049250313e-16 * max(S.n, 32);
-  if (!(th < (it > 1 ? 0.3f : 1.6f))) S.rstate[1] = 1;      // no contraction: leave it to the FP64 sweeps
-  else if ((double)K * th * th < 0.5 * tol) {
-    S.rstate[2] = it;
   }
 }
 
@@ -283,6 +311,7 @@ __global__ void refine_check_kernel(const SvdSector* __restrict__ secs, int coun
 __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdSector* __restrict__ secs, int step) {
   extern __shared__ __align__(128) char smem[];
   __shared__ int s_t[kOzN];
+  __shared__ float s_d[kOzN];      // second-order part of W's diagonal
   const SvdSector S = secs[blockIdx.y];
   if (skip(S)) return;
   const int K = min(S.m, S.n), n = S.n, ns = ns_of(S);
@@ -297,56 +326,78 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
   double2* out = step == 0 ? S.A0 : (onV ? ((step & 1) ? S.V1 : S.V0) : ((step & 1) ? S.A1 : S.A0));
   const int64_t ld = onV ? K : n;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // scale of each column of W: the largest component of s_k W_kc.  The correction E is stored in the
-  // scaled form s_k E_kc / s_c; V's columns have unit scale.
+  // scale of each column of W: the largest component of s_k W_kc, s_k the scale of X's column k.  The
+  // correction E is stored in the scaled form of A's columns, s_k E_kc / s_c.
   for (int c = warp; c < kOzN; c += 8) {
     int top = INT_MIN / 2;
+    float sq = 0.f;
     if (c0 + c < ns) {
+      const int ec = step == 0 ? 0 : S.cexp[c0 + c];
       for (int k = lane; k < kn; k += 32) {
         if (step == 0) {
           const double2 w = S.V0[(int64_t)(c0 + c) * K + k];
           const int e = max((int)((__double_as_longlong(w.x) >> 52) & 0x7ff), (int)((__double_as_longlong(w.y) >> 52) & 0x7ff));
           if (e) top = max(top, e - 1022 + S.cexp[k]);
         } else {
-          float2 w = S.E[(int64_t)(c0 + c) * K + k];
-          if (k == c0 + c) w.x -= 9.3132257e-10f * (float)S.rdiag[k];
+          const float2 w = S.E[(int64_t)(c0 + c) * K + k];
           const int e = max((__float_as_int(w.x) >> 23) & 0xff, (__float_as_int(w.y) >> 23) & 0xff);
-          if (e) top = max(top, e - 126 + (onV ? S.cexp[c0 + c] - S.cexp[k] : 0));
+          const int d = ec - S.cexp[k];      // E_kc = w 2^d
+          if (e) top = max(top, e - 126 + (onV ? d + S.vexp[k] : 0));
+          const float f = exp2f((float)max(-60, min(60, d)));
+          sq = fmaf(w.x * f, w.x * f, fmaf(w.y * f, w.y * f, sq));
         }
       }
     }
-    for (int o = 16; o; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    for (int o = 16; o; o >>= 1) {
+      top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+      sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    if (lane == 0) s_d[c] = -0.5f * sq;
+    // the diagonal's second-order part may be the largest entry
+    if (step > 0 && sq > 0.f) top = max(top, ilogbf(sq) + 1 + (onV ? S.vexp[c0 + c] : 0));
     if (lane == 0) s_t[c] = max(top, -1000);
   }
   __syncthreads();
   char* sB = smem + kOzSlices * kOzABytes;
   OzSum t;
-  auto la = [&](int k0) { load_rows<kOzSlices>(smem, X, ld, r0, nrow, k0, kn, onV ? nullptr : S.cexp); };
+  auto la = [&](int k0) { load_rows<kOzSlices>(smem, X, ld, r0, nrow, k0, kn, onV ? S.vexp : S.cexp); };
   auto lb = [&](int k0) {      // W: column c, contraction k; scaled by s_k / t_c
-#pragma unroll 1
-    for (int r = warp; r < kOzN; r += 8) {
-      const int k = k0 + lane;
-      char* d = sB + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2);
-      const bool in = c0 + r < ns && k < kn;
+    if (lane >= (min(kOzK, kn - k0) + 7) / 8 * 8) return;
+    const int k = k0 + lane, rows = min(kOzN, ns - c0);
+    double2 vd[kOzN / 8];
+    float2 vf[kOzN / 8];
+#pragma unroll
+    for (int a = 0; a < kOzN / 8; ++a) {
+      const int r = warp + 8 * a;
+      const bool in = r < rows && k < kn;
       if (step == 0) {
-        const double2 v = in ? S.V0[(int64_t)(c0 + r) * K + k] : make_double2(0.0, 0.0);
-        oz_store<kOzSlices>(d, kOzBBytes, v, in ? s_t[r] - S.cexp[k] : 0, 0u);
+        vd[a] = in ? S.V0[(int64_t)(c0 + r) * K + k] : make_double2(0.0, 0.0);
       } else {
-        float2 v = in ? S.E[(int64_t)(c0 + r) * K + k] : make_float2(0.f, 0.f);
-        if (in && k == c0 + r) v.x -= 9.3132257e-10f * (float)S.rdiag[k];
-        oz_store<kOzSlices>(d, kOzBBytes, v, in ? (onV ? s_t[r] - (S.cexp[c0 + r] - S.cexp[k]) : s_t[r]) : 0, 0u);
+        vf[a] = in ? S.E[(int64_t)(c0 + r) * K + k] : make_float2(0.f, 0.f);
+        if (in && k == c0 + r) vf[a].x += s_d[r];
       }
     }
+    const int ek = k < kn ? S.cexp[k] : 0, ev = onV && k < kn ? S.vexp[k] : 0;
+#pragma unroll
+    for (int a = 0; a < kOzN / 8; ++a) {
+      const int r = warp + 8 * a;
+      if (r >= rows) continue;
+      char* d = sB + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2);
+      if (step == 0) oz_store<kOzSlices>(d, kOzBBytes, vd[a], s_t[r] - ek, 0u);
+      else oz_store<kOzSlices>(d, kOzBBytes, vf[a], onV ? s_t[r] - (S.cexp[c0 + r] - ek + ev) : s_t[r], 0u);
+    }
   };
-  oz_product<kOzSlices>(t, smem, kn, la, lb);
   const int g = lane >> 2, q = lane & 3, wr = warp & 3, wc = warp >> 2;
+  const bool on = r0 + wr * 16 < nrow && c0 + wc * 16 < ns;
+  oz_product<kOzSlices>(t, smem, kn, on, la, lb);
+  if (!on) return;
 #pragma unroll
   for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
       const int i = r0 + wr * 16 + g + ((x >> 1) << 3), lc = wc * 16 + h * 8 + 2 * q + (x & 1), c = c0 + lc;
       if (i >= nrow || c >= ns) continue;
-      const int e = s_t[lc] - 60 + (step == 0 ? 0 : (onV ? 1 : S.cexp[c]));
+      const int e = s_t[lc] - 60 + (step == 0 || onV ? 0 : S.cexp[c]);
       double2 v = make_double2(oz_double(t.hi[0][h][x], t.lo[0][h][x], e), oz_double(t.hi[1][h][x], t.lo[1][h][x], e));
       if (step > 0) {
         const double2 o = X[(int64_t)c * ld + i];
@@ -361,7 +412,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
 // tile over p <= q.  rstate[4 + it] keeps the largest entry relative to its column.
 __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSector* __restrict__ secs, int it) {
   extern __shared__ __align__(128) char smem[];
-  __shared__ int s_ep[kOzM], s_eq[kOzN], s_one[kOzM];
+  __shared__ int s_ep[kOzM], s_eq[kOzN], s_vp[kOzM], s_vq[kOzN];
   const SvdSector S = secs[blockIdx.y];
   if (skip(S)) return;
   const int K = min(S.m, S.n), n = S.n, ns = ns_of(S);
@@ -374,29 +425,36 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSec
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < kOzM) {
     s_ep[tid] = p0 + tid < ns ? S.cexp[p0 + tid] : 0;
-    s_one[tid] = 1;
+    s_vp[tid] = p0 + tid < ns ? S.vexp[p0 + tid] : 0;
   }
-  if (tid < kOzN) s_eq[tid] = q0 + tid < ns ? S.cexp[q0 + tid] : 0;
+  if (tid < kOzN) {
+    s_eq[tid] = q0 + tid < ns ? S.cexp[q0 + tid] : 0;
+    s_vq[tid] = q0 + tid < ns ? S.vexp[q0 + tid] : 0;
+  }
   __syncthreads();
   char* sB = smem + kOzSlices * kOzABytes;
   const int g = lane >> 2, qq = lane & 3, wr = warp & 3, wc = warp >> 2;
+  const bool on = p0 + wr * 16 < ns && q0 + wc * 16 < ns && p0 + wr * 16 < q0 + wc * 16 + 16;
   OzSum t;
   oz_product<kOzSlices>(
-      t, smem, K, [&](int k0) { load_cols<kOzSlices, kOzM>(smem, kOzABytes, V, K, p0, ns, k0, K, s_one); },
-      [&](int k0) { load_cols<kOzSlices, kOzN>(sB, kOzBBytes, V, K, q0, ns, k0, K, s_one); });
+      t, smem, K, on, [&](int k0) { load_cols<kOzSlices, kOzM>(smem, kOzABytes, V, K, p0, ns, k0, K, s_vp); },
+      [&](int k0) { load_cols<kOzSlices, kOzN>(sB, kOzBBytes, V, K, q0, ns, k0, K, s_vq); });
   float Rr[2][4], Ri[2][4];
 #pragma unroll
   for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
       const int p = p0 + wr * 16 + g + ((x >> 1) << 3), q = q0 + wc * 16 + h * 8 + 2 * qq + (x & 1);
-      // 1 - |v_p|^2 on the diagonal: V's scale is 2, so 1 is 2^58 in the units of the sum
-      Rr[h][x] = -4.f * oz_float(t.hi[0][h][x] - (p == q ? (1LL << 26) : 0), t.lo[0][h][x]);
-      Ri[h][x] = -4.f * oz_float(t.hi[1][h][x], t.lo[1][h][x]);
+      // 1 - |v_p|^2 on the diagonal is taken in integers: 1 is 2^(60 - 2 e) in the units of the sum
+      const int ep = s_vp[wr * 16 + g + ((x >> 1) << 3)], eq = s_vq[wc * 16 + h * 8 + 2 * qq + (x & 1)];
+      const float f = -exp2f((float)(ep + eq));
+      Rr[h][x] = f * oz_float(t.hi[0][h][x] - (p == q ? 1LL << (28 - 2 * max(ep, -16)) : 0), t.lo[0][h][x]);
+      Ri[h][x] = f * oz_float(t.hi[1][h][x], t.lo[1][h][x]);
     }
   oz_product<kOzSlices>(
-      t, smem, n, [&](int k0) { load_cols<kOzSlices, kOzM>(smem, kOzABytes, A, n, p0, ns, k0, n, s_ep); },
+      t, smem, n, on, [&](int k0) { load_cols<kOzSlices, kOzM>(smem, kOzABytes, A, n, p0, ns, k0, n, s_ep); },
       [&](int k0) { load_cols<kOzSlices, kOzN>(sB, kOzBBytes, A, n, q0, ns, k0, n, s_eq); });
+  if (!on) return;
   float worst = 0.f;
   const double floor2 = S.rfloor2[0];
   const float tol = 2.2204460e-16f * (float)max(n, 32);
@@ -418,38 +476,10 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSec
         const float al = (float)(np * pow2(-2 * ep)), be = (float)(nq * pow2(-2 * eq));
         const float rho = exp2f((float)max(-60, min(60, eq - ep)));       // s_q / s_p
         const float gr = oz_float(t.hi[0][h][x], t.lo[0][h][x]), gi = oz_float(t.hi[1][h][x], t.lo[1][h][x]);
-        const float br = be * rho * rho;                  // lambda_q / s_p^2
-        const float dif = br - al;
-        const float rr = Rr[h][x], ri = Ri[h][x];
-        if (fabsf(dif) > 0.03f * fmaxf(al, br)) {
-          const float ip = 1.f / dif, brq = be * rho;
-          epq = make_float2((gr + brq * rr) * ip, (gi + brq * ri) * ip);
-          // E_qp = conj(S_pq + lambda_p R_pq) / (lambda_p - lambda_q)
-          const float f = -rho * ip;
-          eqp = make_float2((gr * rho + al * rr) * f, -(gi * rho + al * ri) * f);
-        } else {      // close values: orthonormalise by R / 2 and turn by the Jacobi angle
-          const float mean = 0.5f * (al / rho + be * rho);
-          const float hr = gr + mean * rr, hi_ = gi + mean * ri, ag = hypotf(hr, hi_);
-          float tx = 0.f, ty = 0.f;
-          if (ag > tol * sqrtf(al * be)) {      // orthogonal to rounding otherwise
-            const float z = dif / (2.f * rho * ag), az = fabsf(z);
-            const float tt = copysignf(1.f, z) / (az + (az < 1e18f ? sqrtf(fmaf(z, z, 1.f)) : az));
-            const float c = rsqrtf(fmaf(tt, tt, 1.f));
-            tx = c * tt * hr / ag;
-            ty = c * tt * hi_ / ag;
-            // the cosine of a large angle, summed exactly (integers) whatever the order of the tiles
-            const int dec = __float2int_rn((tt * tt * c / (1.f + c)) * c * 1073741824.f);
-            if (dec > 0) {
-              atomicAdd(S.rdiag + p, dec);
-              atomicAdd(S.rdiag + q, dec);
-            }
-          }
-          epq = make_float2((0.5f * rr + tx) / rho, (0.5f * ri + ty) / rho);
-          eqp = make_float2((0.5f * rr - tx) * rho, -(0.5f * ri - ty) * rho);
-        }
-        const float a1 = hypotf(epq.x, epq.y), a2 = hypotf(eqp.x, eqp.y);
-        // relative change of the smaller column, absolute change of the larger one's rotation
-        worst = fmaxf(worst, rho <= 1.f ? fmaxf(a1, a2 / rho) : fmaxf(a2, a1 * rho));
+        const RefinePair P = refine_pair(al, be, rho, gr, gi, Rr[h][x], Ri[h][x], tol);
+        epq = P.pq;
+        eqp = P.qp;
+        worst = fmaxf(worst, P.size);
       }
       S.E[(int64_t)q * K + p] = epq;
       S.E[(int64_t)p * K + q] = eqp;
@@ -514,12 +544,14 @@ cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max
   refine_update_kernel<<<dim3(ct * rn, count), kOzThreads, kOzSmem, st>>>(d_secs, 0);
   refine_norm_kernel<<<cols, 256, 0, st>>>(d_secs, 1, 0);
   count_launch(); count_launch(); count_launch();
-  for (int it = 0; it < kRefineSteps; ++it) {
+  // two or three steps settle a sector; launches beyond that find nothing to do (3 us each), and
+  // what is not settled after the last one costs FP64 sweeps, which large sectors can least afford
+  const int steps = max_k < 200 ? 4 : kRefineSteps;
+  for (int it = 0; it < steps; ++it) {
     refine_gram_kernel<<<dim3(ct * rk, count), kOzThreads, kOzSmem, st>>>(d_secs, it);
     refine_update_kernel<<<dim3(ct * (rn + rk), count), kOzThreads, kOzSmem, st>>>(d_secs, it + 1);
     refine_norm_kernel<<<cols, 256, 0, st>>>(d_secs, 1, it + 1);
-    refine_check_kernel<<<cd(count, 64), 64, 0, st>>>(d_secs, count, it + 1);
-    count_launch(); count_launch(); count_launch(); count_launch();
+    count_launch(); count_launch(); count_launch();
   }
   refine_output_kernel<<<cols, 256, 0, st>>>(d_secs);
   count_launch();

@@ -62,6 +62,7 @@
 #include <vector>
 
 #include "mps_internal.h"
+#include "refine_pair.cuh"
 
 namespace mps {
 namespace {
@@ -73,9 +74,11 @@ constexpr int kMaxTeam = 304;           // CTAs of a team: 2 on each of 152 SMs
 constexpr int kSvdTeamExpired = -2;     // a sector's status when a team's wait ran out
 constexpr int kMaxWarps = 16;
 constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps per CTA, 2 CTAs per SM
-// smallest min(m, n) of a refined sector: below it the one-CTA kernel's few sweeps cost less than
-// the dozen launches of the refinement (chi = 64 layers of 31-35 columns, 1.4 ms)
-constexpr int kRefineMinK = 48;
+constexpr int kRefineMinK = 25;         // smallest min(m, n) refined on the tensor cores
+// a refined sector's FP32 sweeps end with one that found no cosine above this: it has left about the square
+constexpr float kFp32Stop = 1e-3f;
+constexpr int kSmallK = 24;             // largest min(m, n) refined inside one CTA
+constexpr int kFrontSmallK = 64;        // largest min(m, n) with a one-CTA front
 // rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
 // a row's dependent FMAs 128)
 constexpr int kAhead = 8;
@@ -707,7 +710,7 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // (possibly tiny) inner product: |g| against tol sqrt(alpha beta), t = tan(theta) from
 // zeta = (beta - alpha) / (2 |g|).
 __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int p, int q, bool valid, int G,
-                              float tol, float floor2) {
+                              float tol, float floor2, float stop) {
   const int gl = threadIdx.x & (G - 1);
   float alpha = 0.f, beta = 0.f;
   if (valid) {
@@ -730,6 +733,7 @@ __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int 
   }
   const float ag = hypotf(gr, gi);
   act = act && (ag > tol * sqrtf(alpha) * sqrtf(beta));
+  const float far = stop * sqrtf(alpha) * sqrtf(beta);
   if (act) {
     const float zeta = (beta - alpha) / (2.f * ag), az = fabsf(zeta);
     const float t = copysignf(1.f, zeta) / (az + (az < 1e18f ? sqrtf(fmaf(zeta, zeta, 1.f)) : az));
@@ -747,7 +751,7 @@ __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int 
       nrm[q] = beta + tg;
     }
   }
-  return act;
+  return act && ag > far;
 }
 
 __device__ __forceinline__ int group_width32(int P, int R, int nwarps) {
@@ -770,6 +774,7 @@ struct JacobiBlocks32 {
   float2* sm;
   float* smn;
   int bsmax, g, gs, cl0;      // as in JacobiBlocks
+  float stop = 0.f;           // a sweep whose rotations all had cosines up to this is the last one
   __device__ int staged_with(int p) const {
     const int q = p / cl0;
     return min(gs, g - q / gs * gs);
@@ -853,7 +858,7 @@ struct JacobiBlocks32 {
                   valid = a < s_len32[j] && b < s_len32[j];
                 }
                 rot |= jacobi_pair32(sm, R, Rr, ld, smn, j * bsmax + min(a, b), j * bsmax + max(a, b), valid, G,
-                                     tol, floor2);
+                                     tol, floor2, stop);
               }
               __syncthreads();
             }
@@ -878,7 +883,7 @@ struct JacobiBlocks32 {
                     q = max(pa, pb);
                   }
                 }
-                rot |= jacobi_pair32(sm, R, Rr, ld, smn, p, q, valid, G, tol, floor2);
+                rot |= jacobi_pair32(sm, R, Rr, ld, smn, p, q, valid, G, tol, floor2, stop);
               }
               __syncthreads();
             }
@@ -1112,7 +1117,7 @@ __device__ void qr_columns(T2* A, int64_t ld, int rows, int ncol, int K, T2* rkk
       u0.y = x0.y - beta.y;
       x[k] = u0;
       __stcg(rkk + k, beta);
-      __stcg(tau + k, uu > 0 ? 2 / uu : 0);
+      __stcg(tau + k, uu > 0 ? 2 / uu : T(0));
     }
     __syncwarp();
   };
@@ -1804,10 +1809,7 @@ __host__ __device__ inline SmemLayout smem_layout(int m, int n) {
   return L;
 }
 
-__global__ void __launch_bounds__(kSvdThreads, 1) jacobi_cta_kernel(const SvdSector* __restrict__ secs,
-                                                                    int max_sweeps) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SvdSector S = secs[blockIdx.x];
+__device__ __forceinline__ void cta_sector(const SvdSector& S, unsigned char* smem_raw, int max_sweeps) {
   const SmemLayout L = smem_layout(S.m, S.n);
   Work w;
   w.W = reinterpret_cast<double2*>(smem_raw + L.W);
@@ -1822,6 +1824,578 @@ __global__ void __launch_bounds__(kSvdThreads, 1) jacobi_cta_kernel(const SvdSec
   w.pi = reinterpret_cast<int*>(smem_raw + L.pi);
   w.scal = reinterpret_cast<double*>(smem_raw + L.scal);
   svd_sector<PlainMem>(S, w, 0, 1, CtaSync{}, max_sweeps, JacobiRoundRobin<PlainMem>{});
+}
+
+__global__ void __launch_bounds__(kSvdThreads, 1) jacobi_cta_kernel(const SvdSector* __restrict__ secs,
+                                                                    int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cta_sector(secs[blockIdx.x], smem_raw, max_sweeps);
+}
+
+// ---------------------------------------------------------------------------------------
+// One CTA, everything in shared memory: the refined SVD of a small sector.  The QR and the FP32 sweeps are
+// those of svd_front; up to kSmallK columns the refinement runs here too (its products are shorter than a
+// kernel launch), above that J and V go to the tensor-core kernels.  The FP64 sweeps of jacobi_cta_kernel
+// paid for every rotation's root and quotient in FP64 (some 1500 cycles of latency a pair); here those
+// are FP32 and the FP64 work is the QR and the refinement's products.
+// ---------------------------------------------------------------------------------------
+struct SmallLayout {
+  int ldm, fld, lda;                  // strides of W, F and A
+  int64_t W, F, V, V32, E, rkk, tau, nu, lam, inv, nrm, perm, sel, rank, total;
+};
+__host__ __device__ inline SmallLayout small_layout(int m, int n, bool full) {
+  auto al = [](int64_t x) { return (x + 15) & ~int64_t(15); };
+  const int K = m < n ? m : n;
+  SmallLayout L;
+  L.ldm = m | 1;
+  L.fld = (n + K) | 1;
+  L.lda = n | 1;
+  int64_t o = 0;
+  L.W = o; o = al(o + 16LL * L.ldm * n);
+  const int64_t f = 8LL * L.fld * K, a = full ? 16LL * L.lda * K : 0;      // A takes F's place
+  L.F = o; o = al(o + (f > a ? f : a));
+  L.V = o; o = al(o + (full ? 16LL * K * K : 0));
+  L.V32 = o; o = al(o + (full ? 8LL * K * K : 0));
+  L.E = o; o = al(o + (full ? 8LL * K * K : 0));
+  L.rkk = o; o = al(o + 16LL * K);
+  L.tau = o; o = al(o + 8LL * K);
+  L.nu = o; o = al(o + 8LL * n);
+  L.lam = o; o = al(o + 8LL * K);
+  L.inv = o; o = al(o + 8LL * K);
+  L.nrm = o; o = al(o + 4LL * K);
+  L.perm = o; o = al(o + 4LL * n);
+  L.sel = o; o = al(o + 4LL * K);
+  L.rank = o; o = al(o + 4LL * K);
+  L.total = o;
+  return L;
+}
+
+// Householder QR of a matrix in shared memory by one CTA (as qr_columns).  An FP64 instruction occupies its
+// quarter of the SM for 64 cycles whatever its lanes do, so a step's chain of them is its time: warp 0
+// takes column k + 1 with all its lanes on the rows and forms the next reflector (its two roots are one
+// instruction sequence on two lanes), while the other warps share the rest, 8, 4 or 2 columns a warp with
+// the rows dealt to 4, 8 or 16 lanes: no lane idles and the sums end in 2-4 shuffles.  35 x 35 took 248 us
+// with a warp per pair of columns, 142 with 8 columns a warp throughout.
+template <class Pos>
+__device__ void qr_small(double2* A, int ld, int rows, int ncol, int K, double2* rkk, double* tau, Pos pos) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  // column j <- (I - tau_k u u^dag) column j by the lanes sub, sub + subs, ... that share it
+  auto apply = [&](const double2* u, double tk, double2* x, int k, int sub, int subs, bool on) {
+    double p = 0.0, q = 0.0, r = 0.0, s = 0.0;
+    if (on)
+      for (int i = k + sub; i < rows; i += subs) {
+        const double2 a = u[i], b = x[i];
+        p = fma(a.x, b.x, p);
+        r = fma(a.y, b.y, r);
+        q = fma(a.x, b.y, q);
+        s = fma(a.y, b.x, s);
+      }
+    p += r;
+    q -= s;
+    for (int o = 32 / subs; o < 32; o <<= 1) {      // lanes of a column differ in the high bits
+      p += __shfl_xor_sync(0xffffffffu, p, o);
+      q += __shfl_xor_sync(0xffffffffu, q, o);
+    }
+    p *= tk;
+    q *= tk;
+    if (on) {
+#pragma unroll 4
+      for (int i = k + sub; i < rows; i += subs) {
+        const double2 a = u[i];
+        double2 b = x[i];
+        b.x = fma(-a.x, p, fma(a.y, q, b.x));
+        b.y = fma(-a.x, q, fma(-a.y, p, b.y));
+        x[i] = b;
+      }
+    }
+  };
+  auto reflector = [&](int k) {      // warp 0: column k is final above row k
+    double2* x = A + (int64_t)pos(k) * ld;
+    double s0 = 0.0, s1 = 0.0;
+    for (int i = k + lane; i < rows; i += 32) {
+      const double2 v = x[i];
+      s0 = fma(v.x, v.x, s0);
+      s1 = fma(v.y, v.y, s1);
+    }
+    const double x2 = warp_sum(s0 + s1);
+    const double2 x0 = x[k];
+    const double a2 = fma(x0.x, x0.x, x0.y * x0.y);
+    const double v = lane == 0 ? x2 : a2, iv = v > 0.0 ? rsqrt(v) : 0.0, sv = v * iv;
+    const double xn = __shfl_sync(0xffffffffu, sv, 0), a0 = __shfl_sync(0xffffffffu, sv, 1);
+    const double ia = __shfl_sync(0xffffffffu, iv, 1);
+    const double f = -ia * xn;
+    const double2 beta = a2 > 0.0 ? make_double2(x0.x * f, x0.y * f) : make_double2(-xn, 0.0);
+    const double uu = x2 + xn * a0;
+    __syncwarp();
+    if (lane == 0) {
+      x[k] = make_double2(x0.x - beta.x, x0.y - beta.y);
+      rkk[k] = beta;
+      tau[k] = uu > 0.0 ? 1.0 / uu : 0.0;
+    }
+    __syncwarp();
+  };
+  if (warp == 0) reflector(0);
+  for (int k = 0; k < K; ++k) {
+    __syncthreads();
+    const double2* u = A + (int64_t)pos(k) * ld;
+    const double tk = tau[k];
+    if (warp == 0) {
+      if (k + 1 < ncol) apply(u, tk, A + (int64_t)pos(k + 1) * ld, k, lane, 32, true);
+      __syncwarp();
+      if (k + 1 < K) reflector(k + 1);
+    } else {
+      const int rest = ncol - k - 2;
+      const int cols = rest > 4 * (nwarps - 1) ? 8 : rest > 2 * (nwarps - 1) ? 4 : 2;
+      const int col = lane & (cols - 1), sub = lane / cols;
+      for (int j0 = k + 2 + (warp - 1) * cols; j0 < ncol; j0 += (nwarps - 1) * cols) {
+        const bool on = j0 + col < ncol;
+        apply(u, tk, A + (int64_t)pos(on ? j0 + col : k) * ld, k, sub, 32 / cols, on);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// The Jacobi rotation of two FP32 columns with squared norms al, be and inner product (gr, gi), from their
+// cosine c and the ratio of their norms, so that nothing is squared below the range of FP32: cs, (u, v) = the
+// sine times the phase, tg = the change of the norms.  False when c <= tol.
+struct Rot32 { float cs, u, v, tg, c; };
+__device__ __forceinline__ bool rotation32(float al, float be, float gr, float gi, float tol, Rot32& R) {
+  const float ra = rsqrt_fast(al), rb = rsqrt_fast(be);
+  const float sr = gr * ra * rb, si = gi * ra * rb;
+  const float c2 = fmaf(sr, sr, si * si);
+  if (!(c2 > tol * tol)) return false;
+  const float ic = rsqrt_fast(c2), sa = al * ra, sb = be * rb;
+  R.c = c2 * ic;
+  const float z = fminf(fmaxf(0.5f * (sb * ra - sa * rb) * ic, -1e17f), 1e17f);
+  const float h = fmaf(z, z, 1.f);
+  const float t = copysignf(rcp_fast(fabsf(z) + h * rsqrt_fast(h)), z);
+  R.cs = rsqrt_fast(fmaf(t, t, 1.f));
+  const float f = R.cs * t * ic;
+  R.u = f * sr;
+  R.v = f * si;
+  R.tg = t * R.c * sa * sb;
+  return true;
+}
+
+// G lanes rotate columns p, q of the FP32 matrix.  Both columns, the rows of the rotations included, are
+// loaded at once and stay in registers when a lane holds at most kHeld of their elements.  Returns the cosine (0: not
+// rotated).
+constexpr int kHeld = 10;
+__device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, float* nrm, int p, int q, bool valid, int G,
+                                            float tol, float floor2) {
+  const int gl = threadIdx.x & (G - 1);
+  float al = 0.f, be = 0.f;
+  if (valid) {
+    al = nrm[p];
+    be = nrm[q];
+  }
+  const bool act = valid && fminf(al, be) > floor2;
+  float2* ap = F + (act ? p : 0) * ld;
+  float2* aq = F + (act ? q : 0) * ld;
+  const bool held = Rr <= kHeld * G;
+  float2 x[kHeld], y[kHeld];
+  float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;
+  if (held) {
+#pragma unroll
+    for (int t = 0; t < kHeld; ++t) {
+      x[t] = y[t] = make_float2(0.f, 0.f);
+      if (act && gl + t * G < Rr) {
+        x[t] = ap[gl + t * G];
+        y[t] = aq[gl + t * G];
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < kHeld; ++t)
+      if (gl + t * G < R) {
+        gr = fmaf(x[t].x, y[t].x, gr);
+        hr = fmaf(x[t].y, y[t].y, hr);
+        gi = fmaf(x[t].x, y[t].y, gi);
+        hi = fmaf(-x[t].y, y[t].x, hi);
+      }
+  } else if (act) {
+#pragma unroll 4
+    for (int i = gl; i < R; i += G) {
+      const float2 u = ap[i], v = aq[i];
+      gr = fmaf(u.x, v.x, gr);
+      hr = fmaf(u.y, v.y, hr);
+      gi = fmaf(u.x, v.y, gi);
+      hi = fmaf(-u.y, v.x, hi);
+    }
+  }
+  gr += hr;
+  gi += hi;
+  for (int o = G >> 1; o; o >>= 1) {
+    gr += __shfl_xor_sync(0xffffffffu, gr, o);
+    gi += __shfl_xor_sync(0xffffffffu, gi, o);
+  }
+  Rot32 T;
+  if (!act || !rotation32(al, be, gr, gi, tol, T)) return 0.f;
+  auto turn = [&](float2& a, float2& b) {
+    const float2 ao = a, bo = b;
+    a = make_float2(fmaf(T.cs, ao.x, -fmaf(T.u, bo.x, T.v * bo.y)), fmaf(T.cs, ao.y, -fmaf(T.u, bo.y, -T.v * bo.x)));
+    b = make_float2(fmaf(T.cs, bo.x, fmaf(T.u, ao.x, -T.v * ao.y)), fmaf(T.cs, bo.y, fmaf(T.u, ao.y, T.v * ao.x)));
+  };
+  if (held) {
+#pragma unroll
+    for (int t = 0; t < kHeld; ++t)
+      if (gl + t * G < Rr) {
+        turn(x[t], y[t]);
+        ap[gl + t * G] = x[t];
+        aq[gl + t * G] = y[t];
+      }
+  } else {
+    for (int i0 = gl; i0 < Rr; i0 += 4 * G) {
+      float2 a[4], b[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (i0 + t * G < Rr) {
+          a[t] = ap[i0 + t * G];
+          b[t] = aq[i0 + t * G];
+        }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (i0 + t * G < Rr) {
+          turn(a[t], b[t]);
+          ap[i0 + t * G] = a[t];
+          aq[i0 + t * G] = b[t];
+        }
+    }
+  }
+  if (gl == 0) {
+    nrm[p] = fmaxf(al - T.tg, 0.f);
+    nrm[q] = be + T.tg;
+  }
+  return T.c;
+}
+
+// Round-robin FP32 sweeps of one CTA until no pair of a sweep was further than kFp32Stop from orthogonal
+// (each sweep squares the distance, so the sweep that found that has left about its square).
+__device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm, float tol, float floor2,
+                             int max_sweeps) {
+  __shared__ int s_far;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int mp = K + (K & 1), ring = mp - 1, P = mp / 2;
+  int G = 8;      // lanes a pair: the widest that still does a round in one pass, 8 at least
+  while (G < 32 && 2 * G * P <= (int)blockDim.x && 4 * G < Rr) G *= 2;
+  const int slots = blockDim.x / G, slot = tid / G;
+  for (int sweep = 0; K > 1 && sweep < max_sweeps; ++sweep) {
+    for (int j = warp; j < K; j += nwarps) {
+      float acc = 0.f;
+      for (int i = lane; i < R; i += 32) {
+        const float2 x = F[j * ld + i];
+        acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
+      }
+      acc = warp_sum_f(acc);
+      if (lane == 0) nrm[j] = acc;
+    }
+    if (tid == 0) s_far = 0;
+    __syncthreads();
+    bool far = false;
+    if (P <= slots) {      // one pass a round: the pair of this slot steps round the ring
+      int a = slot % ring, b = (ring - slot % ring) % ring;      // rr_pair(slot, 0) - 1
+      if (slot == 0) b = 0;
+      for (int r = 0; r < ring; ++r) {
+        const int p = slot == 0 ? 0 : a + 1, q = b + 1;
+        const bool valid = slot < P && p < K && q < K;
+        far |= small_pair(F, R, Rr, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop;
+        if (++a == ring) a = 0;
+        if (++b == ring) b = 0;
+        __syncthreads();
+      }
+    } else {
+      for (int r = 0; r < ring; ++r) {
+        for (int base = 0; base < P; base += slots) {
+          const int k = base + slot;
+          int p = 0, q = 0;
+          if (k < P) rr_pair(k, r, mp, p, q);
+          const bool valid = k < P && p < K && q < K;
+          far |= small_pair(F, R, Rr, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop;
+        }
+        __syncthreads();
+      }
+    }
+    if (far) s_far = 1;
+    __syncthreads();
+    const int go = s_far;
+    __syncthreads();
+    if (!go) break;
+  }
+}
+
+__global__ void __launch_bounds__(kSvdThreads, 1) svd_small_kernel(const SvdSector* __restrict__ secs, int max_sweeps) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_ns, s_theta;
+  const SvdSector S = secs[blockIdx.x];
+  const int m = S.m, n = S.n, K = min(m, n);
+  const bool full = S.F == nullptr;      // else the front of a sector that the tensor cores refine
+  const SmallLayout L = small_layout(m, n, full);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  double2* W = reinterpret_cast<double2*>(smem_raw + L.W);
+  float2* F = reinterpret_cast<float2*>(smem_raw + L.F);
+  double2* rkk = reinterpret_cast<double2*>(smem_raw + L.rkk);
+  double* tau = reinterpret_cast<double*>(smem_raw + L.tau);
+  double* nu = reinterpret_cast<double*>(smem_raw + L.nu);
+  float* nrm = reinterpret_cast<float*>(smem_raw + L.nrm);
+  int* perm = reinterpret_cast<int*>(smem_raw + L.perm);
+  int* sel = reinterpret_cast<int*>(smem_raw + L.sel);
+  for (int e = tid; e < m * n; e += blockDim.x) {
+    const int i = e / n, j = e % n;
+    const double s = S.rowscale ? S.rowscale[i] : 1.0;
+    const double2 x = S.theta[e];
+    W[(int64_t)j * L.ldm + i] = make_double2(s * x.x, s * x.y);
+  }
+  if (!full && tid < 16) S.rstate[tid] = 0;
+  __syncthreads();
+  for (int j = warp; j < n; j += nwarps) {
+    double a0 = 0.0, a1 = 0.0;
+    for (int i = lane; i < m; i += 32) {
+      const double2 x = W[(int64_t)j * L.ldm + i];
+      a0 = fma(x.x, x.x, a0);
+      a1 = fma(x.y, x.y, a1);
+    }
+    a0 = warp_sum(a0 + a1);
+    if (lane == 0) nu[j] = a0;
+  }
+  __syncthreads();
+  double fro2 = 0.0;
+  for (int j = lane; j < n; j += 32) fro2 += nu[j];
+  fro2 = warp_sum(fro2);
+  for (int j = tid; j < n; j += blockDim.x) {      // descending norms, NaN last
+    const double vj = nu[j], v = isnan(vj) ? -1.0 : vj;
+    int rk = 0;
+    for (int q = 0; q < n; ++q) {
+      const double wq = nu[q], x = isnan(wq) ? -1.0 : wq;
+      rk += (x > v) || (x == v && q < j);
+    }
+    perm[rk] = j;
+  }
+  __syncthreads();
+  bool left = !(fro2 > 1e-270 && fro2 < 1e270);      // zero, not finite, or squares out of range
+  if (left) {
+    if (!full) {
+      if (tid == 0) S.rstate[1] = 1;
+      return;
+    }
+  } else {
+    const int sc = -(ilogb(fro2) / 2);
+    const double scale = scalbn(1.0, sc), up = scalbn(1.0, -sc);
+    const double frel = fmax(32.0 * kEps, S.floor_rel);
+    const double floor2 = fmax(frel * frel * fro2, S.floor_abs * S.floor_abs) * scale * scale;
+    qr_small(W, L.ldm, m, n, K, rkk, tau, [&](int j) { return perm[j]; });
+    // R scaled by 2^sc, its diagonal in place; F = [conj R^T; I]
+    for (int e = tid; e < K * n; e += blockDim.x) {
+      const int i = e % K, j = e / K;
+      double2* w = W + (int64_t)perm[j] * L.ldm + i;
+      double2 x = make_double2(0.0, 0.0);
+      if (i <= j) {
+        x = i == j ? rkk[i] : *w;
+        x.x *= scale;
+        x.y *= scale;
+        *w = x;
+      }
+      F[(int64_t)i * L.fld + j] = make_float2((float)x.x, (float)-x.y);
+    }
+    for (int e = tid; e < K * K; e += blockDim.x)
+      F[(int64_t)(e / K) * L.fld + n + e % K] = make_float2(e / K == e % K ? 1.f : 0.f, 0.f);
+    __syncthreads();
+    if (!full)
+      for (int e = tid; e < K * n; e += blockDim.x) {      // J = R^dag for the tensor-core kernels
+        const int i = e / n, j = e % n;
+        double2 x = make_double2(0.0, 0.0);
+        if (i <= j) x = W[(int64_t)perm[j] * L.ldm + i];
+        S.J[e] = make_double2(x.x, -x.y);
+      }
+    const float tol32 = 1.1920929e-07f * (float)max(n, 32), fl32 = (float)(0.01 * floor2);
+    small_sweeps(F, n, n + K, L.fld, K, nrm, tol32, fl32, min(max_sweeps, S.fp32_sweeps + 6));
+    for (int j = warp; j < K; j += nwarps) {
+      float acc = 0.f;
+      for (int i = lane; i < n; i += 32) {
+        const float2 x = F[(int64_t)j * L.fld + i];
+        acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
+      }
+      acc = warp_sum_f(acc);
+      if (lane == 0) nrm[j] = acc;
+    }
+    __syncthreads();
+    if (warp == 0) {      // the kept columns, in column order
+      int ns = 0;
+      for (int c0 = 0; c0 < K; c0 += 32) {
+        const bool keep = c0 + lane < K && nrm[c0 + lane] > fl32;
+        const unsigned mask = __ballot_sync(0xffffffffu, keep);
+        if (keep) sel[ns + __popc(mask & ((1u << lane) - 1))] = c0 + lane;
+        ns += __popc(mask);
+      }
+      if (lane == 0) s_ns = ns;
+    }
+    __syncthreads();
+    const int ns = s_ns;
+    if (!full) {
+      for (int e = tid; e < K * ns; e += blockDim.x) {
+        const float2 v = F[(int64_t)sel[e / K] * L.fld + n + e % K];
+        S.V0[e] = make_double2((double)v.x, (double)v.y);
+      }
+      for (int j = tid; j < n; j += blockDim.x) S.order[j] = perm[j];
+      if (tid == 0) {
+        S.rfloor2[0] = floor2;
+        S.rfloor2[1] = up;
+        S.rstate[0] = ns;
+        if (ns == 0) S.rstate[1] = 1;
+      }
+      return;
+    }
+    // ---- refinement in FP64 (see k_refine.cu) -------------------------------------------------
+    double2* V = reinterpret_cast<double2*>(smem_raw + L.V);
+    float2* V32 = reinterpret_cast<float2*>(smem_raw + L.V32);
+    float2* E = reinterpret_cast<float2*>(smem_raw + L.E);
+    double* lam = reinterpret_cast<double*>(smem_raw + L.lam);
+    double* inv = reinterpret_cast<double*>(smem_raw + L.inv);
+    for (int e = tid; e < K * ns; e += blockDim.x) {
+      const float2 v = F[(int64_t)sel[e / K] * L.fld + n + e % K];
+      V32[e] = v;
+      V[e] = make_double2((double)v.x, (double)v.y);
+    }
+    __syncthreads();
+    double2* A = reinterpret_cast<double2*>(smem_raw + L.F);
+    const float tol = 2.2204460e-16f * (float)max(n, 32);
+    int steps = 0;
+    bool settled = false;
+    left = ns == 0;
+    for (int it = 0; !left; ++it) {
+      for (int e = tid; e < n * ns; e += blockDim.x) {      // A = J V
+        const int j = e % n, c = e / n, top = min(j, K - 1);
+        const double2* r = W + (int64_t)perm[j] * L.ldm;
+        const double2* v = V + (int64_t)c * K;
+        double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
+        for (int i = 0; i <= top; ++i) {
+          a0 = fma(r[i].x, v[i].x, a0);
+          a1 = fma(r[i].y, v[i].y, a1);
+          b0 = fma(r[i].x, v[i].y, b0);
+          b1 = fma(r[i].y, v[i].x, b1);
+        }
+        A[(int64_t)c * L.lda + j] = make_double2(a0 + a1, b0 - b1);
+      }
+      __syncthreads();
+      for (int c = warp; c < ns; c += nwarps) {
+        double a0 = 0.0, a1 = 0.0;
+        for (int j = lane; j < n; j += 32) {
+          const double2 x = A[(int64_t)c * L.lda + j];
+          a0 = fma(x.x, x.x, a0);
+          a1 = fma(x.y, x.y, a1);
+        }
+        a0 = warp_sum(a0 + a1);
+        if (lane == 0) {
+          lam[c] = a0;
+          inv[c] = a0 > 0.0 ? rsqrt(a0) : 0.0;
+        }
+      }
+      if (tid == 0) s_theta = 0;
+      __syncthreads();
+      if (settled || it == kRefineSteps) break;
+      float worst = 0.f;
+      for (int e = tid; e < ns * ns; e += blockDim.x) {
+        const int p = e % ns, q = e / ns;
+        if (p > q) continue;
+        const double2 *a = A + (int64_t)p * L.lda, *b = A + (int64_t)q * L.lda, *v = V + (int64_t)p * K,
+                      *u = V + (int64_t)q * K;
+        double g0 = 0.0, g1 = 0.0, h0 = 0.0, h1 = 0.0;
+        for (int i = 0; i < K; ++i) {
+          g0 = fma(v[i].x, u[i].x, g0);
+          g1 = fma(v[i].y, u[i].y, g1);
+          h0 = fma(v[i].x, u[i].y, h0);
+          h1 = fma(v[i].y, u[i].x, h1);
+        }
+        const float rr = (float)((p == q ? 1.0 : 0.0) - (g0 + g1)), ri = (float)(h1 - h0);
+        if (p == q) {
+          E[q * K + p] = make_float2(0.5f * rr, 0.f);
+          worst = fmaxf(worst, fabsf(rr));
+          continue;
+        }
+        g0 = g1 = h0 = h1 = 0.0;
+        for (int j = 0; j < n; ++j) {
+          g0 = fma(a[j].x, b[j].x, g0);
+          g1 = fma(a[j].y, b[j].y, g1);
+          h0 = fma(a[j].x, b[j].y, h0);
+          h1 = fma(a[j].y, b[j].x, h1);
+        }
+        RefinePair P = {};
+        float rho = 1.f;
+        if (fmin(lam[p], lam[q]) > floor2) {
+          const double f = inv[p] * inv[q];
+          rho = (float)(lam[q] * f);                  // |a_q| / |a_p|
+          P = refine_pair(1.f, 1.f, rho, (float)((g0 + g1) * f), (float)((h0 - h1) * f), rr, ri, tol);
+          worst = fmaxf(worst, P.size);
+        }
+        E[q * K + p] = make_float2(P.pq.x * rho, P.pq.y * rho);
+        E[p * K + q] = make_float2(P.qp.x / rho, P.qp.y / rho);
+        if (!(P.size >= 0.f)) worst = 1e30f;          // NaN: leave it
+      }
+      for (int o = 16; o; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+      if (lane == 0) atomicMax(&s_theta, __float_as_int(worst));
+      __syncthreads();
+      const float th = __int_as_float(s_theta);
+      left = refine_fails(th, it);
+      settled = !left && refine_settles(th, ns, n);
+      steps = it + 1;
+      if (!left)
+        for (int e = tid; e < K * ns; e += blockDim.x) {      // V += V E: E is small, FP32 holds the product
+          const int i = e % K, c = e / K;
+          float x = 0.f, y = 0.f, sq = 0.f;
+          for (int k = 0; k < ns; ++k) {
+            const float2 v = V32[k * K + i], w = E[c * K + k];
+            sq = fmaf(w.x, w.x, fmaf(w.y, w.y, sq));
+            x = fmaf(v.x, w.x, fmaf(-v.y, w.y, x));
+            y = fmaf(v.x, w.y, fmaf(v.y, w.x, y));
+          }
+          const float2 v = V32[e];      // the diagonal's second-order part
+          V[e].x += (double)fmaf(-0.5f * sq, v.x, x);
+          V[e].y += (double)fmaf(-0.5f * sq, v.y, y);
+        }
+      __syncthreads();
+      for (int e = tid; e < K * ns; e += blockDim.x) V32[e] = make_float2((float)V[e].x, (float)V[e].y);
+      __syncthreads();
+    }
+    if (settled) {      // singular values and Y = P A / sigma in descending order; the rest is zero
+      int* rank = reinterpret_cast<int*>(smem_raw + L.rank);
+      for (int c = tid; c < K; c += blockDim.x) {
+        const double v = c < ns && lam[c] > floor2 ? lam[c] : 0.0;
+        int rk = 0;
+        for (int j = 0; j < K; ++j) {
+          const double x = j < ns && lam[j] > floor2 ? lam[j] : 0.0;
+          rk += (x > v) || (x == v && j < c);
+        }
+        const double sg = sqrt(v);
+        S.sigma[rk] = sg * up;
+        rank[c] = rk;
+        inv[c] = v > 0.0 ? 1.0 / sg : 0.0;
+      }
+      __syncthreads();
+      for (int e = tid; e < n * K; e += blockDim.x) {
+        const int j = e % n, c = e / n;
+        double2 z = make_double2(0.0, 0.0);
+        if (c < ns && inv[c] > 0.0) {
+          const double2 a = A[(int64_t)c * L.lda + j];
+          z = make_double2(a.x * inv[c], a.y * inv[c]);
+        }
+        S.Y[(int64_t)rank[c] * n + perm[j]] = z;
+      }
+      if (tid == 0) *S.status = steps;
+      return;
+    }
+  }
+  __syncthreads();
+  cta_sector(S, smem_raw, max_sweeps);      // the FP64 sweeps, from the start
 }
 
 __device__ __forceinline__ Work cluster_work(const SvdSector& S) {
@@ -1908,6 +2482,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSe
   j32.g = S.groups;
   j32.gs = S.staged;
   j32.cl0 = cluster;
+  j32.stop = kFp32Stop;
   j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
   j32.sm = reinterpret_cast<float2*>(smem_raw);
   j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
@@ -1948,6 +2523,8 @@ cudaError_t set_attrs(int* big_out) {
     return cudaSuccess;
   }
   e = cudaFuncSetAttribute(jacobi_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(svd_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBlockSmemMax);
@@ -2019,25 +2596,30 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   if (g.count <= 0) return cudaSuccess;
   const SvdSector* d = d_secs + g.first;
   count_launch();
+  if (g.kind == kSvdSmall || (g.kind == kSvdRefine && g.cl == 1 && !fallback)) {
+    svd_small_kernel<<<g.count, kSvdThreads, g.smem_small, st>>>(d, max_sweeps);
+    return cudaGetLastError();
+  }
+  const int cl = g.kind == kSvdRefine && g.cl == 1 ? 2 : g.cl;      // a one-CTA front falls back to a cluster of 2
   if (g.kind == kSvdSmem) {
     jacobi_cta_kernel<<<g.count, kSvdThreads, g.smem, st>>>(d, max_sweeps);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.count * g.cl);
+  cfg.gridDim = dim3(g.count * cl);
   cfg.blockDim = dim3(g.kind == kSvdCluster ? kSvdThreads : kBlockThreads);
   cfg.dynamicSmemBytes = g.smem;
   cfg.stream = st;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = g.cl;
+  at.val.clusterDim.x = cl;
   at.val.clusterDim.y = 1;
   at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   if (g.kind == kSvdTeam) return launch_teams(d, g, max_sweeps, st);
   if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps);
-  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, g.cl, max_sweeps);
+  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, cl, max_sweeps);
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
 }
 
@@ -2111,13 +2693,26 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
   if (e != cudaSuccess) return e;
   // every sector gets a kernel and a cluster size
   std::vector<std::pair<int, int>> key(secs.size());
-  std::vector<int64_t> smem(secs.size(), 0);
+  std::vector<int64_t> smem(secs.size(), 0), small(secs.size(), 0);
   for (size_t k = 0; k < secs.size(); ++k) {
     const SvdSector S = secs[k];
     if (S.mode == kSvdSmem) {
-      key[k] = {kSvdSmem, 1};
+      key[k] = {S.small ? kSvdSmall : kSvdSmem, 1};
       smem[k] = svd_smem_need(S.m, S.n);
+      if (S.small) small[k] = std::max(smem[k], small_layout(S.m, S.n, true).total);
       continue;
+    }
+    if (S.F && std::min(S.m, S.n) <= kFrontSmallK && small_layout(S.m, S.n, false).total <= kSvdSmemMax) {
+      // a one-CTA front; should the FP64 sweeps be needed, a cluster of 2 stages all its block pairs
+      const int cn = S.wide ? std::min(S.m, S.n) : S.n, bw = std::max(2, tune.bw);
+      const int g = std::max(1, (std::min(S.m, S.n) + bw * 2) / (2 * bw * 2));
+      if (g <= kMaxStaged && block_smem_need(S.m, cn, 2, g, g) <= kBlockSmemMax) {
+        key[k] = {kSvdRefine, 1};
+        smem[k] = block_smem_need(S.m, cn, 2, g, g);
+        small[k] = small_layout(S.m, S.n, false).total;
+        secs[k].groups = secs[k].staged = g;
+        continue;
+      }
     }
     // blocks of about tune.bw columns (6 by default); the smallest cluster (tune.cl_min,
     // then doubling up to 8 CTAs) whose CTAs can stage all of their block pairs of a round
@@ -2195,6 +2790,7 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
     }
     groups.back().count++;
     groups.back().smem = std::max<int>(groups.back().smem, (int)smem[k]);
+    groups.back().smem_small = std::max<int>(groups.back().smem_small, (int)small[k]);
     groups.back().max_k = std::max(groups.back().max_k, std::min(secs[k].m, secs[k].n));
     groups.back().max_n = std::max(groups.back().max_n, secs[k].n);
     if (key[k].first == kSvdTeam) {
@@ -2264,6 +2860,7 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
   L.piv_off.assign(ns, -1);
   L.wide.assign(ns, 0);
   L.exact.assign(ns, 0);
+  L.small.assign(ns, 0);
   L.bar_off = -1;
   const int members = team ? kMaxTeam : kMaxCluster;
   L.w2_off.assign(ns, -1);
@@ -2271,7 +2868,7 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
   for (auto* v : {&L.f32_off, &L.n32_off, &L.vd_off, &L.gm_off, &L.a1_off, &L.sel_off, &L.j_off, &L.v_off2, &L.misc_off})
     v->assign(ns, -1);
   L.smem = 0;
-  const int set_k = svd_mixed_min_k(), own_k = std::min(set_k, kRefineMinK);   // 0: off
+  const int set_k = svd_mixed_min_k(), own_k = set_k > 0 ? kRefineMinK : 0;   // 0: off
   int64_t off = 0;
   auto a256 = [](int64_t x) { return (x + 255) & ~int64_t(255); };
   for (int k = 0; k < ns; ++k) {
@@ -2280,6 +2877,8 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     L.exact[k] = exact && exact[k];
     const bool refine = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) >= own_k;
     if (need <= kSvdSmemMax && std::min(m[k], n[k]) < cluster_min_k && !refine) {
+      L.small[k] = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) <= kSmallK &&
+                   small_layout(m[k], n[k], true).total <= kSvdSmemMax;
       L.smem = std::max<int>(L.smem, (int)need);
       continue;
     }
@@ -2329,6 +2928,9 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
 
 void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base) {
   S.mode = L.mode[k];
+  S.small = L.small[k];
+  S.F = nullptr;
+  S.fp32_sweeps = svd_mixed_sweeps();
   if (S.mode != kSvdCluster) return;
   S.work = reinterpret_cast<double2*>(base + L.work_off[k]);
   S.uwork = reinterpret_cast<double2*>(base + L.v_off[k]);
@@ -2365,7 +2967,7 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
     S.rfloor2 = reinterpret_cast<double*>(p);      p += 16;
     S.rnorm = reinterpret_cast<double*>(p);        p += 8 * K;
     S.cexp = reinterpret_cast<int*>(p);            p += 4 * K;
-    S.rdiag = reinterpret_cast<int*>(p);           p += 4 * K;
+    S.vexp = reinterpret_cast<int*>(p);            p += 4 * K;
     S.nrm32 = reinterpret_cast<float*>(p);         p += 4 * K;
     S.sel = reinterpret_cast<int*>(p);             p += 4 * (K + 1);
     S.F = reinterpret_cast<float2*>(base + ((p - base + 255) & ~int64_t(255)));

@@ -201,10 +201,11 @@ struct ThetaTask {            // one (l, r) block pair of one update: sum_m G * 
 struct TileRef { int task; int ti; int tj; };
 
 constexpr int kSvdSmem = 0;          // one CTA, the whole sector in shared memory
-constexpr int kSvdCluster = 1;       // a thread-block cluster, data in L2, round-robin Jacobi
-constexpr int kSvdTeam = 3;          // block Jacobi by teams of CTAs in one cooperative launch
-constexpr int kSvdRefine = 4;        // QR and FP32 Jacobi on a cluster, then tensor-core refinement
-constexpr int kSvdClusterBlock = 2;  // a thread-block cluster, data in L2, block Jacobi staged in shared memory
+constexpr int kSvdSmall = 1;         // the same, refined inside the CTA instead of FP64 sweeps
+constexpr int kSvdCluster = 2;       // a thread-block cluster, data in L2, round-robin Jacobi
+constexpr int kSvdTeam = 4;          // block Jacobi by teams of CTAs in one cooperative launch
+constexpr int kSvdRefine = 5;        // QR and FP32 Jacobi on a cluster, then tensor-core refinement
+constexpr int kSvdClusterBlock = 3;  // a thread-block cluster, data in L2, block Jacobi staged in shared memory
 
 struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   const double2* theta;       // row-major m x n
@@ -219,7 +220,8 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   double2* Y;                 // out: n x min(m, n) column-major right singular vectors
   int* status;                // out: Jacobi sweeps used, or -1 when not converged
   int m, n;
-  int mode;                   // kSvdSmem, kSvdCluster or kSvdClusterBlock
+  int mode;                   // kSvdSmem or kSvdCluster
+  int small;                  // kSvdSmem: refined inside the CTA
   int groups;                 // block Jacobi: block pairs per CTA and round
   int staged;                 // block Jacobi: block pairs staged in shared memory at once
   double floor_rel;           // columns below floor_rel |M|_F are not rotated, their sigma is 0
@@ -242,9 +244,8 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   float2* E;                  // K x K: the scaled correction of a step (overlays F)
   double* rnorm;              // K squared column norms of the current A
   double* rfloor2;            // [0] the floor in the scale of J, [1] the power of two that undoes that scale
-  int* cexp;                  // K scale exponents of the columns of J or A
-  int* rdiag;                 // K: 1 - cosine of the large angles of a step, in units of 2^-30
-  int* rstate;                // [0] columns kept, [1] left to the FP64 sweeps, [2] steps when settled, [4 + step] size of E
+  int *cexp, *vexp;           // K scale exponents of the columns of J or A, and of V
+  int* rstate;                // 16: [0] columns kept, [1] not 0: left to the FP64 sweeps, [2] steps when settled, [4 + step] size of E
   int fp32_sweeps;            // limit of the FP32 sweeps
   unsigned* teambar;          // barrier of the sector's team (nullptr: no teams in this batch)
   int team_first, team_size;  // the team's CTAs in its launch
@@ -258,7 +259,7 @@ struct SvdScratchLayout {
   std::vector<int64_t> f32_off, n32_off, vd_off, gm_off, a1_off, sel_off;   // mixed precision (-1: off)
   std::vector<int64_t> j_off, v_off2, misc_off;       // refinement (-1: off)
   std::vector<int> wide;
-  std::vector<char> exact;
+  std::vector<char> exact, small;
   int64_t bar_off = -1;       // barriers of teams, 64 bytes a sector
   int smem = 0;               // dynamic shared memory of the one-CTA kernel
   int64_t total = 0;
@@ -400,7 +401,8 @@ cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n
                          cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
 struct SvdGroup {
-  int kind, cl, smem, first, count, max_k, max_n;
+  int kind, cl, smem, first, count, max_k, max_n;   // cl 1 of kSvdRefine: a one-CTA front
+  int smem_small;              // dynamic shared memory of svd_small_kernel
   int ctas;                    // kSvdTeam: CTAs of all teams, and the range of their barriers
   unsigned *bar0, *bar1;
 };
@@ -439,7 +441,7 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
 
 // The refinement of sectors that svd_front_kernel has prepared (k_refine.cu): J V, at most
 // kRefineSteps corrections, and the outputs of the sectors that have settled.
-constexpr int kRefineSteps = 5;
+constexpr int kRefineSteps = 6;
 cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max_n, cudaStream_t st);
 
 cudaError_t launch_select(const SelectSector* d_secs, const SelectTask* d_tasks, int n_tasks,
