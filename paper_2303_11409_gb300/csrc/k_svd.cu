@@ -77,8 +77,8 @@ constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps 
 constexpr int kRefineMinK = 25;         // smallest min(m, n) refined on the tensor cores
 // a refined sector's FP32 sweeps end with one that found no cosine above this: it has left about the square
 constexpr float kFp32Stop = 1e-3f;
+constexpr int kFrontThreads = 384;      // one-CTA fronts
 constexpr int kSmallK = 24;             // largest min(m, n) refined inside one CTA
-constexpr int kFrontSmallK = 64;        // largest min(m, n) with a one-CTA front
 // rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
 // a row's dependent FMAs 128)
 constexpr int kAhead = 8;
@@ -1848,12 +1848,17 @@ __host__ __device__ inline SmallLayout small_layout(int m, int n, bool full) {
   const int K = m < n ? m : n;
   SmallLayout L;
   L.ldm = m | 1;
-  L.fld = (n + K) | 1;
+  L.fld = (n + K + 7) / 16 * 16 + 8;      // two neighbouring columns' 8-lane rows fall into different halves of the banks
   L.lda = n | 1;
   int64_t o = 0;
-  L.W = o; o = al(o + 16LL * L.ldm * n);
-  const int64_t f = 8LL * L.fld * K, a = full ? 16LL * L.lda * K : 0;      // A takes F's place
-  L.F = o; o = al(o + (f > a ? f : a));
+  const int64_t w = 16LL * L.ldm * n, f = 8LL * L.fld * K, a = 16LL * L.lda * K;
+  L.W = o;
+  if (full) {      // A takes F's place
+    o = al(o + w);
+    L.F = o; o = al(o + (f > a ? f : a));
+  } else {         // J goes to global memory, then F takes W's place
+    L.F = o; o = al(o + (f > w ? f : w));
+  }
   L.V = o; o = al(o + (full ? 16LL * K * K : 0));
   L.V32 = o; o = al(o + (full ? 8LL * K * K : 0));
   L.E = o; o = al(o + (full ? 8LL * K * K : 0));
@@ -1989,10 +1994,7 @@ __device__ __forceinline__ bool rotation32(float al, float be, float gr, float g
   return true;
 }
 
-// G lanes rotate columns p, q of the FP32 matrix.  Both columns, the rows of the rotations included, are
-// loaded at once and stay in registers when a lane holds at most kHeld of their elements.  Returns the cosine (0: not
-// rotated).
-constexpr int kHeld = 10;
+// G lanes rotate columns p, q of the FP32 matrix in shared memory.  Returns the cosine (0: not rotated).
 __device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, float* nrm, int p, int q, bool valid, int G,
                                             float tol, float floor2) {
   const int gl = threadIdx.x & (G - 1);
@@ -2004,27 +2006,8 @@ __device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, fl
   const bool act = valid && fminf(al, be) > floor2;
   float2* ap = F + (act ? p : 0) * ld;
   float2* aq = F + (act ? q : 0) * ld;
-  const bool held = Rr <= kHeld * G;
-  float2 x[kHeld], y[kHeld];
   float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;
-  if (held) {
-#pragma unroll
-    for (int t = 0; t < kHeld; ++t) {
-      x[t] = y[t] = make_float2(0.f, 0.f);
-      if (act && gl + t * G < Rr) {
-        x[t] = ap[gl + t * G];
-        y[t] = aq[gl + t * G];
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < kHeld; ++t)
-      if (gl + t * G < R) {
-        gr = fmaf(x[t].x, y[t].x, gr);
-        hr = fmaf(x[t].y, y[t].y, hr);
-        gi = fmaf(x[t].x, y[t].y, gi);
-        hi = fmaf(-x[t].y, y[t].x, hi);
-      }
-  } else if (act) {
+  if (act)
 #pragma unroll 4
     for (int i = gl; i < R; i += G) {
       const float2 u = ap[i], v = aq[i];
@@ -2033,7 +2016,6 @@ __device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, fl
       gi = fmaf(u.x, v.y, gi);
       hi = fmaf(-u.y, v.x, hi);
     }
-  }
   gr += hr;
   gi += hi;
   for (int o = G >> 1; o; o >>= 1) {
@@ -2042,36 +2024,22 @@ __device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, fl
   }
   Rot32 T;
   if (!act || !rotation32(al, be, gr, gi, tol, T)) return 0.f;
-  auto turn = [&](float2& a, float2& b) {
-    const float2 ao = a, bo = b;
-    a = make_float2(fmaf(T.cs, ao.x, -fmaf(T.u, bo.x, T.v * bo.y)), fmaf(T.cs, ao.y, -fmaf(T.u, bo.y, -T.v * bo.x)));
-    b = make_float2(fmaf(T.cs, bo.x, fmaf(T.u, ao.x, -T.v * ao.y)), fmaf(T.cs, bo.y, fmaf(T.u, ao.y, T.v * ao.x)));
-  };
-  if (held) {
+  for (int i0 = gl; i0 < Rr; i0 += 4 * G) {
+    float2 a[4], b[4];
 #pragma unroll
-    for (int t = 0; t < kHeld; ++t)
-      if (gl + t * G < Rr) {
-        turn(x[t], y[t]);
-        ap[gl + t * G] = x[t];
-        aq[gl + t * G] = y[t];
+    for (int t = 0; t < 4; ++t)
+      if (i0 + t * G < Rr) {
+        a[t] = ap[i0 + t * G];
+        b[t] = aq[i0 + t * G];
       }
-  } else {
-    for (int i0 = gl; i0 < Rr; i0 += 4 * G) {
-      float2 a[4], b[4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
-        if (i0 + t * G < Rr) {
-          a[t] = ap[i0 + t * G];
-          b[t] = aq[i0 + t * G];
-        }
-#pragma unroll
-      for (int t = 0; t < 4; ++t)
-        if (i0 + t * G < Rr) {
-          turn(a[t], b[t]);
-          ap[i0 + t * G] = a[t];
-          aq[i0 + t * G] = b[t];
-        }
-    }
+    for (int t = 0; t < 4; ++t)
+      if (i0 + t * G < Rr) {
+        ap[i0 + t * G] = make_float2(fmaf(T.cs, a[t].x, -fmaf(T.u, b[t].x, T.v * b[t].y)),
+                                     fmaf(T.cs, a[t].y, -fmaf(T.u, b[t].y, -T.v * b[t].x)));
+        aq[i0 + t * G] = make_float2(fmaf(T.cs, b[t].x, fmaf(T.u, a[t].x, -T.v * a[t].y)),
+                                     fmaf(T.cs, b[t].y, fmaf(T.u, a[t].y, T.v * a[t].x)));
+      }
   }
   if (gl == 0) {
     nrm[p] = fmaxf(al - T.tg, 0.f);
@@ -2080,16 +2048,87 @@ __device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, fl
   return T.c;
 }
 
-// Round-robin FP32 sweeps of one CTA until no pair of a sweep was further than kFp32Stop from orthogonal
-// (each sweep squares the distance, so the sweep that found that has left about its square).
+// FP32 sweeps of one CTA until no pair of a sweep was further than kFp32Stop from orthogonal (each sweep
+// squares the distance, so the sweep that found that has left about its square).
+//
+// Order: the columns are halved, every column of the second half meets every column of the first, then
+// each half is treated alike (as many sweeps as the round-robin order, on sectors of 51-197 columns).  The
+// 8 lanes of a slot keep their column of the second half in registers through a level and pass over the
+// others, E elements a lane, so a pair moves one column through shared memory instead of two.  Columns longer
+// than 8 E, or more than two per slot, go round-robin with both columns in memory.
+template <int G, int E>
+__device__ bool held_level(float2* F, int R, int Rr, int ld, float* nrm, int own, int base, int len, int i, int steps,
+                           float tol, float floor2) {
+  const int gl = threadIdx.x & (G - 1);
+  float2 x[E], y[E];
+  float al = 0.f;
+  float2* ax = F + max(own, 0) * ld;
+  if (own >= 0) al = nrm[own];
+#pragma unroll
+  for (int t = 0; t < E; ++t)
+    if (gl + G * t < Rr) x[t] = ax[gl + G * t];
+  bool far = false;
+  int c = i;      // partner base + (i + step) mod len
+  for (int s = 0; s < steps; ++s) {
+    const bool live = own >= 0 && s < len;
+    const int q = live ? base + c : 0;
+    if (++c >= len) c = 0;
+    const float be = nrm[q];
+    float2* ay = F + q * ld;
+    float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;
+#pragma unroll
+    for (int t = 0; t < E; ++t)
+      if (gl + G * t < Rr) y[t] = ay[gl + G * t];
+#pragma unroll
+    for (int t = 0; t < E; ++t)
+      if (gl + G * t < R) {
+        gr = fmaf(x[t].x, y[t].x, gr);
+        hr = fmaf(x[t].y, y[t].y, hr);
+        gi = fmaf(x[t].x, y[t].y, gi);
+        hi = fmaf(-x[t].y, y[t].x, hi);
+      }
+    const bool act = live && fminf(al, be) > floor2;
+    gr += hr;
+    gi += hi;
+#pragma unroll
+    for (int o = G / 2; o; o >>= 1) {
+      gr += __shfl_xor_sync(0xffffffffu, gr, o);
+      gi += __shfl_xor_sync(0xffffffffu, gi, o);
+    }
+    Rot32 T;
+    if (act && rotation32(al, be, gr, gi, tol, T)) {
+      far |= T.c > kFp32Stop;
+#pragma unroll
+      for (int t = 0; t < E; ++t)
+        if (gl + G * t < Rr) {
+          const float2 a = x[t], b = y[t];
+          x[t] = make_float2(fmaf(T.cs, a.x, -fmaf(T.u, b.x, T.v * b.y)), fmaf(T.cs, a.y, -fmaf(T.u, b.y, -T.v * b.x)));
+          ay[gl + G * t] = make_float2(fmaf(T.cs, b.x, fmaf(T.u, a.x, -T.v * a.y)),
+                                       fmaf(T.cs, b.y, fmaf(T.u, a.y, T.v * a.x)));
+        }
+      al = fmaxf(al - T.tg, 0.f);
+      if (gl == 0) nrm[q] = be + T.tg;
+    }
+    __syncthreads();
+  }
+  if (own >= 0) {
+#pragma unroll
+    for (int t = 0; t < E; ++t)
+      if (gl + G * t < Rr) ax[gl + G * t] = x[t];
+    if (gl == 0) nrm[own] = al;
+  }
+  __syncthreads();
+  return far;
+}
+
+template <int Lanes, int E>      // Lanes 0: the round-robin order
 __device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm, float tol, float floor2,
                              int max_sweeps) {
   __shared__ int s_far;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int mp = K + (K & 1), ring = mp - 1, P = mp / 2;
-  int G = 8;      // lanes a pair: the widest that still does a round in one pass, 8 at least
-  while (G < 32 && 2 * G * P <= (int)blockDim.x && 4 * G < Rr) G *= 2;
-  const int slots = blockDim.x / G, slot = tid / G;
+  int G = 8;      // lanes a pair of the round-robin order
+  while (G < 32 && 4 * G < Rr && 2 * G * P <= (int)blockDim.x) G *= 2;
   for (int sweep = 0; K > 1 && sweep < max_sweeps; ++sweep) {
     for (int j = warp; j < K; j += nwarps) {
       float acc = 0.f;
@@ -2103,23 +2142,36 @@ __device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm
     if (tid == 0) s_far = 0;
     __syncthreads();
     bool far = false;
-    if (P <= slots) {      // one pass a round: the pair of this slot steps round the ring
-      int a = slot % ring, b = (ring - slot % ring) % ring;      // rr_pair(slot, 0) - 1
-      if (slot == 0) b = 0;
-      for (int r = 0; r < ring; ++r) {
-        const int p = slot == 0 ? 0 : a + 1, q = b + 1;
-        const bool valid = slot < P && p < K && q < K;
-        far |= small_pair(F, R, Rr, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop;
-        if (++a == ring) a = 0;
-        if (++b == ring) b = 0;
-        __syncthreads();
+    if constexpr (Lanes > 0) {
+      for (int level = 0; (K - 1) >> level; ++level) {
+        // slot u's column: the u-th of the second halves of this level's segments
+        int u = tid / Lanes, own = -1, base = 0, len = 0;
+        for (int g = 0; g < 1 << level; ++g) {
+          int a = 0, b = K;
+          for (int k = level - 1; k >= 0; --k) {
+            const int h = a + (b - a + 1) / 2;
+            if (g >> k & 1) a = h; else b = h;
+          }
+          const int n2 = (b - a) / 2;
+          if (u < n2) {
+            base = a;
+            len = b - a - n2;
+            own = a + len + u;
+            break;
+          }
+          u -= n2;
+        }
+        const int steps = (((K - 1) >> level) + 2) / 2;      // half of the longest segment, rounded up
+        far |= held_level<Lanes, E>(F, R, Rr, ld, nrm, own, base, len, u, steps, tol, floor2);
       }
     } else {
+      const int slots = blockDim.x / G, slot = tid / G;
       for (int r = 0; r < ring; ++r) {
-        for (int base = 0; base < P; base += slots) {
-          const int k = base + slot;
-          int p = 0, q = 0;
-          if (k < P) rr_pair(k, r, mp, p, q);
+#pragma unroll 1
+        for (int k = slot; k < P + slot; k += slots) {      // rr_pair(k, r), the sums being below 2 ring
+          const int a = k + r - (k + r >= ring ? ring : 0);
+          const int b = k == 0 ? r : ring - k + r - (r >= k ? ring : 0);
+          const int p = k == 0 ? 0 : a + 1, q = b + 1;
           const bool valid = k < P && p < K && q < K;
           far |= small_pair(F, R, Rr, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop;
         }
@@ -2134,12 +2186,15 @@ __device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm
   }
 }
 
-__global__ void __launch_bounds__(kSvdThreads, 1) svd_small_kernel(const SvdSector* __restrict__ secs, int max_sweeps) {
+// Threads: kSvdThreads for whole refinements (up to kSmallK columns), kFrontThreads for fronts: 4 a column, so
+// every pair of a round of up to 96 columns has its 8 lanes.
+template <int Threads>
+__global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* __restrict__ secs, int max_sweeps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_ns, s_theta;
   const SvdSector S = secs[blockIdx.x];
   const int m = S.m, n = S.n, K = min(m, n);
-  const bool full = S.F == nullptr;      // else the front of a sector that the tensor cores refine
+  constexpr bool full = Threads == kSvdThreads;      // else the front of a sector that the tensor cores refine
   const SmallLayout L = small_layout(m, n, full);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   double2* W = reinterpret_cast<double2*>(smem_raw + L.W);
@@ -2194,31 +2249,43 @@ __global__ void __launch_bounds__(kSvdThreads, 1) svd_small_kernel(const SvdSect
     const double frel = fmax(32.0 * kEps, S.floor_rel);
     const double floor2 = fmax(frel * frel * fro2, S.floor_abs * S.floor_abs) * scale * scale;
     qr_small(W, L.ldm, m, n, K, rkk, tau, [&](int j) { return perm[j]; });
-    // R scaled by 2^sc, its diagonal in place; F = [conj R^T; I]
-    for (int e = tid; e < K * n; e += blockDim.x) {
-      const int i = e % K, j = e / K;
-      double2* w = W + (int64_t)perm[j] * L.ldm + i;
-      double2 x = make_double2(0.0, 0.0);
-      if (i <= j) {
-        x = i == j ? rkk[i] : *w;
-        x.x *= scale;
-        x.y *= scale;
-        *w = x;
+    // R scaled by 2^sc; F = [fl32(R^dag); I]
+    if (full) {      // R stays in W, its diagonal in place
+      for (int e = tid; e < K * n; e += blockDim.x) {
+        const int i = e % K, j = e / K;
+        double2* w = W + (int64_t)perm[j] * L.ldm + i;
+        double2 x = make_double2(0.0, 0.0);
+        if (i <= j) {
+          x = i == j ? rkk[i] : *w;
+          x.x *= scale;
+          x.y *= scale;
+          *w = x;
+        }
+        F[(int64_t)i * L.fld + j] = make_float2((float)x.x, (float)-x.y);
       }
-      F[(int64_t)i * L.fld + j] = make_float2((float)x.x, (float)-x.y);
+    } else {         // J = R^dag for the tensor-core kernels
+      for (int e = tid; e < K * n; e += blockDim.x) {
+        const int i = e / n, j = e % n;
+        double2 x = make_double2(0.0, 0.0);
+        if (i <= j) x = i == j ? rkk[i] : W[(int64_t)perm[j] * L.ldm + i];
+        S.J[e] = make_double2(scale * x.x, -scale * x.y);
+      }
+      __syncthreads();
+      for (int e = tid; e < K * n; e += blockDim.x) {
+        const double2 x = S.J[e];
+        F[(int64_t)(e / n) * L.fld + e % n] = make_float2((float)x.x, (float)x.y);
+      }
     }
     for (int e = tid; e < K * K; e += blockDim.x)
       F[(int64_t)(e / K) * L.fld + n + e % K] = make_float2(e / K == e % K ? 1.f : 0.f, 0.f);
     __syncthreads();
-    if (!full)
-      for (int e = tid; e < K * n; e += blockDim.x) {      // J = R^dag for the tensor-core kernels
-        const int i = e / n, j = e % n;
-        double2 x = make_double2(0.0, 0.0);
-        if (i <= j) x = W[(int64_t)perm[j] * L.ldm + i];
-        S.J[e] = make_double2(x.x, -x.y);
-      }
     const float tol32 = 1.1920929e-07f * (float)max(n, 32), fl32 = (float)(0.01 * floor2);
-    small_sweeps(F, n, n + K, L.fld, K, nrm, tol32, fl32, min(max_sweeps, S.fp32_sweeps + 6));
+    const int slots = K / 2, Rr = n + K, sweeps = min(max_sweeps, S.fp32_sweeps + 6);
+    if (full && slots <= Threads / 32 && Rr <= 96) small_sweeps<32, 3>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (slots <= Threads / 16 && Rr <= 96) small_sweeps<16, 6>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (slots <= Threads / 16 && Rr <= 192) small_sweeps<16, 12>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (!full && slots <= Threads / 8 && Rr <= 192) small_sweeps<8, 24>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
+    else small_sweeps<0, 0>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
     for (int j = warp; j < K; j += nwarps) {
       float acc = 0.f;
       for (int i = lane; i < n; i += 32) {
@@ -2395,7 +2462,7 @@ __global__ void __launch_bounds__(kSvdThreads, 1) svd_small_kernel(const SvdSect
     }
   }
   __syncthreads();
-  cta_sector(S, smem_raw, max_sweeps);      // the FP64 sweeps, from the start
+  if constexpr (full) cta_sector(S, smem_raw, max_sweeps);      // the FP64 sweeps, from the start
 }
 
 __device__ __forceinline__ Work cluster_work(const SvdSector& S) {
@@ -2497,6 +2564,7 @@ int64_t svd_smem_need(int m, int n) { return smem_layout(m, n).total; }
 namespace {
 
 constexpr int kBlockSmemMax = 110 * 1024;   // two block-Jacobi CTAs per SM
+constexpr int kFrontSmemMax = 216 * 1024;   // one-CTA fronts
 // 8 CTAs per large sector: the GPU places about twice as many 8-CTA clusters as
 // 16-CTA ones, which keeps more SMs busy when a layer has hundreds of large sectors
 constexpr int kBigCluster = 8;
@@ -2524,7 +2592,10 @@ cudaError_t set_attrs(int* big_out) {
   }
   e = cudaFuncSetAttribute(jacobi_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemMax);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(svd_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSvdSmemMax);
+    e = cudaFuncSetAttribute(svd_small_kernel<kSvdThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFrontSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(svd_small_kernel<kFrontThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kFrontSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBlockSmemMax);
@@ -2597,7 +2668,10 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   const SvdSector* d = d_secs + g.first;
   count_launch();
   if (g.kind == kSvdSmall || (g.kind == kSvdRefine && g.cl == 1 && !fallback)) {
-    svd_small_kernel<<<g.count, kSvdThreads, g.smem_small, st>>>(d, max_sweeps);
+    if (g.kind == kSvdRefine)
+      svd_small_kernel<kFrontThreads><<<g.count, kFrontThreads, g.smem_small, st>>>(d, max_sweeps);
+    else
+      svd_small_kernel<kSvdThreads><<<g.count, kSvdThreads, g.smem_small, st>>>(d, max_sweeps);
     return cudaGetLastError();
   }
   const int cl = g.kind == kSvdRefine && g.cl == 1 ? 2 : g.cl;      // a one-CTA front falls back to a cluster of 2
@@ -2702,7 +2776,7 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
       if (S.small) small[k] = std::max(smem[k], small_layout(S.m, S.n, true).total);
       continue;
     }
-    if (S.F && std::min(S.m, S.n) <= kFrontSmallK && small_layout(S.m, S.n, false).total <= kSvdSmemMax) {
+    if (S.F && small_layout(S.m, S.n, false).total <= kFrontSmemMax) {
       // a one-CTA front; should the FP64 sweeps be needed, a cluster of 2 stages all its block pairs
       const int cn = S.wide ? std::min(S.m, S.n) : S.n, bw = std::max(2, tune.bw);
       const int g = std::max(1, (std::min(S.m, S.n) + bw * 2) / (2 * bw * 2));

@@ -401,7 +401,7 @@ cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n
                          cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
 struct SvdGroup {
-  int kind, cl, smem, first, count, max_k, max_n;   // cl 1 of kSvdRefine: a one-CTA front
+  int kind, cl, smem, first, count, max_k, max_n;   // cl 1, 0 of kSvdRefine: one-CTA fronts
   int smem_small;              // dynamic shared memory of svd_small_kernel
   int ctas;                    // kSvdTeam: CTAs of all teams, and the range of their barriers
   unsigned *bar0, *bar1;
