@@ -62,6 +62,7 @@
 #include <vector>
 
 #include "mps_internal.h"
+#include "jacobi32.cuh"
 #include "refine_pair.cuh"
 
 namespace mps {
@@ -710,7 +711,7 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // (possibly tiny) inner product: |g| against tol sqrt(alpha beta), t = tan(theta) from
 // zeta = (beta - alpha) / (2 |g|).
 __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int p, int q, bool valid, int G,
-                              float tol, float floor2, float stop) {
+                              float tol, float floor2) {
   const int gl = threadIdx.x & (G - 1);
   float alpha = 0.f, beta = 0.f;
   if (valid) {
@@ -733,7 +734,6 @@ __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int 
   }
   const float ag = hypotf(gr, gi);
   act = act && (ag > tol * sqrtf(alpha) * sqrtf(beta));
-  const float far = stop * sqrtf(alpha) * sqrtf(beta);
   if (act) {
     const float zeta = (beta - alpha) / (2.f * ag), az = fabsf(zeta);
     const float t = copysignf(1.f, zeta) / (az + (az < 1e18f ? sqrtf(fmaf(zeta, zeta, 1.f)) : az));
@@ -751,7 +751,7 @@ __device__ bool jacobi_pair32(float2* A, int R, int Rr, int ld, float* nrm, int 
       nrm[q] = beta + tg;
     }
   }
-  return act && ag > far;
+  return act;
 }
 
 __device__ __forceinline__ int group_width32(int P, int R, int nwarps) {
@@ -774,7 +774,6 @@ struct JacobiBlocks32 {
   float2* sm;
   float* smn;
   int bsmax, g, gs, cl0;      // as in JacobiBlocks
-  float stop = 0.f;           // a sweep whose rotations all had cosines up to this is the last one
   __device__ int staged_with(int p) const {
     const int q = p / cl0;
     return min(gs, g - q / gs * gs);
@@ -858,7 +857,7 @@ struct JacobiBlocks32 {
                   valid = a < s_len32[j] && b < s_len32[j];
                 }
                 rot |= jacobi_pair32(sm, R, Rr, ld, smn, j * bsmax + min(a, b), j * bsmax + max(a, b), valid, G,
-                                     tol, floor2, stop);
+                                     tol, floor2);
               }
               __syncthreads();
             }
@@ -883,7 +882,7 @@ struct JacobiBlocks32 {
                     q = max(pa, pb);
                   }
                 }
-                rot |= jacobi_pair32(sm, R, Rr, ld, smn, p, q, valid, G, tol, floor2, stop);
+                rot |= jacobi_pair32(sm, R, Rr, ld, smn, p, q, valid, G, tol, floor2);
               }
               __syncthreads();
             }
@@ -1182,9 +1181,228 @@ __device__ void qr_columns(T2* A, int64_t ld, int rows, int ncol, int K, T2* rkk
   sync();
 }
 
+// FP32 block-Jacobi sweeps of a front: the K columns of F (column c at F + c * ld, its rows in pairs) in
+// 2 cl g blocks, paired by the round-robin order, CTA `rank` at its positions rank g .. rank g + g - 1.  Between
+// two rounds every position passes its blocks on to its neighbours, so of the 2 g blocks that a CTA holds it
+// keeps all but two in shared memory: it stores those to F and, past the cluster barrier, loads the two that
+// arrive.  A CTA whose shared memory holds only gs < g pairs goes through them gs at a time.
+// A block pair's shorter block is held in registers, E row pairs a lane of the G lanes of a slot, and meets
+// the columns of the other (G = 0: columns too long for that, both in memory).
+// A round's exchange takes some 6 us (stores 2.5, the barrier and its slowest CTA 2, loads 1.5), a step 1-1.7 us.
+// With every block staged in every round and (re, im) columns read and written for each rotation, a layer at
+// chi = 333 (L = 33) took 32.1 ms and one at chi = 512 (L = 32) 86.9, now 28.6 and 73.6.
+struct FrontBlocks {
+  float2* sm;
+  float* smn;
+  int bsmax, g, gs, cl;
+
+  struct Tables {      // one per CTA
+    int held[2 * kMaxStaged];      // the block in each slot (-1: none)
+    int col[2 * kMaxStaged], len[2 * kMaxStaged];
+    int at[2 * kMaxStaged];        // the slot of each block of the stage: pair j's at 2 j and 2 j + 1
+    int fresh[2 * kMaxStaged];     // the slot was loaded for this stage
+    int swap[kMaxStaged];          // pair j's shorter block is the second
+    int most;                      // columns of the stage's longest block
+    uint64_t bar;
+  };
+
+  // Makes the slots hold the blocks of stage (r, c0), or none with r < 0; barrier(): between stores and loads.
+  template <class Barrier>
+  __device__ __forceinline__ void stage(Tables& T, float2* F, int ld, int K, float* nrm, int rank, int r, int c0,
+                                        uint32_t& parity, Barrier barrier) const {
+    const int tid = threadIdx.x, lane = tid & 31, nb = 2 * cl * g, slots = 2 * gs;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+    int to = -1, want = -1, col = 0, len = 0;
+    if (tid < 32) {
+      const int held = lane < slots ? T.held[lane] : -1, j = lane >> 1;
+      if (r >= 0 && lane < slots && c0 + j < g) {
+        int bp, bq;
+        rr_pair(rank * g + c0 + j, r, nb, bp, bq);
+        want = lane & 1 ? bq : bp;
+        col = (int)((int64_t)K * want / nb);
+        len = (int)((int64_t)K * (want + 1) / nb) - col;
+      }
+      bool stays = false;
+      for (int s = 0; s < slots; ++s) {
+        if (__shfl_sync(0xffffffffu, held, s) == want && want >= 0) to = s;
+        if (__shfl_sync(0xffffffffu, want, s) == held && held >= 0) stays = true;
+      }
+      if (held >= 0 && !stays) {
+        const int from = T.col[lane], n = T.len[lane];
+        for (int c = 0; c < n; ++c) {
+          bulk_store(F + (int64_t)(from + c) * ld, sm + (lane * bsmax + c) * ld, (uint32_t)ld * 8u);
+          __stcg(nrm + from + c, smn[lane * bsmax + c]);
+        }
+      }
+      bulk_store_drain();
+      unsigned room = __ballot_sync(0xffffffffu, lane < slots && !stays);
+      const bool load = want >= 0 && to < 0;
+      const unsigned loads = __ballot_sync(0xffffffffu, load);
+      for (int i = __popc(loads & ((1u << lane) - 1)); i; --i) room &= room - 1;
+      if (load) to = __ffs(room) - 1;
+      __syncwarp();
+      if (lane < slots) {
+        T.fresh[lane] = 0;
+        if (!stays) T.held[lane] = -1;
+      }
+      __syncwarp();
+      if (want >= 0) {
+        T.at[lane] = to;
+        T.held[to] = want;
+        T.col[to] = col;
+        T.len[to] = len;
+        T.fresh[to] = load;
+      }
+      const int other = __shfl_xor_sync(0xffffffffu, len, 1);
+      if (want >= 0 && !(lane & 1)) T.swap[j] = len > other;
+      const int most = __reduce_max_sync(0xffffffffu, len);
+      if (lane == 0) T.most = most;
+      __syncwarp();
+    }
+    barrier();
+    if (r < 0) return;
+    if (tid < 32) {
+      const bool load = want >= 0 && T.fresh[to];
+      int bytes = load ? len * ld * 8 : 0;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
+      fence_to_async();
+      if (lane == 0) stage_expect(&T.bar, (uint32_t)bytes);
+      __syncwarp();
+      if (load)
+        for (int c = 0; c < len; ++c)
+          bulk_load(sm + (to * bsmax + c) * ld, F + (int64_t)(col + c) * ld, (uint32_t)ld * 8u, &T.bar);
+    }
+    for (int e = tid; e < slots * bsmax; e += blockDim.x) {
+      const int s = e / bsmax, c = e % bsmax;
+      if (T.held[s] >= 0 && T.fresh[s] && c < T.len[s]) smn[e] = __ldcg(nrm + T.col[s] + c);
+    }
+    stage_wait(&T.bar, parity);
+    parity ^= 1u;
+    __syncthreads();
+  }
+
+  template <int G, int E, class Sync>
+  __device__ void sweeps(Tables& T, float2* F, int R2, int Rr2, int ld, int K, float* nrm, int* flags, int rank,
+                         Sync sync, float tol, float floor2, int max_sweeps) const {
+    const int tid = threadIdx.x, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int ring = 2 * cl * g - 1;
+    uint32_t parity = 0;
+    if (tid == 0) stage_bar_init(&T.bar);
+    if (tid < 2 * gs) T.held[tid] = -1;
+    __syncthreads();
+    stage(T, F, ld, K, nrm, rank, 0, 0, parity, [] { __syncthreads(); });
+    for (int sweep = 0;; ++sweep) {
+      bool far = false;
+      for (int r = 0; r < ring; ++r)
+        for (int c0 = 0; c0 < g; c0 += gs) {
+          const int ns = min(gs, g - c0);
+          if (r == 0) {      // fresh norms, and the pairs inside each block
+            for (int e = warp; e < 2 * ns * bsmax; e += nwarps) {
+              const int s = T.at[e / bsmax], c = e % bsmax;
+              if (c < T.len[s]) norm32(sm + (s * bsmax + c) * ld, R2, smn + s * bsmax + c);
+            }
+            __syncthreads();
+            const int mpb = bsmax + (bsmax & 1), P = 2 * ns * (mpb / 2);
+            const int W = group_width32(P, 2 * R2, nwarps), slots = blockDim.x / W;
+            for (int rr = 0; rr < mpb - 1; ++rr) {
+              for (int k0 = 0; k0 < P; k0 += slots) {
+                const int k = k0 + tid / W;
+                int a = 0, b = 0, s = 0;
+                bool valid = k < P;
+                if (valid) {
+                  s = T.at[k / (mpb / 2)];
+                  rr_pair(k % (mpb / 2), rr, mpb, a, b);
+                  valid = a < T.len[s] && b < T.len[s];
+                }
+                far |= pair32(sm, R2, Rr2, ld, smn, s * bsmax + min(a, b), s * bsmax + max(a, b), valid, W, tol,
+                              floor2) > kFp32Stop * kFp32Stop;
+              }
+              __syncthreads();
+            }
+          }
+          const int most = T.most, P = ns * most;
+          if constexpr (G > 0) {
+            constexpr int slots = kBlockThreads / G;
+            for (int k0 = 0; k0 < P; k0 += slots) {
+              const int k = k0 + tid / G, j = k / most, i = k % most;
+              int own = 0, base = 0, sb = 0;
+              bool on = k < P;
+              if (on) {
+                const int sa = T.at[2 * j + T.swap[j]], so = T.at[2 * j + 1 - T.swap[j]];
+                own = sa * bsmax + i;
+                base = so * bsmax;
+                sb = T.len[so];
+                on = i < T.len[sa];
+              }
+              Held32<G, E> x;
+              if (on) x.load(sm + own * ld, Rr2, smn[own]);
+              int c = i;      // it meets base + (i + t) mod sb
+              for (int t = 0; t < most; ++t) {
+                const bool live = on && t < sb;
+                const int q = live ? base + c : 0;
+                if (++c >= sb) c = 0;
+                far |= x.meet(sm + q * ld, smn + q, R2, Rr2, live, tol, floor2) > kFp32Stop * kFp32Stop;
+                __syncthreads();
+              }
+              if (on) {
+                x.store(sm + own * ld, Rr2);
+                if ((tid & (G - 1)) == 0) smn[own] = x.al;
+              }
+            }
+          } else {
+            const int W = group_width32(P, 2 * R2, nwarps), slots = blockDim.x / W;
+            for (int t = 0; t < most; ++t) {
+              for (int k0 = 0; k0 < P; k0 += slots) {
+                const int k = k0 + tid / W, j = k / most, i = k % most;
+                int p = 0, q = 0;
+                bool valid = k < P;
+                if (valid) {
+                  const int sa = T.at[2 * j + T.swap[j]], so = T.at[2 * j + 1 - T.swap[j]];
+                  valid = i < T.len[sa] && t < T.len[so];
+                  if (valid) {
+                    p = sa * bsmax + i;
+                    q = so * bsmax + (i + t) % T.len[so];
+                  }
+                }
+                far |= pair32(sm, R2, Rr2, ld, smn, p, q, valid, W, tol, floor2) > kFp32Stop * kFp32Stop;
+              }
+              __syncthreads();
+            }
+          }
+          const bool over = c0 + gs >= g, last = over && r + 1 == ring;
+          if (!last) {
+            if (over) stage(T, F, ld, K, nrm, rank, r + 1, 0, parity, sync);
+            else stage(T, F, ld, K, nrm, rank, r, c0 + gs, parity, [] { __syncthreads(); });
+          }
+        }
+      if (__syncthreads_or(far) && tid == 0) __stcg(flags + sweep, 1);
+      bool done = false;
+      stage(T, F, ld, K, nrm, rank, 0, 0, parity, [&] {
+        sync();
+        done = __ldcg(flags + sweep) == 0 || sweep + 1 >= max_sweeps;
+      });
+      if (done) break;
+    }
+    stage(T, F, ld, K, nrm, rank, -1, 0, parity, sync);
+  }
+
+  template <class Sync>
+  __device__ void operator()(float2* F, int R2, int Rr2, int ld, int K, float* nrm, int* flags, int rank, Sync sync,
+                             float tol, float floor2, int max_sweeps) const {
+    __shared__ Tables T;
+    if (max_sweeps < 1) return;
+    if (Rr2 <= 192) sweeps<16, 12>(T, F, R2, Rr2, ld, K, nrm, flags, rank, sync, tol, floor2, max_sweeps);
+    else if (Rr2 <= 256) sweeps<32, 8>(T, F, R2, Rr2, ld, K, nrm, flags, rank, sync, tol, floor2, max_sweeps);
+    else if (Rr2 <= 384) sweeps<32, 12>(T, F, R2, Rr2, ld, K, nrm, flags, rank, sync, tol, floor2, max_sweeps);
+    else sweeps<0, 0>(T, F, R2, Rr2, ld, K, nrm, flags, rank, sync, tol, floor2, max_sweeps);
+  }
+};
+
 template <class Sync>
 __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas, Sync sync, int max_sweeps,
-                          const JacobiBlocks32& j32, unsigned char* smem) {
+                          const FrontBlocks& j32, unsigned char* smem) {
   const int m = S.m, n = S.n, K = min(m, n);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int tid_all = rank * blockDim.x + tid, threads_all = nctas * blockDim.x;
@@ -1249,10 +1467,9 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
   double2* J = S.J;
   const bool wide = S.wide;
   const int jlen = wide ? K : n;
-  const int Rr = jlen + K, fld = (Rr + 1) & ~1;   // even: columns 16-byte aligned for bulk copies
+  const int vr = even32(jlen), fld = vr + even32(K);      // the rotations' first row, the columns' stride
   float2* F = S.F;
-  float2* F1 = wide ? reinterpret_cast<float2*>(S.A1) : F;     // FP32 J: n x K for the second QR, or in place
-  const int64_t ld1 = wide ? n : fld;
+  float2* F1 = reinterpret_cast<float2*>(S.A1);     // wide: FP32 J, n x K, for a second QR
   {
     const int tr = (K + 3) / 4, tc = (n + 7) / 8;
     for (int64_t t = worker; t < (int64_t)tr * tc; t += workers) {
@@ -1264,7 +1481,9 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
         x.x *= scale;
         x.y *= -scale;
         J[(int64_t)i * n + j] = x;
-        __stcg(F1 + (int64_t)i * ld1 + j, make_float2((float)x.x, (float)x.y));
+        const float2 f = make_float2((float)x.x, (float)x.y);
+        if (wide) __stcg(F1 + (int64_t)i * n + j, f);
+        else set_row32(F + (int64_t)i * fld, j, f);
       }
     }
   }
@@ -1280,12 +1499,12 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
       float2 v = make_float2(0.f, 0.f);
       if (i == c) v = __ldcg(rk + c);
       else if (i < c) v = __ldcg(F1 + (int64_t)c * n + i);
-      __stcg(F + (int64_t)c * fld + i, v);
+      set_row32(F + (int64_t)c * fld, i, v);
     }
   }
   for (int64_t e = tid_all; e < (int64_t)K * (fld - jlen); e += threads_all) {   // V = I below
-    const int c = (int)(e / (fld - jlen)), i = (int)(e % (fld - jlen));
-    __stcg(F + (int64_t)c * fld + jlen + i, make_float2(i == c ? 1.f : 0.f, 0.f));
+    const int c = (int)(e / (fld - jlen)), i = jlen + (int)(e % (fld - jlen));
+    set_row32(F + (int64_t)c * fld, i, make_float2(i - vr == c ? 1.f : 0.f, 0.f));
   }
   sync();
   // ---- FP32 sweeps to FP32 convergence; the floor is a tenth of the FP64 one -------------------
@@ -1293,12 +1512,11 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
   __syncthreads();
   const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
   const float fl32 = (float)(0.01 * floor2);
-  bool conv32 = false;
-  j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps + 6), conv32);
-  for (int j = worker; j < K; j += workers) {   // final FP32 norms
+  j32(F, vr / 2, fld / 2, fld, K, S.nrm32, w.flags, rank, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps + 6));
+  for (int j = worker; j < K; j += workers) {   // final FP32 norms, past what L1 holds of the columns
     const float2* a = F + (int64_t)j * fld;
     float acc = 0.f;
-    for (int i = lane; i < jlen; i += 32) {
+    for (int i = lane; i < vr; i += 32) {
       const float2 x = __ldcg(a + i);
       acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
     }
@@ -1323,8 +1541,8 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
   const int ns = __ldcg(S.rstate);
   for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) {
     const int t = (int)(e / K), k = (int)(e % K);
-    const float2 v = __ldcg(F + (int64_t)__ldcg(S.sel + t) * fld + jlen + k);
-    S.V0[e] = make_double2((double)v.x, (double)v.y);
+    const float* v = reinterpret_cast<const float*>(F + (int64_t)__ldcg(S.sel + t) * fld + vr + (k & ~1)) + (k & 1);
+    S.V0[e] = make_double2((double)__ldcg(v), (double)__ldcg(v + 2));
   }
 }
 
@@ -1848,7 +2066,7 @@ __host__ __device__ inline SmallLayout small_layout(int m, int n, bool full) {
   const int K = m < n ? m : n;
   SmallLayout L;
   L.ldm = m | 1;
-  L.fld = (n + K + 7) / 16 * 16 + 8;      // two neighbouring columns' 8-lane rows fall into different halves of the banks
+  L.fld = even32(n) + even32(K);
   L.lda = n | 1;
   int64_t o = 0;
   const int64_t w = 16LL * L.ldm * n, f = 8LL * L.fld * K, a = 16LL * L.lda * K;
@@ -1961,184 +2179,20 @@ __device__ void qr_small(double2* A, int ld, int rows, int ncol, int K, double2*
   __syncthreads();
 }
 
-__device__ __forceinline__ float rsqrt_fast(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float rcp_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// The Jacobi rotation of two FP32 columns with squared norms al, be and inner product (gr, gi), from their
-// cosine c and the ratio of their norms, so that nothing is squared below the range of FP32: cs, (u, v) = the
-// sine times the phase, tg = the change of the norms.  False when c <= tol.
-struct Rot32 { float cs, u, v, tg, c; };
-__device__ __forceinline__ bool rotation32(float al, float be, float gr, float gi, float tol, Rot32& R) {
-  const float ra = rsqrt_fast(al), rb = rsqrt_fast(be);
-  const float sr = gr * ra * rb, si = gi * ra * rb;
-  const float c2 = fmaf(sr, sr, si * si);
-  if (!(c2 > tol * tol)) return false;
-  const float ic = rsqrt_fast(c2), sa = al * ra, sb = be * rb;
-  R.c = c2 * ic;
-  const float z = fminf(fmaxf(0.5f * (sb * ra - sa * rb) * ic, -1e17f), 1e17f);
-  const float h = fmaf(z, z, 1.f);
-  const float t = copysignf(rcp_fast(fabsf(z) + h * rsqrt_fast(h)), z);
-  R.cs = rsqrt_fast(fmaf(t, t, 1.f));
-  const float f = R.cs * t * ic;
-  R.u = f * sr;
-  R.v = f * si;
-  R.tg = t * R.c * sa * sb;
-  return true;
-}
-
-// G lanes rotate columns p, q of the FP32 matrix in shared memory.  Returns the cosine (0: not rotated).
-__device__ __forceinline__ float small_pair(float2* F, int R, int Rr, int ld, float* nrm, int p, int q, bool valid, int G,
-                                            float tol, float floor2) {
-  const int gl = threadIdx.x & (G - 1);
-  float al = 0.f, be = 0.f;
-  if (valid) {
-    al = nrm[p];
-    be = nrm[q];
-  }
-  const bool act = valid && fminf(al, be) > floor2;
-  float2* ap = F + (act ? p : 0) * ld;
-  float2* aq = F + (act ? q : 0) * ld;
-  float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;
-  if (act)
-#pragma unroll 4
-    for (int i = gl; i < R; i += G) {
-      const float2 u = ap[i], v = aq[i];
-      gr = fmaf(u.x, v.x, gr);
-      hr = fmaf(u.y, v.y, hr);
-      gi = fmaf(u.x, v.y, gi);
-      hi = fmaf(-u.y, v.x, hi);
-    }
-  gr += hr;
-  gi += hi;
-  for (int o = G >> 1; o; o >>= 1) {
-    gr += __shfl_xor_sync(0xffffffffu, gr, o);
-    gi += __shfl_xor_sync(0xffffffffu, gi, o);
-  }
-  Rot32 T;
-  if (!act || !rotation32(al, be, gr, gi, tol, T)) return 0.f;
-  for (int i0 = gl; i0 < Rr; i0 += 4 * G) {
-    float2 a[4], b[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-      if (i0 + t * G < Rr) {
-        a[t] = ap[i0 + t * G];
-        b[t] = aq[i0 + t * G];
-      }
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-      if (i0 + t * G < Rr) {
-        ap[i0 + t * G] = make_float2(fmaf(T.cs, a[t].x, -fmaf(T.u, b[t].x, T.v * b[t].y)),
-                                     fmaf(T.cs, a[t].y, -fmaf(T.u, b[t].y, -T.v * b[t].x)));
-        aq[i0 + t * G] = make_float2(fmaf(T.cs, b[t].x, fmaf(T.u, a[t].x, -T.v * a[t].y)),
-                                     fmaf(T.cs, b[t].y, fmaf(T.u, a[t].y, T.v * a[t].x)));
-      }
-  }
-  if (gl == 0) {
-    nrm[p] = fmaxf(al - T.tg, 0.f);
-    nrm[q] = be + T.tg;
-  }
-  return T.c;
-}
-
 // FP32 sweeps of one CTA until no pair of a sweep was further than kFp32Stop from orthogonal (each sweep
 // squares the distance, so the sweep that found that has left about its square).
 //
 // Order: the columns are halved, every column of the second half meets every column of the first, then
 // each half is treated alike (as many sweeps as the round-robin order, on sectors of 51-197 columns).  The
-// 8 lanes of a slot keep their column of the second half in registers through a level and pass over the
-// others, E elements a lane, so a pair moves one column through shared memory instead of two.  Columns longer
-// than 8 E, or more than two per slot, go round-robin with both columns in memory.
-template <int G, int E>
-__device__ bool held_level(float2* F, int R, int Rr, int ld, float* nrm, int own, int base, int len, int i, int steps,
-                           float tol, float floor2) {
-  const int gl = threadIdx.x & (G - 1);
-  float2 x[E], y[E];
-  float al = 0.f;
-  float2* ax = F + max(own, 0) * ld;
-  if (own >= 0) al = nrm[own];
-#pragma unroll
-  for (int t = 0; t < E; ++t)
-    if (gl + G * t < Rr) x[t] = ax[gl + G * t];
-  bool far = false;
-  int c = i;      // partner base + (i + step) mod len
-  for (int s = 0; s < steps; ++s) {
-    const bool live = own >= 0 && s < len;
-    const int q = live ? base + c : 0;
-    if (++c >= len) c = 0;
-    const float be = nrm[q];
-    float2* ay = F + q * ld;
-    float gr = 0.f, gi = 0.f, hr = 0.f, hi = 0.f;
-#pragma unroll
-    for (int t = 0; t < E; ++t)
-      if (gl + G * t < Rr) y[t] = ay[gl + G * t];
-#pragma unroll
-    for (int t = 0; t < E; ++t)
-      if (gl + G * t < R) {
-        gr = fmaf(x[t].x, y[t].x, gr);
-        hr = fmaf(x[t].y, y[t].y, hr);
-        gi = fmaf(x[t].x, y[t].y, gi);
-        hi = fmaf(-x[t].y, y[t].x, hi);
-      }
-    const bool act = live && fminf(al, be) > floor2;
-    gr += hr;
-    gi += hi;
-#pragma unroll
-    for (int o = G / 2; o; o >>= 1) {
-      gr += __shfl_xor_sync(0xffffffffu, gr, o);
-      gi += __shfl_xor_sync(0xffffffffu, gi, o);
-    }
-    Rot32 T;
-    if (act && rotation32(al, be, gr, gi, tol, T)) {
-      far |= T.c > kFp32Stop;
-#pragma unroll
-      for (int t = 0; t < E; ++t)
-        if (gl + G * t < Rr) {
-          const float2 a = x[t], b = y[t];
-          x[t] = make_float2(fmaf(T.cs, a.x, -fmaf(T.u, b.x, T.v * b.y)), fmaf(T.cs, a.y, -fmaf(T.u, b.y, -T.v * b.x)));
-          ay[gl + G * t] = make_float2(fmaf(T.cs, b.x, fmaf(T.u, a.x, -T.v * a.y)),
-                                       fmaf(T.cs, b.y, fmaf(T.u, a.y, T.v * a.x)));
-        }
-      al = fmaxf(al - T.tg, 0.f);
-      if (gl == 0) nrm[q] = be + T.tg;
-    }
-    __syncthreads();
-  }
-  if (own >= 0) {
-#pragma unroll
-    for (int t = 0; t < E; ++t)
-      if (gl + G * t < Rr) ax[gl + G * t] = x[t];
-    if (gl == 0) nrm[own] = al;
-  }
-  __syncthreads();
-  return far;
-}
-
-template <int Lanes, int E>      // Lanes 0: the round-robin order
-__device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm, float tol, float floor2,
+// Lanes lanes of a slot hold their column of the second half in registers through a level.  Columns longer than
+// 2 Lanes E rows, or more of them than slots, go round-robin with both columns in memory (Lanes = 0).
+template <int Lanes, int E>
+__device__ void small_sweeps(float2* F, int R2, int Rr2, int ld, int K, float* nrm, float tol, float floor2,
                              int max_sweeps) {
   __shared__ int s_far;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  const int mp = K + (K & 1), ring = mp - 1, P = mp / 2;
-  int G = 8;      // lanes a pair of the round-robin order
-  while (G < 32 && 4 * G < Rr && 2 * G * P <= (int)blockDim.x) G *= 2;
+  const int tid = threadIdx.x, warp = tid >> 5, nwarps = blockDim.x >> 5;
   for (int sweep = 0; K > 1 && sweep < max_sweeps; ++sweep) {
-    for (int j = warp; j < K; j += nwarps) {
-      float acc = 0.f;
-      for (int i = lane; i < R; i += 32) {
-        const float2 x = F[j * ld + i];
-        acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
-      }
-      acc = warp_sum_f(acc);
-      if (lane == 0) nrm[j] = acc;
-    }
+    for (int j = warp; j < K; j += nwarps) norm32(F + j * ld, R2, nrm + j);
     if (tid == 0) s_far = 0;
     __syncthreads();
     bool far = false;
@@ -2162,9 +2216,26 @@ __device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm
           u -= n2;
         }
         const int steps = (((K - 1) >> level) + 2) / 2;      // half of the longest segment, rounded up
-        far |= held_level<Lanes, E>(F, R, Rr, ld, nrm, own, base, len, u, steps, tol, floor2);
+        Held32<Lanes, E> x;
+        x.load(F + max(own, 0) * ld, Rr2, nrm[max(own, 0)]);
+        int c = u;                                           // it meets base + (u + step) mod len
+        for (int s = 0; s < steps; ++s) {
+          const bool live = own >= 0 && s < len;
+          const int q = live ? base + c : 0;
+          if (++c >= len) c = 0;
+          far |= x.meet(F + q * ld, nrm + q, R2, Rr2, live, tol, floor2) > kFp32Stop * kFp32Stop;
+          __syncthreads();
+        }
+        if (own >= 0) {
+          x.store(F + own * ld, Rr2);
+          if ((tid & (Lanes - 1)) == 0) nrm[own] = x.al;
+        }
+        __syncthreads();
       }
     } else {
+      const int mp = K + (K & 1), ring = mp - 1, P = mp / 2;
+      int G = 8;
+      while (G < 32 && 4 * G < Rr2 && 2 * G * P <= (int)blockDim.x) G *= 2;
       const int slots = blockDim.x / G, slot = tid / G;
       for (int r = 0; r < ring; ++r) {
 #pragma unroll 1
@@ -2173,7 +2244,7 @@ __device__ void small_sweeps(float2* F, int R, int Rr, int ld, int K, float* nrm
           const int b = k == 0 ? r : ring - k + r - (r >= k ? ring : 0);
           const int p = k == 0 ? 0 : a + 1, q = b + 1;
           const bool valid = k < P && p < K && q < K;
-          far |= small_pair(F, R, Rr, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop;
+          far |= pair32(F, R2, Rr2, ld, nrm, min(p, q), max(p, q), valid, G, tol, floor2) > kFp32Stop * kFp32Stop;
         }
         __syncthreads();
       }
@@ -2261,7 +2332,7 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
           x.y *= scale;
           *w = x;
         }
-        F[(int64_t)i * L.fld + j] = make_float2((float)x.x, (float)-x.y);
+        set_row32(F + i * L.fld, j, make_float2((float)x.x, (float)-x.y));
       }
     } else {         // J = R^dag for the tensor-core kernels
       for (int e = tid; e < K * n; e += blockDim.x) {
@@ -2273,28 +2344,23 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
       __syncthreads();
       for (int e = tid; e < K * n; e += blockDim.x) {
         const double2 x = S.J[e];
-        F[(int64_t)(e / n) * L.fld + e % n] = make_float2((float)x.x, (float)x.y);
+        set_row32(F + e / n * L.fld, e % n, make_float2((float)x.x, (float)x.y));
       }
     }
-    for (int e = tid; e < K * K; e += blockDim.x)
-      F[(int64_t)(e / K) * L.fld + n + e % K] = make_float2(e / K == e % K ? 1.f : 0.f, 0.f);
+    const int vr = even32(n);      // the rotations' first row
+    for (int e = tid; e < K * (L.fld - n); e += blockDim.x) {
+      const int j = e / (L.fld - n), i = n + e % (L.fld - n);
+      set_row32(F + j * L.fld, i, make_float2(i - vr == j ? 1.f : 0.f, 0.f));
+    }
     __syncthreads();
     const float tol32 = 1.1920929e-07f * (float)max(n, 32), fl32 = (float)(0.01 * floor2);
-    const int slots = K / 2, Rr = n + K, sweeps = min(max_sweeps, S.fp32_sweeps + 6);
-    if (full && slots <= Threads / 32 && Rr <= 96) small_sweeps<32, 3>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
-    else if (slots <= Threads / 16 && Rr <= 96) small_sweeps<16, 6>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
-    else if (slots <= Threads / 16 && Rr <= 192) small_sweeps<16, 12>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
-    else if (!full && slots <= Threads / 8 && Rr <= 192) small_sweeps<8, 24>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
-    else small_sweeps<0, 0>(F, n, Rr, L.fld, K, nrm, tol32, fl32, sweeps);
-    for (int j = warp; j < K; j += nwarps) {
-      float acc = 0.f;
-      for (int i = lane; i < n; i += 32) {
-        const float2 x = F[(int64_t)j * L.fld + i];
-        acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
-      }
-      acc = warp_sum_f(acc);
-      if (lane == 0) nrm[j] = acc;
-    }
+    const int slots = K / 2, R2 = vr / 2, Rr2 = L.fld / 2, sweeps = min(max_sweeps, S.fp32_sweeps + 6);
+    if (full && slots <= Threads / 32 && Rr2 <= 64) small_sweeps<32, 2>(F, R2, Rr2, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (slots <= Threads / 16 && Rr2 <= 48) small_sweeps<16, 3>(F, R2, Rr2, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (slots <= Threads / 16 && Rr2 <= 96) small_sweeps<16, 6>(F, R2, Rr2, L.fld, K, nrm, tol32, fl32, sweeps);
+    else if (!full && slots <= Threads / 8 && Rr2 <= 96) small_sweeps<8, 12>(F, R2, Rr2, L.fld, K, nrm, tol32, fl32, sweeps);
+    else small_sweeps<0, 0>(F, R2, Rr2, L.fld, K, nrm, tol32, fl32, sweeps);
+    for (int j = warp; j < K; j += nwarps) norm32(F + j * L.fld, R2, nrm + j);
     __syncthreads();
     if (warp == 0) {      // the kept columns, in column order
       int ns = 0;
@@ -2310,7 +2376,7 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
     const int ns = s_ns;
     if (!full) {
       for (int e = tid; e < K * ns; e += blockDim.x) {
-        const float2 v = F[(int64_t)sel[e / K] * L.fld + n + e % K];
+        const float2 v = row32(F + sel[e / K] * L.fld, vr + e % K);
         S.V0[e] = make_double2((double)v.x, (double)v.y);
       }
       for (int j = tid; j < n; j += blockDim.x) S.order[j] = perm[j];
@@ -2329,7 +2395,7 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
     double* lam = reinterpret_cast<double*>(smem_raw + L.lam);
     double* inv = reinterpret_cast<double*>(smem_raw + L.inv);
     for (int e = tid; e < K * ns; e += blockDim.x) {
-      const float2 v = F[(int64_t)sel[e / K] * L.fld + n + e % K];
+      const float2 v = row32(F + sel[e / K] * L.fld, vr + e % K);
       V32[e] = v;
       V[e] = make_double2((double)v.x, (double)v.y);
     }
@@ -2544,15 +2610,14 @@ __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSe
   const int rank = (int)cluster_rank();
   const SvdSector S = secs[blockIdx.x / cluster];
   const int K = min(S.m, S.n);
-  // FP32 columns of jlen + K <= 2 jlen complex values in the staging area sized for FP64 ones
-  JacobiBlocks32 j32;
+  const int fld = even32(S.wide ? K : S.n) + even32(K);
+  FrontBlocks j32;
   j32.g = S.groups;
-  j32.gs = S.staged;
-  j32.cl0 = cluster;
-  j32.stop = kFp32Stop;
+  j32.gs = S.front_staged;
+  j32.cl = cluster;
   j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
   j32.sm = reinterpret_cast<float2*>(smem_raw);
-  j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * ((((S.wide ? K : S.n) + K) + 1) & ~1));
+  j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * fld);
   svd_front(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, j32, smem_raw);
 }
 
@@ -2565,6 +2630,7 @@ namespace {
 
 constexpr int kBlockSmemMax = 110 * 1024;   // two block-Jacobi CTAs per SM
 constexpr int kFrontSmemMax = 216 * 1024;   // one-CTA fronts
+constexpr int kPairSmemMax = 114900;        // cluster fronts, two CTAs per SM
 // 8 CTAs per large sector: the GPU places about twice as many 8-CTA clusters as
 // 16-CTA ones, which keeps more SMs busy when a layer has hundreds of large sectors
 constexpr int kBigCluster = 8;
@@ -2578,6 +2644,11 @@ int g_big_cluster[kMaxDevices] = {};
 int64_t block_smem_need(int m, int n, int cl, int g, int gs) {
   const int64_t K = std::min(m, n), bs = (K + 2 * cl * g - 1) / (2 * cl * g);
   return 16 * 2 * gs * bs * n + 16 * 2 * gs * bs + 64;   // norms, and the FP32 staging's even-stride padding
+}
+// of a front: FP32 columns of at most n + 1 + K + 1 rows, and norms
+int64_t front_smem_need(int m, int n, int cl, int g, int gs) {
+  const int64_t K = std::min(m, n), bs = (K + 2 * cl * g - 1) / (2 * cl * g);
+  return 8 * 2 * gs * bs * (even32(n) + even32((int)K)) + 4 * 2 * gs * bs;
 }
 
 cudaError_t set_attrs(int* big_out) {
@@ -2600,7 +2671,7 @@ cudaError_t set_attrs(int* big_out) {
     e = cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBlockSmemMax);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
+    e = cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(jacobi_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmemMax);
   if (e != cudaSuccess) return e;
@@ -2682,7 +2753,7 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g.count * cl);
   cfg.blockDim = dim3(g.kind == kSvdCluster ? kSvdThreads : kBlockThreads);
-  cfg.dynamicSmemBytes = g.smem;
+  cfg.dynamicSmemBytes = g.kind == kSvdRefine && !fallback ? g.smem_small : g.smem;
   cfg.stream = st;
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
@@ -2788,6 +2859,7 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
         continue;
       }
     }
+    if (16LL * std::max(S.m, S.n) > kBlockSmemMax) secs[k].F = nullptr;   // no room for a reflector
     // blocks of about tune.bw columns (6 by default); the smallest cluster (tune.cl_min,
     // then doubling up to 8 CTAs) whose CTAs can stage all of their block pairs of a round
     // at once, so that a step offers the warp groups about K / (2 cl) * bw / 2 disjoint
@@ -2795,39 +2867,52 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
     // when a single one does not fit
     const int bw = std::max(2, tune.bw);
     const int cn = S.wide ? std::min(S.m, S.n) : S.n;   // Jacobi column length
+    auto need = [&](int cl, int g, int gs) {
+      return S.F ? front_smem_need(S.m, cn, cl, g, gs) : block_smem_need(S.m, cn, cl, g, gs);
+    };
+    const int64_t room = S.F ? kPairSmemMax : kBlockSmemMax;
+    auto blocks = [&](int cl) {      // of a front: at most bw columns each, its 6 warps' slots a pair of them
+      const int K = std::min(S.m, S.n);
+      return S.F ? (K + 2 * bw * cl - 1) / (2 * bw * cl) : std::max(1, (K + bw * cl) / (2 * bw * cl));
+    };
     int pick_cl = 0, pick_g = 0, pick_gs = 0;
     for (int cl = std::max(2, std::min(tune.cl_min, kBigCluster)); cl <= kBigCluster && !pick_cl; cl *= 2) {
-      const int g = std::max(1, (std::min(S.m, S.n) + bw * cl) / (2 * bw * cl));
-      if (g <= kMaxStaged && block_smem_need(S.m, cn, cl, g, g) <= kBlockSmemMax) {
+      const int g = blocks(cl);
+      if (g <= kMaxStaged && need(cl, g, g) <= room) {
         pick_cl = cl; pick_g = g; pick_gs = g;
       }
     }
     if (!pick_cl) {
       const int cl = kBigCluster;
-      int g = std::max(1, (std::min(S.m, S.n) + bw * cl) / (2 * bw * cl));
-      while (g < 64 && block_smem_need(S.m, cn, cl, g, 1) > kBlockSmemMax) ++g;
+      int g = blocks(cl);
+      while (g < 64 && need(cl, g, 1) > room) ++g;
       int gs = 1;
-      while (gs < std::min(g, kMaxStaged) && block_smem_need(S.m, cn, cl, g, gs + 1) <= kBlockSmemMax) ++gs;
-      if (block_smem_need(S.m, cn, cl, g, gs) <= kBlockSmemMax) {
+      while (gs < std::min(g, kMaxStaged) && need(cl, g, gs + 1) <= room) ++gs;
+      if (need(cl, g, gs) <= room) {
         pick_cl = cl; pick_g = g; pick_gs = gs;
       }
     }
     if (std::min(S.m, S.n) >= tune.c16_min_k && big_cluster >= 16) {   // a 16-CTA cluster
       const int cl = 16;
-      int g = std::max(1, (std::min(S.m, S.n) + bw * cl) / (2 * bw * cl));
-      while (g < 64 && block_smem_need(S.m, cn, cl, g, 1) > kBlockSmemMax) ++g;
+      int g = blocks(cl);
+      while (g < 64 && need(cl, g, 1) > room) ++g;
       int gs = 1;
-      while (gs < std::min(g, kMaxStaged) && block_smem_need(S.m, cn, cl, g, gs + 1) <= kBlockSmemMax) ++gs;
-      if (block_smem_need(S.m, cn, cl, g, gs) <= kBlockSmemMax) {
+      while (gs < std::min(g, kMaxStaged) && need(cl, g, gs + 1) <= room) ++gs;
+      if (need(cl, g, gs) <= room) {
         pick_cl = cl; pick_g = g; pick_gs = gs;
       }
     }
     if (std::min(S.m, S.n) >= tune.rr_min_k) pick_cl = 0;
-    if (16LL * std::max(S.m, S.n) > kBlockSmemMax) secs[k].F = nullptr;   // no room for a reflector
+    if (pick_cl && S.F) {      // the FP64 sweeps, should they be needed, stage FP64 columns of the same blocks
+      secs[k].front_staged = pick_gs;
+      small[k] = std::max<int64_t>(need(pick_cl, pick_g, pick_gs),
+                                   16LL * std::max(S.m, S.n));      // the QR's copy of a reflector
+      while (pick_gs > 0 && block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs) > kBlockSmemMax) --pick_gs;
+      if (pick_gs == 0) pick_cl = 0;
+    }
     if (pick_cl) {
       key[k] = {secs[k].F ? kSvdRefine : kSvdClusterBlock, pick_cl};
-      smem[k] = std::max<int64_t>(block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs),
-                                  secs[k].F ? 16LL * std::max(S.m, S.n) : 0);      // the QR's copy of a reflector
+      smem[k] = block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs);
       secs[k].groups = pick_g;
       secs[k].staged = pick_gs;
     } else {
@@ -2894,12 +2979,23 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
     for (int g = 1; g < ng; ++g)
       if ((e = cudaStreamWaitEvent(side[g - 1], fork, 0)) != cudaSuccess) return e;
   }
+  // Clusters of 8 need free places on several SMs at once, so with them the one-CTA kernels, which take up to a
+  // whole SM and end first, go behind the last smaller clusters instead of beside them (a layer of 77 sectors at
+  // chi = 333: fronts done after 17.7 instead of 20 ms).
+  auto one_cta = [&](int g) {
+    return groups[g].kind <= kSvdSmall || (groups[g].kind == kSvdRefine && groups[g].cl == 1);
+  };
+  const bool behind = groups[0].kind == kSvdRefine && groups[0].cl == kBigCluster;
+  auto lane = [&](int g) {
+    while (behind && g > 1 && one_cta(g)) --g;
+    return g;
+  };
   for (int g = 0; g < ng; ++g) {
-    cudaStream_t s = (fan && g > 0) ? side[g - 1] : st;
+    cudaStream_t s = (fan && g > 0) ? side[lane(g) - 1] : st;
     if ((e = launch_group(d_secs, groups[g], max_sweeps, s)) != cudaSuccess) return e;
   }
   auto joined = [&](int g) -> cudaError_t {
-    cudaError_t e2 = cudaEventRecord(join[g - 1], side[g - 1]);
+    cudaError_t e2 = cudaEventRecord(join[g - 1], side[lane(g) - 1]);
     return e2 == cudaSuccess ? cudaStreamWaitEvent(st, join[g - 1], 0) : e2;
   };
   // the refined groups come first (group 0 on st): refine them together once their fronts are done,

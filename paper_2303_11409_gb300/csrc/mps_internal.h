@@ -224,6 +224,7 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   int small;                  // kSvdSmem: refined inside the CTA
   int groups;                 // block Jacobi: block pairs per CTA and round
   int staged;                 // block Jacobi: block pairs staged in shared memory at once
+  int front_staged;           // the same of a refined sector's FP32 sweeps
   double floor_rel;           // columns below floor_rel |M|_F are not rotated, their sigma is 0
                               // (0: the rounding-noise level 32 eps)
   double floor_abs;           // the same for an absolute level (0: none)
@@ -401,8 +402,8 @@ cudaError_t launch_theta(const ThetaTask* d_tasks, const TileRef* d_tiles, int n
                          cudaStream_t st);
 // Sectors grouped by kernel and cluster size (a group is a contiguous run of the array).
 struct SvdGroup {
-  int kind, cl, smem, first, count, max_k, max_n;   // cl 1, 0 of kSvdRefine: one-CTA fronts
-  int smem_small;              // dynamic shared memory of svd_small_kernel
+  int kind, cl, smem, first, count, max_k, max_n;   // cl 1 of kSvdRefine: one-CTA fronts
+  int smem_small;              // dynamic shared memory of svd_small_kernel and svd_front_kernel
   int ctas;                    // kSvdTeam: CTAs of all teams, and the range of their barriers
   unsigned *bar0, *bar1;
 };
