@@ -1680,13 +1680,13 @@ int mps_sample(mps_t h, int n, const double* uniforms, int32_t* configs_out, dou
   // per site, per charge of its left bond, per occupation: the block and the next charge's index
   std::vector<int> site_off(L);
   std::vector<SampleEntry> table;
-  int cap = 1;
+  int rows = 1, width = 1;
   for (int s = 0; s < L; ++s) {
     const BondTable &Lb = h->bonds[s], &Rb = h->bonds[s + 1];
-    cap = std::max(cap, std::max(Lb.total(), Rb.total()));
     site_off[s] = (int)table.size();
     const double2* slot = h->slot_ptr(s, h->cur[s]);
-    for (int li = 0; li < Lb.size(); ++li)
+    for (int li = 0; li < Lb.size(); ++li) {
+      int across = 0;
       for (int i = 0; i < d; ++i) {
         SampleEntry e{nullptr, 0, 0, -1, 0};
         const int bi = h->sites[s].find(Lb.charge[li], h->rule.wrap(Lb.charge[li] - h->rule.charge_of(i)));
@@ -1696,9 +1696,13 @@ int mps_sample(mps_t h, int n, const double* uniforms, int32_t* configs_out, dou
           e.Dl = B.Dl;
           e.Dm = B.Dm;
           e.next = B.im;
+          rows = std::max(rows, e.Dl);
+          across += e.Dm;
         }
         table.push_back(e);
       }
+      width = std::max(width, across);
+    }
   }
   const int64_t b_table = a256(sizeof(SampleEntry) * (int64_t)table.size());
   const int64_t b_off = a256(sizeof(int) * (int64_t)L);
@@ -1721,7 +1725,7 @@ int mps_sample(mps_t h, int n, const double* uniforms, int32_t* configs_out, dou
   double* d_prob = reinterpret_cast<double*>(base + in_bytes + b_cfg);
   // the work depends on the drawn patterns (the blocks visited), so none is counted
   CUDA_OR_FAIL(h, timed(h, MPS_K_SAMPLE, true, 0.0, 0.0, [&] {
-    return launch_sample(reinterpret_cast<SampleEntry*>(base), reinterpret_cast<int*>(base + b_table), L, d, cap,
+    return launch_sample(reinterpret_cast<SampleEntry*>(base), reinterpret_cast<int*>(base + b_table), L, d, rows, width,
                          reinterpret_cast<double*>(base + b_table + b_off), n, d_cfg, d_prob, h->stream);
   }));
   CUDA_OR_FAIL(h, cudaMemcpyAsync(h->pin_out.p, d_cfg, b_cfg + b_prob, cudaMemcpyDeviceToHost, h->stream));

@@ -18,8 +18,8 @@
 // occupation i with a block (c_s, c_s - i) gets w_i = |v B^[s][c_s, c_s - i]|^2; i is the
 // first occupation (ascending) whose cumulative w_i / sum_j w_j exceeds the caller's
 // uniform u_s; v becomes v B rescaled to unit norm, and the pattern's probability is the
-// product of the conditionals.  One CTA per sample: a pass computes every w_i (fixed-order
-// reductions), thread 0 takes the decision, a second pass forms the chosen product.
+// product of the conditionals.  One CTA per sample: it forms every v B and w_i (fixed-order
+// reductions), thread 0 takes the decision.
 //
 // entropy_kernel: the bond entropy S_b = -sum_a lambda_a^2 ln lambda_a^2 over all
 // sectors of bond b (lambda are the Schmidt values of Sec. II; zero values add
@@ -94,59 +94,94 @@ __global__ void entropy_kernel(const double* __restrict__ lam, int n, double* __
   if (threadIdx.x == 0) *out = red[0];
 }
 
-__device__ __forceinline__ double block_sum(double x, double* red) {
-  red[threadIdx.x] = x;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
-}
+// w[c] = sum_a v[a] B[a, c] for c < C by the whole CTA, a column a lane: locate(c, Dm) is column c's first
+// element, Dm its row stride.  FP64 issue binds it (a warp instruction takes its scheduler 64 cycles at any lane
+// count), so when the columns fill few warps the rows are shared by several, at least 16 each, whose parts are
+// added in order.
+// w holds rowbuf(C) values.
+constexpr int kRowThreads = 256;
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowParts = 128;      // two parts or more: up to 4 warps of columns, so w is free from here for them
+__host__ __device__ inline int rowbuf(int C) { return C > kRowParts + 32 * kRowWarps ? C : kRowParts + 32 * kRowWarps; }
 
-// w[j] = sum_a v[a] B[a, j] for j < Dm (B row-major Dl x Dm); returns |w|^2 when keep, else
-// only the norm (w untouched)
-__device__ __forceinline__ double row_times_block(const double2* v, const SampleEntry& e, double2* w, bool keep,
-                                                  double* red) {
-  double part = 0.0;
-  for (int j = threadIdx.x; j < e.Dm; j += blockDim.x) {
+template <class Locate>
+__device__ __forceinline__ void row_times_columns(const double2* v, int Dl, int C, double2* w, Locate locate) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int chunks = (C + 31) / 32, parts = chunks > 0 ? max(1, min(kRowWarps / chunks, Dl / 16)) : 1;
+  for (int t = warp; t < chunks * parts; t += kRowWarps) {
+    const int c = t % chunks * 32 + lane, q = t / chunks;
     double2 acc = make_double2(0.0, 0.0);
-    for (int a = 0; a < e.Dl; ++a) {
-      const double2 x = v[a], b = e.blk[(int64_t)a * e.Dm + j];
-      acc.x = fma(x.x, b.x, fma(-x.y, b.y, acc.x));
-      acc.y = fma(x.x, b.y, fma(x.y, b.x, acc.y));
+    if (c < C) {
+      int Dm, a = Dl * q / parts;
+      const int a1 = Dl * (q + 1) / parts;
+      const double2* B = locate(c, Dm);
+      B += (int64_t)a * Dm;
+#pragma unroll 4
+      for (; a < a1; ++a, B += Dm) {
+        const double2 x = v[a], b = *B;
+        acc.x = fma(x.x, b.x, fma(-x.y, b.y, acc.x));
+        acc.y = fma(x.x, b.y, fma(x.y, b.x, acc.y));
+      }
     }
-    if (keep) w[j] = acc;
-    part = fma(acc.x, acc.x, fma(acc.y, acc.y, part));
+    if (parts > 1) w[kRowParts + t * 32 + lane] = acc;
+    else if (c < C) w[c] = acc;
   }
-  return block_sum(part, red);
+  __syncthreads();
+  if (parts == 1) return;
+  for (int c = threadIdx.x; c < C; c += blockDim.x) {
+    double2 acc = w[kRowParts + c];
+    for (int q = 1; q < parts; ++q) {
+      const double2 x = w[kRowParts + q * chunks * 32 + c];
+      acc.x += x.x;
+      acc.y += x.y;
+    }
+    w[c] = acc;
+  }
+  __syncthreads();
 }
 
-__global__ void sample_kernel(const SampleEntry* __restrict__ table, const int* __restrict__ site_off, int L, int d,
-                              int cap, const double* __restrict__ uniforms, int* __restrict__ configs,
-                              double* __restrict__ probs) {
+// One CTA a sample.  The columns of all d products v B of a site lie side by side over the lanes and every product
+// is kept, so the chosen one is not formed again.  512 samples at chi = 128 (L = 32, d = 5): 741 -> 315 us, where
+// one occupation after the other left most lanes idle and the chosen product was formed twice.
+__global__ void __launch_bounds__(kRowThreads) sample_kernel(const SampleEntry* __restrict__ table,
+                                                                const int* __restrict__ site_off, int L, int d,
+                                                                int rows, const double* __restrict__ uniforms,
+                                                                int* __restrict__ configs, double* __restrict__ probs) {
   extern __shared__ __align__(16) unsigned char raw[];
   double2* v = reinterpret_cast<double2*>(raw);
-  double2* w = v + cap;
-  __shared__ double red[256];
+  double2* w = v + rows;
+  __shared__ SampleEntry E[MPS_MAX_D];
   __shared__ double wn[MPS_MAX_D];
   __shared__ int pick, bad;
-  const int k = blockIdx.x;
-  if (threadIdx.x == 0) { v[0] = make_double2(1.0, 0.0); bad = 0; }
-  __syncthreads();
+  const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) { v[0] = make_double2(1.0, 0.0); bad = 0; }
   int li = 0;                     // sector index of the current right-charge in its bond table
   double p = 1.0;
   for (int s = 0; s < L; ++s) {
-    const SampleEntry* row = table + site_off[s] + (int64_t)li * d;
+    if (tid < d) E[tid] = table[site_off[s] + (int64_t)li * d + tid];
+    __syncthreads();
+    int C = 0, Dl = 0;
     for (int i = 0; i < d; ++i) {
-      const SampleEntry e = row[i];
-      const double n2 = e.blk ? row_times_block(v, e, w, false, red) : -1.0;
-      if (threadIdx.x == 0) wn[i] = n2;
+      C += E[i].Dm;
+      Dl = max(Dl, E[i].Dl);
+    }
+    row_times_columns(v, Dl, C, w, [&](int c, int& Dm) {
+      int i = 0;
+      while (c >= E[i].Dm) c -= E[i++].Dm;
+      Dm = E[i].Dm;
+      return E[i].blk + c;
+    });
+    for (int i = warp; i < d; i += kRowWarps) {
+      int off = 0;
+      for (int j = 0; j < i; ++j) off += E[j].Dm;
+      double n2 = 0.0;
+      for (int c = lane; c < E[i].Dm; c += 32) n2 = fma(w[off + c].x, w[off + c].x, fma(w[off + c].y, w[off + c].y, n2));
+#pragma unroll
+      for (int o = 16; o; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      if (lane == 0) wn[i] = E[i].blk ? n2 : -1.0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       double tot = 0.0;
       int last = -1;
       for (int i = 0; i < d; ++i)
@@ -169,28 +204,28 @@ __global__ void sample_kernel(const SampleEntry* __restrict__ table, const int* 
     }
     __syncthreads();
     if (bad) break;
-    const SampleEntry e = row[pick];
-    const double n2 = row_times_block(v, e, w, true, red);
-    const double scale = 1.0 / sqrt(n2);
-    for (int j = threadIdx.x; j < e.Dm; j += blockDim.x) v[j] = make_double2(w[j].x * scale, w[j].y * scale);
-    li = e.next;
+    int off = 0;
+    for (int j = 0; j < pick; ++j) off += E[j].Dm;
+    const double scale = 1.0 / sqrt(wn[pick]);
+    for (int j = tid; j < E[pick].Dm; j += blockDim.x) v[j] = make_double2(w[off + j].x * scale, w[off + j].y * scale);
+    li = E[pick].next;
     __syncthreads();
   }
-  if (threadIdx.x == 0) probs[k] = bad ? 0.0 : p;
+  if (tid == 0) probs[k] = bad ? 0.0 : p;
 }
 
 }  // namespace
 
-cudaError_t launch_sample(const SampleEntry* d_table, const int* d_site_off, int L, int d, int cap,
+cudaError_t launch_sample(const SampleEntry* d_table, const int* d_site_off, int L, int d, int rows, int width,
                           const double* d_uniforms, int n, int* d_configs, double* d_probs, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const size_t smem = sizeof(double2) * 2 * (size_t)cap;
+  const size_t smem = sizeof(double2) * ((size_t)rows + rowbuf(width));
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   count_launch();
-  sample_kernel<<<n, 256, smem, st>>>(d_table, d_site_off, L, d, cap, d_uniforms, d_configs, d_probs);
+  sample_kernel<<<n, kRowThreads, smem, st>>>(d_table, d_site_off, L, d, rows, d_uniforms, d_configs, d_probs);
   return cudaGetLastError();
 }
 

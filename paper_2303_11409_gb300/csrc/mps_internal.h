@@ -522,7 +522,8 @@ struct AmpStep { const double2* blk; int Dl, Dm; };
 // s for the li-th charge c of bond s (blk == nullptr when absent) and the index of c - i in
 // bond s+1's table.
 struct SampleEntry { const double2* blk; int Dl, Dm; int next; int pad; };
-cudaError_t launch_sample(const SampleEntry* d_table, const int* d_site_off, int L, int d, int cap,
+// rows: the largest block height, width: the largest sum of a charge's block widths.
+cudaError_t launch_sample(const SampleEntry* d_table, const int* d_site_off, int L, int d, int rows, int width,
                           const double* d_uniforms, int n, int* d_configs, double* d_probs, cudaStream_t st);
 // -sum lambda^2 ln lambda^2 over n values into *d_out (one CTA).
 cudaError_t launch_entropy(const double* d_lambda, int n, double* d_out, cudaStream_t st);
