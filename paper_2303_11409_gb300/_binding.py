@@ -7,6 +7,7 @@ importing this module fails loudly otherwise.  There is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import warnings
 
@@ -150,6 +151,12 @@ def _ptr(a: np.ndarray, t):
     return a.ctypes.data_as(t)
 
 
+def _ptr_array(arrays):
+    """double *[] of the arrays' addresses (they must outlive the call it is passed to)."""
+    addr = (ctypes.c_void_p * len(arrays))(*[a.__array_interface__["data"][0] for a in arrays])
+    return ctypes.cast(addr, ctypes.POINTER(_dblp))
+
+
 def _i32(a) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
@@ -172,6 +179,7 @@ def _default_stream():
     return None
 
 
+@functools.lru_cache(maxsize=None)
 def gate_length(d: int) -> int:
     """Complex numbers in one flattened gate: sum over n of s_n^2."""
     tot = 0
@@ -359,9 +367,10 @@ class MPS:
         gs = [self._gate_flat(g) for g in gates]
         if len(gs) != len(sites):
             raise ValueError("one gate per site")
-        if any(g.size != self.gate_length() for g in gs):
+        length = self.gate_length()
+        if any(g.size != length for g in gs):
             raise ValueError("a gate has the wrong number of entries")
-        arr = (_dblp * len(gs))(*[g.ctypes.data_as(_dblp) for g in gs])
+        arr = _ptr_array(gs)
         te = np.zeros(len(gs))
         rc = lib.mps_apply_layer(self._h, len(gs), _ptr(sites, _intp), arr, chi, cutoff, _ptr(te, _dblp))
         self._check(rc, "mps_apply_layer")
@@ -614,7 +623,7 @@ class Executor:
         gs = [_c128_flat(it[2]) for it in items]
         if any(g.size != it[0].gate_length() for g, it in zip(gs, items)):
             raise ValueError("a gate has the wrong number of entries")
-        garr = (_dblp * n)(*[g.ctypes.data_as(_dblp) for g in gs])
+        garr = _ptr_array(gs)
         chis = np.array([it[3] for it in items], dtype=np.intc)
         cuts = np.array([it[4] for it in items], dtype=np.float64)
         te = np.zeros(n)
@@ -754,7 +763,7 @@ def apply_gate2_batch(items, stream_owner: MPS | None = None):
     gs = [it[0]._gate_flat(it[2]) for it in items]
     if any(g.size != it[0].gate_length() for g, it in zip(gs, items)):
         raise ValueError("a gate has the wrong number of entries")
-    garr = (_dblp * n)(*[g.ctypes.data_as(_dblp) for g in gs])
+    garr = _ptr_array(gs)
     chis = np.array([it[3] for it in items], dtype=np.intc)
     cuts = np.array([it[4] for it in items], dtype=np.float64)
     te = np.zeros(n)

@@ -272,11 +272,33 @@ struct Stager {
     size = a256(off + (int64_t)sizeof(T) * count);
     return off;
   }
+  // room for count values that the caller writes in place
+  template <typename T> T* room(int64_t count, int64_t* off) {
+    *off = size;
+    size = a256(size + (int64_t)sizeof(T) * count);
+    return reinterpret_cast<T*>(host + *off);
+  }
 };
 
 struct Req {
   mps_s* h; int site; const double* gate; int chi; double cutoff;
   int status = MPS_OK; double trunc = 0.0;
+};
+
+// A dense table over (row, column) sector indices, -1 where nothing is: looked up for every product of every
+// update instead of searching the block lists (of a batch of 176 updates: 0.35 ms of host time).
+struct BlockIndex {
+  std::vector<int> v;
+  size_t cols = 0;
+  void clear(size_t rows, size_t c) {
+    cols = c;
+    v.assign(rows * c, -1);
+  }
+  void of(const SiteTable& S, const BondTable& left, const BondTable& right) {
+    clear(left.size(), right.size());
+    for (size_t b = 0; b < S.blocks.size(); ++b) (*this)(S.blocks[b].il, S.blocks[b].im) = (int)b;
+  }
+  int& operator()(size_t i, size_t j) { return v[i * cols + j]; }
 };
 
 // Per-update scratch bookkeeping of one batch.
@@ -306,7 +328,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   Range batch_range("mps.update_call");
   // ---- K0: plan every update and size the workspace --------------------------------
   int64_t ws = 0;
-  int n_sec_total = 0, n_tiles = 0, n_tasks = 0, max_tri = 0;
+  int n_sec_total = 0, n_tiles = 0, n_tasks = 0;
   // reduced-precision updates ([0] TF32, [1] BF16x3): shadow slots, shadow tiles, products,
   // gate-mix tasks, and the complex64 buffer of the products T_m
   int64_t tc_slots[2] = {0, 0}, tc_shtiles[2] = {0, 0}, tc_jobs[2] = {0, 0}, tc_mix[2] = {0, 0};
@@ -319,7 +341,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   for (int u = 0; u < nreq; ++u) {
     mps_s* h = reqs[u].h;
     const int s = reqs[u].site;
-    plan_update(h->bonds[s], h->bonds[s + 1], h->bonds[s + 2], h->rule, W[u].plan);
+    plan_update(h->bonds[s], h->bonds[s + 1], h->bonds[s + 2], h->rule, W[u].plan, false);
     if (h->chi_deflate > 0.0 && (int)h->cut_est.size() == h->L + 1) {
       W[u].cut_est = h->cut_est[s + 1];
       // a cut recorded by the previous update call on this handle (the same layer kind in a row,
@@ -329,7 +351,6 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       const bool fresh = (int)h->cut_call.size() == h->L + 1 && h->calls - h->cut_call[s + 1] <= 1;
       W[u].chi_level = fresh ? h->chi_deflate : h->chi_deflate / 30.0;
     }
-    max_tri = std::max<int>(max_tri, (int)W[u].plan.triple_l.size());
     n_sec_total += (int)W[u].plan.sectors.size();
     if (W[u].plan.sectors.empty()) return fail(owner, MPS_EINVAL, "update has no charge sectors");
   }
@@ -485,8 +506,11 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   for (int u = 0; u < nreq; ++u) W[u].gate_off = desc_off + sg.put(reqs[u].gate, 2 * reqs[u].h->rule.gate_len());
 
   // ---- build phase-1 descriptors ------------------------------------------------------
-  std::vector<ThetaTask> tasks; tasks.reserve(n_tasks);
-  std::vector<TileRef> tiles; tiles.reserve(n_tiles);
+  // the products of Theta', written where they are uploaded from (a batch of 176 updates has 2.4 MB of them)
+  int64_t o_tasks, o_tiles;
+  ThetaTask* const tasks = sg.room<ThetaTask>(n_tasks, &o_tasks);
+  TileRef* const tiles = sg.room<TileRef>(n_tiles, &o_tiles);
+  int task_n = 0, tile_n = 0;
   // reduced-precision updates, per precision ([0] TF32, [1] BF16x3)
   std::vector<ShadowTask> shtask[2];
   std::vector<ShadowTile> shtile[2];
@@ -504,9 +528,10 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   std::vector<LambdaTask> gath;
   int64_t gath_next = 0;
   int sec_global = 0;
+  BlockIndex at_l, at_r, row_at, col_at;
   for (int u = 0; u < nreq; ++u) {
     mps_s* h = reqs[u].h;
-    const int s = reqs[u].site, d = h->d;
+    const int s = reqs[u].site;
     const BondTable &Lb = h->bonds[s], &Mb = h->bonds[s + 1], &Rb = h->bonds[s + 2];
     const SiteTable &SL = h->sites[s], &SR = h->sites[s + 1];
     const double2* slotL = h->slot_ptr(s, h->cur[s]);
@@ -557,18 +582,27 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
         }
       }
     }
+    at_l.of(SL, Lb, Mb);
+    at_r.of(SR, Mb, Rb);
+    row_at.clear(P.sectors.size(), Lb.size());
+    col_at.clear(P.sectors.size(), Rb.size());
+    for (size_t si = 0; si < P.sectors.size(); ++si) {
+      const SectorPlanEntry& E = P.sectors[si];
+      for (size_t a = 0; a < E.li.size(); ++a) row_at(si, E.li[a]) = E.loff[a];
+      for (size_t a = 0; a < E.ri.size(); ++a) col_at(si, E.ri[a]) = E.coff[a];
+    }
     for (int li = 0; li < Lb.size(); ++li)
       for (int ri = 0; ri < Rb.size(); ++ri) {
         const int l = Lb.charge[li], r = Rb.charge[ri];
         const int n = rule.pair(l, r);           // the gate block of this pair
         if (n < 0) continue;
-        ThetaTask T;
+        ThetaTask mixed;      // of a reduced-precision update: not uploaded
+        ThetaTask& T = tc || task_n == n_tasks ? mixed : tasks[task_n];
         std::memset(&T, 0, sizeof(T));
-        T.nm = 0;
         for (int mi = 0; mi < Mb.size(); ++mi) {
           const int m = Mb.charge[mi];
           if (rule.phys(l, m) < 0 || rule.phys(m, r) < 0) continue;
-          const int bl = SL.find(l, m), br = SR.find(m, r);
+          const int bl = at_l(li, mi), br = at_r(mi, ri);
           if (bl < 0 || br < 0) return fail(owner, MPS_EINVAL, "internal: missing block");
           T.A[T.nm] = slotL + SL.blocks[bl].off;
           T.B[T.nm] = slotR + SR.blocks[br].off;
@@ -577,6 +611,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
           T.nm++;
         }
         if (T.nm == 0) continue;
+        if (!tc && task_n == n_tasks) return fail(owner, MPS_EINVAL, "internal: product count");
         T.nc = 0;
         int cs[MPS_MAX_D];
         const int ncs = rule.mids(l, r, cs);
@@ -585,8 +620,8 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
           const int si = sector_of(c);
           if (si < 0) return fail(owner, MPS_EINVAL, "internal: missing sector");
           const SectorPlanEntry& E = P.sectors[si];
-          const int roff = E.row_off(li);
-          const int coff = E.col_off(ri);
+          const int roff = row_at(si, li);
+          const int coff = col_at(si, ri);
           if (roff < 0 || coff < 0) return fail(owner, MPS_EINVAL, "internal: sector layout");
           T.out[T.nc] = reinterpret_cast<double2*>(dptr(W[u].theta_off[si])) + (int64_t)roff * E.cols + coff;
           T.ldo[T.nc] = E.cols;
@@ -648,10 +683,11 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
           tc_th_flops += 8.0 * T.nm * T.nc * T.Dl * T.Dr;
           continue;
         }
-        const int task_id = (int)tasks.size();
-        tasks.push_back(T);
-        for (int ti = 0; ti < (T.Dl + kTile - 1) / kTile; ++ti)
-          for (int tj = 0; tj < (T.Dr + kTile - 1) / kTile; ++tj) tiles.push_back(TileRef{task_id, ti, tj});
+        const int task_id = task_n++;
+        const int rows = (T.Dl + kTile - 1) / kTile, cols = (T.Dr + kTile - 1) / kTile;
+        if (tile_n + rows * cols > n_tiles) return fail(owner, MPS_EINVAL, "internal: tile count");
+        for (int ti = 0; ti < rows; ++ti)
+          for (int tj = 0; tj < cols; ++tj) tiles[tile_n++] = TileRef{task_id, ti, tj};
       }
     W[u].sel_first = (int)selsec.size();
     for (size_t si = 0; si < P.sectors.size(); ++si, ++sec_global) {
@@ -711,7 +747,9 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       }
     }
   }
-  std::vector<std::vector<SvdSector>> svd_sorted(n_cand, svd);
+  std::vector<std::vector<SvdSector>> svd_sorted(n_cand);
+  for (int c = 0; c + 1 < n_cand; ++c) svd_sorted[c] = svd;
+  svd_sorted[n_cand - 1] = std::move(svd);
   std::vector<std::vector<SvdGroup>> svd_groups(n_cand);
   for (int c = 0; c < n_cand; ++c) {
     const SvdTune tune = n_cand > 1 ? svd_tune_candidate(c) : (chosen >= 0 ? svd_tune_candidate(chosen) : SvdTune());
@@ -719,8 +757,6 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   }
 
   // ---- descriptors into the staging buffer (uploaded in one copy) ---------------------
-  const int64_t o_tasks = sg.put(tasks.data(), (int64_t)tasks.size());
-  const int64_t o_tiles = sg.put(tiles.data(), (int64_t)tiles.size());
   std::vector<int64_t> o_svd(n_cand);
   for (int c = 0; c < n_cand; ++c) o_svd[c] = sg.put(svd_sorted[c].data(), (int64_t)svd_sorted[c].size());
   const int64_t o_selsec = sg.put(selsec.data(), (int64_t)selsec.size());
@@ -751,7 +787,8 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   // ---- algorithmic work of the three kernels (flops: complex multiply-add = 8) -------
   double th_flops = 0, th_bytes = (double)(theta_bytes_end - theta_bytes_begin);   // Theta' written
   int th_rows = 1, th_cols = 1;
-  for (const ThetaTask& T : tasks) {
+  for (int k = 0; k < task_n; ++k) {
+    const ThetaTask& T = tasks[k];
     th_rows = std::max(th_rows, T.Dl);
     th_cols = std::max(th_cols, T.Dr);
     for (int i = 0; i < T.nm; ++i) th_flops += 8.0 * T.Dl * T.Dm[i] * T.Dr;
@@ -803,10 +840,10 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
         return launch_lambda(reinterpret_cast<LambdaTask*>(dptr(desc_off + o_gath)), (int)gath.size(), st);
       });
     if (e != cudaSuccess) return e;
-    const bool any_theta = !tiles.empty() || !mixes[0].empty() || !mixes[1].empty();
+    const bool any_theta = tile_n > 0 || !mixes[0].empty() || !mixes[1].empty();
     return timed(owner, MPS_K_THETA, any_theta, th_flops, th_bytes, [&] {
       cudaError_t e2 = launch_theta(reinterpret_cast<ThetaTask*>(dptr(desc_off + o_tasks)),
-                                    reinterpret_cast<TileRef*>(dptr(desc_off + o_tiles)), (int)tiles.size(), th_rows,
+                                    reinterpret_cast<TileRef*>(dptr(desc_off + o_tiles)), tile_n, th_rows,
                                     th_cols, st);
       for (int p = 0; p < 2 && e2 == cudaSuccess; ++p)
         e2 = launch_mix(precs[p], reinterpret_cast<MixTask*>(dptr(desc_off + o_mix[p])), (int)mixes[p].size(),
@@ -836,7 +873,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     CUDA_OR_FAIL(owner, run_phase(owner, 0, [&]() -> cudaError_t {
       cudaError_t e = upload_and_theta();
       if (e == cudaSuccess)
-        e = timed(owner, MPS_K_SVD, !svd.empty(), svd_flops, svd_bytes, [&] { return svd_launch(0); });
+        e = timed(owner, MPS_K_SVD, n_sec_total > 0, svd_flops, svd_bytes, [&] { return svd_launch(0); });
       if (e == cudaSuccess) e = select_and_readback();
       return e;
     }));
@@ -949,6 +986,10 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   std::vector<ScatterTask> sc;
   std::vector<GemmTask> gm;
   std::vector<TileRef> gt;
+  lam.reserve(lam_bound);
+  sc.reserve(scatter_bound);
+  gm.reserve(gemm_tasks_bound);
+  gt.reserve(gemm_tiles_bound);
   // reduced-precision reassembly ([0] TF32, [1] BF16x3): Y(c)[:, :k] as B tiles, appended to the
   // phase-1 slots (the reassembly A tiles of Theta' written by the mix are still there)
   std::vector<ShadowTask> yshtask[2];
@@ -1020,6 +1061,8 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     const double scale = 1.0 / R.norm_kept;
     double2* dstL = h->slot_ptr(s, h->cur[s] ^ 1);
     double2* dstR = h->slot_ptr(s + 1, h->cur[s + 1] ^ 1);
+    at_l.of(newL[u], Lb, M);
+    at_r.of(newR[u], M, Rb);
     int mi = 0;
     for (size_t si = 0; si < P.sectors.size(); ++si) {
       const int k = kept[W[u].sel_first + si];
@@ -1031,7 +1074,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       lam.push_back(LambdaTask{sig, h->lambda_ptr(s + 1) + M.off[mi], k, scale});
       for (size_t ra = 0; ra < E.ri.size(); ++ra) {
         const int ri = E.ri[ra];
-        const int b = newR[u].find(E.c, Rb.charge[ri]);
+        const int b = at_r(mi, ri);
         ScatterTask T;
         T.Y = Y;
         T.out = dstR + newR[u].blocks[b].off;
@@ -1059,7 +1102,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       }
       for (size_t la = 0; la < E.li.size(); ++la) {
         const int li = E.li[la];
-        const int b = newL[u].find(Lb.charge[li], E.c);
+        const int b = at_l(li, mi);
         if (tc) {   // B^[s][l, c] = (Theta'(c)[rows of l] . Y(c)[:, :k]) / |S_kept| on the tensor cores
           const int Dl = Lb.dim[li];
           const int64_t a0 = ra_slot[u][si][la];
@@ -1098,7 +1141,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
     }
     Stats& S = h->stats;
     S.n_sectors = (int)P.sectors.size();
-    S.n_triples = (int)P.triple_l.size();
+    S.n_triples = (int)P.n_triples;
     S.max_sweeps = max_sweeps;
     S.tie_band = R.band;
     S.norm_all = R.norm_all;

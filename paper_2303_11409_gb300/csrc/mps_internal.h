@@ -176,12 +176,14 @@ struct SectorPlanEntry {
 };
 struct UpdatePlan {
   std::vector<SectorPlanEntry> sectors;                 // c ascending
-  std::vector<int> triple_l, triple_m, triple_r;        // sector indices, lexicographic
+  std::vector<int> triple_l, triple_m, triple_r;        // sector indices, lexicographic, when listed
+  int64_t n_triples = 0;
 };
 void plan_update(const BondTable& left, const BondTable& mid, const BondTable& right, int d,
                  UpdatePlan& plan);
+// list_triples: also plan.triple_*, which only the planner's own callers read
 void plan_update(const BondTable& left, const BondTable& mid, const BondTable& right, const ChargeRule& rule,
-                 UpdatePlan& plan);
+                 UpdatePlan& plan, bool list_triples = true);
 
 // ---------------------------------------------------------------------------
 // Kernel descriptors (plain structs, copied to device memory in one upload).

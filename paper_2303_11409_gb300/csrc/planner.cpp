@@ -10,6 +10,7 @@
 // columns of every Theta(c) are contiguous ranges of the left and right tables
 // (the "charge-sorted memory alignment" of Sec. II).
 #include <algorithm>
+#include <numeric>
 #include <new>
 #include <cstring>
 
@@ -117,6 +118,8 @@ void ChargeRule::init_zn() {
 static void fill_lists(const BondTable& left, const BondTable& right, SectorPlanEntry& e) {
   e.loff.clear();
   e.coff.clear();
+  e.loff.reserve(e.li.size());
+  e.coff.reserve(e.ri.size());
   int o = 0;
   for (int i : e.li) { e.loff.push_back(o); o += left.dim[i]; }
   e.rows = o;
@@ -128,18 +131,26 @@ static void fill_lists(const BondTable& left, const BondTable& right, SectorPlan
 }
 
 void plan_update(const BondTable& left, const BondTable& mid, const BondTable& right, const ChargeRule& rule,
-                 UpdatePlan& plan) {
+                 UpdatePlan& plan, bool list_triples) {
   const int d = rule.d;
   plan.sectors.clear();
+  plan.n_triples = 0;
   plan.triple_l.clear(); plan.triple_m.clear(); plan.triple_r.clear();
-  for (int i = 0; i < left.size(); ++i)
-    for (int j = 0; j < mid.size(); ++j) {
-      if (rule.phys(left.charge[i], mid.charge[j]) < 0) continue;
-      for (int k = 0; k < right.size(); ++k) {
-        if (rule.phys(mid.charge[j], right.charge[k]) < 0) continue;
-        plan.triple_l.push_back(i); plan.triple_m.push_back(j); plan.triple_r.push_back(k);
+  for (int j = 0; j < mid.size(); ++j) {
+    int64_t rows = 0, cols = 0;
+    for (int i = 0; i < left.size(); ++i) rows += rule.phys(left.charge[i], mid.charge[j]) >= 0;
+    for (int k = 0; k < right.size(); ++k) cols += rule.phys(mid.charge[j], right.charge[k]) >= 0;
+    plan.n_triples += rows * cols;
+  }
+  if (list_triples)
+    for (int i = 0; i < left.size(); ++i)
+      for (int j = 0; j < mid.size(); ++j) {
+        if (rule.phys(left.charge[i], mid.charge[j]) < 0) continue;
+        for (int k = 0; k < right.size(); ++k) {
+          if (rule.phys(mid.charge[j], right.charge[k]) < 0) continue;
+          plan.triple_l.push_back(i); plan.triple_m.push_back(j); plan.triple_r.push_back(k);
+        }
       }
-    }
   if (left.size() == 0 || right.size() == 0) return;
   if (rule.tabled()) {
     // several U(1) charges, or Z_n with d < n: every middle charge some (l, r) pair reaches,
@@ -184,6 +195,7 @@ void plan_update(const BondTable& left, const BondTable& mid, const BondTable& r
   // Candidate middle charges: c with some left l in [c, c+d-1] and right r in [c-d+1, c].
   int cmin = std::max(right.charge.front(), left.charge.front() - (d - 1));
   int cmax = std::min(left.charge.back(), right.charge.back() + (d - 1));
+  plan.sectors.reserve(std::max(0, cmax - cmin + 1));
   for (int c = cmin; c <= cmax; ++c) {
     // rows: left sectors with c <= l <= c + d - 1 (contiguous in the sorted table)
     int l0 = (int)(std::lower_bound(left.charge.begin(), left.charge.end(), c) - left.charge.begin());
@@ -191,12 +203,14 @@ void plan_update(const BondTable& left, const BondTable& mid, const BondTable& r
     int r0 = (int)(std::lower_bound(right.charge.begin(), right.charge.end(), c - (d - 1)) - right.charge.begin());
     int r1 = (int)(std::upper_bound(right.charge.begin(), right.charge.end(), c) - right.charge.begin());
     if (l0 >= l1 || r0 >= r1) continue;
-    SectorPlanEntry e;
+    plan.sectors.emplace_back();
+    SectorPlanEntry& e = plan.sectors.back();
     e.c = c; e.l0 = l0; e.l1 = l1; e.r0 = r0; e.r1 = r1;
-    for (int i = l0; i < l1; ++i) e.li.push_back(i);
-    for (int k = r0; k < r1; ++k) e.ri.push_back(k);
+    e.li.resize(l1 - l0);
+    e.ri.resize(r1 - r0);
+    std::iota(e.li.begin(), e.li.end(), l0);
+    std::iota(e.ri.begin(), e.ri.end(), r0);
     fill_lists(left, right, e);
-    plan.sectors.push_back(e);
   }
 }
 
