@@ -255,6 +255,9 @@ __device__ __forceinline__ void load_rows(char* dst, const double2* X, int64_t l
   }
 }
 
+// Two or three steps settle a sector; launches beyond that find nothing to do (3 us each), and what is
+// not settled after the last one costs FP64 sweeps, which large sectors can least afford.
+__host__ __device__ constexpr int refine_steps(int K) { return K < 200 ? 4 : kRefineSteps; }
 constexpr int kLeftAt = 100;       // rstate[1] when step it leaves the sector: kLeftAt + it
 __device__ __forceinline__ int ns_of(const SvdSector& S) { return __ldg(S.rstate); }
 __device__ __forceinline__ bool skip(const SvdSector& S) { return S.rstate[1] != 0 || S.rstate[2] != 0; }
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(256) refine_norm_kernel(const SvdSector* __res
     const float th = __int_as_float(S.rstate[4 + it - 1]);
     if (refine_fails(th, it - 1)) S.rstate[1] = kLeftAt + it;
     else if (refine_settles(th, ncol, n)) S.rstate[2] = it;
+    else if (it >= refine_steps(K)) S.rstate[1] = kLeftAt + it;      // whatever its batch has launched
   }
   const double2* X = which == 0 ? S.J : ((it & 1) ? S.A1 : S.A0);
   for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < ncol; c += gridDim.x * 8) {
@@ -544,9 +548,7 @@ cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max
   refine_update_kernel<<<dim3(ct * rn, count), kOzThreads, kOzSmem, st>>>(d_secs, 0);
   refine_norm_kernel<<<cols, 256, 0, st>>>(d_secs, 1, 0);
   count_launch(); count_launch(); count_launch();
-  // two or three steps settle a sector; launches beyond that find nothing to do (3 us each), and
-  // what is not settled after the last one costs FP64 sweeps, which large sectors can least afford
-  const int steps = max_k < 200 ? 4 : kRefineSteps;
+  const int steps = refine_steps(max_k);
   for (int it = 0; it < steps; ++it) {
     refine_gram_kernel<<<dim3(ct * rk, count), kOzThreads, kOzSmem, st>>>(d_secs, it);
     refine_update_kernel<<<dim3(ct * (rn + rk), count), kOzThreads, kOzSmem, st>>>(d_secs, it + 1);

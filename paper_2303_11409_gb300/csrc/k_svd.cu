@@ -2994,27 +2994,42 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
     cudaStream_t s = (fan && g > 0) ? side[lane(g) - 1] : st;
     if ((e = launch_group(d_secs, groups[g], max_sweeps, s)) != cudaSuccess) return e;
   }
-  auto joined = [&](int g) -> cudaError_t {
-    cudaError_t e2 = cudaEventRecord(join[g - 1], side[lane(g) - 1]);
-    return e2 == cudaSuccess ? cudaStreamWaitEvent(st, join[g - 1], 0) : e2;
+  auto joined = [&](int g, cudaStream_t into) -> cudaError_t {
+    cudaStream_t from = side[lane(g) - 1];
+    if (from == into) return cudaSuccess;
+    cudaError_t e2 = cudaEventRecord(join[g - 1], from);
+    return e2 == cudaSuccess ? cudaStreamWaitEvent(into, join[g - 1], 0) : e2;
   };
-  // the refined groups come first (group 0 on st): refine them together once their fronts are done,
-  // while the other groups go on
-  int nr = 0, count = 0, max_k = 0, max_n = 0;
-  for (; nr < ng && groups[nr].kind == kSvdRefine; ++nr) {
-    count += groups[nr].count;
-    max_k = std::max(max_k, groups[nr].max_k);
-    max_n = std::max(max_n, groups[nr].max_n);
-    if (fan && nr > 0 && (e = joined(nr)) != cudaSuccess) return e;
-  }
-  if (nr > 0) {
-    if ((e = launch_refine(d_secs + groups[0].first, count, max_k, max_n, st)) != cudaSuccess) return e;
-    for (int g = 0; g < nr; ++g)
-      if ((e = launch_group(d_secs, groups[g], max_sweeps, st, true)) != cudaSuccess) return e;
+  auto refine = [&](int g0, int g1, cudaStream_t s) -> cudaError_t {      // groups g0 .. g1 - 1, their fronts done
+    int count = 0, max_k = 0, max_n = 0;
+    for (int g = g0; g < g1; ++g) {
+      count += groups[g].count;
+      max_k = std::max(max_k, groups[g].max_k);
+      max_n = std::max(max_n, groups[g].max_n);
+    }
+    cudaError_t e2 = launch_refine(d_secs + groups[g0].first, count, max_k, max_n, s);
+    for (int g = g0; g < g1 && e2 == cudaSuccess; ++g) e2 = launch_group(d_secs, groups[g], max_sweeps, s, true);
+    return e2;
+  };
+  // The refined groups come first.  Clusters of 8 run on when the other fronts are done, and leave SMs free by then,
+  // so those sectors are refined meanwhile; without clusters of 8 all are refined together.
+  int nr = 0;
+  while (nr < ng && groups[nr].kind == kSvdRefine) ++nr;
+  const int first = fan && behind && nr > 1 ? 1 : 0;      // the first group of the refinement beside
+  if (first) {
+    cudaStream_t s = side[lane(nr - 1) - 1];
+    for (int g = 1; g < nr; ++g)
+      if ((e = joined(g, s)) != cudaSuccess) return e;
+    if ((e = refine(1, nr, s)) != cudaSuccess || (e = refine(0, 1, st)) != cudaSuccess) return e;
+  } else {
+    if (fan)
+      for (int g = 1; g < nr; ++g)
+        if ((e = joined(g, st)) != cudaSuccess) return e;
+    if (nr > 0 && (e = refine(0, nr, st)) != cudaSuccess) return e;
   }
   if (fan)
-    for (int g = std::max(nr, 1); g < ng; ++g)
-      if ((e = joined(g)) != cudaSuccess) return e;
+    for (int g = first ? 1 : std::max(nr, 1); g < ng; ++g)
+      if ((e = joined(g, st)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
