@@ -22,11 +22,12 @@
 // Storage: M is kept row-major with an odd leading dimension ld >= n, so the QR
 // rank-1 updates are coalesced (32 consecutive columns per warp) and, once R's
 // rows are conjugated in place, they are the contiguous columns of R^dag.
-// Sectors from min(m, n) = 48 (but those of reduced-precision updates) do not run these FP64 sweeps:
-// svd_front_kernel does an unpivoted QR and FP32 sweeps, and k_refine.cu finishes them with exact
-// tensor-core products; the kernels below take what that leaves.  A layer of 16 updates at chi = 512
-// (Bose-Hubbard, L = 32) takes 95 ms with it, 272 ms with the FP64 sweeps; three layers at chi = 128
-// (L = 24) 19 and 60 ms.
+// Sectors of FP64 updates do not run these FP64 sweeps: svd_small_kernel (one CTA) and svd_front_kernel (a
+// cluster) do an unpivoted QR and FP32 sweeps, and exact products finish them, in the CTA up to kSmallK columns
+// and on the tensor cores above (k_refine.cu); the kernels below take what that leaves, and the sectors
+// of reduced-precision updates.  A layer of 16 updates at chi = 512 (Bose-Hubbard, L = 32) takes 72 ms with
+// it, 272 ms with the FP64 sweeps; three layers at chi = 128 (L = 24) 10.2 and 61 ms, at chi = 64 (XXZ, L = 16)
+// 2.6 and 6.9.
 //
 // GB300 runs FP64 at 2 FMA/clk/SM, so one SM per large sector would leave a
 // layer waiting on its largest sectors.  Three kernels share the work:
@@ -79,7 +80,9 @@ constexpr int kRefineMinK = 25;         // smallest min(m, n) refined on the ten
 // a refined sector's FP32 sweeps end with one that found no cosine above this: it has left about the square
 constexpr float kFp32Stop = 1e-3f;
 constexpr int kFrontThreads = 384;      // one-CTA fronts
-constexpr int kSmallK = 24;             // largest min(m, n) refined inside one CTA
+// largest min(m, n) refined inside one CTA: its FP64 products at 24 columns take as long (2 x 60 us) as the
+// refinement's launches do beside other sectors', and grow with the cube
+constexpr int kSmallK = 24;
 // rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
 // a row's dependent FMAs 128)
 constexpr int kAhead = 8;
@@ -2055,7 +2058,10 @@ __global__ void __launch_bounds__(kSvdThreads, 1) jacobi_cta_kernel(const SvdSec
 // those of svd_front; up to kSmallK columns the refinement runs here too (its products are shorter than a
 // kernel launch), above that J and V go to the tensor-core kernels.  The FP64 sweeps of jacobi_cta_kernel
 // paid for every rotation's root and quotient in FP64 (some 1500 cycles of latency a pair); here those
-// are FP32 and the FP64 work is the QR and the refinement's products.
+// are FP32 and the FP64 work is the QR and the refinement's products.  A front of 95 x 95 takes 2.07 ms, 0.84
+// of it the QR (0.6 at the SM's FP64 rate), 1.17 the FP32 sweeps; on a cluster of 8 over L2 it took 3.3.  A whole 15 x 15
+// sector takes 116 us, 39 in the QR, 28 in the sweeps, 42 in two refinement steps: chains of FP64 roots, quotients
+// and sums.
 // ---------------------------------------------------------------------------------------
 struct SmallLayout {
   int ldm, fld, lda;                  // strides of W, F and A
