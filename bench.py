@@ -657,7 +657,10 @@ def run_ours(args, world, rank, local):
                 "frac_of_measured_fp64": achieved / fp64_measured if unit == "GFLOP/s" else None,
                 "kernels": {k: {"launches": v["launches"], "ms": round(v["ms"], 3), "share": v["ms"] / tot_ms}
                             for k, v in ks.items() if v["launches"]}}
-    if dom == "svd":
+    if dom == "svd" and args.precision == "fp64":
+        roofline["flops_note"] = ("nominal QR and Jacobi flops against the FP64 peak: above 1 because FP64 updates sweep "
+                                  "in FP32 and finish on the tensor cores")
+    elif dom == "svd":
         # ncu DRAM bytes of the cluster SVD on the saturated L=24, chi<=1024 chain (bench.py --case
         # small_tf32, the first cluster-SVD launch of the layer): 9.05 + 28.21 GB for a launch of
         # 3.21e11 nominal flops.  The write-back of staged column blocks grows with the sweep work,

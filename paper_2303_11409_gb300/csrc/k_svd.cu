@@ -1198,6 +1198,7 @@ struct FrontBlocks {
   float2* sm;
   float* smn;
   int bsmax, g, gs, cl;
+  int* left;      // set when a bounded wait expires: the sector then goes to the FP64 sweeps
 
   struct Tables {      // one per CTA
     int held[2 * kMaxStaged];      // the block in each slot (-1: none)
@@ -1281,7 +1282,7 @@ struct FrontBlocks {
       const int s = e / bsmax, c = e % bsmax;
       if (T.held[s] >= 0 && T.fresh[s] && c < T.len[s]) smn[e] = __ldcg(nrm + T.col[s] + c);
     }
-    stage_wait(&T.bar, parity);
+    if (!stage_wait(&T.bar, parity)) *left = 1;
     parity ^= 1u;
     __syncthreads();
   }
@@ -2621,6 +2622,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSe
   j32.g = S.groups;
   j32.gs = S.front_staged;
   j32.cl = cluster;
+  j32.left = S.rstate + 1;
   j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
   j32.sm = reinterpret_cast<float2*>(smem_raw);
   j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * fld);
