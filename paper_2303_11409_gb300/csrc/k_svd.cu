@@ -410,7 +410,8 @@ __device__ __forceinline__ int group_slot(int G) {
 // matrix is contiguous in global memory and in the staging area, 16-byte aligned, a multiple of
 // 16 bytes long.  One thread issues them; the CTA waits on an mbarrier (loads) or the issuing
 // thread on the bulk group (stores).  Global data crosses between the generic and the async
-// proxy only behind fence.proxy.async and the cluster barrier.
+// proxy only behind fence.proxy.async and the cluster barrier, staged data behind the same fence for
+// shared memory and a CTA barrier.
 __device__ __forceinline__ uint32_t sh_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void stage_bar_init(uint64_t* b) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(sh_addr(b)) : "memory");
@@ -436,6 +437,8 @@ __device__ __forceinline__ void bulk_store_drain() {
   asm volatile("fence.proxy.async.global;\n" ::: "memory");
 }
 __device__ __forceinline__ void fence_to_async() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
+// Every thread, between its accesses of staged columns and the barrier before a bulk copy reads or overwrites them.
+__device__ __forceinline__ void fence_stage() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 // Bounded wait (about 2 s) for the staging barrier's phase; false when it expired.
 __device__ __forceinline__ bool stage_wait(uint64_t* b, uint32_t parity) {
   const uint32_t a = sh_addr(b);
@@ -664,6 +667,7 @@ struct JacobiBlocks {
                 else
                   rot |= jacobi_pair_mw(sm, n, n, smn, p, q, valid, G, tol2, floor2, s_red, mw_phase, 1 + slot);
               }
+              if (t + 1 == bsmax) fence_stage();
               __syncthreads();
             }
           }
@@ -887,6 +891,7 @@ struct JacobiBlocks32 {
                 }
                 rot |= jacobi_pair32(sm, R, Rr, ld, smn, p, q, valid, G, tol, floor2);
               }
+              if (t + 1 == bsmax) fence_stage();
               __syncthreads();
             }
           }
@@ -1215,7 +1220,7 @@ struct FrontBlocks {
   __device__ __forceinline__ void stage(Tables& T, float2* F, int ld, int K, float* nrm, int rank, int r, int c0,
                                         uint32_t& parity, Barrier barrier) const {
     const int tid = threadIdx.x, lane = tid & 31, nb = 2 * cl * g, slots = 2 * gs;
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    fence_stage();
     __syncthreads();
     int to = -1, want = -1, col = 0, len = 0;
     if (tid < 32) {
@@ -1512,7 +1517,7 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
   }
   sync();
   // ---- FP32 sweeps to FP32 convergence; the floor is a tenth of the FP64 one -------------------
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the staging area held reflectors
+  fence_stage();      // the staging area held reflectors
   __syncthreads();
   const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
   const float fl32 = (float)(0.01 * floor2);
