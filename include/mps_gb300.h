@@ -471,6 +471,14 @@ MPS_API int mps_autotune_min_flops(double flops);
 MPS_API int mps_last_batch_sweeps(mps_t h, int* n_sectors, int64_t* sweeps_sum, int* sweeps_max);
 
 /*
+ * mps_last_batch_paths - how the sectors of the last update call on h were decomposed (any may
+ * be NULL): the number finished by refinement (MPS_SVD_REFINED), by FP64 Jacobi sweeps
+ * (MPS_SVD_SWEEPS), of those the ones that FP32 sweeps went ahead of (MPS_SVD_FP32_START) and the
+ * ones that ran on a team of CTAs (MPS_SVD_TEAM).  Diagnostics; no counterpart in the paper.
+ */
+MPS_API int mps_last_batch_paths(mps_t h, int* refined, int* swept, int* fp32_start, int* on_teams);
+
+/*
  * mps_save - writes the current state of h (its charge rule: U(1), Z_n or several U(1)
  * charges; bond charge tables and Schmidt values, site blocks, and each bond's deflation
  * history) to the file `path` (created or truncated).  The file holds the
@@ -683,6 +691,30 @@ MPS_API int mps_svd_sectors(int n_sectors, const int* m, const int* n,
                     double* d_sigma, const int64_t* sig_off,
                     double* d_y, const int64_t* y_off,
                     int* d_status, void* d_work, int64_t work_bytes, void* cuda_stream);
+
+/*
+ * mps_svd_sectors_path - mps_svd_sectors with a choice of the finish and a record of the path.
+ *   keep_phases   0: as FP64 updates and mps_svd_sectors do (refinement where mps_svd_mixed_min_k
+ *                 allows it); otherwise as TF32 and BF16x3 updates do, whose rounding of Y sees the
+ *                 phases of its columns: pivoted QR and FP64 Jacobi sweeps for every sector
+ *   d_path        n_sectors ints on the device, or NULL: the MPS_SVD_* bits of each sector
+ *                 (written when it has ended with a status of -1 or above)
+ * d_work holds at least mps_svd_path_work_bytes(...) for the same sizes and keep_phases.
+ * Diagnostics of the per-sector SVDs of Sec. II; no counterpart in the paper.
+ */
+#define MPS_SVD_REFINED 1        /* FP32 sweeps, then FP64-accurate corrections */
+#define MPS_SVD_SWEEPS 2         /* FP64 Jacobi sweeps */
+#define MPS_SVD_FP32_START 4     /* FP32 sweeps ahead of the FP64 ones */
+#define MPS_SVD_TEAM 8           /* a team of CTAs in a cooperative launch */
+#define MPS_SVD_ROUND_ROBIN 16   /* the round-robin cluster kernel */
+MPS_API int64_t mps_svd_path_work_bytes(int n_sectors, const int* m, const int* n, int keep_phases);
+MPS_API int mps_svd_sectors_path(int n_sectors, const int* m, const int* n,
+                    const double* d_mats, const int64_t* mat_off,
+                    const double* d_rowscale, const int64_t* row_off,
+                    double* d_sigma, const int64_t* sig_off,
+                    double* d_y, const int64_t* y_off,
+                    int* d_status, int keep_phases, int* d_path,
+                    void* d_work, int64_t work_bytes, void* cuda_stream);
 
 /*
  * mps_svd_mixed_min_k - from which min(m, n) a sector SVD starts with one-sided Jacobi sweeps in

@@ -19,6 +19,7 @@ LIB_PATH = os.path.join(_HERE, "_lib", "libmps_gb300.so")
 MPS_OK, MPS_EINVAL, MPS_ECHARGE, MPS_ENOMEM, MPS_ENOCONV, MPS_ECUDA, MPS_ETIMEOUT = 0, -1, -2, -3, -4, -5, -6
 MPS_FP64, MPS_TF32, MPS_BF16X3 = 0, 1, 2
 MPS_MAX_D = 8
+MPS_SVD_REFINED, MPS_SVD_SWEEPS, MPS_SVD_FP32_START, MPS_SVD_TEAM, MPS_SVD_ROUND_ROBIN = 1, 2, 4, 8, 16
 MPS_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 KERNEL_KINDS = ("theta", "svd", "select", "lambda", "scatter", "gemm", "expect", "amplitude", "sample", "tcgemm",
                 "shadow")
@@ -95,6 +96,7 @@ _SIGS = {
     "mps_gate_layout": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, _i32p, _i32p, ctypes.c_int,
                                        _intp, _i64p]),
     "mps_last_batch_sweeps": (ctypes.c_int, [_h, _intp, _i64p, _intp]),
+    "mps_last_batch_paths": (ctypes.c_int, [_h, _intp, _intp, _intp, _intp]),
     "mps_set_profiling": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_kernel_stats": (ctypes.c_int, [_h, ctypes.c_int, _i64p, _dblp, _dblp, _dblp]),
     "mps_reset_kernel_stats": (ctypes.c_int, [_h]),
@@ -107,6 +109,9 @@ _SIGS = {
                                                _vp, _i64p, _vp, _vp]),
     "mps_svd_sectors": (ctypes.c_int, [ctypes.c_int, _intp, _intp, _vp, _i64p, _vp, _i64p, _vp, _i64p, _vp,
                                        _i64p, _vp, _vp, ctypes.c_int64, _vp]),
+    "mps_svd_path_work_bytes": (ctypes.c_int64, [ctypes.c_int, _intp, _intp, ctypes.c_int]),
+    "mps_svd_sectors_path": (ctypes.c_int, [ctypes.c_int, _intp, _intp, _vp, _i64p, _vp, _i64p, _vp, _i64p, _vp,
+                                            _i64p, _vp, ctypes.c_int, _vp, _vp, ctypes.c_int64, _vp]),
     "mps_set_graphs": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_set_sweep_limit": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_tc_inject_stall": (ctypes.c_int, [ctypes.c_int]),
@@ -476,6 +481,12 @@ class MPS:
         n, tot, mx = ctypes.c_int(), ctypes.c_int64(), ctypes.c_int()
         lib.mps_last_batch_sweeps(self._h, ctypes.byref(n), ctypes.byref(tot), ctypes.byref(mx))
         return dict(sectors=n.value, mean=tot.value / max(n.value, 1), max=mx.value)
+
+    def last_batch_paths(self) -> dict:
+        """Sectors of the last update call by how they were decomposed (mps_last_batch_paths)."""
+        v = [ctypes.c_int() for _ in range(4)]
+        self._check(lib.mps_last_batch_paths(self._h, *[ctypes.byref(x) for x in v]), "mps_last_batch_paths")
+        return dict(zip(("refined", "swept", "fp32_start", "on_teams"), (x.value for x in v)))
 
     def set_profiling(self, on: bool = True):
         self._check(lib.mps_set_profiling(self._h, int(bool(on))), "mps_set_profiling")
@@ -874,9 +885,20 @@ def svd_work_bytes(ms, ns) -> int:
 def svd_sectors(mats, rowscales=None, stream=None):
     """Batched sector SVD on the GPU through mps_svd_sectors (torch supplies device memory).
 
-    mats: list of complex128 host arrays (m_k x n_k).  Returns [(sigma, Y, sweeps)] with
-    M_k = diag(rowscale_k) mats_k = X S Y^dag.
+    mats: list of complex128 host arrays (m_k x n_k).  Returns [(sigma, Y, steps)] with
+    M_k = diag(rowscale_k) mats_k = X S Y^dag; steps counts refinement steps or FP64 sweeps.
     """
+    return [r[:3] for r in _svd_sectors(mats, rowscales, stream, None)]
+
+
+def svd_sectors_path(mats, rowscales=None, keep_phases=False, stream=None):
+    """svd_sectors through mps_svd_sectors_path: [(sigma, Y, steps, path)], path the MPS_SVD_* bits;
+    keep_phases: finished as TF32 and BF16x3 updates do."""
+    return _svd_sectors(mats, rowscales, stream, bool(keep_phases))
+
+
+def _svd_sectors(mats, rowscales, stream, keep_phases):
+    """keep_phases None: mps_svd_sectors, else mps_svd_sectors_path."""
     import torch
     dev = torch.device("cuda")
     ms = [a.shape[0] for a in mats]
@@ -891,29 +913,36 @@ def svd_sectors(mats, rowscales=None, stream=None):
     d_sig = torch.zeros(sum(ks), dtype=torch.float64, device=dev)
     d_y = torch.zeros(2 * sum(n * k for n, k in zip(ns, ks)), dtype=torch.float64, device=dev)
     d_st = torch.zeros(len(mats), dtype=torch.int32, device=dev)
-    wb = svd_work_bytes(ms, ns)
-    d_work = torch.zeros(max(wb, 256), dtype=torch.uint8, device=dev)
+    d_path = torch.zeros(len(mats), dtype=torch.int32, device=dev)
     d_rs = None
     if rowscales is not None:
         d_rs = torch.from_numpy(np.concatenate([np.asarray(r, np.float64) for r in rowscales])).to(dev)
     st = torch.cuda.current_stream().cuda_stream if stream is None else stream
     m_a = np.asarray(ms, np.intc)
     n_a = np.asarray(ns, np.intc)
-    rc = lib.mps_svd_sectors(len(mats), _ptr(m_a, _intp), _ptr(n_a, _intp), d_mats.data_ptr(),
-                             _ptr(mat_off, _i64p), d_rs.data_ptr() if d_rs is not None else None,
-                             _ptr(r_off, _i64p) if d_rs is not None else None,
-                             d_sig.data_ptr(), _ptr(s_off, _i64p), d_y.data_ptr(), _ptr(y_off, _i64p),
-                             d_st.data_ptr(), d_work.data_ptr(), d_work.numel(), st)
+    args = (len(mats), _ptr(m_a, _intp), _ptr(n_a, _intp), d_mats.data_ptr(),
+            _ptr(mat_off, _i64p), d_rs.data_ptr() if d_rs is not None else None,
+            _ptr(r_off, _i64p) if d_rs is not None else None,
+            d_sig.data_ptr(), _ptr(s_off, _i64p), d_y.data_ptr(), _ptr(y_off, _i64p), d_st.data_ptr())
+    if keep_phases is None:
+        wb = svd_work_bytes(ms, ns)
+    else:
+        wb = int(lib.mps_svd_path_work_bytes(len(mats), _ptr(m_a, _intp), _ptr(n_a, _intp), int(keep_phases)))
+    d_work = torch.zeros(max(wb, 256), dtype=torch.uint8, device=dev)
+    if keep_phases is None:
+        rc = lib.mps_svd_sectors(*args, d_work.data_ptr(), d_work.numel(), st)
+    else:
+        rc = lib.mps_svd_sectors_path(*args, int(keep_phases), d_path.data_ptr(), d_work.data_ptr(), d_work.numel(), st)
     if rc != MPS_OK:
-        raise MPSError(rc, "mps_svd_sectors")
+        raise MPSError(rc, "mps_svd_sectors" if keep_phases is None else "mps_svd_sectors_path")
     torch.cuda.synchronize()
     sig = d_sig.cpu().numpy()
     y = d_y.cpu().numpy().view(np.complex128)
-    sts = d_st.cpu().numpy()
+    sts, paths = d_st.cpu().numpy(), d_path.cpu().numpy()
     out = []
     for k in range(len(mats)):
         Y = y[y_off[k]:y_off[k] + ns[k] * ks[k]].reshape(ks[k], ns[k]).T   # column-major n x k
-        out.append((sig[s_off[k]:s_off[k] + ks[k]].copy(), Y.copy(), int(sts[k])))
+        out.append((sig[s_off[k]:s_off[k] + ks[k]].copy(), Y.copy(), int(sts[k]), int(paths[k])))
     return out
 
 

@@ -398,6 +398,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   for (int u = 0; u < nreq; ++u) gates_bytes += a256(16LL * reqs[u].h->rule.gate_len());
   const int64_t kept_off = ws; ws = a256(ws + 4LL * n_sec_total);
   const int64_t status_off = ws; ws = a256(ws + 4LL * n_sec_total);
+  const int64_t path_off = ws; ws = a256(ws + 4LL * n_sec_total);
   const int64_t res_off = ws; ws = a256(ws + (int64_t)sizeof(SelectResult) * nreq);
   // the left lambdas of sectors whose rows are not one run of the bond table (several-U(1)
   // handles), gathered so that the SVD reads its row scale contiguously
@@ -711,6 +712,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       S.sigma = reinterpret_cast<double*>(dptr(W[u].sig_off[si]));
       S.Y = reinterpret_cast<double2*>(dptr(W[u].y_off[si]));
       S.status = reinterpret_cast<int*>(dptr(status_off)) + sec_global;
+      S.path = reinterpret_cast<int*>(dptr(path_off)) + sec_global;
       svd.push_back(S);
       selsec.push_back(SelectSector{S.sigma, std::min(E.rows, E.cols)});
     }
@@ -922,6 +924,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   }
   const int* kept = (const int*)owner->pin_out.p;
   const int* sstat = (const int*)((char*)owner->pin_out.p + (status_off - kept_off));
+  const int* spath = (const int*)((char*)owner->pin_out.p + (path_off - kept_off));
   const SelectResult* res = (const SelectResult*)((char*)owner->pin_out.p + (res_off - kept_off));
 
   // ---- deflation check: an update whose new cut fell below level / kChiGuard x the estimate its
@@ -1000,13 +1003,18 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   int64_t sc_elems = 0;
   std::vector<char> apply(nreq, 0);
   {
-    int bmax = 0;
+    int bmax = 0, path[4] = {};
     int64_t bsum = 0;
     for (int k = 0; k < n_sec_total; ++k) {
       if (sstat[k] < -1) return fail(owner, MPS_ETIMEOUT, "a bounded wait inside the sector SVD expired");
       bmax = std::max(bmax, sstat[k]);
       bsum += std::max(sstat[k], 0);
+      for (int x = 0; x < 4; ++x) path[x] += spath[k] >> x & 1;
     }
+    owner->stats.batch_refined = path[0];
+    owner->stats.batch_swept = path[1];
+    owner->stats.batch_fp32 = path[2];
+    owner->stats.batch_team = path[3];
     owner->stats.batch_sectors = n_sec_total;
     owner->stats.batch_sweeps_sum = bsum;
     owner->stats.batch_sweeps_max = bmax;
@@ -2026,6 +2034,15 @@ int mps_last_batch_sweeps(mps_t h, int* n_sectors, int64_t* sweeps_sum, int* swe
   if (n_sectors) *n_sectors = h->stats.batch_sectors;
   if (sweeps_sum) *sweeps_sum = h->stats.batch_sweeps_sum;
   if (sweeps_max) *sweeps_max = h->stats.batch_sweeps_max;
+  return MPS_OK;
+}
+
+int mps_last_batch_paths(mps_t h, int* refined, int* swept, int* fp32_start, int* on_teams) {
+  if (!h) return MPS_EINVAL;
+  if (refined) *refined = h->stats.batch_refined;
+  if (swept) *swept = h->stats.batch_swept;
+  if (fp32_start) *fp32_start = h->stats.batch_fp32;
+  if (on_teams) *on_teams = h->stats.batch_team;
   return MPS_OK;
 }
 

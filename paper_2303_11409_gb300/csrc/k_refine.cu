@@ -522,7 +522,10 @@ __global__ void __launch_bounds__(256) refine_output_kernel(const SvdSector* __r
       y[S.order[j]] = z;
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *S.status = it;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *S.status = it;
+    if (S.path) *S.path = MPS_SVD_REFINED;
+  }
 }
 
 }  // namespace

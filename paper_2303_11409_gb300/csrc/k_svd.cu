@@ -476,6 +476,7 @@ __host__ __device__ inline int odd_ld(int n) { return n | 1; }
 // share the sector, one barrier per round.
 template <class Mem>
 struct JacobiRoundRobin {
+  static constexpr int kPath = Mem::kCache ? MPS_SVD_ROUND_ROBIN : 0;
   template <class Sync>
   __device__ int operator()(double2* W, int n, int ld, int K, const Work& w, int rank, int nctas, Sync sync,
                             double tol2, double floor2, int max_sweeps, bool& converged) const {
@@ -539,6 +540,7 @@ struct JacobiRoundRobin {
 // separated by CTA barriers, the round by one cluster barrier.  Every pair is visited
 // once per sweep.
 struct JacobiBlocks {
+  static constexpr int kPath = 0;
   double2* sm;   // 2 * gs * bsmax columns of n complex (shared memory)
   double* smn;   // 2 * gs * bsmax norms (shared memory)
   int bsmax;
@@ -1967,13 +1969,19 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
       S.Y[(int64_t)r * n + Mem::ld(w.perm + j)] = y;
     }
   }
-  if (tid_all == 0) *S.status = converged ? sweep : -1;
+  if (tid_all == 0) {
+    *S.status = converged ? sweep : -1;
+    const bool start = std::is_same<J32, JacobiBlocks32>::value && S.f32 && K >= 2;
+    if (S.path) *S.path = MPS_SVD_SWEEPS | (start ? MPS_SVD_FP32_START : 0) | Sync::kPath | Jacobi::kPath;
+  }
 }
 
 struct CtaSync {
+  static constexpr int kPath = 0;
   __device__ void operator()() const { __syncthreads(); }
 };
 struct ClusterSync {
+  static constexpr int kPath = 0;
   __device__ void operator()() const { cluster_sync_all(); }
 };
 
@@ -1981,6 +1989,7 @@ struct ClusterSync {
 // arrivals, zero at the launch.  The wait is bounded (about 20 s): a CTA whose wait expires marks the
 // sector and leaves; no bulk copy is in flight at a barrier, so nothing outlives it.
 struct TeamSync {
+  static constexpr int kPath = MPS_SVD_TEAM;
   unsigned* bar;
   int* status;
   unsigned size;
@@ -2535,7 +2544,10 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
         }
         S.Y[(int64_t)rank[c] * n + perm[j]] = z;
       }
-      if (tid == 0) *S.status = steps;
+      if (tid == 0) {
+        *S.status = steps;
+        if (S.path) *S.path = MPS_SVD_REFINED;
+      }
       return;
     }
   }
@@ -3202,17 +3214,88 @@ extern "C" int mps_svd_mixed_sweeps(int max_sweeps) {
   return MPS_OK;
 }
 
-namespace mps {
-
-}  // namespace mps
-
 using namespace mps;
 
-extern "C" int64_t mps_svd_work_bytes(int n_sectors, const int* m, const int* n) {
+extern "C" int64_t mps_svd_path_work_bytes(int n_sectors, const int* m, const int* n, int keep_phases) {
   if (n_sectors < 0 || (n_sectors > 0 && (!m || !n))) return -1;
   SvdScratchLayout L;
-  if (!svd_layout(n_sectors, m, n, L)) return -1;
+  const std::vector<char> exact(n_sectors, keep_phases != 0);
+  if (!svd_layout(n_sectors, m, n, L, -1, exact.data())) return -1;
   return ((int64_t)sizeof(SvdSector) * n_sectors + 255) / 256 * 256 + L.total;
+}
+
+extern "C" int64_t mps_svd_work_bytes(int n_sectors, const int* m, const int* n) {
+  return mps_svd_path_work_bytes(n_sectors, m, n, 0);
+}
+
+namespace {
+// The sectors of one call, in scratch laid out by L behind desc bytes of descriptors.
+struct SectorCall {
+  int n_sectors;
+  const int *m, *n;
+  const double* d_mats;
+  const int64_t* mat_off;
+  const double* d_rowscale;
+  const int64_t* row_off;
+  double* d_sigma;
+  const int64_t* sig_off;
+  double* d_y;
+  const int64_t* y_off;
+  int *d_status, *d_path;
+  bool valid() const {
+    return n_sectors > 0 && m && n && d_mats && mat_off && d_sigma && sig_off && d_y && y_off && d_status &&
+           !(d_rowscale && !row_off);
+  }
+  int64_t desc() const { return ((int64_t)sizeof(SvdSector) * n_sectors + 255) / 256 * 256; }
+  int run(const SvdScratchLayout& L, void* d_work, cudaStream_t st) const {
+    std::vector<SvdSector> cta, cl;
+    char* base = (char*)d_work + desc();
+    for (int k = 0; k < n_sectors; ++k) {
+      SvdSector S = {};
+      S.theta = reinterpret_cast<const double2*>(d_mats) + mat_off[k];
+      S.rowscale = d_rowscale ? d_rowscale + row_off[k] : nullptr;
+      S.m = m[k];
+      S.n = n[k];
+      svd_fill_scratch(S, L, k, base);
+      S.sigma = d_sigma + sig_off[k];
+      S.Y = reinterpret_cast<double2*>(d_y) + y_off[k];
+      S.status = d_status + k;
+      S.path = d_path ? d_path + k : nullptr;
+      (S.mode == kSvdCluster ? cl : cta).push_back(S);
+    }
+    std::vector<SvdSector> all(cta);
+    all.insert(all.end(), cl.begin(), cl.end());
+    std::vector<SvdGroup> groups;
+    SvdTune tune;
+    svd_forced_tune(tune);
+    if (svd_group(all, groups, tune) != cudaSuccess) return MPS_ECUDA;
+    if (cudaMemcpyAsync(d_work, all.data(), sizeof(SvdSector) * all.size(), cudaMemcpyHostToDevice, st) !=
+        cudaSuccess)
+      return MPS_ECUDA;
+    const SvdSector* d_all = reinterpret_cast<const SvdSector*>(d_work);
+    if (launch_svd_groups(d_all, groups, st, nullptr, 0, nullptr, nullptr) != cudaSuccess) return MPS_ECUDA;
+    // the descriptors came from pageable host memory: finish before returning
+    return cudaStreamSynchronize(st) == cudaSuccess ? MPS_OK : MPS_ECUDA;
+  }
+};
+}  // namespace
+
+extern "C" int mps_svd_sectors_path(int n_sectors, const int* m, const int* n,
+                                    const double* d_mats, const int64_t* mat_off,
+                                    const double* d_rowscale, const int64_t* row_off,
+                                    double* d_sigma, const int64_t* sig_off,
+                                    double* d_y, const int64_t* y_off,
+                                    int* d_status, int keep_phases, int* d_path,
+                                    void* d_work, int64_t work_bytes, void* cuda_stream) {
+  if (n_sectors == 0) return MPS_OK;
+  const SectorCall C{n_sectors, m,       n,   d_mats, mat_off,  d_rowscale, row_off,
+                     d_sigma,   sig_off, d_y, y_off,  d_status, d_path};
+  if (!C.valid() || !d_work) return MPS_EINVAL;
+  SvdScratchLayout L;
+  const std::vector<char> exact(n_sectors, keep_phases != 0);
+  if (!svd_layout(n_sectors, m, n, L, -1, exact.data())) return MPS_EINVAL;
+  if (work_bytes < C.desc() + L.total) return MPS_EINVAL;
+  return C.run(L, d_work, (cudaStream_t)cuda_stream);
 }
 
 extern "C" int mps_svd_sectors(int n_sectors, const int* m, const int* n,
@@ -3221,44 +3304,8 @@ extern "C" int mps_svd_sectors(int n_sectors, const int* m, const int* n,
                                double* d_sigma, const int64_t* sig_off,
                                double* d_y, const int64_t* y_off,
                                int* d_status, void* d_work, int64_t work_bytes, void* cuda_stream) {
-  if (n_sectors == 0) return MPS_OK;
-  if (n_sectors < 0 || !m || !n || !d_mats || !mat_off || !d_sigma || !sig_off || !d_y || !y_off ||
-      !d_status || !d_work)
-    return MPS_EINVAL;
-  if (d_rowscale && !row_off) return MPS_EINVAL;
-  SvdScratchLayout L;
-  if (!svd_layout(n_sectors, m, n, L)) return MPS_EINVAL;
-  const int64_t desc = ((int64_t)sizeof(SvdSector) * n_sectors + 255) / 256 * 256;
-  if (work_bytes < desc + L.total) return MPS_EINVAL;
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  std::vector<SvdSector> cta, cl;
-  char* base = (char*)d_work + desc;
-  for (int k = 0; k < n_sectors; ++k) {
-    SvdSector S = {};
-    S.theta = reinterpret_cast<const double2*>(d_mats) + mat_off[k];
-    S.rowscale = d_rowscale ? d_rowscale + row_off[k] : nullptr;
-    S.m = m[k];
-    S.n = n[k];
-    svd_fill_scratch(S, L, k, base);
-    S.sigma = d_sigma + sig_off[k];
-    S.Y = reinterpret_cast<double2*>(d_y) + y_off[k];
-    S.status = d_status + k;
-    (S.mode == kSvdCluster ? cl : cta).push_back(S);
-  }
-  std::vector<SvdSector> all(cta);
-  all.insert(all.end(), cl.begin(), cl.end());
-  std::vector<SvdGroup> groups;
-  SvdTune tune;
-  svd_forced_tune(tune);
-  if (svd_group(all, groups, tune) != cudaSuccess) return MPS_ECUDA;
-  if (cudaMemcpyAsync(d_work, all.data(), sizeof(SvdSector) * all.size(), cudaMemcpyHostToDevice, st) !=
-      cudaSuccess)
-    return MPS_ECUDA;
-  const SvdSector* d_all = reinterpret_cast<const SvdSector*>(d_work);
-  if (launch_svd_groups(d_all, groups, st, nullptr, 0, nullptr, nullptr) != cudaSuccess) return MPS_ECUDA;
-  // the descriptors came from pageable host memory: finish before returning
-  if (cudaStreamSynchronize(st) != cudaSuccess) return MPS_ECUDA;
-  return MPS_OK;
+  return mps_svd_sectors_path(n_sectors, m, n, d_mats, mat_off, d_rowscale, row_off, d_sigma, sig_off, d_y, y_off,
+                              d_status, 0, nullptr, d_work, work_bytes, cuda_stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -3281,17 +3328,16 @@ extern "C" int mps_svd_sectors_noalloc(int n_sectors, const int* m, const int* n
                                        double* d_y, const int64_t* y_off,
                                        int* d_status, void* cuda_stream) {
   if (n_sectors == 0) return MPS_OK;
-  if (n_sectors < 0 || !m || !n || !d_mats || !mat_off || !d_sigma || !sig_off || !d_y || !y_off || !d_status)
-    return MPS_EINVAL;
-  if (d_rowscale && !row_off) return MPS_EINVAL;
+  const SectorCall C{n_sectors, m,       n,   d_mats, mat_off,  d_rowscale, row_off,
+                     d_sigma,   sig_off, d_y, y_off,  d_status, nullptr};
+  if (!C.valid()) return MPS_EINVAL;
   SvdScratchLayout L;
   if (!svd_layout(n_sectors, m, n, L)) return MPS_EINVAL;
-  const int64_t desc = ((int64_t)sizeof(SvdSector) * n_sectors + 255) / 256 * 256;
-  if (desc + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) {   // the FP64 sweeps need less scratch
+  if (C.desc() + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) {   // the FP64 sweeps need less scratch
     const std::vector<char> plain(n_sectors, 1);
     if (!svd_layout(n_sectors, m, n, L, -1, plain.data())) return MPS_EINVAL;
   }
-  if (desc + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) return MPS_ENOMEM;   // over the fixed scratch
+  if (C.desc() + L.total > (int64_t)MPS_NOALLOC_SCRATCH_BYTES) return MPS_ENOMEM;   // over the fixed scratch
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return MPS_ECUDA;
   if (dev < 0 || dev >= kNoAllocMaxDevices) return MPS_EINVAL;
@@ -3305,32 +3351,5 @@ extern "C" int mps_svd_sectors_noalloc(int n_sectors, const int* m, const int* n
     }
     d_work = g_noalloc_addr[dev];
   }
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  std::vector<SvdSector> cta, cl;
-  char* base = (char*)d_work + desc;
-  for (int k = 0; k < n_sectors; ++k) {
-    SvdSector S = {};
-    S.theta = reinterpret_cast<const double2*>(d_mats) + mat_off[k];
-    S.rowscale = d_rowscale ? d_rowscale + row_off[k] : nullptr;
-    S.m = m[k];
-    S.n = n[k];
-    svd_fill_scratch(S, L, k, base);
-    S.sigma = d_sigma + sig_off[k];
-    S.Y = reinterpret_cast<double2*>(d_y) + y_off[k];
-    S.status = d_status + k;
-    (S.mode == kSvdCluster ? cl : cta).push_back(S);
-  }
-  std::vector<SvdSector> all(cta);
-  all.insert(all.end(), cl.begin(), cl.end());
-  std::vector<SvdGroup> groups;
-  SvdTune tune;
-  svd_forced_tune(tune);
-  if (svd_group(all, groups, tune) != cudaSuccess) return MPS_ECUDA;
-  if (cudaMemcpyAsync(d_work, all.data(), sizeof(SvdSector) * all.size(), cudaMemcpyHostToDevice, st) !=
-      cudaSuccess)
-    return MPS_ECUDA;
-  const SvdSector* d_all = reinterpret_cast<const SvdSector*>(d_work);
-  if (launch_svd_groups(d_all, groups, st, nullptr, 0, nullptr, nullptr) != cudaSuccess) return MPS_ECUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return MPS_ECUDA;
-  return MPS_OK;
+  return C.run(L, d_work, (cudaStream_t)cuda_stream);
 }

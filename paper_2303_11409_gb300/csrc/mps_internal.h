@@ -220,7 +220,8 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   double* pivv;               // cluster mode: per-CTA pivot values, then two scalars
   double* sigma;              // out: min(m, n) values, descending
   double2* Y;                 // out: n x min(m, n) column-major right singular vectors
-  int* status;                // out: Jacobi sweeps used, or -1 when not converged
+  int* status;                // out: refinement steps or Jacobi sweeps used, or -1 when not converged
+  int* path;                  // out (or nullptr): MPS_SVD_* bits of how it was finished
   int m, n;
   int mode;                   // kSvdSmem or kSvdCluster
   int small;                  // kSvdSmem: refined inside the CTA
@@ -332,6 +333,7 @@ struct Stats {
   double norm_all = 0, norm_kept = 0;
   int batch_sectors = 0, batch_sweeps_max = 0;   // over every update of the last call
   int64_t batch_sweeps_sum = 0;
+  int batch_refined = 0, batch_swept = 0, batch_fp32 = 0, batch_team = 0;
   int64_t deflated_updates = 0, deflation_redos = 0;   // cut-estimate deflation, cumulative
 };
 

@@ -51,3 +51,75 @@ def test_staged_blocks_give_the_same_bits_each_time(gpu_lib):
     for out in others:
         for (s, y, _), (s1, y1, _) in zip(first, out):
             assert np.array_equal(s, s1) and np.array_equal(y, y1)
+
+
+@pytest.mark.parametrize("decades", [0.0, 8.0])
+def test_sweeps_of_reduced_precision_updates_match_lapack(gpu_lib, decades):
+    """Pivoted QR and FP64 sweeps in one CTA (up to about 95 columns) and on clusters, from 192 columns behind FP32
+    sweeps and a Cholesky QR of their rotations."""
+    m = gpu_lib
+    shapes = [(15, 16), (48, 48), (95, 95), (112, 112), (130, 238), (192, 192), (193, 193), (257, 255), (300, 310),
+              (420, 260), (230, 480), (640, 610)]
+    mats, scales = _graded(shapes, decades, 21 + int(decades))
+    for A, w, (s, y, sweeps, path) in zip(mats, scales, m.svd_sectors_path(mats, scales, keep_phases=True)):
+        start = m.MPS_SVD_FP32_START if min(A.shape) >= 192 else 0
+        assert path == m.MPS_SVD_SWEEPS | start and sweeps > 0
+        _check(w[:, None] * A, s, y)
+
+
+def test_which_sectors_are_refined(gpu_lib):
+    """Spectra without large degenerate groups settle at every size; large groups of equal values and zero matrices
+    are left to the FP64 sweeps."""
+    m = gpu_lib
+    from tests import test_gpu_svd_fronts as F
+    from tests import test_gpu_svd_refine as T
+    for decades in (0.0, 8.0):
+        mats, scales = _graded(T.SHAPES + F.SMALL + F.ONE_CTA + F.CLUSTER, decades, 5)
+        assert all(r[3] == m.MPS_SVD_REFINED for r in m.svd_sectors_path(mats, scales))
+    rng = np.random.default_rng(7)
+    Q, P = W.haar_unitary(72, rng), W.haar_unitary(72, rng)
+    left = [Q @ np.diag(np.repeat([1.0, 0.5, 0.25], 24)) @ P,
+            Q @ np.diag(np.concatenate([1 + 1e-10 * np.arange(36), 0.2 + 1e-5 * np.arange(36)])) @ P,
+            np.zeros((50, 60), complex)]
+    settled = [W.random_complex((80, 13), rng) @ W.random_complex((13, 70), rng), np.eye(64, dtype=complex),
+               1e-130 * W.random_complex((50, 50), rng), W.haar_unitary(300, rng)]
+    assert [r[3] for r in m.svd_sectors_path(left)] == [m.MPS_SVD_SWEEPS] * len(left)
+    assert [r[3] for r in m.svd_sectors_path(settled)] == [m.MPS_SVD_REFINED] * len(settled)
+
+
+@pytest.mark.parametrize("L,chi", [(10, 300), (12, 700)])
+def test_when_teams_are_formed(gpu_lib, L, chi):
+    """Few large sectors of a TF32 update take teams of CTAs, unless the phases are captured; an FP64 update's are refined,
+    but for those up to 24 columns that one CTA cannot hold (13 x 522 here)."""
+    import torch
+    from oracle import gates
+    from tests.helpers import load_state, random_state
+    m = gpu_lib
+    st = random_state(L, 5, L, chi, seed=chi)
+    stream = torch.cuda.Stream()
+    for precision, graphs in ((m.MPS_TF32, False), (m.MPS_TF32, True), (m.MPS_FP64, False)):
+        g = m.MPS(5, [1] * L, chi, precision=precision, stream=stream.cuda_stream)
+        load_state(g, st)
+        g.set_graphs(graphs)
+        s = L // 2 - 1
+        g.apply_gate2(s, gates.bh_gate(L, s, 5, 1.0, 2.0, 0.3), chi, 1e-10)
+        p = g.last_batch_paths()
+        if precision == m.MPS_FP64:
+            assert p["refined"] >= 10 and p["swept"] <= 1 and p["fp32_start"] == p["on_teams"] == 0
+        else:
+            assert p["refined"] == 0 and p["swept"] > 0 and (p["on_teams"] > 0) == (not graphs)
+        g.close()
+
+
+@pytest.mark.parametrize("min_k", [0, 16])
+def test_small_sectors_on_one_cta_and_on_block_clusters(gpu_lib, min_k):
+    m = gpu_lib
+    mats, scales = _graded([(16, 16), (17, 40), (48, 48), (64, 31), (85, 85), (90, 120), (130, 70)], 8.0, 31)
+    try:
+        m.svd_cluster_min_k(min_k)
+        out = m.svd_sectors_path(mats, scales, keep_phases=True)
+    finally:
+        m.svd_cluster_min_k(0)
+    for A, w, (s, y, sweeps, path) in zip(mats, scales, out):
+        assert path == m.MPS_SVD_SWEEPS and sweeps > 0
+        _check(w[:, None] * A, s, y)
