@@ -407,9 +407,15 @@ MPS_API int64_t mps_launch_count(void);
  * call returns it with the state unchanged).  For tests of the timeout path without
  * faulting or hanging the GPU; nothing is in flight when the kernel frees its tensor
  * memory.  The paper has no counterpart.
+ *
+ * mps_svd_inject_stall - the same for the waits for staged columns in the sector SVD (any handle, and
+ * mps_svd_sectors), by bits: 1, the block-Jacobi sweeps, whose sectors then end with status -2 and
+ * whose calls report MPS_ETIMEOUT; 0: off.  The barriers then expect 16 bytes more than are copied, and
+ * the wait runs out after about 50 ms instead of 2 s.  MPS_EINVAL for other bits.  The paper has no counterpart.
  */
 MPS_API int mps_set_sweep_limit(mps_t h, int max_sweeps);
 MPS_API int mps_tc_inject_stall(int on);
+MPS_API int mps_svd_inject_stall(int what);
 
 /*
  * mps_set_graphs - when on, each update call on h (mps_apply_gate2/_layer, and the
@@ -679,7 +685,8 @@ MPS_API int mps_gate_layout(int d, int zn, int ncomp, const int32_t* phys_charge
  *   d_sigma + sig_off[k]   min(m_k, n_k) singular values, descending
  *   d_y + y_off[k]         the right singular vectors as an n_k x min(m_k,n_k)
  *                          column-major complex128 matrix Y (M = X S Y^dag)
- *   d_status[k]            Jacobi sweeps used, or -1 if not converged
+ *   d_status[k]            refinement steps or Jacobi sweeps used, -1 if not converged, -2 when a
+ *                          bounded wait inside the kernel expired (no values then)
  * mat_off, row_off, sig_off, y_off, m, n are host int64/int arrays of length
  * n_sectors; d_work is device scratch of work_bytes bytes, at least
  * mps_svd_work_bytes(...) for the same sizes.

@@ -13,7 +13,7 @@ from ._binding import MPS_NOALLOC_SCRATCH_BYTES, svd_sectors_noalloc, svd_sector
 from ._binding import (MPS_SVD_REFINED, MPS_SVD_SWEEPS, MPS_SVD_FP32_START, MPS_SVD_TEAM,  # noqa: F401
                        MPS_SVD_ROUND_ROBIN)
 from ._binding import Executor, footprint_bytes, fp64_peak_probe, zgemm_tc  # noqa: F401
-from ._binding import tc_inject_stall, svd_mixed_min_k, svd_mixed_sweeps, svd_cluster_min_k  # noqa: F401
+from ._binding import tc_inject_stall, svd_inject_stall, svd_mixed_min_k, svd_mixed_sweeps, svd_cluster_min_k  # noqa: F401
 from ._binding import (autotune_clear, autotune_force, autotune_freeze, autotune_min_flops,  # noqa: F401
                        autotune_stats, autotune_table)
 from . import models, tebd, serve  # noqa: F401

@@ -115,6 +115,7 @@ _SIGS = {
     "mps_set_graphs": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_set_sweep_limit": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_tc_inject_stall": (ctypes.c_int, [ctypes.c_int]),
+    "mps_svd_inject_stall": (ctypes.c_int, [ctypes.c_int]),
     "mps_graph_stats": (ctypes.c_int, [_h, _i64p, _i64p, _i64p]),
     "mps_set_autotune": (ctypes.c_int, [_h, ctypes.c_int]),
     "mps_autotune_stats": (ctypes.c_int, [_i64p, _i64p, _i64p]),
@@ -688,6 +689,13 @@ def autotune_force(candidate: int) -> None:
 def autotune_freeze(frozen: bool = True) -> None:
     """Frozen: sector-size histograms not yet in the table keep the default shape, untuned."""
     lib.mps_autotune_freeze(int(bool(frozen)))
+
+
+def svd_inject_stall(what: int) -> None:
+    """Bits of the sector SVD's staging waits that are made to run out (1: the block sweeps; 0: none)."""
+    rc = lib.mps_svd_inject_stall(int(what))
+    if rc != MPS_OK:
+        raise MPSError(rc, "mps_svd_inject_stall")
 
 
 def svd_mixed_min_k(min_k: int) -> None:

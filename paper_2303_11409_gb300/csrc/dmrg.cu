@@ -1612,6 +1612,8 @@ struct Dmrg {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     resolve();
     if (e != cudaSuccess) return fail(MPS_ECUDA, std::string("DMRG SVD: ") + cudaGetErrorString(e));
+    for (int k = 0; k < ns; ++k)
+      if (stat_h[k] < -1) return fail(MPS_ETIMEOUT, "DMRG: a bounded wait inside the sector SVD expired");
     if (res_h->status != 0) return fail(MPS_EINVAL, "DMRG: all singular values vanish");
     bool noconv = false;
     for (int k = 0; k < ns; ++k) noconv = noconv || stat_h[k] < 0;
@@ -1913,6 +1915,8 @@ struct Dmrg {
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       resolve();
       if (e != cudaSuccess) return fail(MPS_ECUDA, std::string("DMRG canonical form: ") + cudaGetErrorString(e));
+      for (int k = 0; k < ns; ++k)
+        if (stat_h[k] < -1) return fail(MPS_ETIMEOUT, "DMRG: a bounded wait inside the sector SVD expired");
       if (res_h->status != 0) return fail(MPS_EINVAL, "DMRG canonical form: all singular values vanish");
       for (int k = 0; k < ns; ++k)
         if (stat_h[k] < 0) rc = MPS_ENOCONV;

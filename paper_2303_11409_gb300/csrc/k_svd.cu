@@ -73,7 +73,7 @@ constexpr double kEps = 2.220446049250313e-16;
 constexpr int kMaxCached = 16;          // rows cached in registers per lane (n <= 512)
 constexpr int kMaxCluster = 16;
 constexpr int kMaxTeam = 304;           // CTAs of a team: 2 on each of 152 SMs
-constexpr int kSvdTeamExpired = -2;     // a sector's status when a team's wait ran out
+constexpr int kSvdExpired = -2;         // a sector's status when a bounded wait ran out
 constexpr int kMaxWarps = 16;
 constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps per CTA, 2 CTAs per SM
 constexpr int kRefineMinK = 25;         // smallest min(m, n) refined on the tensor cores
@@ -86,6 +86,7 @@ constexpr int kSmallK = 24;
 // rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
 // a row's dependent FMAs 128)
 constexpr int kAhead = 8;
+constexpr int kStallBlocks = 1;         // bits of mps_svd_inject_stall: the block sweeps
 constexpr int kMaxStaged = 16;          // block pairs staged at once by one block-Jacobi CTA
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -439,8 +440,11 @@ __device__ __forceinline__ void bulk_store_drain() {
 __device__ __forceinline__ void fence_to_async() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
 // Every thread, between its accesses of staged columns and the barrier before a bulk copy reads or overwrites them.
 __device__ __forceinline__ void fence_stage() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-// Bounded wait (about 2 s) for the staging barrier's phase; false when it expired.
-__device__ __forceinline__ bool stage_wait(uint64_t* b, uint32_t parity) {
+// Bounded wait (about 2 s; 50 ms when the barrier is made to expect bytes that never come) for the
+// staging barrier's phase; false when it expired.  The CTA then leaves its columns alone, keeps to the
+// barriers that it shares with others, and waits once more for its copies in flight before it ends.
+__device__ __forceinline__ bool stage_wait(uint64_t* b, uint32_t parity, bool stall) {
+  const long long limit = stall ? 100000000LL : 4000000000LL;
   const uint32_t a = sh_addr(b);
   const long long t0 = clock64();
   for (;;) {
@@ -451,7 +455,7 @@ __device__ __forceinline__ bool stage_wait(uint64_t* b, uint32_t parity) {
         : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
-    if (clock64() - t0 > 4000000000LL) return false;
+    if (clock64() - t0 > limit) return false;
   }
 }
 
@@ -547,6 +551,7 @@ struct JacobiBlocks {
   int g;         // a round has cl0 * g block pairs; CTA `rank` takes the pairs rank, rank + nctas, ...
   int gs;        // block pairs staged at once
   int cl0;       // the cluster size that fixes the block ordering (nctas itself on a cluster)
+  bool stall;    // expect bytes that no copy brings
   // how many block pairs a cluster's CTA stages together with pair p
   __device__ int staged_with(int p) const {
     const int q = p / cl0;
@@ -568,6 +573,7 @@ struct JacobiBlocks {
     const int worker = rank * nwarps + warp, workers = nctas * nwarps;
     const int nb = 2 * cl0 * g, own = (cl0 * g - rank + nctas - 1) / nctas;
     const bool team = nctas != cl0;   // one pair at a time, in the lane groups the cluster would use
+    bool dead = false;                // a wait of this CTA expired
     int sweep = 0;
     converged = K < 2;
     for (; !converged && sweep < max_sweeps; ++sweep) {
@@ -587,7 +593,7 @@ struct JacobiBlocks {
       if (tid == 0) s_rot = 0;
       bool rot = false;
       for (int r = 0; r < nb - 1; ++r) {
-        for (int c0 = 0; c0 < own; c0 += team ? 1 : gs) {        // chunks of gs block pairs of this CTA
+        for (int c0 = 0; c0 < own && !dead; c0 += team ? 1 : gs) {        // chunks of gs block pairs of this CTA
           const int ns = team ? 1 : min(gs, g - c0);
           const int ns_ref = team ? staged_with(rank + c0 * nctas) : ns;
           if (tid < 2 * gs) {
@@ -610,7 +616,7 @@ struct JacobiBlocks {
             uint32_t bytes = 0;
             for (int j = 0; j < 2 * ns; ++j) bytes += (uint32_t)s_len[j] * (uint32_t)n * 16u;
             fence_to_async();
-            stage_expect(&s_bar, bytes);
+            stage_expect(&s_bar, bytes + (stall ? 16u : 0u));
             for (int j = 0; j < 2 * ns; ++j)
               for (int c = 0; c < s_len[j]; ++c)
                 bulk_load(sm + ((int64_t)j * bsmax + c) * n, W + (int64_t)(s_col[j] + c) * ld, (uint32_t)n * 16u,
@@ -618,9 +624,9 @@ struct JacobiBlocks {
           }
           for (int j = 0; j < 2 * ns; ++j)
             for (int c = tid; c < s_len[j]; c += blockDim.x) smn[j * bsmax + c] = __ldcg(w.nrm + s_col[j] + c);
-          stage_wait(&s_bar, stage_parity);
+          dead = __syncthreads_or(!stage_wait(&s_bar, stage_parity, stall));
+          if (dead) break;
           stage_parity ^= 1u;
-          __syncthreads();
           if (r == 0) {   // pairs inside each staged block, round-robin within the block
             const int mpb = bsmax + (bsmax & 1);
             const int P = 2 * ns * (mpb / 2);
@@ -688,8 +694,13 @@ struct JacobiBlocks {
       if (rot) s_rot = 1;
       __syncthreads();
       if (tid == 0 && s_rot) __stcg(w.flags + sweep, 1);
+      if (tid == 0 && dead) __stcg(w.flags + max_sweeps, 1);
       sync();
       converged = __ldcg(w.flags + sweep) == 0;
+      if (__ldcg(w.flags + max_sweeps) != 0) {      // some CTA's wait
+        if (dead) stage_wait(&s_bar, stage_parity, stall);
+        return kSvdExpired;
+      }
     }
     return sweep;
   }
@@ -778,11 +789,12 @@ __device__ __forceinline__ int group_width32(int P, int R, int nwarps) {
 // ordering as JacobiBlocks, columns of Rr FP32 complex staged whole in shared memory (the
 // FP64 kernel's staging area holds them: 8 (jlen + K) <= 16 jlen bytes per column), dot
 // products over the first R rows.  Returns the sweeps used (converged: a sweep without a
-// rotation).  flags: max_sweeps + 1 ints, zero on entry.
+// rotation) or kSvdExpired.  flags: max_sweeps + 1 ints, zero on entry (the last for a wait that expired).
 struct JacobiBlocks32 {
   float2* sm;
   float* smn;
   int bsmax, g, gs, cl0;      // as in JacobiBlocks
+  bool stall;
   __device__ int staged_with(int p) const {
     const int q = p / cl0;
     return min(gs, g - q / gs * gs);
@@ -801,6 +813,7 @@ struct JacobiBlocks32 {
     const int worker = rank * nwarps + warp, workers = nctas * nwarps;
     const int nb = 2 * cl0 * g, own = (cl0 * g - rank + nctas - 1) / nctas;
     const bool team = nctas != cl0;
+    bool dead = false;
     int sweep = 0;
     converged = K < 2;
     for (; !converged && sweep < max_sweeps; ++sweep) {
@@ -818,7 +831,7 @@ struct JacobiBlocks32 {
       if (tid == 0) s_rot32 = 0;
       bool rot = false;
       for (int r = 0; r < nb - 1; ++r) {
-        for (int c0 = 0; c0 < own; c0 += team ? 1 : gs) {
+        for (int c0 = 0; c0 < own && !dead; c0 += team ? 1 : gs) {
           const int ns = team ? 1 : min(gs, g - c0);
           const int ns_ref = team ? staged_with(rank + c0 * nctas) : ns;
           if (tid < 2 * gs) {
@@ -841,7 +854,7 @@ struct JacobiBlocks32 {
             uint32_t bytes = 0;
             for (int j = 0; j < 2 * ns; ++j) bytes += (uint32_t)s_len32[j] * (uint32_t)ld * 8u;
             fence_to_async();
-            stage_expect(&s_bar32, bytes);
+            stage_expect(&s_bar32, bytes + (stall ? 16u : 0u));
             for (int j = 0; j < 2 * ns; ++j)
               for (int c = 0; c < s_len32[j]; ++c)
                 bulk_load(sm + ((int64_t)j * bsmax + c) * ld, F + (int64_t)(s_col32[j] + c) * ld, (uint32_t)ld * 8u,
@@ -849,9 +862,9 @@ struct JacobiBlocks32 {
           }
           for (int j = 0; j < 2 * ns; ++j)
             for (int c = tid; c < s_len32[j]; c += blockDim.x) smn[j * bsmax + c] = __ldcg(nrm + s_col32[j] + c);
-          stage_wait(&s_bar32, stage_parity);
+          dead = __syncthreads_or(!stage_wait(&s_bar32, stage_parity, stall));
+          if (dead) break;
           stage_parity ^= 1u;
-          __syncthreads();
           if (r == 0) {
             const int mpb = bsmax + (bsmax & 1);
             const int P = 2 * ns * (mpb / 2);
@@ -912,8 +925,13 @@ struct JacobiBlocks32 {
       if (rot) s_rot32 = 1;
       __syncthreads();
       if (tid == 0 && s_rot32) __stcg(flags + sweep, 1);
+      if (tid == 0 && dead) __stcg(flags + max_sweeps, 1);
       sync();
       converged = __ldcg(flags + sweep) == 0;
+      if (__ldcg(flags + max_sweeps) != 0) {
+        if (dead) stage_wait(&s_bar32, stage_parity, stall);
+        return kSvdExpired;
+      }
     }
     return sweep;
   }
@@ -922,9 +940,10 @@ struct NoJacobi32 {};
 
 // The mixed-precision start of a cluster sector's sweeps (see above).  J: jlen x K, column c at
 // J + c * jld (FP64, L2).  On return the FP64 Jacobi matrix is S.a1 (same jld), its first
-// *nsel_out columns J V and the rest zero.  Every CTA of the cluster calls it.
+// *nsel_out columns J V and the rest zero.  Every CTA of the cluster calls it.  False when a
+// wait expired (in every CTA alike).
 template <class Sync>
-__device__ void mixed_precondition(const SvdSector& S, const Work& w, const double2* J, int jlen, int jld, int K,
+__device__ bool mixed_precondition(const SvdSector& S, const Work& w, const double2* J, int jlen, int jld, int K,
                                    int rank, int nctas, Sync sync, double floor2, int max_sweeps,
                                    const JacobiBlocks32& j32, int* nsel_out) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -953,8 +972,9 @@ __device__ void mixed_precondition(const SvdSector& S, const Work& w, const doub
   const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
   const float fl32 = (float)(0.01 * floor2 * sc * sc);
   bool conv32 = false;
-  j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps),
-      conv32);
+  if (j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps),
+          conv32) == kSvdExpired)
+    return false;
   for (int j = worker; j < K; j += workers) {   // final FP32 norms
     const float2* a = F + (int64_t)j * fld;
     float acc = 0.f;
@@ -1063,6 +1083,7 @@ __device__ void mixed_precondition(const SvdSector& S, const Work& w, const doub
   for (int s = tid_all; s <= max_sweeps; s += threads_all) L2Mem::st(w.flags + s, 0);
   sync();
   *nsel_out = ns;
+  return true;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1289,7 +1310,7 @@ struct FrontBlocks {
       const int s = e / bsmax, c = e % bsmax;
       if (T.held[s] >= 0 && T.fresh[s] && c < T.len[s]) smn[e] = __ldcg(nrm + T.col[s] + c);
     }
-    if (!stage_wait(&T.bar, parity)) *left = 1;
+    if (!stage_wait(&T.bar, parity, false)) *left = 1;
     parity ^= 1u;
     __syncthreads();
   }
@@ -1869,7 +1890,10 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   if constexpr (std::is_same<J32, JacobiBlocks32>::value) {
     if (S.f32 && K >= 2) {       // FP32 sweeps first; the FP64 sweeps then start from J V
       int ns = K;
-      mixed_precondition(S, w, J, jlen, jld, K, rank, nctas, sync, floor2, max_sweeps, j32, &ns);
+      if (!mixed_precondition(S, w, J, jlen, jld, K, rank, nctas, sync, floor2, max_sweeps, j32, &ns)) {
+        if (tid_all == 0) *S.status = kSvdExpired;
+        return;
+      }
       J = S.a1;
       Kj = ns;
       for (int j = worker; j < K; j += workers) {   // column norms of the new Jacobi matrix
@@ -1886,6 +1910,10 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
     }
   }
   const int sweep = jacobi(J, jlen, jld, Kj, w, rank, nctas, sync, tol2, floor2, max_sweeps, converged);
+  if (sweep == kSvdExpired) {
+    if (tid_all == 0) *S.status = kSvdExpired;
+    return;
+  }
 
   // ---- singular values (noise floor -> 0), descending, ties by column index -----------
   for (int j = worker; j < K; j += workers) {
@@ -2014,7 +2042,7 @@ struct TeamSync {
       }
       asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
       s_expired = expired;
-      if (expired) *status = kSvdTeamExpired;
+      if (expired) *status = kSvdExpired;
     }
     __syncthreads();
     if (s_expired) asm volatile("exit;\n");
@@ -2581,9 +2609,10 @@ __global__ void __launch_bounds__(kSvdThreads) jacobi_cluster_kernel(const SvdSe
 // The block-Jacobi SVD of one sector by nctas CTAs in the ordering of a cluster of cl0.
 template <class Sync>
 __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* smem, int rank, int nctas, int cl0,
-                                           Sync sync, int max_sweeps) {
+                                           Sync sync, int max_sweeps, int stall) {
   const int K = min(S.m, S.n);
   JacobiBlocks jb;
+  jb.stall = stall & kStallBlocks;
   jb.g = S.groups;
   jb.gs = S.staged;
   jb.cl0 = cl0;
@@ -2593,6 +2622,7 @@ __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* sm
   // the FP32 sweeps of a mixed-precision sector stage columns of jlen + K <= 2 jlen FP32
   // complex values in the same area
   JacobiBlocks32 j32;
+  j32.stall = jb.stall;
   j32.g = jb.g;
   j32.gs = jb.gs;
   j32.cl0 = cl0;
@@ -2603,11 +2633,11 @@ __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* sm
 }
 
 __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(const SvdSector* __restrict__ secs,
-                                                                                int cluster, int max_sweeps) {
+                                                                                int cluster, int max_sweeps, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SvdSector S = secs[blockIdx.x / cluster];
   if (S.F && S.rstate[1] == 0 && S.rstate[2] > 0) return;   // settled by the refinement
-  svd_blocks(S, smem_raw, (int)cluster_rank(), cluster, cluster, ClusterSync{}, max_sweeps);
+  svd_blocks(S, smem_raw, (int)cluster_rank(), cluster, cluster, ClusterSync{}, max_sweeps, stall);
 }
 
 // The same for batches with few large sectors: one cooperative launch, in which a sector has a team
@@ -2617,7 +2647,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(
 // sector kept 8 SMs busy for 1.23 s takes 165 ms (a team of 104), three updates at chi = 1024 297 -> 125 ms;
 // there the FP64 pipes of the whole chip are the bound.
 __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const SvdSector* __restrict__ secs, int count,
-                                                                       int max_sweeps) {
+                                                                       int max_sweeps, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int k = 0;
   while (k + 1 < count && (int)blockIdx.x >= secs[k + 1].team_first) ++k;
@@ -2625,7 +2655,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const Svd
   __shared__ unsigned s_target;
   if (threadIdx.x == 0) s_target = 0;
   svd_blocks(S, smem_raw, (int)blockIdx.x - S.team_first, S.team_size, S.team_cl0,
-             TeamSync{S.teambar, S.status, (unsigned)S.team_size, &s_target}, max_sweeps);
+             TeamSync{S.teambar, S.status, (unsigned)S.team_size, &s_target}, max_sweeps, stall);
 }
 
 __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSector* __restrict__ secs, int cluster,
@@ -2753,7 +2783,7 @@ cudaError_t launch_teams(const SvdSector* d, const SvdGroup& g, int max_sweeps, 
   at.val.cooperative = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, jacobi_team_kernel, d, g.count, max_sweeps);
+  e = cudaLaunchKernelEx(&cfg, jacobi_team_kernel, d, g.count, max_sweeps, svd_stall());
   return e == cudaSuccess ? cudaEventRecord(last[dev], st) : e;
 }
 
@@ -2789,7 +2819,7 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   cfg.numAttrs = 1;
   if (g.kind == kSvdTeam) return launch_teams(d, g, max_sweeps, st);
   if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps);
-  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, cl, max_sweeps);
+  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, cl, max_sweeps, svd_stall());
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
 }
 
@@ -3189,7 +3219,9 @@ namespace {
 std::atomic<int> g_mixed_min_k{192};
 std::atomic<int> g_mixed_sweeps{8};
 std::atomic<int> g_cluster_min_k{1 << 30};
+std::atomic<int> g_svd_stall{0};
 }
+int svd_stall() { return g_svd_stall.load(); }
 int svd_mixed_min_k() { return g_mixed_min_k.load(); }
 int svd_cluster_min_k() { return g_cluster_min_k.load(); }
 int svd_mixed_sweeps() { return g_mixed_sweeps.load(); }
@@ -3199,6 +3231,12 @@ int svd_mixed_sweeps() { return g_mixed_sweeps.load(); }
 extern "C" int mps_svd_mixed_min_k(int min_k) {
   if (min_k < 0) return MPS_EINVAL;
   mps::g_mixed_min_k.store(min_k);
+  return MPS_OK;
+}
+
+extern "C" int mps_svd_inject_stall(int what) {
+  if (what & ~mps::kStallBlocks) return MPS_EINVAL;
+  mps::g_svd_stall.store(what);
   return MPS_OK;
 }
 

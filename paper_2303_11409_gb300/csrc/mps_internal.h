@@ -277,6 +277,7 @@ struct SvdScratchLayout {
 bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int cluster_min_k = -1,
                 const char* exact = nullptr, bool team = false);
 int svd_cluster_min_k();
+int svd_stall();      // what mps_svd_inject_stall set
 // Cluster sectors with min(m, n) >= this run FP32 Jacobi sweeps first and finish in FP64
 // (0: every sector FP64 only); mps_svd_mixed_min_k sets it.
 int svd_mixed_min_k();

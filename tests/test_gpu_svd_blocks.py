@@ -123,3 +123,68 @@ def test_small_sectors_on_one_cta_and_on_block_clusters(gpu_lib, min_k):
     for A, w, (s, y, sweeps, path) in zip(mats, scales, out):
         assert path == m.MPS_SVD_SWEEPS and sweeps > 0
         _check(w[:, None] * A, s, y)
+
+
+def test_expired_staging_waits_end_the_call_with_a_status(gpu_lib):
+    """FP64 sweeps, FP32 sweeps ahead of them, and a sector of one CTA, which stages nothing."""
+    m = gpu_lib
+    mats, scales = _graded([(112, 112), (300, 310), (48, 48)], 4.0, 41)
+    m.svd_inject_stall(1)
+    try:
+        out = m.svd_sectors_path(mats, scales, keep_phases=True)
+    finally:
+        m.svd_inject_stall(0)
+    assert [r[2] for r in out[:2]] == [-2, -2] and [r[3] for r in out[:2]] == [0, 0]
+    assert out[2][2] > 0 and out[2][3] == m.MPS_SVD_SWEEPS
+    for A, w, (s, y, sweeps, path) in zip(mats, scales, m.svd_sectors_path(mats, scales, keep_phases=True)):
+        assert sweeps > 0
+        _check(w[:, None] * A, s, y)
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_expired_staging_waits_of_an_update_leave_the_state(gpu_lib, graphs):
+    """With graphs off the large sectors are on teams of CTAs, with graphs on clusters."""
+    import torch
+    from oracle import gates
+    from tests.helpers import load_state, random_state
+    m = gpu_lib
+    L, chi, s = 10, 300, 4
+    stream = torch.cuda.Stream()
+    g = m.MPS(5, [1] * L, chi, precision=m.MPS_BF16X3, stream=stream.cuda_stream)
+    load_state(g, random_state(L, 5, L, chi, seed=1))
+    g.set_graphs(graphs)
+    G = gates.bh_gate(L, s, 5, 1.0, 2.0, 0.3)
+    before = [g.bond(s + 1), g.site(s), g.site(s + 1)]
+    m.svd_inject_stall(1)
+    try:
+        with pytest.raises(m.MPSError) as e:
+            g.apply_gate2(s, G, chi, 1e-10)
+        assert e.value.code == m.MPS_ETIMEOUT
+    finally:
+        m.svd_inject_stall(0)
+    for a, b in zip(before, [g.bond(s + 1), g.site(s), g.site(s + 1)]):
+        assert a.keys() == b.keys() and all(np.array_equal(a[k], b[k]) for k in a)
+    g.apply_gate2(s, G, chi, 1e-10)
+    assert abs(sum(float(np.sum(v ** 2)) for v in g.bond(s + 1).values()) - 1.0) < 1e-12
+    g.close()
+
+
+def test_expired_staging_waits_of_dmrg(gpu_lib):
+    from tests.helpers import load_state, random_state
+    m = gpu_lib
+    L, chi = 10, 300
+    terms = m.models.chain_bond_terms("bh", L, 5, J=1.0, U=2.0)
+    g = m.MPS(5, [1] * L, chi)
+    load_state(g, random_state(L, 5, L, chi, seed=2))
+    m.svd_mixed_min_k(0)
+    m.svd_inject_stall(1)
+    try:
+        with pytest.raises(m.MPSError) as e:
+            g.dmrg(terms, 1, chi, 1e-12)
+        assert e.value.code == m.MPS_ETIMEOUT
+    finally:
+        m.svd_inject_stall(0)
+        m.svd_mixed_min_k(192)
+    g.close()
+    with pytest.raises(m.MPSError):
+        m.svd_inject_stall(64)
