@@ -410,7 +410,8 @@ MPS_API int64_t mps_launch_count(void);
  *
  * mps_svd_inject_stall - the same for the waits for staged columns in the sector SVD (any handle, and
  * mps_svd_sectors), by bits: 1, the block-Jacobi sweeps, whose sectors then end with status -2 and
- * whose calls report MPS_ETIMEOUT; 0: off.  The barriers then expect 16 bytes more than are copied, and
+ * whose calls report MPS_ETIMEOUT; 2, the FP32 sweeps of refined sectors on clusters, which then
+ * take the FP64 sweeps; 0: off.  The barriers then expect 16 bytes more than are copied, and
  * the wait runs out after about 50 ms instead of 2 s.  MPS_EINVAL for other bits.  The paper has no counterpart.
  */
 MPS_API int mps_set_sweep_limit(mps_t h, int max_sweeps);

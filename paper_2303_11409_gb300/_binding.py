@@ -692,7 +692,8 @@ def autotune_freeze(frozen: bool = True) -> None:
 
 
 def svd_inject_stall(what: int) -> None:
-    """Bits of the sector SVD's staging waits that are made to run out (1: the block sweeps; 0: none)."""
+    """Bits of the sector SVD's staging waits that are made to run out (1: the block sweeps, 2: the FP32
+    sweeps of refined sectors; 0: none)."""
     rc = lib.mps_svd_inject_stall(int(what))
     if rc != MPS_OK:
         raise MPSError(rc, "mps_svd_inject_stall")

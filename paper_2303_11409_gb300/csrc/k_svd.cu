@@ -86,7 +86,7 @@ constexpr int kSmallK = 24;
 // rows a thread loads ahead of their use in the QR's column loops (an L2 load takes some 800 cycles,
 // a row's dependent FMAs 128)
 constexpr int kAhead = 8;
-constexpr int kStallBlocks = 1;         // bits of mps_svd_inject_stall: the block sweeps
+constexpr int kStallBlocks = 1, kStallFronts = 2;      // bits of mps_svd_inject_stall
 constexpr int kMaxStaged = 16;          // block pairs staged at once by one block-Jacobi CTA
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1227,6 +1227,7 @@ struct FrontBlocks {
   float* smn;
   int bsmax, g, gs, cl;
   int* left;      // set when a bounded wait expires: the sector then goes to the FP64 sweeps
+  bool stall;     // expect bytes that no copy brings
 
   struct Tables {      // one per CTA
     int held[2 * kMaxStaged];      // the block in each slot (-1: none)
@@ -1235,6 +1236,7 @@ struct FrontBlocks {
     int fresh[2 * kMaxStaged];     // the slot was loaded for this stage
     int swap[kMaxStaged];          // pair j's shorter block is the second
     int most;                      // columns of the stage's longest block
+    int dead;                      // a wait of this CTA expired: it holds no columns any more
     uint64_t bar;
   };
 
@@ -1245,6 +1247,10 @@ struct FrontBlocks {
     const int tid = threadIdx.x, lane = tid & 31, nb = 2 * cl * g, slots = 2 * gs;
     fence_stage();
     __syncthreads();
+    if (T.dead) {
+      barrier();
+      return;
+    }
     int to = -1, want = -1, col = 0, len = 0;
     if (tid < 32) {
       const int held = lane < slots ? T.held[lane] : -1, j = lane >> 1;
@@ -1300,7 +1306,7 @@ struct FrontBlocks {
 #pragma unroll
       for (int o = 16; o; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
       fence_to_async();
-      if (lane == 0) stage_expect(&T.bar, (uint32_t)bytes);
+      if (lane == 0) stage_expect(&T.bar, (uint32_t)bytes + (stall ? 16u : 0u));
       __syncwarp();
       if (load)
         for (int c = 0; c < len; ++c)
@@ -1310,9 +1316,19 @@ struct FrontBlocks {
       const int s = e / bsmax, c = e % bsmax;
       if (T.held[s] >= 0 && T.fresh[s] && c < T.len[s]) smn[e] = __ldcg(nrm + T.col[s] + c);
     }
-    if (!stage_wait(&T.bar, parity, false)) *left = 1;
+    if (__syncthreads_or(!stage_wait(&T.bar, parity, stall))) {
+      if (tid < slots) {
+        T.at[tid] = tid;
+        T.len[tid] = 0;
+      }
+      if (tid == 0) {
+        *left = T.dead = 1;
+        T.most = 0;
+      }
+      __syncthreads();
+      return;
+    }
     parity ^= 1u;
-    __syncthreads();
   }
 
   template <int G, int E, class Sync>
@@ -1321,7 +1337,10 @@ struct FrontBlocks {
     const int tid = threadIdx.x, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int ring = 2 * cl * g - 1;
     uint32_t parity = 0;
-    if (tid == 0) stage_bar_init(&T.bar);
+    if (tid == 0) {
+      stage_bar_init(&T.bar);
+      T.dead = 0;
+    }
     if (tid < 2 * gs) T.held[tid] = -1;
     __syncthreads();
     stage(T, F, ld, K, nrm, rank, 0, 0, parity, [] { __syncthreads(); });
@@ -1410,14 +1429,16 @@ struct FrontBlocks {
           }
         }
       if (__syncthreads_or(far) && tid == 0) __stcg(flags + sweep, 1);
+      if (tid == 0 && T.dead) __stcg(flags + max_sweeps, 1);
       bool done = false;
       stage(T, F, ld, K, nrm, rank, 0, 0, parity, [&] {
         sync();
-        done = __ldcg(flags + sweep) == 0 || sweep + 1 >= max_sweeps;
+        done = __ldcg(flags + sweep) == 0 || sweep + 1 >= max_sweeps || __ldcg(flags + max_sweeps) != 0;
       });
       if (done) break;
     }
     stage(T, F, ld, K, nrm, rank, -1, 0, parity, sync);
+    if (T.dead) stage_wait(&T.bar, parity, stall);
   }
 
   template <class Sync>
@@ -2659,7 +2680,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const Svd
 }
 
 __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSector* __restrict__ secs, int cluster,
-                                                                     int max_sweeps) {
+                                                                     int max_sweeps, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int rank = (int)cluster_rank();
   const SvdSector S = secs[blockIdx.x / cluster];
@@ -2670,6 +2691,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) svd_front_kernel(const SvdSe
   j32.gs = S.front_staged;
   j32.cl = cluster;
   j32.left = S.rstate + 1;
+  j32.stall = stall & kStallFronts;
   j32.bsmax = (K + 2 * cluster * j32.g - 1) / (2 * cluster * j32.g);
   j32.sm = reinterpret_cast<float2*>(smem_raw);
   j32.smn = reinterpret_cast<float*>(smem_raw + 8LL * 2 * j32.gs * j32.bsmax * fld);
@@ -2818,7 +2840,7 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   if (g.kind == kSvdTeam) return launch_teams(d, g, max_sweeps, st);
-  if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps);
+  if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps, svd_stall());
   if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, cl, max_sweeps, svd_stall());
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
 }
@@ -3235,7 +3257,7 @@ extern "C" int mps_svd_mixed_min_k(int min_k) {
 }
 
 extern "C" int mps_svd_inject_stall(int what) {
-  if (what & ~mps::kStallBlocks) return MPS_EINVAL;
+  if (what & ~(mps::kStallBlocks | mps::kStallFronts)) return MPS_EINVAL;
   mps::g_svd_stall.store(what);
   return MPS_OK;
 }

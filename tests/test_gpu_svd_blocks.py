@@ -188,3 +188,26 @@ def test_expired_staging_waits_of_dmrg(gpu_lib):
     g.close()
     with pytest.raises(m.MPSError):
         m.svd_inject_stall(64)
+
+
+def test_expired_waits_of_the_fp32_sweeps_leave_the_sector_to_the_fp64_sweeps(gpu_lib):
+    """Fronts on clusters, with blocks that stay in shared memory and that do not; a one-CTA front stages nothing."""
+    import time
+    m = gpu_lib
+    mats, scales = _graded([(130, 238), (240, 241), (257, 384), (390, 430), (112, 112)], 4.0, 43)
+    clean = m.svd_sectors_path(mats, scales)
+    assert all(r[3] == m.MPS_SVD_REFINED for r in clean)
+    m.svd_inject_stall(2)
+    try:
+        t0 = time.perf_counter()
+        out = m.svd_sectors_path(mats, scales)
+        took = time.perf_counter() - t0
+    finally:
+        m.svd_inject_stall(0)
+    assert [r[3] for r in out] == [m.MPS_SVD_SWEEPS] * 4 + [m.MPS_SVD_REFINED]
+    assert took < 2.0      # one wait of 50 ms a CTA and another for its copies, not one a round
+    for A, w, (s, y, sweeps, path) in zip(mats, scales, out):
+        assert sweeps > 0
+        _check(w[:, None] * A, s, y)
+    for (s, y, _, _), (s1, y1, _, _) in zip(clean, m.svd_sectors_path(mats, scales)):
+        assert np.array_equal(s, s1) and np.array_equal(y, y1)
