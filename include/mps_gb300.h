@@ -715,6 +715,14 @@ MPS_API int mps_svd_sectors(int n_sectors, const int* m, const int* n,
 #define MPS_SVD_FP32_START 4     /* FP32 sweeps ahead of the FP64 ones */
 #define MPS_SVD_TEAM 8           /* a team of CTAs in a cooperative launch */
 #define MPS_SVD_ROUND_ROBIN 16   /* the round-robin cluster kernel */
+/*
+ * mps_svd_sector_plan - the route of one m x n sector with the present settings (host code, no GPU
+ * needed; any output may be NULL): path, the MPS_SVD_* bits it ends with unless its spectrum leaves the refinement
+ * unsettled; ctas, the CTAs that share it; block_pairs and staged, the column-block pairs per CTA and round of its
+ * sweeps, and how many of them a CTA holds in shared memory at once (0 where one CTA holds everything).
+ * Teams depend on the whole batch and are not shown.  MPS_EINVAL for m or n below 1.
+ */
+MPS_API int mps_svd_sector_plan(int m, int n, int keep_phases, int* path, int* ctas, int* block_pairs, int* staged);
 MPS_API int64_t mps_svd_path_work_bytes(int n_sectors, const int* m, const int* n, int keep_phases);
 MPS_API int mps_svd_sectors_path(int n_sectors, const int* m, const int* n,
                     const double* d_mats, const int64_t* mat_off,

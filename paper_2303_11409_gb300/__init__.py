@@ -9,7 +9,7 @@ from ._binding import (EXPORTED, LIB_PATH, MPS, MPS_BF16X3, MPS_EINVAL, MPS_ECHA
                        JacobiNotConverged, KERNEL_KINDS, MPSError, apply_gate2_batch, gate_length, launch_count, lib,
                        plan_sectors, plan_sectors_rule, gate_layout,
                        svd_sectors, svd_work_bytes)
-from ._binding import MPS_NOALLOC_SCRATCH_BYTES, svd_sectors_noalloc, svd_sectors_path  # noqa: F401
+from ._binding import MPS_NOALLOC_SCRATCH_BYTES, svd_sectors_noalloc, svd_sectors_path, svd_sector_plan  # noqa: F401
 from ._binding import (MPS_SVD_REFINED, MPS_SVD_SWEEPS, MPS_SVD_FP32_START, MPS_SVD_TEAM,  # noqa: F401
                        MPS_SVD_ROUND_ROBIN)
 from ._binding import Executor, footprint_bytes, fp64_peak_probe, zgemm_tc  # noqa: F401

@@ -109,6 +109,7 @@ _SIGS = {
                                                _vp, _i64p, _vp, _vp]),
     "mps_svd_sectors": (ctypes.c_int, [ctypes.c_int, _intp, _intp, _vp, _i64p, _vp, _i64p, _vp, _i64p, _vp,
                                        _i64p, _vp, _vp, ctypes.c_int64, _vp]),
+    "mps_svd_sector_plan": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, _intp, _intp, _intp, _intp]),
     "mps_svd_path_work_bytes": (ctypes.c_int64, [ctypes.c_int, _intp, _intp, ctypes.c_int]),
     "mps_svd_sectors_path": (ctypes.c_int, [ctypes.c_int, _intp, _intp, _vp, _i64p, _vp, _i64p, _vp, _i64p, _vp,
                                             _i64p, _vp, ctypes.c_int, _vp, _vp, ctypes.c_int64, _vp]),
@@ -889,6 +890,15 @@ def svd_work_bytes(ms, ns) -> int:
     m = np.ascontiguousarray(np.asarray(ms, dtype=np.intc))
     n = np.ascontiguousarray(np.asarray(ns, dtype=np.intc))
     return int(lib.mps_svd_work_bytes(len(m), _ptr(m, _intp), _ptr(n, _intp)))
+
+
+def svd_sector_plan(m: int, n: int, keep_phases: bool = False) -> dict:
+    """The route of an m x n sector (mps_svd_sector_plan; needs no GPU)."""
+    v = [ctypes.c_int() for _ in range(4)]
+    rc = lib.mps_svd_sector_plan(int(m), int(n), int(keep_phases), *[ctypes.byref(x) for x in v])
+    if rc != MPS_OK:
+        raise MPSError(rc, "mps_svd_sector_plan")
+    return dict(zip(("path", "ctas", "block_pairs", "staged"), (x.value for x in v)))
 
 
 def svd_sectors(mats, rowscales=None, stream=None):

@@ -2909,6 +2909,84 @@ cudaError_t form_teams(std::vector<SvdSector>& secs, std::vector<std::pair<int, 
   return cudaSuccess;
 }
 
+// The kernel and the cluster size of one sector, its block pairs (groups, staged, front_staged) and the dynamic
+// shared memory of the FP64 sweeps and of the front.  Host arithmetic alone; clears F where the sector is not refined.
+struct SvdShape {
+  int kind, cl;
+  int64_t smem, small;
+};
+SvdShape sector_shape(SvdSector& S, const SvdTune& tune, int big_cluster) {
+  SvdShape r = {};
+  if (S.mode == kSvdSmem) {
+    r.kind = S.small ? kSvdSmall : kSvdSmem;
+    r.cl = 1;
+    r.smem = svd_smem_need(S.m, S.n);
+    if (S.small) r.small = std::max(r.smem, small_layout(S.m, S.n, true).total);
+    return r;
+  }
+  const int K = std::min(S.m, S.n), bw = std::max(2, tune.bw);
+  const int cn = S.wide ? K : S.n;   // Jacobi column length
+  if (S.F && small_layout(S.m, S.n, false).total <= kFrontSmemMax) {
+    // a one-CTA front; should the FP64 sweeps be needed, a cluster of 2 stages all its block pairs
+    const int g = std::max(1, (K + bw * 2) / (2 * bw * 2));
+    if (g <= kMaxStaged && block_smem_need(S.m, cn, 2, g, g) <= kBlockSmemMax) {
+      S.groups = S.staged = g;
+      return SvdShape{kSvdRefine, 1, block_smem_need(S.m, cn, 2, g, g), small_layout(S.m, S.n, false).total};
+    }
+  }
+  if (16LL * std::max(S.m, S.n) > kBlockSmemMax) S.F = nullptr;   // no room for a reflector
+  // blocks of about tune.bw columns (6 by default); the smallest cluster (tune.cl_min,
+  // then doubling up to 8 CTAs) whose CTAs can stage all of their block pairs of a round
+  // at once, so that a step offers the warp groups about K / (2 cl) * bw / 2 disjoint
+  // pairs; failing that, 8 CTAs staging as many pairs as fit, with more pairs per CTA
+  // when a single one does not fit.  A front's blocks serve its FP32 sweeps and the FP64 sweeps that may have to
+  // follow, whose columns are longer in bytes unless n is well below K: one pair of either has to fit.
+  auto need = [&](int cl, int g, int gs) {
+    return S.F ? front_smem_need(S.m, cn, cl, g, gs) : block_smem_need(S.m, cn, cl, g, gs);
+  };
+  const int64_t room = S.F ? kPairSmemMax : kBlockSmemMax;
+  auto fits = [&](int cl, int g, int gs) {
+    return need(cl, g, gs) <= room && block_smem_need(S.m, cn, cl, g, 1) <= kBlockSmemMax;
+  };
+  auto blocks = [&](int cl) {      // of a front: at most bw columns each, its 6 warps' slots a pair of them
+    return S.F ? (K + 2 * bw * cl - 1) / (2 * bw * cl) : std::max(1, (K + bw * cl) / (2 * bw * cl));
+  };
+  int pick_cl = 0, pick_g = 0, pick_gs = 0;
+  for (int cl = std::max(2, std::min(tune.cl_min, kBigCluster)); cl <= kBigCluster && !pick_cl; cl *= 2) {
+    const int g = blocks(cl);
+    if (g <= kMaxStaged && fits(cl, g, g)) {
+      pick_cl = cl; pick_g = g; pick_gs = g;
+    }
+  }
+  auto in_chunks = [&](int cl) {
+    int g = blocks(cl);
+    while (g < 64 && !fits(cl, g, 1)) ++g;
+    int gs = 1;
+    while (gs < std::min(g, kMaxStaged) && fits(cl, g, gs + 1)) ++gs;
+    if (fits(cl, g, gs)) {
+      pick_cl = cl; pick_g = g; pick_gs = gs;
+    }
+  };
+  if (!pick_cl) in_chunks(kBigCluster);
+  if (K >= tune.c16_min_k && big_cluster >= 16) in_chunks(16);
+  if (K >= tune.rr_min_k || !pick_cl) {
+    S.F = nullptr;        // the round-robin kernel runs in FP64 alone
+    return SvdShape{kSvdCluster, big_cluster, 0, 0};
+  }
+  r.kind = S.F ? kSvdRefine : kSvdClusterBlock;
+  r.cl = pick_cl;
+  S.groups = pick_g;
+  if (S.F) {
+    S.front_staged = pick_gs;
+    r.small = std::max<int64_t>(need(pick_cl, pick_g, pick_gs),
+                                16LL * std::max(S.m, S.n));      // the QR's copy of a reflector
+    while (block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs) > kBlockSmemMax) --pick_gs;      // 1 fits
+  }
+  S.staged = pick_gs;
+  r.smem = block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs);
+  return r;
+}
+
 cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& groups, const SvdTune& tune, bool team) {
   int big_cluster = 0;
   cudaError_t e = set_attrs(&big_cluster);
@@ -2917,85 +2995,10 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
   std::vector<std::pair<int, int>> key(secs.size());
   std::vector<int64_t> smem(secs.size(), 0), small(secs.size(), 0);
   for (size_t k = 0; k < secs.size(); ++k) {
-    const SvdSector S = secs[k];
-    if (S.mode == kSvdSmem) {
-      key[k] = {S.small ? kSvdSmall : kSvdSmem, 1};
-      smem[k] = svd_smem_need(S.m, S.n);
-      if (S.small) small[k] = std::max(smem[k], small_layout(S.m, S.n, true).total);
-      continue;
-    }
-    if (S.F && small_layout(S.m, S.n, false).total <= kFrontSmemMax) {
-      // a one-CTA front; should the FP64 sweeps be needed, a cluster of 2 stages all its block pairs
-      const int cn = S.wide ? std::min(S.m, S.n) : S.n, bw = std::max(2, tune.bw);
-      const int g = std::max(1, (std::min(S.m, S.n) + bw * 2) / (2 * bw * 2));
-      if (g <= kMaxStaged && block_smem_need(S.m, cn, 2, g, g) <= kBlockSmemMax) {
-        key[k] = {kSvdRefine, 1};
-        smem[k] = block_smem_need(S.m, cn, 2, g, g);
-        small[k] = small_layout(S.m, S.n, false).total;
-        secs[k].groups = secs[k].staged = g;
-        continue;
-      }
-    }
-    if (16LL * std::max(S.m, S.n) > kBlockSmemMax) secs[k].F = nullptr;   // no room for a reflector
-    // blocks of about tune.bw columns (6 by default); the smallest cluster (tune.cl_min,
-    // then doubling up to 8 CTAs) whose CTAs can stage all of their block pairs of a round
-    // at once, so that a step offers the warp groups about K / (2 cl) * bw / 2 disjoint
-    // pairs; failing that, 8 CTAs staging as many pairs as fit, with more pairs per CTA
-    // when a single one does not fit
-    const int bw = std::max(2, tune.bw);
-    const int cn = S.wide ? std::min(S.m, S.n) : S.n;   // Jacobi column length
-    auto need = [&](int cl, int g, int gs) {
-      return S.F ? front_smem_need(S.m, cn, cl, g, gs) : block_smem_need(S.m, cn, cl, g, gs);
-    };
-    const int64_t room = S.F ? kPairSmemMax : kBlockSmemMax;
-    auto blocks = [&](int cl) {      // of a front: at most bw columns each, its 6 warps' slots a pair of them
-      const int K = std::min(S.m, S.n);
-      return S.F ? (K + 2 * bw * cl - 1) / (2 * bw * cl) : std::max(1, (K + bw * cl) / (2 * bw * cl));
-    };
-    int pick_cl = 0, pick_g = 0, pick_gs = 0;
-    for (int cl = std::max(2, std::min(tune.cl_min, kBigCluster)); cl <= kBigCluster && !pick_cl; cl *= 2) {
-      const int g = blocks(cl);
-      if (g <= kMaxStaged && need(cl, g, g) <= room) {
-        pick_cl = cl; pick_g = g; pick_gs = g;
-      }
-    }
-    if (!pick_cl) {
-      const int cl = kBigCluster;
-      int g = blocks(cl);
-      while (g < 64 && need(cl, g, 1) > room) ++g;
-      int gs = 1;
-      while (gs < std::min(g, kMaxStaged) && need(cl, g, gs + 1) <= room) ++gs;
-      if (need(cl, g, gs) <= room) {
-        pick_cl = cl; pick_g = g; pick_gs = gs;
-      }
-    }
-    if (std::min(S.m, S.n) >= tune.c16_min_k && big_cluster >= 16) {   // a 16-CTA cluster
-      const int cl = 16;
-      int g = blocks(cl);
-      while (g < 64 && need(cl, g, 1) > room) ++g;
-      int gs = 1;
-      while (gs < std::min(g, kMaxStaged) && need(cl, g, gs + 1) <= room) ++gs;
-      if (need(cl, g, gs) <= room) {
-        pick_cl = cl; pick_g = g; pick_gs = gs;
-      }
-    }
-    if (std::min(S.m, S.n) >= tune.rr_min_k) pick_cl = 0;
-    if (pick_cl && S.F) {      // the FP64 sweeps, should they be needed, stage FP64 columns of the same blocks
-      secs[k].front_staged = pick_gs;
-      small[k] = std::max<int64_t>(need(pick_cl, pick_g, pick_gs),
-                                   16LL * std::max(S.m, S.n));      // the QR's copy of a reflector
-      while (pick_gs > 0 && block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs) > kBlockSmemMax) --pick_gs;
-      if (pick_gs == 0) pick_cl = 0;
-    }
-    if (pick_cl) {
-      key[k] = {secs[k].F ? kSvdRefine : kSvdClusterBlock, pick_cl};
-      smem[k] = block_smem_need(S.m, cn, pick_cl, pick_g, pick_gs);
-      secs[k].groups = pick_g;
-      secs[k].staged = pick_gs;
-    } else {
-      key[k] = {kSvdCluster, big_cluster};
-      secs[k].F = nullptr;        // the round-robin kernel runs in FP64 alone
-    }
+    const SvdShape r = sector_shape(secs[k], tune, big_cluster);
+    key[k] = {r.kind, r.cl};
+    smem[k] = r.smem;
+    small[k] = r.small;
   }
   if (team && (e = form_teams(secs, key, smem)) != cudaSuccess) return e;
   // group by (kind, cluster size); the most expensive sectors first inside a group
@@ -3286,6 +3289,30 @@ extern "C" int64_t mps_svd_path_work_bytes(int n_sectors, const int* m, const in
 
 extern "C" int64_t mps_svd_work_bytes(int n_sectors, const int* m, const int* n) {
   return mps_svd_path_work_bytes(n_sectors, m, n, 0);
+}
+
+extern "C" int mps_svd_sector_plan(int m, int n, int keep_phases, int* path, int* ctas, int* block_pairs,
+                                   int* staged) {
+  SvdScratchLayout L;
+  const char exact = keep_phases != 0;
+  if (m < 1 || n < 1 || !svd_layout(1, &m, &n, L, -1, &exact)) return MPS_EINVAL;
+  alignas(256) static char none[256];      // addresses are formed from it, nothing is read or written
+  SvdSector S = {};
+  S.m = m;
+  S.n = n;
+  svd_fill_scratch(S, L, 0, none);
+  SvdTune tune;
+  svd_forced_tune(tune);
+  const SvdShape r = sector_shape(S, tune, kMaxCluster);
+  const bool start = r.kind == kSvdClusterBlock && S.f32 && std::min(m, n) >= 2;
+  if (path)
+    *path = r.kind == kSvdRefine || r.kind == kSvdSmall
+                ? MPS_SVD_REFINED
+                : MPS_SVD_SWEEPS | (start ? MPS_SVD_FP32_START : 0) | (r.kind == kSvdCluster ? MPS_SVD_ROUND_ROBIN : 0);
+  if (ctas) *ctas = r.cl;
+  if (block_pairs) *block_pairs = S.groups;
+  if (staged) *staged = S.front_staged ? S.front_staged : S.staged;
+  return MPS_OK;
 }
 
 namespace {

@@ -56,3 +56,19 @@ def test_fronts_do_not_depend_on_their_batch(gpu_lib):
     for A, (s, y, _) in zip(mats, every):
         s1, y1, _ = m.svd_sectors([A])[0]
         assert np.array_equal(s, s1) and np.array_equal(y, y1)
+
+
+def test_fronts_whose_block_pair_just_fits(gpu_lib):
+    """Sizes at which a pair of FP32 blocks fits shared memory and the same pair of FP64 blocks would not."""
+    m = gpu_lib
+    rng = np.random.default_rng(17)
+    mats = [W.random_complex(s, rng) for s in [(590, 590), (598, 660), (710, 710)]]
+    scales = [np.sort(10.0 ** (-6.0 * rng.random(A.shape[0])))[::-1].copy() for A in mats]
+    for A, w, (s, y, steps, path) in zip(mats, scales, m.svd_sectors_path(mats, scales)):
+        M = w[:, None] * A
+        N = max(M.shape)
+        assert path == m.MPS_SVD_REFINED and steps > 0
+        S = scipy.linalg.svd(M, compute_uv=False, lapack_driver="gesvd")
+        assert np.max(np.abs(s - S)) <= 4 * N * EPS * S[0], M.shape
+        Y = y[:, s > 64 * N * EPS * S[0]]
+        assert np.max(np.abs(Y.conj().T @ Y - np.eye(Y.shape[1]))) <= 4 * EPS * M.shape[1] + 8 * EPS * N, M.shape

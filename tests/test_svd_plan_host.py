@@ -1,0 +1,32 @@
+"""The route of a sector by its size (host arithmetic, no GPU)."""
+import os
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def m():
+    import __graft_entry__ as g
+    b = g._build_module()
+    if not os.path.exists(b.LIB):
+        b.build()
+    import paper_2303_11409_gb300
+    return paper_2303_11409_gb300
+
+
+SIZES = {"square": lambda k: (k, k), "flat": lambda k: (int(0.85 * k), k), "wide": lambda k: (k, 2 * k),
+         "tall": lambda k: (2 * k, k)}
+
+
+@pytest.mark.parametrize("shape", SIZES)
+def test_no_size_falls_out_of_the_block_sweeps(m, shape):
+    """One block pair has to fit the shared memory of the FP32 sweeps and of the FP64 sweeps behind them: from 586
+    columns there are sizes at which a pair that just fits the first does not fit the second."""
+    for k in range(26, 1500):
+        rows, cols = SIZES[shape](k)
+        plan = m.svd_sector_plan(rows, cols)
+        if min(rows, cols) > 24:
+            assert plan["path"] == m.MPS_SVD_REFINED, (rows, cols)
+        kept = m.svd_sector_plan(rows, cols, keep_phases=True)
+        start = m.MPS_SVD_FP32_START if min(rows, cols) >= 192 else 0
+        assert kept["path"] == m.MPS_SVD_SWEEPS | start, (rows, cols)
