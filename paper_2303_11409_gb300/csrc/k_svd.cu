@@ -2934,7 +2934,6 @@ SvdShape sector_shape(SvdSector& S, const SvdTune& tune, int big_cluster) {
       return SvdShape{kSvdRefine, 1, block_smem_need(S.m, cn, 2, g, g), small_layout(S.m, S.n, false).total};
     }
   }
-  if (16LL * std::max(S.m, S.n) > kBlockSmemMax) S.F = nullptr;   // no room for a reflector
   // blocks of about tune.bw columns (6 by default); the smallest cluster (tune.cl_min,
   // then doubling up to 8 CTAs) whose CTAs can stage all of their block pairs of a round
   // at once, so that a step offers the warp groups about K / (2 cl) * bw / 2 disjoint
@@ -3140,7 +3139,9 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     if (m[k] < 1 || n[k] < 1) return false;
     const int64_t need = svd_smem_need(m[k], n[k]);
     L.exact[k] = exact && exact[k];
-    const bool refine = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) >= own_k;
+    // a front's CTAs hold a copy of the QR's reflector; longer columns keep the FP32 start of the other sectors
+    const bool refine = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) >= own_k &&
+                        16LL * std::max(m[k], n[k]) <= kBlockSmemMax;
     if (need <= kSvdSmemMax && std::min(m[k], n[k]) < cluster_min_k && !refine) {
       L.small[k] = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) <= kSmallK &&
                    small_layout(m[k], n[k], true).total <= kSvdSmemMax;

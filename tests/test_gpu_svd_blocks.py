@@ -211,3 +211,13 @@ def test_expired_waits_of_the_fp32_sweeps_leave_the_sector_to_the_fp64_sweeps(gp
         _check(w[:, None] * A, s, y)
     for (s, y, _, _), (s1, y1, _, _) in zip(clean, m.svd_sectors_path(mats, scales)):
         assert np.array_equal(s, s1) and np.array_equal(y, y1)
+
+
+def test_columns_too_long_for_a_front(gpu_lib):
+    m = gpu_lib
+    mats, scales = _graded([(7100, 195), (7100, 40)], 3.0, 47)
+    out = m.svd_sectors_path(mats, scales)
+    assert [r[3] for r in out] == [m.MPS_SVD_SWEEPS | m.MPS_SVD_FP32_START, m.MPS_SVD_SWEEPS]
+    for A, w, (s, y, sweeps, path) in zip(mats, scales, out):
+        assert sweeps > 0
+        _check(w[:, None] * A, s, y)

@@ -30,3 +30,13 @@ def test_no_size_falls_out_of_the_block_sweeps(m, shape):
         kept = m.svd_sector_plan(rows, cols, keep_phases=True)
         start = m.MPS_SVD_FP32_START if min(rows, cols) >= 192 else 0
         assert kept["path"] == m.MPS_SVD_SWEEPS | start, (rows, cols)
+
+
+@pytest.mark.parametrize("rows,cols", [(7041, 191), (7041, 192), (7040, 192), (9000, 640), (200, 7100), (7100, 30)])
+def test_columns_too_long_for_a_front_keep_the_fp32_start(m, rows, cols):
+    """A front copies the QR's reflector, 16 bytes a row, to shared memory (7040 rows)."""
+    path = m.svd_sector_plan(rows, cols)["path"]
+    if max(rows, cols) <= 7040:
+        assert path == m.MPS_SVD_REFINED
+    else:
+        assert path == m.MPS_SVD_SWEEPS | (m.MPS_SVD_FP32_START if min(rows, cols) >= 192 else 0)
