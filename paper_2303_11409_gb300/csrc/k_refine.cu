@@ -544,6 +544,10 @@ cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max
       return e;
     if (dev < 64) done.fetch_or(1ull << dev);
   }
+  // the sector is blockIdx.y, which ends at 65535
+  constexpr int kMaxSectors = 65535;
+  for (; count > kMaxSectors; d_secs += kMaxSectors, count -= kMaxSectors)
+    if ((e = launch_refine(d_secs, kMaxSectors, max_k, max_n, st)) != cudaSuccess) return e;
   auto cd = [](int a, int b) { return (a + b - 1) / b; };
   const dim3 cols(std::min(cd(max_k, 8), 64), count);
   const int ct = cd(max_k, kOzN), rk = cd(max_k, kOzM), rn = cd(max_n, kOzM);

@@ -96,3 +96,15 @@ def test_teams_give_the_bits_of_the_clusters(gpu_lib, L, chi):
     for a, b in zip(*out):
         assert a.keys() == b.keys()
         assert all(np.array_equal(a[k], b[k]) for k in a)
+
+
+def test_more_sectors_than_a_grid_has_rows(gpu_lib):
+    """70,000 refined sectors in one call; those on both sides of 65,535 against LAPACK."""
+    m = gpu_lib
+    rng = np.random.default_rng(70)
+    n, k = 70000, 25
+    A = rng.standard_normal((n, k, k)) + 1j * rng.standard_normal((n, k, k))
+    out = m.svd_sectors_path(list(A))
+    assert all(r[3] == m.MPS_SVD_REFINED for r in out)
+    for i in [0, 1, *range(65530, 65540), n - 1, *rng.integers(0, n, 200)]:
+        _check(A[i], *out[i][:3])
