@@ -23,9 +23,9 @@
 // are cut while a tile is staged in shared memory, so the operands stay FP64 in global memory.
 #include <algorithm>
 #include <atomic>
-#include <climits>
 
 #include "mps_internal.h"
+#include "refine_fixed.cuh"
 #include "refine_pair.cuh"
 
 namespace mps {
@@ -39,32 +39,6 @@ constexpr int kOzAhead = 4;                         // operand loads in flight a
 constexpr int kOzSmem = kOzSlices * (kOzABytes + kOzBBytes);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// x 2^(54 - e) rounded to an integer, plus 128 in every one of the 7 low bytes (balanced digits are
-// then byte - 128); |x| < 2^e.
-__device__ __forceinline__ uint64_t oz_fixed(double x, int e) {
-  const long long b = __double_as_longlong(x);
-  const int E = (int)((b >> 52) & 0x7ff);
-  const long long mant = (b & 0xfffffffffffffLL) | 0x10000000000000LL;
-  const int s = E - 1021 - e;
-  long long q;
-  if (s >= 0) q = mant << min(s, 1);
-  else q = s < -54 ? 0 : (mant + (1LL << (-s - 1))) >> (-s);
-  if (b < 0) q = -q;
-  return (uint64_t)(q + 0x0080808080808080LL);
-}
-__device__ __forceinline__ uint64_t oz_fixed(float x, int e) {
-  const int b = __float_as_int(x);
-  const int E = (b >> 23) & 0xff;
-  const long long mant = (b & 0x7fffff) | 0x800000;
-  const int s = E - 96 - e;      // x = mant 2^(E - 150)
-  long long q;
-  if (E == 0) q = 0;
-  else if (s >= 0) q = mant << min(s, 30);
-  else q = s < -25 ? 0 : (mant + (1LL << (-s - 1))) >> (-s);
-  if (b < 0) q = -q;
-  return (uint64_t)(q + 0x0080808080808080LL);
-}
 
 // The slices of one complex number into its row: word = (BF16 re, BF16 im), neg flips im.
 template <int NS, typename T2>
@@ -333,33 +307,30 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
   // scale of each column of W: the largest component of s_k W_kc, s_k the scale of X's column k.  The
   // correction E is stored in the scaled form of A's columns, s_k E_kc / s_c.
   for (int c = warp; c < kOzN; c += 8) {
-    int top = INT_MIN / 2;
-    float sq = 0.f;
+    CorrectionScale cs;
     if (c0 + c < ns) {
       const int ec = step == 0 ? 0 : S.cexp[c0 + c];
       for (int k = lane; k < kn; k += 32) {
         if (step == 0) {
           const double2 w = S.V0[(int64_t)(c0 + c) * K + k];
           const int e = max((int)((__double_as_longlong(w.x) >> 52) & 0x7ff), (int)((__double_as_longlong(w.y) >> 52) & 0x7ff));
-          if (e) top = max(top, e - 1022 + S.cexp[k]);
+          if (e) cs.top = max(cs.top, e - 1022 + S.cexp[k]);
         } else {
           const float2 w = S.E[(int64_t)(c0 + c) * K + k];
-          const int e = max((__float_as_int(w.x) >> 23) & 0xff, (__float_as_int(w.y) >> 23) & 0xff);
           const int d = ec - S.cexp[k];      // E_kc = w 2^d
-          if (e) top = max(top, e - 126 + (onV ? d + S.vexp[k] : 0));
-          const float f = exp2f((float)max(-60, min(60, d)));
-          sq = fmaf(w.x * f, w.x * f, fmaf(w.y * f, w.y * f, sq));
+          cs.add(w.x, w.y, d, onV ? d + S.vexp[k] : 0, k == c0 + c);
         }
       }
     }
     for (int o = 16; o; o >>= 1) {
-      top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-      sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      cs.top = max(cs.top, __shfl_xor_sync(0xffffffffu, cs.top, o));
+      cs.sq += __shfl_xor_sync(0xffffffffu, cs.sq, o);
+      cs.diag += __shfl_xor_sync(0xffffffffu, cs.diag, o);      // one lane holds it
     }
-    if (lane == 0) s_d[c] = -0.5f * sq;
-    // the diagonal's second-order part may be the largest entry
-    if (step > 0 && sq > 0.f) top = max(top, ilogbf(sq) + 1 + (onV ? S.vexp[c0 + c] : 0));
-    if (lane == 0) s_t[c] = max(top, -1000);
+    if (lane == 0) {
+      s_d[c] = cs.second_order();
+      s_t[c] = cs.scale(onV && c0 + c < ns ? S.vexp[c0 + c] : 0);
+    }
   }
   __syncthreads();
   char* sB = smem + kOzSlices * kOzABytes;
