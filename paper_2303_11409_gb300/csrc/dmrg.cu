@@ -289,16 +289,17 @@ __global__ void __launch_bounds__(kVecThreads) dots_reduce_kernel(const double2*
 }
 
 // ---- one Lanczos step's Gram-Schmidt in four launches -------------------------------------------
-// A CTA owns a chunk of 128 E elements of w.  gs_dots_kernel leaves the chunk's partial products with
-// every basis vector; gs_update_kernel sums all CTAs' partials itself (fixed order, so every CTA gets
-// the same coefficients), subtracts, and forms the next partials from the chunk it still holds (the
-// second pass's products, or the norm); gs_scale_kernel closes the step.  The separate kernels for
+// A CTA owns chunks of 128 E elements of w, a single one up to 620,000 elements.  gs_dots_kernel leaves
+// their partial products with every basis vector; gs_update_kernel sums all CTAs' partials itself (fixed
+// order, so every CTA gets the same coefficients), subtracts, and forms the next partials from the chunk it
+// still holds (the second pass's products, or the norm); gs_scale_kernel closes the step.  The separate kernels for
 // products, sums, subtraction, norm, scalars and scaling were ten launches, and on the vectors of
 // short chains (10-20 thousand elements) launch latency was all of their time: 230 us a step under
 // event timing at L = 10, chi <= 96, now 45.  FP64 adds are what the reductions cost (2 a clock and SM), so a warp
 // sums 8 vectors' products together: 18 adds instead of 80.
 constexpr int kGsThreads = 128;
 constexpr int kGsMaxK = 64;
+constexpr int kGsBlocks = 608;      // 4 x 152 SMs
 
 // v[0..7] of the 32 lanes summed over the lanes: lane 4 k holds the sum of v[k] (k = 0..7)
 __device__ __forceinline__ double sum8(double (&v)[8], int lane) {
@@ -317,10 +318,11 @@ __device__ __forceinline__ double sum8(double (&v)[8], int lane) {
   return s;
 }
 
-// partial[k * gridDim.x + blockIdx.x] = sum over the CTA's elements of conj(V_k) w, k < nk
+// partial[k * gridDim.x + blockIdx.x] = sum over the CTA's elements of conj(V_k) w, k < nk; this chunk's part is added
+// to what the CTA's earlier ones left unless it is the first
 template <int E>
 __device__ void gs_partials(const double2* V, int64_t ldv, int nk, const double2 (&w)[E], int64_t e0,
-                            int64_t n, double2* partial, double2 (*red)[8]) {
+                            int64_t n, bool first, double2* partial, double2 (*red)[8]) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int k0 = 0; k0 < nk; k0 += 8) {
     double sx[8], sy[8];
@@ -349,7 +351,12 @@ __device__ void gs_partials(const double2* V, int64_t ldv, int nk, const double2
         s.x += red[x][tid].x;
         s.y += red[x][tid].y;
       }
-      partial[(int64_t)(k0 + tid) * gridDim.x + blockIdx.x] = s;
+      double2* p = partial + (int64_t)(k0 + tid) * gridDim.x + blockIdx.x;
+      if (!first) {
+        s.x += p->x;
+        s.y += p->y;
+      }
+      *p = s;
     }
     __syncthreads();
   }
@@ -383,11 +390,14 @@ __global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(const double2* V, i
   __shared__ double2 red[kGsThreads / 32][8];
   next_may_launch();
   wait_for_previous();
-  const int64_t e0 = (int64_t)blockIdx.x * kGsThreads * E + threadIdx.x;
-  double2 x[E];
+  const int64_t all = (int64_t)gridDim.x * kGsThreads * E;
+  for (int64_t c0 = (int64_t)blockIdx.x * kGsThreads * E; c0 < n; c0 += all) {
+    const int64_t e0 = c0 + threadIdx.x;
+    double2 x[E];
 #pragma unroll
-  for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
-  gs_partials<E>(V, ldv, nk, x, e0, n, partial, red);
+    for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
+    gs_partials<E>(V, ldv, nk, x, e0, n, c0 < all, partial, red);
+  }
 }
 
 // w -= sum_k h_k V_k with h from pin, then the partials of the new w: its products with the basis
@@ -404,33 +414,37 @@ __global__ void __launch_bounds__(kGsThreads) gs_update_kernel(const double2* V,
   gs_sums(pin, gridDim.x, nk, h);
   if (blockIdx.x == 0)
     for (int k = threadIdx.x; k < nk; k += kGsThreads) hout[k] = h[k];
-  const int64_t e0 = (int64_t)blockIdx.x * kGsThreads * E + threadIdx.x;
-  double2 x[E];
+  const int64_t all = (int64_t)gridDim.x * kGsThreads * E;
+  double2 s = make_double2(0.0, 0.0);
+  for (int64_t c0 = (int64_t)blockIdx.x * kGsThreads * E; c0 < n; c0 += all) {
+    const int64_t e0 = c0 + threadIdx.x;
+    double2 x[E];
 #pragma unroll
-  for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
+    for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
 #pragma unroll 4
-  for (int k = 0; k < nk; ++k) {
-    const double2 c = h[k];
+    for (int k = 0; k < nk; ++k) {
+      const double2 c = h[k];
 #pragma unroll
-    for (int i = 0; i < E; ++i) {
-      const int64_t e = e0 + i * kGsThreads;
-      if (e < n) {
-        const double2 v = V[(int64_t)k * ldv + e];
-        x[i].x = fma(-c.x, v.x, fma(c.y, v.y, x[i].x));
-        x[i].y = fma(-c.x, v.y, fma(-c.y, v.x, x[i].y));
+      for (int i = 0; i < E; ++i) {
+        const int64_t e = e0 + i * kGsThreads;
+        if (e < n) {
+          const double2 v = V[(int64_t)k * ldv + e];
+          x[i].x = fma(-c.x, v.x, fma(c.y, v.y, x[i].x));
+          x[i].y = fma(-c.x, v.y, fma(-c.y, v.x, x[i].y));
+        }
       }
     }
-  }
 #pragma unroll
-  for (int i = 0; i < E; ++i)
-    if (e0 + i * kGsThreads < n) w[e0 + i * kGsThreads] = x[i];
-  if (!last) {
-    gs_partials<E>(V, ldv, nk, x, e0, n, pout, red);
-    return;
-  }
-  double2 s = make_double2(0.0, 0.0);
+    for (int i = 0; i < E; ++i)
+      if (e0 + i * kGsThreads < n) w[e0 + i * kGsThreads] = x[i];
+    if (!last) {
+      gs_partials<E>(V, ldv, nk, x, e0, n, c0 < all, pout, red);
+    } else {
 #pragma unroll
-  for (int i = 0; i < E; ++i) s.x = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, s.x));
+      for (int i = 0; i < E; ++i) s.x = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, s.x));
+    }
+  }
+  if (!last) return;
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = s;
   __syncthreads();
@@ -457,14 +471,15 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(double2* dst, cons
     alpha[j] = h[j].x + g[j].x;
     beta[j] = b;
   }
+  for (int64_t c0 = (int64_t)blockIdx.x * kGsThreads * E; c0 < n; c0 += (int64_t)gridDim.x * kGsThreads * E)
 #pragma unroll
-  for (int i = 0; i < E; ++i) {
-    const int64_t e = ((int64_t)blockIdx.x * E + i) * kGsThreads + threadIdx.x;
-    if (e < n) {
-      const double2 v = w[e];
-      dst[e] = make_double2(f * v.x, f * v.y);
+    for (int i = 0; i < E; ++i) {
+      const int64_t e = c0 + i * kGsThreads + threadIdx.x;
+      if (e < n) {
+        const double2 v = w[e];
+        dst[e] = make_double2(f * v.x, f * v.y);
+      }
     }
-  }
 }
 
 __global__ void inv_norm_kernel(const double2* __restrict__ nrm2, double* __restrict__ inv) {
@@ -1218,10 +1233,14 @@ struct Dmrg {
     b.nb = std::max(1, std::min(kDotBlocks, (int)((dim + kVecThreads - 1) / kVecThreads)));
     b.vb = vec_blocks(dim);
     // the fewest elements a thread that leave at most two CTAs an SM: FP64 issue bounds a chunk, so
-    // short vectors want every SM, and the sums of the partials grow with the number of CTAs
+    // short vectors want every SM, and the sums of the partials, which every CTA forms, grow with the number of
+    // CTAs.  Beyond 8 elements a thread the grid grows to four CTAs an SM, then each takes several chunks
+    // (without that limit the sums grow with the square of the length).  A step against 12 vectors, us, one
+    // chunk a CTA | 2, 4, 6, 8 CTAs an SM: 1 M elements 587 | 790, 532, 590, 604; 4 M 3792 | 2837, 1607, 1804, 1735;
+    // 8 M 11549 | 5575, 2992, 3593, 3042.
     b.ge = 1;
     while (b.ge < 8 && dim > (int64_t)kDotBlocks * kGsThreads * b.ge) b.ge *= 2;
-    b.gb = (int)((dim + (int64_t)kGsThreads * b.ge - 1) / ((int64_t)kGsThreads * b.ge));
+    b.gb = (int)std::min<int64_t>(kGsBlocks, (dim + (int64_t)kGsThreads * b.ge - 1) / ((int64_t)kGsThreads * b.ge));
     const int64_t npart = (int64_t)(b.K + 1) * std::max(b.nb, b.gb);
     const int64_t o_w = (int64_t)(b.K + 1) * b.ldv, o_t = o_w + b.ldv, o_part = o_t + b.ldv;
     const int64_t o_sc = o_part + 2 * npart;
