@@ -10,10 +10,13 @@
 // descending list, so the result is one count per sector.
 //
 // One CTA per update.  The spectra are staged in shared memory (those of up to kSelSectors sectors and
-// kSelValues values; larger ones are read where they are), and every value finds its own place among all of
-// them by binary searches: v is the value x with #{sigma > x} < chi <= #{sigma >= x}.  The bisection on the
-// bit pattern of v that did this in 64 rounds of counts and block sums took 86-160 us an update, all of it
-// latency; this takes 27-90.  All sums are fixed-order block reductions (deterministic).
+// kSelValues values; larger ones are read where they are).  v is searched between the cutoff and the largest value by
+// its bit pattern: a round counts the values above 2^p - 1 thresholds by binary searches, one a thread, so the range
+// shrinks 2^p-fold (p = 1 to 5, by the number of sectors).  It takes a warp reduction, a few atomics and one barrier a
+// round, whatever the spectra.  One update, us, by the bisection with two searches a sector and a block sum in each of
+// 64 rounds | by letting every value search its own place | so: 20 sectors of 20 values 111 | 62 | 36, 30 of 150
+// 172 | 211 | 47, 30 of 600 226 | 1643 | 72, 600 of 8 917 | 16657 | 476, 16 of 280 equal values 158 | 4015 | 41.
+// All sums are fixed-order block reductions (deterministic).
 #include "mps_internal.h"
 
 namespace mps {
@@ -48,21 +51,8 @@ __device__ T block_sum(T v, T* red) {
 // Singular values are not negative, so their bit patterns order like the values; integer comparisons
 // keep the searches off the FP64 pipe (where one costs a warp 64 cycles).
 __device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
-// number of entries of a descending array that are > x
-__device__ int count_gt(const double* a, int k, double x) {
-  if (x < 0.0) return k;
-  const long long b = bits(x);
-  int lo = 0, hi = k;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (bits(a[mid]) > b) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-// number of entries of a descending array that are >= x
-__device__ int count_ge(const double* a, int k, double x) {
-  if (x <= 0.0) return k;
-  const long long b = bits(x);
+// number of entries of a descending array whose bits are >= b
+__device__ __forceinline__ int count_from(const double* a, int k, long long b) {
   int lo = 0, hi = k;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
@@ -70,6 +60,9 @@ __device__ int count_ge(const double* a, int k, double x) {
   }
   return lo;
 }
+// number of entries of a descending array that are > x, and that are >= x
+__device__ int count_gt(const double* a, int k, double x) { return x < 0.0 ? k : count_from(a, k, bits(x) + 1); }
+__device__ int count_ge(const double* a, int k, double x) { return x <= 0.0 ? k : count_from(a, k, bits(x)); }
 
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector* __restrict__ secs,
                                                              const SelectTask* __restrict__ tasks,
@@ -80,7 +73,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
   __shared__ double s_val[kSelValues];
   __shared__ const double* s_sig[kSelSectors];
   __shared__ int s_k[kSelSectors], s_cand[kSelSectors], s_above[kSelSectors], s_band[kSelSectors];
-  __shared__ double s_v;
+  __shared__ int s_count[3][32];
   const SelectTask T = tasks[blockIdx.x];
   const int tid = threadIdx.x;
   const int ns = T.s1 - T.s0;
@@ -107,6 +100,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
       __syncthreads();
     }
   }
+  // 2^p - 1 thresholds a round of the search, as many as give every (sector, threshold) a thread
+  int p = 5;
+  while (p > 1 && ns << p > kSelThreads) --p;
+  if (tid < 32) s_count[0][tid] = 0;      // before the barriers of the sums below
   auto sector = [&](int s) { return listed ? SelectSector{s_sig[s], s_k[s]} : secs[T.s0 + s]; };
   // |sigma|^2 and sigma_max
   double part = 0.0, vmax = 0.0;
@@ -140,28 +137,29 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
   const long long nc = block_sum(nc_part, ired);
   int band_total = 0;
   if (nc > T.chi) {
-    // the chi-th largest candidate: the value whose equals straddle place chi
-    for (int s = 0, first = 0; s < ns; ++s) {
-      const SelectSector S = sector(s);
-      const int cand = listed ? s_cand[s] : kept[T.s0 + s];
-      // the candidates of all sectors dealt to the threads in one row
-      const int j0 = (tid - first % kSelThreads + kSelThreads) % kSelThreads;
-      first += cand;
-      for (int j = j0; j < cand; j += kSelThreads) {
-        const double x = S.sigma[j];
-        int gt = 0, ge = 0;
-        for (int q = 0; q < ns && gt < T.chi; ++q) {
-          const SelectSector Q = sector(q);
-          const int c = count_gt(Q.sigma, Q.k, x);
-          gt += c;
-          ge += c;
-          for (int i = c; i < Q.k && bits(Q.sigma[i]) == bits(x); ++i) ++ge;
+    // v, the largest x with #{sigma >= x} >= chi, is the chi-th largest candidate
+    long long lo = thr >= 0.0 ? bits(thr) + 1 : 0, hi = bits(vmax) + 1;      // #{>= lo} >= chi > #{>= hi}
+    const int g = p == 1 ? 0 : p, j = tid & ((1 << g) - 1);      // thresholds sit in neighbouring lanes
+    for (int r = 0; hi - lo > 1; r = r == 2 ? 0 : r + 1) {
+      const long long step = max(1LL, (hi - lo) >> p), x = lo + step * (j + 1);
+      const bool tried = j + 1 < 1 << p && x < hi;
+      int c = 0;
+      if (tried)
+        for (int t = tid; t < ns << g; t += kSelThreads) {
+          const SelectSector S = sector(t >> g);
+          c += count_from(S.sigma, S.k, x);
         }
-        if (gt < T.chi && ge >= T.chi) s_v = x;      // every value equal to it writes the same
-      }
+      for (int o = 1 << g; o < 32; o <<= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if ((tid & 31) < 1 << g && c) atomicAdd(&s_count[r][j], c);
+      if (tid < 32) s_count[r == 2 ? 0 : r + 1][tid] = 0;      // last read two barriers ago
+      __syncthreads();
+      const unsigned enough =
+          __ballot_sync(0xffffffffu, (tid & 31) < 1 << g && tried && s_count[r][j] >= T.chi);
+      const int above = enough ? 32 - __clz(enough) : 0;      // the thresholds that still have chi values
+      if (lo + step * (above + 1) < hi && above + 1 < 1 << p) hi = lo + step * (above + 1);
+      lo += step * above;
     }
-    __syncthreads();
-    const double v = s_v;
+    const double v = __longlong_as_double(lo);
     const double delta = kTieRel * vmax;
     const double upper = v + delta, lower = v - delta;
     long long above_part = 0, band_part = 0;
@@ -173,13 +171,15 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
       if (listed) {
         s_above[s] = above;
         s_band[s] = inband;
+        s_cand[s] = above + inband;      // from here on: the number kept
       }
+      kept[T.s0 + s] = above + inband;
       above_part += above;
       band_part += inband;
     }
     const long long above_total = block_sum(above_part, ired);
     band_total = (int)block_sum(band_part, ired);
-    if (tid == 0) {
+    if (tid == 0 && band_total > T.chi - above_total) {      // more ties than places: in sector order
       long long left = T.chi - above_total;
       for (int s = 0; s < ns; ++s) {
         int above, inband;
@@ -189,10 +189,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
         } else {
           const SelectSector S = secs[T.s0 + s];
           above = count_gt(S.sigma, S.k, upper);
-          inband = min(count_ge(S.sigma, S.k, lower), count_gt(S.sigma, S.k, thr)) - above;
+          inband = kept[T.s0 + s] - above;
         }
         const long long take = min((long long)inband, left);
-        if (listed) s_cand[s] = above + (int)take;      // from here on: the number kept
+        if (listed) s_cand[s] = above + (int)take;
         kept[T.s0 + s] = above + (int)take;
         left -= take;
       }

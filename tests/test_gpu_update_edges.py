@@ -85,3 +85,39 @@ def test_selection_over_more_values_than_a_table(gpu_lib):
     tables = [{c: 230 for c in range(lo, lo + 10)} for lo in (9, 8, 7)]
     g, st = _update(gpu_lib, 3, 24, 24, 11, tables, 900, rng)
     _same(g, st, 11, 3)
+
+
+@pytest.mark.parametrize("dim, charges, chi", [(40, 11, 100), (150, 11, 700), (300, 11, 2000), (600, 9, 2500), (2, 281, 401)])
+def test_selection_among_equal_values(gpu_lib, dim, charges, chi):
+    """Unitary blocks between equal charges and equal Schmidt values: Theta'(c) is a product of unitaries, the values of
+    all sectors are equal up to rounding, and the ties go to the sectors in ascending order until chi are kept (up to
+    and past the values and the sectors that are staged in shared memory)."""
+    m = gpu_lib
+    rng = np.random.default_rng(dim)
+    d, L = 2, 2 * charges + 20
+    s = L // 2 - 1
+    st = U1MPS.product(d, [k % 2 for k in range(L)])
+    table = {5 + q: dim for q in range(charges)}
+    for b in (s, s + 1, s + 2):
+        st.bond[b] = dict(table)
+        st.lam[b] = {c: np.ones(dim) / np.sqrt(dim * charges) for c in table}
+    for k in (s, s + 1):
+        st.B[k] = {(c, r): np.zeros((dim, dim), complex) for c in table for r in table if 0 <= c - r < d}
+        for c in table:
+            st.B[k][(c, c)] = np.linalg.qr(rng.standard_normal((dim, dim)) + 1j * rng.standard_normal((dim, dim)))[0]
+    g = m.MPS(d, [k % 2 for k in range(L)], max(chi, dim * charges))
+    for b in (s, s + 1, s + 2):
+        g.set_bond(b, st.lam[b])
+    for k in (s, s + 1):
+        g.set_site(k, st.B[k])
+    gate = [np.eye(1, dtype=complex), np.eye(2, dtype=complex), np.eye(1, dtype=complex)]
+    g.apply_gate2(s, gate, chi, 1e-10)
+    kept = {c: len(v) for c, v in g.bond(s + 1).items()}
+    want, left = {}, chi
+    for c in table:
+        if left > 0:
+            want[c] = min(dim, left)
+            left -= want[c]
+    assert kept == want
+    for c, v in g.bond(s + 1).items():
+        assert np.max(np.abs(v - 1 / np.sqrt(chi))) <= 1e-12
