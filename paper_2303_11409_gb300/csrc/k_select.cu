@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectSector*
     for (int s = tid; s < ns; s += kSelThreads) kept[T.s0 + s] = 0;
     return;
   }
-  const double thr = T.cutoff * R.norm_all;
+  double thr = T.cutoff * R.norm_all;
+  if (thr == 0.0) thr = 0.0;      // -0.0 has the lowest bits of all
   long long nc_part = 0;
   for (int s = tid; s < ns; s += kSelThreads) {
     const SelectSector S = sector(s);

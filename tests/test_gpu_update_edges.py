@@ -121,3 +121,23 @@ def test_selection_among_equal_values(gpu_lib, dim, charges, chi):
     assert kept == want
     for c, v in g.bond(s + 1).items():
         assert np.max(np.abs(v - 1 / np.sqrt(chi))) <= 1e-12
+
+
+@pytest.mark.parametrize("cutoff", [0.0, -0.0])
+def test_a_cutoff_of_minus_zero_is_zero(gpu_lib, cutoff):
+    """Values of exactly 0 (empty rows and columns) are not kept by either."""
+    m = gpu_lib
+    d, L, s, dim = 2, 12, 5, 8
+    table = {3: dim, 2: dim}
+    g = m.MPS(d, [k % 2 for k in range(L)], 64)
+    rng = np.random.default_rng(3)
+    for b in (s, s + 1, s + 2):
+        g.set_bond(b, {c: np.ones(dim) / np.sqrt(2 * dim) for c in table})
+    B = {(c, r): np.zeros((dim, dim), complex) for c in table for r in table if 0 <= c - r < d}
+    for c in table:
+        B[(c, c)][:3, :3] = rng.standard_normal((3, 3))
+    for k in (s, s + 1):
+        g.set_site(k, B)
+    g.apply_gate2(s, [np.eye(1, dtype=complex), np.eye(2, dtype=complex), np.eye(1, dtype=complex)], 64, cutoff)
+    assert {c: len(v) for c, v in g.bond(s + 1).items()} == {2: 3, 3: 3}
+    assert all(np.all(v > 0) for v in g.bond(s + 1).values())
