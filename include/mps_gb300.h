@@ -737,8 +737,9 @@ MPS_API int mps_svd_sectors_path(int n_sectors, const int* m, const int* n,
  * FP32 (default 192; 0: none does).  The FP32 sweeps run on the Jacobi matrix stacked on the
  * identity, which accumulates the rotations V.  Sectors of TF32 and BF16x3 handles then make V
  * unitary in FP64 (one Cholesky QR) and go on with FP64 sweeps from the Jacobi matrix times V.
- * All other sectors do so whatever their size, unless min_k is 0, and are finished by FP64-accurate products
- * (on the tensor cores from 25 columns) instead of FP64 sweeps.  Results meet the same FP64 accuracy; FP32 runs at 61x the FP64
+ * All other sectors are finished by FP64-accurate products (on the tensor cores from 25 columns) instead of FP64
+ * sweeps, whatever their size while min_k is 1..192; above the default only from min_k on, so that a
+ * caller can keep smaller sectors in FP64 throughout.  Results meet the same FP64 accuracy; FP32 runs at 61x the FP64
  * rate on this part.  A process setting, read when an update call or mps_svd_sectors lays out its
  * scratch (more scratch per such sector from 25 columns: about 8 (jlen + K) K + 32 (n + K) K bytes).  MPS_EINVAL for
  * min_k < 0.  A tuning of the per-sector SVDs of Sec. II; no counterpart in the paper.

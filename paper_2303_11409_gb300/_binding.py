@@ -701,7 +701,8 @@ def svd_inject_stall(what: int) -> None:
 
 
 def svd_mixed_min_k(min_k: int) -> None:
-    """Cluster SVD sectors with min(m, n) >= min_k start with FP32 Jacobi sweeps (0: off)."""
+    """Sector SVDs with min(m, n) >= min_k start with FP32 Jacobi sweeps (0: none; FP64 handles: all while
+    min_k is at most its default, 192)."""
     rc = lib.mps_svd_mixed_min_k(int(min_k))
     if rc != MPS_OK:
         raise MPSError(rc, "mps_svd_mixed_min_k")

@@ -76,6 +76,7 @@ constexpr int kMaxTeam = 304;           // CTAs of a team: 2 on each of 152 SMs
 constexpr int kSvdExpired = -2;         // a sector's status when a bounded wait ran out
 constexpr int kMaxWarps = 16;
 constexpr int kBlockThreads = 192;      // block-Jacobi cluster kernel: 6 warps per CTA, 2 CTAs per SM
+constexpr int kMixedMinK = 192;         // default of mps_svd_mixed_min_k
 constexpr int kRefineMinK = 25;         // smallest min(m, n) refined on the tensor cores
 // a refined sector's FP32 sweeps end with one that found no cosine above this: it has left about the square
 constexpr float kFp32Stop = 1e-3f;
@@ -3132,7 +3133,11 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
   for (auto* v : {&L.f32_off, &L.n32_off, &L.vd_off, &L.gm_off, &L.a1_off, &L.sel_off, &L.j_off, &L.v_off2, &L.misc_off})
     v->assign(ns, -1);
   L.smem = 0;
-  const int set_k = svd_mixed_min_k(), own_k = set_k > 0 ? kRefineMinK : 0;   // 0: off
+  // FP64 updates refine at every size unless the caller has asked for FP64 sweeps, at all sizes (0) or up to a size
+  // above the default
+  const int set_k = svd_mixed_min_k();
+  const bool any_k = set_k > 0 && set_k <= kMixedMinK;
+  const int own_k = any_k ? kRefineMinK : set_k;
   int64_t off = 0;
   auto a256 = [](int64_t x) { return (x + 255) & ~int64_t(255); };
   for (int k = 0; k < ns; ++k) {
@@ -3143,7 +3148,7 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     const bool refine = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) >= own_k &&
                         16LL * std::max(m[k], n[k]) <= kBlockSmemMax;
     if (need <= kSvdSmemMax && std::min(m[k], n[k]) < cluster_min_k && !refine) {
-      L.small[k] = !L.exact[k] && own_k > 0 && std::min(m[k], n[k]) <= kSmallK &&
+      L.small[k] = !L.exact[k] && any_k && std::min(m[k], n[k]) <= kSmallK &&
                    small_layout(m[k], n[k], true).total <= kSvdSmemMax;
       L.smem = std::max<int>(L.smem, (int)need);
       continue;
@@ -3242,7 +3247,7 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
 }
 
 namespace {
-std::atomic<int> g_mixed_min_k{192};
+std::atomic<int> g_mixed_min_k{kMixedMinK};
 std::atomic<int> g_mixed_sweeps{8};
 std::atomic<int> g_cluster_min_k{1 << 30};
 std::atomic<int> g_svd_stall{0};

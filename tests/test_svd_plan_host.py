@@ -40,3 +40,22 @@ def test_columns_too_long_for_a_front_keep_the_fp32_start(m, rows, cols):
         assert path == m.MPS_SVD_REFINED
     else:
         assert path == m.MPS_SVD_SWEEPS | (m.MPS_SVD_FP32_START if min(rows, cols) >= 192 else 0)
+
+
+def test_raising_the_fp32_limit_keeps_smaller_sectors_in_fp64(m):
+    sizes = [(15, 15), (24, 24), (60, 60), (250, 260), (399, 900), (400, 400), (700, 500)]
+    try:
+        for k in (1, 64, 192):
+            m.svd_mixed_min_k(k)
+            assert all(m.svd_sector_plan(*s)["path"] == m.MPS_SVD_REFINED for s in sizes)
+            for s in sizes:
+                start = m.MPS_SVD_FP32_START if min(s) >= max(k, 96) else 0      # from the block clusters' sizes
+                assert m.svd_sector_plan(*s, keep_phases=True)["path"] == m.MPS_SVD_SWEEPS | start
+        m.svd_mixed_min_k(400)
+        for s in sizes:
+            assert m.svd_sector_plan(*s)["path"] == (m.MPS_SVD_REFINED if min(s) >= 400 else m.MPS_SVD_SWEEPS)
+        m.svd_mixed_min_k(0)
+        for s in sizes:
+            assert m.svd_sector_plan(*s)["path"] == m.svd_sector_plan(*s, keep_phases=True)["path"] == m.MPS_SVD_SWEEPS
+    finally:
+        m.svd_mixed_min_k(192)
