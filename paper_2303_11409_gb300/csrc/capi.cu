@@ -756,6 +756,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   for (int c = 0; c < n_cand; ++c) {
     const SvdTune tune = n_cand > 1 ? svd_tune_candidate(c) : (chosen >= 0 ? svd_tune_candidate(chosen) : SvdTune());
     CUDA_OR_FAIL(owner, svd_group(svd_sorted[c], svd_groups[c], tune, teams));
+    CUDA_OR_FAIL(owner, svd_side_streams(owner, (int)svd_groups[c].size() - 1));
   }
 
   // ---- descriptors into the staging buffer (uploaded in one copy) ---------------------
@@ -855,7 +856,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
   };
   auto svd_launch = [&](int c) -> cudaError_t {   // one or more kernels
     const SvdSector* d_svd = reinterpret_cast<SvdSector*>(dptr(desc_off + o_svd[c]));
-    return launch_svd_groups(d_svd, svd_groups[c], st, owner->side, kSvdSideStreams, owner->fork, owner->join,
+    return launch_svd_groups(d_svd, svd_groups[c], st, owner->side, owner->n_side, owner->fork, owner->join,
                              owner->sweep_limit);
   };
   auto select_and_readback = [&]() -> cudaError_t {
@@ -966,6 +967,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
       // the tile shape the first run used for these sectors
       const SvdTune tune = n_cand > 1 ? svd_tune_candidate(c_used) : (chosen >= 0 ? svd_tune_candidate(chosen) : SvdTune());
       CUDA_OR_FAIL(owner, svd_group(sub, sub_groups, tune, teams));
+      CUDA_OR_FAIL(owner, svd_side_streams(owner, (int)sub_groups.size() - 1));
       // the phase-1 SVD descriptors are no longer read (the stream is synchronised): reuse them
       char* hsrc = (char*)owner->pin_in.p + o_svd[c_used];
       std::memcpy(hsrc, sub.data(), sizeof(SvdSector) * sub.size());
@@ -973,7 +975,7 @@ int run_batch(std::vector<Req>& reqs, mps_s* owner) {
                                           cudaMemcpyHostToDevice, st));
       const SvdSector* d_sub = reinterpret_cast<SvdSector*>(dptr(desc_off + o_svd[c_used]));
       CUDA_OR_FAIL(owner, timed(owner, MPS_K_SVD, !sub.empty(), sub_flops, sub_bytes, [&] {
-        return launch_svd_groups(d_sub, sub_groups, st, owner->side, kSvdSideStreams, owner->fork, owner->join,
+        return launch_svd_groups(d_sub, sub_groups, st, owner->side, owner->n_side, owner->fork, owner->join,
                                  owner->sweep_limit);
       }));
       CUDA_OR_FAIL(owner, select_and_readback());
@@ -1430,10 +1432,7 @@ static int create_handle(mps_t* out, int L, int d, const int32_t* site_charges, 
   cudaError_t e = cudaMalloc(&h->d_lambda, sizeof(double) * lam_total);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_sites, sizeof(double2) * site_total);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->staged, cudaEventDisableTiming);
-  for (int i = 0; i < kSvdSideStreams && e == cudaSuccess; ++i) {
-    e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->join[i], cudaEventDisableTiming);
-  }
+  if (e == cudaSuccess) e = svd_side_streams(h, kSvdSideAtFirst);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     if (h->d_lambda) cudaFree(h->d_lambda);
@@ -1549,10 +1548,7 @@ int mps_exec_create(mps_exec_t* out, void* cuda_stream) {
   mps_s* h = new mps_s();
   h->stream = (cudaStream_t)cuda_stream;
   cudaError_t e = cudaEventCreateWithFlags(&h->staged, cudaEventDisableTiming);
-  for (int i = 0; i < kSvdSideStreams && e == cudaSuccess; ++i) {
-    e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->join[i], cudaEventDisableTiming);
-  }
+  if (e == cudaSuccess) e = svd_side_streams(h, kSvdSideAtFirst);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     mps_destroy(h);

@@ -1592,6 +1592,7 @@ struct Dmrg {
     if (spread) tune.cl_min = 8;
     svd_forced_tune(tune);
     e = svd_group(secs, groups, tune);
+    if (e == cudaSuccess) e = svd_side_streams(h, (int)groups.size() - 1);
     if (e != cudaSuccess) return fail(MPS_ECUDA, "DMRG SVD grouping");
     SelectTask task{0, ns, chi, cutoff};
     // descriptors of the SVD and the selection, then the transposes
@@ -1613,7 +1614,7 @@ struct Dmrg {
       const SvdSector* d_secs = reinterpret_cast<const SvdSector*>(dd.p);
       if (e == cudaSuccess)
         e = timed(3, svd_flops, [&] {
-          return launch_svd_groups(d_secs, groups, st, h->side, kSvdSideStreams, h->fork, h->join, h->sweep_limit);
+          return launch_svd_groups(d_secs, groups, st, h->side, h->n_side, h->fork, h->join, h->sweep_limit);
         });
       if (e == cudaSuccess)
         e = launch_select(reinterpret_cast<const SelectSector*>((char*)dd.p + o_sel),
@@ -1899,7 +1900,8 @@ struct Dmrg {
       SvdTune tune;
       if (spread) tune.cl_min = 8;
       svd_forced_tune(tune);
-      if (svd_group(secs, groups, tune) != cudaSuccess) return fail(MPS_ECUDA, "DMRG SVD grouping");
+      if (svd_group(secs, groups, tune) != cudaSuccess || svd_side_streams(h, (int)groups.size() - 1) != cudaSuccess)
+        return fail(MPS_ECUDA, "DMRG SVD grouping");
       SelectTask task{0, ns, 1 << 30, 0.0};
       const int64_t sel_bytes = a256(sizeof(SvdSector) * ns) + a256(sizeof(SelectSector) * ns) + 256;
       if (reserve_desc(sel_bytes + desc_bytes(bp)) != cudaSuccess) return fail(MPS_ENOMEM, "DMRG descriptors");
@@ -1917,7 +1919,7 @@ struct Dmrg {
       const SvdSector* d_secs = reinterpret_cast<const SvdSector*>(dd.p);
       if (e == cudaSuccess)
         e = timed(3, svd_flops, [&] {
-          return launch_svd_groups(d_secs, groups, st, h->side, kSvdSideStreams, h->fork, h->join, h->sweep_limit);
+          return launch_svd_groups(d_secs, groups, st, h->side, h->n_side, h->fork, h->join, h->sweep_limit);
         });
       if (e == cudaSuccess)
         e = launch_select(reinterpret_cast<const SelectSector*>((char*)dd.p + o_sel),

@@ -3045,6 +3045,17 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
   return cudaSuccess;
 }
 
+cudaError_t svd_side_streams(mps_s* h, int n) {
+  for (n = std::min(n, kSvdSideStreams); h->n_side < n; ++h->n_side) {
+    cudaStream_t& s = h->side[h->n_side];
+    cudaEvent_t& j = h->join[h->n_side];
+    cudaError_t e = s ? cudaSuccess : cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !j) e = cudaEventCreateWithFlags(&j, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGroup>& groups, cudaStream_t st,
                               const cudaStream_t* side, int n_side, cudaEvent_t fork, const cudaEvent_t* join,
                               int max_sweeps) {

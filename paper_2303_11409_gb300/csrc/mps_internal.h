@@ -11,7 +11,8 @@
 
 namespace mps {
 
-constexpr int kSvdSideStreams = 8;      // side streams for concurrent SVD kernel groups
+constexpr int kSvdSideStreams = 8;      // most side streams for concurrent SVD kernel groups
+constexpr int kSvdSideAtFirst = 4;      // created with a handle (15 us each with its event), the others when a call needs them
 
 // ---------------------------------------------------------------------------
 // Charge arithmetic.  U(1) (zn = 0, Sec. II): block (l, m) of a site carries the physical
@@ -371,6 +372,7 @@ struct mps_s {
   mps::PinnedBuf pin_in, pin_out;         // staging of descriptors and results
   cudaEvent_t staged = nullptr;           // last upload out of pin_in has completed
   cudaStream_t side[mps::kSvdSideStreams] = {};     // side streams for concurrent SVD kernel groups
+  int n_side = 0;                                   // created so far
   cudaEvent_t fork = nullptr, join[mps::kSvdSideStreams] = {};
   std::string err;
   mps::Stats stats;
@@ -440,6 +442,8 @@ cudaError_t svd_group(std::vector<SvdSector>& secs, std::vector<SvdGroup>& group
                       const SvdTune& tune = SvdTune(), bool team = false);
 // The candidate mps_autotune_force set (true), or false when none is forced.
 bool svd_forced_tune(SvdTune& t);
+// Side streams and join events of h up to n of them (at most kSvdSideStreams); before a capture that uses them.
+cudaError_t svd_side_streams(mps_s* h, int n);
 // Group 0 on st, group g > 0 on side[g-1] when n_side >= groups - 1; st then waits for all.
 cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGroup>& groups, cudaStream_t st,
                               const cudaStream_t* side, int n_side, cudaEvent_t fork, const cudaEvent_t* join,
