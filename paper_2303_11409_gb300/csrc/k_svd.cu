@@ -3065,11 +3065,6 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
   const int ng = (int)groups.size();
   if (ng == 0) return cudaSuccess;
   const bool fan = side && n_side >= ng - 1 && ng > 1;
-  if (fan) {
-    if ((e = cudaEventRecord(fork, st)) != cudaSuccess) return e;
-    for (int g = 1; g < ng; ++g)
-      if ((e = cudaStreamWaitEvent(side[g - 1], fork, 0)) != cudaSuccess) return e;
-  }
   // Clusters of 8 need free places on several SMs at once, so with them the one-CTA kernels, which take up to a
   // whole SM and end first, go behind the last smaller clusters instead of beside them (a layer of 77 sectors at
   // chi = 333: fronts done after 17.7 instead of 20 ms).
@@ -3081,6 +3076,11 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
     while (behind && g > 1 && one_cta(g)) --g;
     return g;
   };
+  if (fan) {      // only the streams that get work: each is joined below, as a capture wants
+    if ((e = cudaEventRecord(fork, st)) != cudaSuccess) return e;
+    for (int g = 1; g < ng; ++g)
+      if (lane(g) == g && (e = cudaStreamWaitEvent(side[g - 1], fork, 0)) != cudaSuccess) return e;
+  }
   for (int g = 0; g < ng; ++g) {
     cudaStream_t s = (fan && g > 0) ? side[lane(g) - 1] : st;
     if ((e = launch_group(d_secs, groups[g], max_sweeps, s)) != cudaSuccess) return e;

@@ -108,3 +108,32 @@ def test_more_sectors_than_a_grid_has_rows(gpu_lib):
     assert all(r[3] == m.MPS_SVD_REFINED for r in out)
     for i in [0, 1, *range(65530, 65540), n - 1, *rng.integers(0, n, 200)]:
         _check(A[i], *out[i][:3])
+
+
+def test_captured_layer_with_every_kind_of_front(gpu_lib):
+    """A layer whose sectors take clusters of 8, smaller clusters, one CTA and the whole refinement in one CTA, on side
+    streams and behind one another: with captured phases the same bits as without, call after call."""
+    import torch
+    from oracle import gates
+    from tests.helpers import load_state, random_state
+    m = gpu_lib
+    L, chi, sites = 14, 700, [2, 4, 6, 8, 10]
+    st = random_state(L, 5, L, chi, seed=8)
+    stream = torch.cuda.Stream()
+    out = []
+    for graphs in (False, True):
+        g = m.MPS(5, [1] * L, chi, stream=stream.cuda_stream)
+        load_state(g, st)
+        g.set_graphs(graphs)
+        for _ in range(3):
+            g.apply_layer(sites, [gates.bh_gate(L, s, 5, 1.0, 2.0, 0.1) for s in sites], chi, 1e-10)
+            assert g.last_batch_paths()["refined"] > 30
+        out.append([g.bond(b) for b in range(L + 1)] + [g.site(s) for s in range(L)])
+        if graphs:
+            assert g.graph_stats()["launches"] >= 6
+        g.close()
+    plans = [m.svd_sector_plan(*s) for s in ((300, 300), (130, 140), (60, 60), (20, 20))]
+    assert [p["ctas"] for p in plans] == [8, 4, 1, 1], plans
+    for a, b in zip(*out):
+        assert a.keys() == b.keys()
+        assert all(np.array_equal(a[k], b[k]) for k in a)
