@@ -7,7 +7,7 @@ importing this module fails loudly otherwise.  There is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
-import functools
+import operator
 import os
 import warnings
 
@@ -186,14 +186,10 @@ def _default_stream():
     return None
 
 
-@functools.lru_cache(maxsize=None)
 def gate_length(d: int) -> int:
-    """Complex numbers in one flattened gate: sum over n of s_n^2."""
-    tot = 0
-    for n in range(2 * d - 1):
-        s = min(d - 1, n) - max(0, n - d + 1) + 1
-        tot += s * s
-    return tot
+    """Complex numbers in one flattened gate: the sum of s_n^2 over its blocks, s_n = 1, ..., d, ..., 1."""
+    d = max(0, operator.index(d))
+    return d * (2 * d * d + 1) // 3
 
 
 def multi_pair_blocks(charges):

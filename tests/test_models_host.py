@@ -104,3 +104,12 @@ def test_gate_lengths(pkg):
             t = (a[0] + b[0], a[1] + b[1])
             total[t] = total.get(t, 0) + 1
     assert sum(len(p) ** 2 for p in pairs.values()) == sum(k * k for k in total.values())
+
+
+def test_gate_length_takes_what_it_took(pkg):
+    """Any integer (numpy scalars and 0-d arrays too), 0 for what has no blocks, and no float, whatever was asked before."""
+    assert pkg.gate_length(5) == pkg.gate_length(np.int32(5)) == pkg.gate_length(np.array(5)) == 85
+    assert pkg.gate_length(0) == pkg.gate_length(-2) == 0
+    for bad in (5.0, np.float64(5), "5"):
+        with pytest.raises(TypeError):
+            pkg.gate_length(bad)
