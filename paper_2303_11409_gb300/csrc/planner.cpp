@@ -195,7 +195,8 @@ void plan_update(const BondTable& left, const BondTable& mid, const BondTable& r
   // Candidate middle charges: c with some left l in [c, c+d-1] and right r in [c-d+1, c].
   int cmin = std::max(right.charge.front(), left.charge.front() - (d - 1));
   int cmax = std::min(left.charge.back(), right.charge.back() + (d - 1));
-  plan.sectors.reserve(std::max(0, cmax - cmin + 1));
+  // at most d charges below every left one, however far apart those are
+  plan.sectors.reserve((size_t)std::max<int64_t>(0, std::min<int64_t>((int64_t)cmax - cmin + 1, (int64_t)d * left.size())));
   for (int c = cmin; c <= cmax; ++c) {
     // rows: left sectors with c <= l <= c + d - 1 (contiguous in the sorted table)
     int l0 = (int)(std::lower_bound(left.charge.begin(), left.charge.end(), c) - left.charge.begin());

@@ -243,3 +243,13 @@ def test_gate_layout_matches_the_oracles_gate_bases(built):
         m.gate_layout(3, zn=2)                                     # Z_n needs d <= n
     with pytest.raises(m.MPSError):
         m.gate_layout(2, charges=[(1, 0), (0, 1)])                 # not ascending
+
+
+@pytest.mark.slow
+def test_planner_takes_charges_far_apart(built):
+    """Two sectors per table, 10^9 charges apart: the plan has as many sectors as the tables allow, and its memory
+    follows those and not the range of the charges."""
+    import paper_2303_11409_gb300 as m
+    n = 10 ** 9
+    triples, sectors = m.plan_sectors(3, {0: 2, n: 1}, {0: 1, n: 1}, {0: 1, n: 3})
+    assert len(triples) == 2 and len(sectors) == 2
