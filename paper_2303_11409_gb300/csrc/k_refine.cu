@@ -232,7 +232,6 @@ __device__ __forceinline__ void load_rows(char* dst, const double2* X, int64_t l
 // Two or three steps settle a sector; launches beyond that find nothing to do (3 us each), and what is
 // not settled after the last one costs FP64 sweeps, which large sectors can least afford.
 __host__ __device__ constexpr int refine_steps(int K) { return K < 200 ? 4 : kRefineSteps; }
-constexpr int kLeftAt = 100;       // rstate[1] when step it leaves the sector: kLeftAt + it
 __device__ __forceinline__ int ns_of(const SvdSector& S) { return __ldg(S.rstate); }
 __device__ __forceinline__ bool skip(const SvdSector& S) { return S.rstate[1] != 0 || S.rstate[2] != 0; }
 

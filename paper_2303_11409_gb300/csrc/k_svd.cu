@@ -939,70 +939,17 @@ struct JacobiBlocks32 {
 };
 struct NoJacobi32 {};
 
-// The mixed-precision start of a cluster sector's sweeps (see above).  J: jlen x K, column c at
-// J + c * jld (FP64, L2).  On return the FP64 Jacobi matrix is S.a1 (same jld), its first
-// *nsel_out columns J V and the rest zero.  Every CTA of the cluster calls it.  False when a
-// wait expired (in every CTA alike).
+// S.vd holds ns columns V of K (ld K), unitary to about 1e-5: one Cholesky QR makes V unitary (V^dag V = U^dag U,
+// V <- V U^-1), and S.a1 (column c at S.a1 + c * jld) becomes J V in its first ns columns, zero in the rest.  Every
+// CTA of the cluster calls it.
 template <class Sync>
-__device__ bool mixed_precondition(const SvdSector& S, const Work& w, const double2* J, int jlen, int jld, int K,
-                                   int rank, int nctas, Sync sync, double floor2, int max_sweeps,
-                                   const JacobiBlocks32& j32, int* nsel_out) {
+__device__ void orthonormal_start(const SvdSector& S, const Work& w, const double2* J, int jlen, int jld, int K, int ns,
+                                  int rank, int nctas, Sync sync, int max_sweeps) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int tid_all = rank * blockDim.x + tid, threads_all = nctas * blockDim.x;
   const int worker = rank * nwarps + warp, workers = nctas * nwarps;
-  const int Rr = jlen + K, fld = (Rr + 1) & ~1;   // even: columns 16-byte aligned for bulk copies
-  float2* F = S.f32;
-  // scale so that the largest column has norm 1 (keeps the FP32 squares far from underflow)
-  double cmax = 0.0;
-  for (int j = 0; j < K; ++j) cmax = fmax(cmax, L2Mem::ld(w.nrm + j));
-  const double sc = cmax > 0.0 ? 1.0 / sqrt(cmax) : 1.0;
-  for (int64_t e = tid_all; e < (int64_t)K * Rr; e += threads_all) {
-    const int c = (int)(e / Rr), i = (int)(e % Rr);
-    float2 v = make_float2(0.f, 0.f);
-    if (i < jlen) {
-      const double2 x = L2Mem::ld(J + (int64_t)c * jld + i);
-      v = make_float2((float)(x.x * sc), (float)(x.y * sc));
-    } else if (i - jlen == c) {
-      v.x = 1.f;
-    }
-    __stcg(F + (int64_t)c * fld + i, v);
-  }
-  for (int s = tid_all; s <= max_sweeps; s += threads_all) L2Mem::st(w.flags + s, 0);
-  sync();
-  // FP32 sweeps to FP32 convergence; the floor is a tenth of the FP64 one (in the scaled units)
-  const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
-  const float fl32 = (float)(0.01 * floor2 * sc * sc);
-  bool conv32 = false;
-  if (j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps),
-          conv32) == kSvdExpired)
-    return false;
-  for (int j = worker; j < K; j += workers) {   // final FP32 norms
-    const float2* a = F + (int64_t)j * fld;
-    float acc = 0.f;
-    for (int i = lane; i < jlen; i += 32) {
-      const float2 x = __ldcg(a + i);
-      acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
-    }
-    acc = warp_sum_f(acc);
-    if (lane == 0) __stcg(S.nrm32 + j, acc);
-  }
-  sync();
-  if (tid_all == 0) {   // the kept columns, in column order
-    int ns = 0;
-    for (int c = 0; c < K; ++c)
-      if (__ldcg(S.nrm32 + c) > fl32) __stcg(S.sel + ns++, c);
-    __stcg(S.sel + K, ns);
-  }
-  sync();
-  const int ns = __ldcg(S.sel + K);
   double2* Vd = S.vd;     // K x ns, column-major (ld K)
   double2* G = S.gm;      // ns x ns, column-major
-  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) {
-    const int t = (int)(e / K), k = (int)(e % K);
-    const float2 v = __ldcg(F + (int64_t)__ldcg(S.sel + t) * fld + jlen + k);
-    L2Mem::st(Vd + e, make_double2((double)v.x, (double)v.y));
-  }
-  sync();
   // Gram matrix G = Vd^dag Vd (upper triangle; a warp per entry)
   for (int64_t e = worker; e < (int64_t)ns * ns; e += workers) {
     const int a = (int)(e % ns), b = (int)(e / ns);
@@ -1083,6 +1030,71 @@ __device__ bool mixed_precondition(const SvdSector& S, const Work& w, const doub
   }
   for (int s = tid_all; s <= max_sweeps; s += threads_all) L2Mem::st(w.flags + s, 0);
   sync();
+}
+
+// The mixed-precision start of a cluster sector's sweeps (see above).  J: jlen x K, column c at
+// J + c * jld (FP64, L2).  On return the FP64 Jacobi matrix is S.a1 (same jld), its first
+// *nsel_out columns J V and the rest zero.  Every CTA of the cluster calls it.  False when a
+// wait expired (in every CTA alike).
+template <class Sync>
+__device__ bool mixed_precondition(const SvdSector& S, const Work& w, const double2* J, int jlen, int jld, int K,
+                                   int rank, int nctas, Sync sync, double floor2, int max_sweeps,
+                                   const JacobiBlocks32& j32, int* nsel_out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int tid_all = rank * blockDim.x + tid, threads_all = nctas * blockDim.x;
+  const int worker = rank * nwarps + warp, workers = nctas * nwarps;
+  const int Rr = jlen + K, fld = (Rr + 1) & ~1;   // even: columns 16-byte aligned for bulk copies
+  float2* F = S.f32;
+  // scale so that the largest column has norm 1 (keeps the FP32 squares far from underflow)
+  double cmax = 0.0;
+  for (int j = 0; j < K; ++j) cmax = fmax(cmax, L2Mem::ld(w.nrm + j));
+  const double sc = cmax > 0.0 ? 1.0 / sqrt(cmax) : 1.0;
+  for (int64_t e = tid_all; e < (int64_t)K * Rr; e += threads_all) {
+    const int c = (int)(e / Rr), i = (int)(e % Rr);
+    float2 v = make_float2(0.f, 0.f);
+    if (i < jlen) {
+      const double2 x = L2Mem::ld(J + (int64_t)c * jld + i);
+      v = make_float2((float)(x.x * sc), (float)(x.y * sc));
+    } else if (i - jlen == c) {
+      v.x = 1.f;
+    }
+    __stcg(F + (int64_t)c * fld + i, v);
+  }
+  for (int s = tid_all; s <= max_sweeps; s += threads_all) L2Mem::st(w.flags + s, 0);
+  sync();
+  // FP32 sweeps to FP32 convergence; the floor is a tenth of the FP64 one (in the scaled units)
+  const float tol32 = 1.1920929e-07f * (float)max(jlen, 32);
+  const float fl32 = (float)(0.01 * floor2 * sc * sc);
+  bool conv32 = false;
+  if (j32(F, jlen, Rr, fld, K, S.nrm32, w.flags, rank, nctas, sync, tol32, fl32, min(max_sweeps, S.fp32_sweeps),
+          conv32) == kSvdExpired)
+    return false;
+  for (int j = worker; j < K; j += workers) {   // final FP32 norms
+    const float2* a = F + (int64_t)j * fld;
+    float acc = 0.f;
+    for (int i = lane; i < jlen; i += 32) {
+      const float2 x = __ldcg(a + i);
+      acc = fmaf(x.x, x.x, fmaf(x.y, x.y, acc));
+    }
+    acc = warp_sum_f(acc);
+    if (lane == 0) __stcg(S.nrm32 + j, acc);
+  }
+  sync();
+  if (tid_all == 0) {   // the kept columns, in column order
+    int ns = 0;
+    for (int c = 0; c < K; ++c)
+      if (__ldcg(S.nrm32 + c) > fl32) __stcg(S.sel + ns++, c);
+    __stcg(S.sel + K, ns);
+  }
+  sync();
+  const int ns = __ldcg(S.sel + K);
+  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) {
+    const int t = (int)(e / K), k = (int)(e % K);
+    const float2 v = __ldcg(F + (int64_t)__ldcg(S.sel + t) * fld + jlen + k);
+    L2Mem::st(S.vd + e, make_double2((double)v.x, (double)v.y));
+  }
+  sync();
+  orthonormal_start(S, w, J, jlen, jld, K, ns, rank, nctas, sync, max_sweeps);
   *nsel_out = ns;
   return true;
 }
@@ -1598,6 +1610,8 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
     const float* v = reinterpret_cast<const float*>(F + (int64_t)__ldcg(S.sel + t) * fld + vr + (k & ~1)) + (k & 1);
     S.V0[e] = make_double2((double)__ldcg(v), (double)__ldcg(v + 2));
   }
+  sync();      // F is read
+  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) S.V32[e] = make_float2((float)S.V0[e].x, (float)S.V0[e].y);
 }
 
 template <class Mem, class Sync, class Jacobi, class J32 = NoJacobi32>
@@ -1611,75 +1625,71 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   const int tid_all = rank * blockDim.x + tid, threads_all = nctas * blockDim.x;
   const int worker = rank * nwarps + warp, workers = nctas * nwarps;
   double2* W = w.W;
-
-  // ---- load M = diag(lambda) Theta' (row-major), column norms, identity permutation ----
-  const int64_t mn = (int64_t)m * n;
-  for (int64_t e = tid_all; e < mn; e += threads_all) {
-    const int i = (int)(e / n), j = (int)(e % n);
-    const double s = S.rowscale ? S.rowscale[i] : 1.0;
-    const double2 t = S.theta[e];
-    Mem::st(W + (int64_t)i * ld + j, make_double2(s * t.x, s * t.y));
-  }
-  for (int s = tid_all; s <= max_sweeps; s += threads_all) Mem::st(w.flags + s, 0);
-  sync();
-  for (int j = tid_all; j < n; j += threads_all) {
-    double acc = 0.0;
-    for (int i = 0; i < m; ++i) {
-      const double2 x = Mem::ld(W + (int64_t)i * ld + j);
-      acc = fma(x.x, x.x, fma(x.y, x.y, acc));
+  // A sector whose refinement did not settle (large groups of close values) goes on from the front's J and rotations: no
+  // second QR, no second FP32 sweeps.  300 x 300 with its values in equal pairs: 147 -> 78 ms.
+  bool resume = false;
+  if constexpr (std::is_same<J32, JacobiBlocks32>::value) resume = S.F && __ldcg(S.rstate + 1) >= kLeftAt;
+  if (resume) {
+    const double up = S.rfloor2[1];      // J is scaled
+    for (int64_t e = tid_all; e < (int64_t)K * n; e += threads_all) {
+      const double2 x = S.J[e];
+      Mem::st(W + e / n * ld + e % n, make_double2(up * x.x, up * x.y));
     }
-    Mem::st(w.nu + j, acc);
-    Mem::st(w.nu0 + j, acc);
-    Mem::st(w.perm + j, j);
-  }
-  sync();
-  if (tid_all == 0) {
-    double f = 0.0;
-    for (int j = 0; j < n; ++j) f += Mem::ld(w.nu + j);
-    Mem::st(w.scal + 1, f);
-  }
-  sync();
-  const double fro2 = Mem::ld(w.scal + 1);
-
-  // ---- Householder QR with column pivoting: M P = Q R ---------------------------------
-  for (int k = 0; k < K; ++k) {
-    // pivot: largest remaining partial norm, ties to the smaller index
-    double bv = -1.0;
-    int bi = n;
-    for (int j = k + tid_all; j < n; j += threads_all) {
-      const double v = Mem::ld(w.nu + j);
-      if (v > bv || (v == bv && j < bi)) { bv = v; bi = j; }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
-    if (lane == 0) { red_v[warp] = bv; red_i[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      for (int x = 1; x < nwarps; ++x)
-        if (red_v[x] > bv || (red_v[x] == bv && red_i[x] < bi)) { bv = red_v[x]; bi = red_i[x]; }
-      Mem::st(w.pv + rank, bv);
-      Mem::st(w.pi + rank, bi);
+    for (int s = tid_all; s <= max_sweeps; s += threads_all) Mem::st(w.flags + s, 0);
+    sync();
+    for (int j = worker; j < K; j += workers) {
+      double acc = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        const double2 x = Mem::ld(W + (int64_t)j * ld + i);
+        acc = fma(x.x, x.x, fma(x.y, x.y, acc));
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) Mem::st(w.nu + j, acc);
     }
     sync();
-    if (nctas <= kMaxCluster) {
-      bv = Mem::ld(w.pv);
-      bi = Mem::ld(w.pi);
-      for (int x = 1; x < nctas; ++x) {
-        const double v = Mem::ld(w.pv + x);
-        const int ix = Mem::ld(w.pi + x);
-        if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+    if (tid_all == 0) {
+      double f = 0.0;
+      for (int j = 0; j < K; ++j) f += Mem::ld(w.nu + j);
+      Mem::st(w.scal + 1, f);
+    }
+    sync();
+  } else {
+    // ---- load M = diag(lambda) Theta' (row-major), column norms, identity permutation ----
+    const int64_t mn = (int64_t)m * n;
+    for (int64_t e = tid_all; e < mn; e += threads_all) {
+      const int i = (int)(e / n), j = (int)(e % n);
+      const double s = S.rowscale ? S.rowscale[i] : 1.0;
+      const double2 t = S.theta[e];
+      Mem::st(W + (int64_t)i * ld + j, make_double2(s * t.x, s * t.y));
+    }
+    for (int s = tid_all; s <= max_sweeps; s += threads_all) Mem::st(w.flags + s, 0);
+    sync();
+    for (int j = tid_all; j < n; j += threads_all) {
+      double acc = 0.0;
+      for (int i = 0; i < m; ++i) {
+        const double2 x = Mem::ld(W + (int64_t)i * ld + j);
+        acc = fma(x.x, x.x, fma(x.y, x.y, acc));
       }
-    } else {
-      bv = -1.0;
-      bi = n;
-      for (int x = lane; x < nctas; x += 32) {
-        const double v = Mem::ld(w.pv + x);
-        const int ix = Mem::ld(w.pi + x);
-        if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+      Mem::st(w.nu + j, acc);
+      Mem::st(w.nu0 + j, acc);
+      Mem::st(w.perm + j, j);
+    }
+    sync();
+    if (tid_all == 0) {
+      double f = 0.0;
+      for (int j = 0; j < n; ++j) f += Mem::ld(w.nu + j);
+      Mem::st(w.scal + 1, f);
+    }
+    sync();
+
+    // ---- Householder QR with column pivoting: M P = Q R ---------------------------------
+    for (int k = 0; k < K; ++k) {
+      // pivot: largest remaining partial norm, ties to the smaller index
+      double bv = -1.0;
+      int bi = n;
+      for (int j = k + tid_all; j < n; j += threads_all) {
+        const double v = Mem::ld(w.nu + j);
+        if (v > bv || (v == bv && j < bi)) { bv = v; bi = j; }
       }
 #pragma unroll
       for (int o = 16; o; o >>= 1) {
@@ -1687,141 +1697,173 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
       }
-    }
-    const int p = (bi < n) ? bi : k;
-    if (p != k) {
-      for (int i = tid_all; i < m; i += threads_all) {
-        double2* rowp = W + (int64_t)i * ld;
-        const double2 a = Mem::ld(rowp + k), b = Mem::ld(rowp + p);
-        Mem::st(rowp + k, b);
-        Mem::st(rowp + p, a);
+      if (lane == 0) { red_v[warp] = bv; red_i[warp] = bi; }
+      __syncthreads();
+      if (tid == 0) {
+        for (int x = 1; x < nwarps; ++x)
+          if (red_v[x] > bv || (red_v[x] == bv && red_i[x] < bi)) { bv = red_v[x]; bi = red_i[x]; }
+        Mem::st(w.pv + rank, bv);
+        Mem::st(w.pi + rank, bi);
       }
-      if (tid_all == 0) {
-        double a = Mem::ld(w.nu + k), b = Mem::ld(w.nu + p);
-        Mem::st(w.nu + k, b); Mem::st(w.nu + p, a);
-        a = Mem::ld(w.nu0 + k); b = Mem::ld(w.nu0 + p);
-        Mem::st(w.nu0 + k, b); Mem::st(w.nu0 + p, a);
-        const int ia = Mem::ld(w.perm + k), ib = Mem::ld(w.perm + p);
-        Mem::st(w.perm + k, ib); Mem::st(w.perm + p, ia);
+      sync();
+      if (nctas <= kMaxCluster) {
+        bv = Mem::ld(w.pv);
+        bi = Mem::ld(w.pi);
+        for (int x = 1; x < nctas; ++x) {
+          const double v = Mem::ld(w.pv + x);
+          const int ix = Mem::ld(w.pi + x);
+          if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+        }
+      } else {
+        bv = -1.0;
+        bi = n;
+        for (int x = lane; x < nctas; x += 32) {
+          const double v = Mem::ld(w.pv + x);
+          const int ix = Mem::ld(w.pi + x);
+          if (v > bv || (v == bv && ix < bi)) { bv = v; bi = ix; }
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+          const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+          if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+        }
       }
-    }
-    sync();
-    // reflector H = I - (2 / u^dag u) u u^dag with H x = beta e_k, |beta| = |x|
-    if (worker == 0) {
-      double x2 = 0.0;
-      for (int i = k + lane; i < m; i += 32) {
-        const double2 x = Mem::ld(W + (int64_t)i * ld + k);
-        x2 = fma(x.x, x.x, fma(x.y, x.y, x2));
+      const int p = (bi < n) ? bi : k;
+      if (p != k) {
+        for (int i = tid_all; i < m; i += threads_all) {
+          double2* rowp = W + (int64_t)i * ld;
+          const double2 a = Mem::ld(rowp + k), b = Mem::ld(rowp + p);
+          Mem::st(rowp + k, b);
+          Mem::st(rowp + p, a);
+        }
+        if (tid_all == 0) {
+          double a = Mem::ld(w.nu + k), b = Mem::ld(w.nu + p);
+          Mem::st(w.nu + k, b); Mem::st(w.nu + p, a);
+          a = Mem::ld(w.nu0 + k); b = Mem::ld(w.nu0 + p);
+          Mem::st(w.nu0 + k, b); Mem::st(w.nu0 + p, a);
+          const int ia = Mem::ld(w.perm + k), ib = Mem::ld(w.perm + p);
+          Mem::st(w.perm + k, ib); Mem::st(w.perm + p, ia);
+        }
       }
-      x2 = warp_sum(x2);
-      const double xn = sqrt(x2);
-      const double2 x0 = Mem::ld(W + (int64_t)k * ld + k);
-      const double a0 = hypot(x0.x, x0.y);
-      double2 beta;
-      if (a0 > 0.0) beta = make_double2(-x0.x / a0 * xn, -x0.y / a0 * xn);
-      else beta = make_double2(-xn, 0.0);
-      const double uu = 2.0 * x2 + 2.0 * xn * a0;
-      for (int i = k + lane; i < m; i += 32) {
-        double2 x = Mem::ld(W + (int64_t)i * ld + k);
-        if (i == k) x = make_double2(x.x - beta.x, x.y - beta.y);
-        Mem::st(w.u + i, x);
-        Mem::st(W + (int64_t)i * ld + k, i == k ? beta : make_double2(0.0, 0.0));
+      sync();
+      // reflector H = I - (2 / u^dag u) u u^dag with H x = beta e_k, |beta| = |x|
+      if (worker == 0) {
+        double x2 = 0.0;
+        for (int i = k + lane; i < m; i += 32) {
+          const double2 x = Mem::ld(W + (int64_t)i * ld + k);
+          x2 = fma(x.x, x.x, fma(x.y, x.y, x2));
+        }
+        x2 = warp_sum(x2);
+        const double xn = sqrt(x2);
+        const double2 x0 = Mem::ld(W + (int64_t)k * ld + k);
+        const double a0 = hypot(x0.x, x0.y);
+        double2 beta;
+        if (a0 > 0.0) beta = make_double2(-x0.x / a0 * xn, -x0.y / a0 * xn);
+        else beta = make_double2(-xn, 0.0);
+        const double uu = 2.0 * x2 + 2.0 * xn * a0;
+        for (int i = k + lane; i < m; i += 32) {
+          double2 x = Mem::ld(W + (int64_t)i * ld + k);
+          if (i == k) x = make_double2(x.x - beta.x, x.y - beta.y);
+          Mem::st(w.u + i, x);
+          Mem::st(W + (int64_t)i * ld + k, i == k ? beta : make_double2(0.0, 0.0));
+        }
+        if (lane == 0) Mem::st(w.scal, uu > 0.0 ? 2.0 / uu : 0.0);
       }
-      if (lane == 0) Mem::st(w.scal, uu > 0.0 ? 2.0 / uu : 0.0);
-    }
-    sync();
-    // trailing update W[k:, j] -= (2/u^dag u) u (u^dag W[k:, j]) for j > k: a CTA takes tiles of tc columns,
-    // each column's dot product in nwarps interleaved row chunks (summed in order whatever the tile
-    // width).  32 columns fill the CTA's warps; with more CTAs than such tiles narrower ones put the
-    // chunks of several columns into a warp, so that every CTA has FP64 work.
-    constexpr int ahead = Mem::kCache ? kAhead : 1;      // shared memory answers at once
-    const double sc = Mem::ld(w.scal);
-    const int ncols = n - k - 1;
-    int tc = 32;
-    if constexpr (Mem::kCache)
-      while (nctas > kMaxCluster && tc > 8 && (ncols + tc / 2 - 1) / (tc / 2) <= nctas) tc >>= 1;
-    const int ntiles = (ncols + tc - 1) / tc;
-    const int tcol = tid % tc, chunk = tid / tc;      // chunks beyond nwarps have no rows in the dot product
-    if (sc != 0.0) {
-      for (int tile = rank; tile < ntiles; tile += nctas) {
-        const int j = k + 1 + tile * tc + tcol;
-        double pr = 0.0, pim = 0.0;
-        if (j < n && chunk < nwarps) {
+      sync();
+      // trailing update W[k:, j] -= (2/u^dag u) u (u^dag W[k:, j]) for j > k: a CTA takes tiles of tc columns,
+      // each column's dot product in nwarps interleaved row chunks (summed in order whatever the tile
+      // width).  32 columns fill the CTA's warps; with more CTAs than such tiles narrower ones put the
+      // chunks of several columns into a warp, so that every CTA has FP64 work.
+      constexpr int ahead = Mem::kCache ? kAhead : 1;      // shared memory answers at once
+      const double sc = Mem::ld(w.scal);
+      const int ncols = n - k - 1;
+      int tc = 32;
+      if constexpr (Mem::kCache)
+        while (nctas > kMaxCluster && tc > 8 && (ncols + tc / 2 - 1) / (tc / 2) <= nctas) tc >>= 1;
+      const int ntiles = (ncols + tc - 1) / tc;
+      const int tcol = tid % tc, chunk = tid / tc;      // chunks beyond nwarps have no rows in the dot product
+      if (sc != 0.0) {
+        for (int tile = rank; tile < ntiles; tile += nctas) {
+          const int j = k + 1 + tile * tc + tcol;
+          double pr = 0.0, pim = 0.0;
+          if (j < n && chunk < nwarps) {
 #pragma unroll ahead
-          for (int i = k + chunk; i < m; i += nwarps) {
-            const double2 ui = Mem::ld(w.u + i);
-            const double2 x = Mem::ld(W + (int64_t)i * ld + j);
-            pr = fma(ui.x, x.x, fma(ui.y, x.y, pr));      // conj(u_i) x
-            pim = fma(ui.x, x.y, fma(-ui.y, x.x, pim));
-          }
-        }
-        if (chunk < nwarps) red_d[chunk][tcol] = pr;
-        __syncthreads();
-        double wr = 0.0;
-        for (int x = 0; x < nwarps; ++x) wr += red_d[x][tcol];
-        __syncthreads();
-        if (chunk < nwarps) red_d[chunk][tcol] = pim;
-        __syncthreads();
-        double wi = 0.0;
-        for (int x = 0; x < nwarps; ++x) wi += red_d[x][tcol];
-        __syncthreads();
-        wr *= sc;
-        wi *= sc;
-        if (j < n) {
-          const int step = (int)blockDim.x / tc;
-          for (int i0 = k + chunk; i0 < m; i0 += ahead * step) {
-            double2 ui[ahead], x[ahead];
-#pragma unroll
-            for (int a = 0; a < ahead; ++a)
-              if (i0 + a * step < m) {
-                ui[a] = Mem::ld(w.u + i0 + a * step);
-                x[a] = Mem::ld(W + (int64_t)(i0 + a * step) * ld + j);
-              }
-#pragma unroll
-            for (int a = 0; a < ahead; ++a)
-              if (i0 + a * step < m) {
-                x[a].x -= ui[a].x * wr - ui[a].y * wi;
-                x[a].y -= ui[a].x * wi + ui[a].y * wr;
-                Mem::st(W + (int64_t)(i0 + a * step) * ld + j, x[a]);
-              }
-          }
-        }
-        __syncthreads();
-        if (chunk == 0 && j < n) {       // downdate the partial norm, recompute on cancellation
-          const double2 r = Mem::ld(W + (int64_t)k * ld + j);
-          double v = Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y);
-          if (v <= 1.4901161193847656e-8 * Mem::ld(w.nu0 + j)) {
-            v = 0.0;
-            for (int i = k + 1; i < m; ++i) {
+            for (int i = k + chunk; i < m; i += nwarps) {
+              const double2 ui = Mem::ld(w.u + i);
               const double2 x = Mem::ld(W + (int64_t)i * ld + j);
-              v = fma(x.x, x.x, fma(x.y, x.y, v));
+              pr = fma(ui.x, x.x, fma(ui.y, x.y, pr));      // conj(u_i) x
+              pim = fma(ui.x, x.y, fma(-ui.y, x.x, pim));
             }
-            Mem::st(w.nu0 + j, v);
           }
-          Mem::st(w.nu + j, v);
+          if (chunk < nwarps) red_d[chunk][tcol] = pr;
+          __syncthreads();
+          double wr = 0.0;
+          for (int x = 0; x < nwarps; ++x) wr += red_d[x][tcol];
+          __syncthreads();
+          if (chunk < nwarps) red_d[chunk][tcol] = pim;
+          __syncthreads();
+          double wi = 0.0;
+          for (int x = 0; x < nwarps; ++x) wi += red_d[x][tcol];
+          __syncthreads();
+          wr *= sc;
+          wi *= sc;
+          if (j < n) {
+            const int step = (int)blockDim.x / tc;
+            for (int i0 = k + chunk; i0 < m; i0 += ahead * step) {
+              double2 ui[ahead], x[ahead];
+#pragma unroll
+              for (int a = 0; a < ahead; ++a)
+                if (i0 + a * step < m) {
+                  ui[a] = Mem::ld(w.u + i0 + a * step);
+                  x[a] = Mem::ld(W + (int64_t)(i0 + a * step) * ld + j);
+                }
+#pragma unroll
+              for (int a = 0; a < ahead; ++a)
+                if (i0 + a * step < m) {
+                  x[a].x -= ui[a].x * wr - ui[a].y * wi;
+                  x[a].y -= ui[a].x * wi + ui[a].y * wr;
+                  Mem::st(W + (int64_t)(i0 + a * step) * ld + j, x[a]);
+                }
+            }
+          }
+          __syncthreads();
+          if (chunk == 0 && j < n) {       // downdate the partial norm, recompute on cancellation
+            const double2 r = Mem::ld(W + (int64_t)k * ld + j);
+            double v = Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y);
+            if (v <= 1.4901161193847656e-8 * Mem::ld(w.nu0 + j)) {
+              v = 0.0;
+              for (int i = k + 1; i < m; ++i) {
+                const double2 x = Mem::ld(W + (int64_t)i * ld + j);
+                v = fma(x.x, x.x, fma(x.y, x.y, v));
+              }
+              Mem::st(w.nu0 + j, v);
+            }
+            Mem::st(w.nu + j, v);
+          }
+        }
+      } else {
+        for (int tile = rank; tile < ntiles; tile += nctas) {
+          const int j = k + 1 + tile * tc + tcol;
+          if (chunk == 0 && j < n) {
+            const double2 r = Mem::ld(W + (int64_t)k * ld + j);
+            Mem::st(w.nu + j, fmax(Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y), 0.0));
+          }
         }
       }
-    } else {
-      for (int tile = rank; tile < ntiles; tile += nctas) {
-        const int j = k + 1 + tile * tc + tcol;
-        if (chunk == 0 && j < n) {
-          const double2 r = Mem::ld(W + (int64_t)k * ld + j);
-          Mem::st(w.nu + j, fmax(Mem::ld(w.nu + j) - (r.x * r.x + r.y * r.y), 0.0));
-        }
-      }
+      sync();
+    }
+
+    // ---- R^dag: conjugate rows 0..K-1 in place; they are the Jacobi columns ------------
+    for (int64_t e = tid_all; e < (int64_t)K * n; e += threads_all) {
+      const int i = (int)(e / n), j = (int)(e % n);
+      double2* a = W + (int64_t)i * ld + j;
+      const double2 x = Mem::ld(a);
+      Mem::st(a, make_double2(x.x, -x.y));
     }
     sync();
   }
-
-  // ---- R^dag: conjugate rows 0..K-1 in place; they are the Jacobi columns ------------
-  const int64_t kn = (int64_t)K * n;
-  for (int64_t e = tid_all; e < kn; e += threads_all) {
-    const int i = (int)(e / n), j = (int)(e % n);
-    double2* a = W + (int64_t)i * ld + j;
-    const double2 x = Mem::ld(a);
-    Mem::st(a, make_double2(x.x, -x.y));
-  }
-  sync();
+  const double fro2 = Mem::ld(w.scal + 1);
 
   // ---- wide sectors (K = m < n): R^dag = Q2 [R2; 0] by unpivoted Householder QR of its
   // K columns.  Rotations that orthogonalise the columns of R^dag orthogonalise those of
@@ -1910,9 +1952,15 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   bool converged = false;
   int Kj = K;                    // columns the FP64 sweeps rotate
   if constexpr (std::is_same<J32, JacobiBlocks32>::value) {
-    if (S.f32 && K >= 2) {       // FP32 sweeps first; the FP64 sweeps then start from J V
+    if (resume || (S.f32 && K >= 2)) {       // the FP64 sweeps start from J V, V the rotations of FP32 sweeps
       int ns = K;
-      if (!mixed_precondition(S, w, J, jlen, jld, K, rank, nctas, sync, floor2, max_sweeps, j32, &ns)) {
+      if (resume) {
+        ns = __ldcg(S.rstate);
+        for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all)
+          Mem::st(S.vd + e, make_double2((double)S.V32[e].x, (double)S.V32[e].y));
+        sync();
+        orthonormal_start(S, w, J, jlen, jld, K, ns, rank, nctas, sync, max_sweeps);
+      } else if (!mixed_precondition(S, w, J, jlen, jld, K, rank, nctas, sync, floor2, max_sweeps, j32, &ns)) {
         if (tid_all == 0) *S.status = kSvdExpired;
         return;
       }
@@ -2007,7 +2055,7 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
     }
   } else {
     // Y[perm[j], r] = column ord[r] of R^dag, row j, divided by its norm
-    for (int64_t e = tid_all; e < kn; e += threads_all) {
+    for (int64_t e = tid_all; e < (int64_t)K * n; e += threads_all) {
       const int r = (int)(e / n), j = (int)(e % n);
       const int c = Mem::ld(w.ord + r);
       const double sv = Mem::ld(w.nrm + c);
@@ -2021,7 +2069,7 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   }
   if (tid_all == 0) {
     *S.status = converged ? sweep : -1;
-    const bool start = std::is_same<J32, JacobiBlocks32>::value && S.f32 && K >= 2;
+    const bool start = std::is_same<J32, JacobiBlocks32>::value && (resume || (S.f32 && K >= 2));
     if (S.path) *S.path = MPS_SVD_SWEEPS | (start ? MPS_SVD_FP32_START : 0) | Sync::kPath | Jacobi::kPath;
   }
 }
@@ -2449,6 +2497,7 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
       for (int e = tid; e < K * ns; e += blockDim.x) {
         const float2 v = row32(F + sel[e / K] * L.fld, vr + e % K);
         S.V0[e] = make_double2((double)v.x, (double)v.y);
+        S.V32[e] = v;
       }
       for (int j = tid; j < n; j += blockDim.x) S.order[j] = perm[j];
       if (tid == 0) {
@@ -3175,14 +3224,14 @@ bool svd_layout(int ns, const int* m, const int* n, SvdScratchLayout& L, int clu
     const bool wide = 4LL * n[k] >= 5LL * m[k];   // the Jacobi sweeps run on the K x K factor R2
     L.wide[k] = wide;
     if (refine) {   // FP32 start and refinement (svd_front, k_refine.cu); the FP64 sweeps that may
-                    // follow use A1 and V's space for their second QR
+                    // follow use the same space (svd_fill_scratch)
       const int64_t jlen = wide ? Kk : N;
       L.j_off[k] = off;    off = a256(off + 16 * N * Kk);
-      L.a1_off[k] = off;   off = a256(off + 16 * N * Kk);
+      L.a1_off[k] = off;   off = a256(off + 16 * odd_ld(n[k]) * Kk);
       L.v_off2[k] = off;   off = a256(off + 2 * 16 * Kk * odd_ld((int)Kk));
       L.misc_off[k] = off; off = a256(off + 64 + 16 + 8 * Kk + 4 * (4 * Kk + 1) + 16);
       off = a256(off + 8 * (jlen + Kk + 2) * Kk);      // F, behind the small arrays
-      L.w2_off[k] = L.v_off2[k];
+      L.w2_off[k] = L.v_off2[k] + 16 * Kk * odd_ld((int)Kk);
       L.yt_off[k] = L.a1_off[k];
     } else {
       if (wide) {
@@ -3254,6 +3303,12 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
     S.sel = reinterpret_cast<int*>(p);             p += 4 * (K + 1);
     S.F = reinterpret_cast<float2*>(base + ((p - base + 255) & ~int64_t(255)));
     S.E = S.F;
+    S.V32 = S.F + K * K;
+    // for the FP64 sweeps that go on from J and V32 (copied to work and vd first): J's space holds the Gram matrix; J V is in
+    // A1's, or in F's where a wide sector has Q2's product in A1's (R2 is in V1's)
+    S.vd = S.V0;
+    S.gm = S.J;
+    S.a1 = S.wide ? reinterpret_cast<double2*>(S.F) : S.A1;
   }
 }
 

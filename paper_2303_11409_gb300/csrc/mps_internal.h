@@ -247,10 +247,11 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   double2 *J, *A0, *A1;       // n x K column-major: R^dag, and J V of even / odd refinement steps (A0 overlays work)
   double2 *V0, *V1;           // K x K: the rotations of even / odd steps
   float2* E;                  // K x K: the scaled correction of a step (overlays F)
+  float2* V32;                // K x K: the kept columns' rotations as the FP32 sweeps left them (F's second half)
   double* rnorm;              // K squared column norms of the current A
   double* rfloor2;            // [0] the floor in the scale of J, [1] the power of two that undoes that scale
   int *cexp, *vexp;           // K scale exponents of the columns of J or A, and of V
-  int* rstate;                // 16: [0] columns kept, [1] not 0: left to the FP64 sweeps, [2] steps when settled, [4 + step] size of E
+  int* rstate;                // 16: [0] columns kept, [1] not 0: left to the FP64 sweeps (from kLeftAt on with the front's J and rotations), [2] steps when settled, [4 + step] size of E
   int fp32_sweeps;            // limit of the FP32 sweeps
   unsigned* teambar;          // barrier of the sector's team (nullptr: no teams in this batch)
   int team_first, team_size;  // the team's CTAs in its launch
@@ -452,6 +453,7 @@ cudaError_t launch_svd_groups(const SvdSector* d_secs, const std::vector<SvdGrou
 // The refinement of sectors that svd_front_kernel has prepared (k_refine.cu): J V, at most
 // kRefineSteps corrections, and the outputs of the sectors that have settled.
 constexpr int kRefineSteps = 6;
+constexpr int kLeftAt = 100;         // SvdSector::rstate[1] when step it leaves the sector: kLeftAt + it
 cudaError_t launch_refine(const SvdSector* d_secs, int count, int max_k, int max_n, cudaStream_t st);
 
 cudaError_t launch_select(const SelectSector* d_secs, const SelectTask* d_tasks, int n_tasks,

@@ -83,7 +83,8 @@ def test_which_sectors_are_refined(gpu_lib):
             np.zeros((50, 60), complex)]
     settled = [W.random_complex((80, 13), rng) @ W.random_complex((13, 70), rng), np.eye(64, dtype=complex),
                1e-130 * W.random_complex((50, 50), rng), W.haar_unitary(300, rng)]
-    assert [r[3] for r in m.svd_sectors_path(left)] == [m.MPS_SVD_SWEEPS] * len(left)
+    swept = m.MPS_SVD_SWEEPS | m.MPS_SVD_FP32_START
+    assert [r[3] for r in m.svd_sectors_path(left)] == [swept, swept, m.MPS_SVD_SWEEPS]
     assert [r[3] for r in m.svd_sectors_path(settled)] == [m.MPS_SVD_REFINED] * len(settled)
 
 
@@ -221,3 +222,22 @@ def test_columns_too_long_for_a_front(gpu_lib):
     for A, w, (s, y, sweeps, path) in zip(mats, scales, out):
         assert sweeps > 0
         _check(w[:, None] * A, s, y)
+
+
+@pytest.mark.parametrize("group", [2, 3, 8, 24])
+def test_degenerate_values_go_on_from_the_fp32_rotations(gpu_lib, group):
+    """Values in equal groups over four decades, which the refinement leaves: one-CTA fronts, cluster fronts, wide and tall.
+    The FP64 sweeps start from the front's QR and rotations, so they are few."""
+    m = gpu_lib
+    rng = np.random.default_rng(group)
+    mats = []
+    for a, b in [(72, 72), (30, 96), (150, 144), (120, 200), (300, 300), (260, 420), (420, 240), (200, 210)]:
+        k = min(a, b)
+        v = np.repeat(10.0 ** (-4.0 * np.arange(-(-k // group)) * group / k), group)[:k]
+        mats.append((W.haar_unitary(a, rng)[:, :k] * v) @ W.haar_unitary(b, rng)[:k])
+    swept = m.MPS_SVD_SWEEPS | m.MPS_SVD_FP32_START
+    out = m.svd_sectors_path(mats)
+    assert sum(r[3] == swept for r in out) >= 6
+    for A, (s, y, steps, path) in zip(mats, out):
+        assert path in (swept, m.MPS_SVD_REFINED) and steps > 0
+        _check(A, s, y)
