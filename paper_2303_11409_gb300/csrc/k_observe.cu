@@ -220,8 +220,11 @@ cudaError_t launch_sample(const SampleEntry* d_table, const int* d_site_off, int
                           const double* d_uniforms, int n, int* d_configs, double* d_probs, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const size_t smem = sizeof(double2) * ((size_t)rows + rowbuf(width));
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // 48 KB without asking, of which the kernel's own tables take some; one value for all usual sizes, so that threads with
+  // different ones do not lower each other's
+  if (smem > 40 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)std::max<size_t>(smem, 224 * 1024));
     if (e != cudaSuccess) return e;
   }
   count_launch();

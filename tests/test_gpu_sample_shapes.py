@@ -56,3 +56,23 @@ def _gate(rng, d):
     def unitary(n):
         return np.linalg.qr(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))[0]
     return [unitary(min(q, d - 1) - max(0, q - d + 1) + 1) for q in range(2 * d - 1)]
+
+
+@pytest.mark.parametrize("dim", [1400, 1527, 1530, 1536, 1540, 5000])
+def test_rows_and_columns_that_just_fill_the_default_shared_memory(gpu_lib, dim):
+    """One charge of dim states on two neighbouring bonds: dim rows and dim columns side by side, 16 bytes each, around
+    48 KB and well beyond."""
+    m = gpu_lib
+    rng = np.random.default_rng(dim)
+    L, s = 30, 14
+    occ = [1, 0] * (L // 2)
+    q = [sum(occ[b:]) for b in range(L + 1)]
+    g = m.MPS(2, occ, dim)
+    for b in (s, s + 1):
+        g.set_bond(b, {q[b]: np.ones(dim) / np.sqrt(dim)})
+    for x, shape in ((s - 1, (1, dim)), (s, (dim, dim)), (s + 1, (dim, 1))):
+        g.set_site(x, {(q[x], q[x + 1]): rng.standard_normal(shape) + 1j * rng.standard_normal(shape)})
+    got, prob = g.sample(W.uniforms(5, L, seed=1))
+    assert np.array_equal(got, [occ] * 5)
+    assert np.max(np.abs(prob - 1.0)) <= 1e-12
+    g.close()
