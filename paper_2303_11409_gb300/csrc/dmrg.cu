@@ -383,7 +383,8 @@ __device__ void gs_sums(const double2* partial, int nb, int nk, double2* out) {
   __syncthreads();
 }
 
-template <int E>
+// Many: the CTAs have more than one chunk each (a loop around a single one costs 1% of a step)
+template <int E, bool Many>
 __global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(const double2* V, int64_t ldv, int nk,
                                                              const double2* w, int64_t n,
                                                              double2* partial) {
@@ -396,13 +397,14 @@ __global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(const double2* V, i
     double2 x[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) x[i] = e0 + i * kGsThreads < n ? w[e0 + i * kGsThreads] : make_double2(0.0, 0.0);
-    gs_partials<E>(V, ldv, nk, x, e0, n, c0 < all, partial, red);
+    gs_partials<E>(V, ldv, nk, x, e0, n, !Many || c0 < all, partial, red);
+    if (!Many) break;
   }
 }
 
 // w -= sum_k h_k V_k with h from pin, then the partials of the new w: its products with the basis
 // (last == 0) or its squared norm.  CTA 0 keeps h in hout.
-template <int E>
+template <int E, bool Many>
 __global__ void __launch_bounds__(kGsThreads) gs_update_kernel(const double2* V, int64_t ldv, int nk,
                                                                double2* w, int64_t n,
                                                                const double2* pin, int last,
@@ -438,11 +440,12 @@ __global__ void __launch_bounds__(kGsThreads) gs_update_kernel(const double2* V,
     for (int i = 0; i < E; ++i)
       if (e0 + i * kGsThreads < n) w[e0 + i * kGsThreads] = x[i];
     if (!last) {
-      gs_partials<E>(V, ldv, nk, x, e0, n, c0 < all, pout, red);
+      gs_partials<E>(V, ldv, nk, x, e0, n, !Many || c0 < all, pout, red);
     } else {
 #pragma unroll
       for (int i = 0; i < E; ++i) s.x = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, s.x));
     }
+    if (!Many) break;
   }
   if (!last) return;
   s = warp_sum(s);
@@ -456,7 +459,7 @@ __global__ void __launch_bounds__(kGsThreads) gs_update_kernel(const double2* V,
 }
 
 // alpha_j = Re(h_j + g_j) (the two passes), beta_j = |w|, V_{j+1} = w / |w|
-template <int E>
+template <int E, bool Many>
 __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(double2* dst, const double2* w,
                                                               int64_t n, const double2* pin, int j,
                                                               const double2* h,
@@ -471,7 +474,7 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(double2* dst, cons
     alpha[j] = h[j].x + g[j].x;
     beta[j] = b;
   }
-  for (int64_t c0 = (int64_t)blockIdx.x * kGsThreads * E; c0 < n; c0 += (int64_t)gridDim.x * kGsThreads * E)
+  for (int64_t c0 = (int64_t)blockIdx.x * kGsThreads * E; c0 < n; c0 += (int64_t)gridDim.x * kGsThreads * E) {
 #pragma unroll
     for (int i = 0; i < E; ++i) {
       const int64_t e = c0 + i * kGsThreads + threadIdx.x;
@@ -480,6 +483,8 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(double2* dst, cons
         dst[e] = make_double2(f * v.x, f * v.y);
       }
     }
+    if (!Many) break;
+  }
 }
 
 __global__ void inv_norm_kernel(const double2* __restrict__ nrm2, double* __restrict__ inv) {
@@ -1268,19 +1273,19 @@ struct Dmrg {
 
   // Step j of the Lanczos recursion after the product: classical Gram-Schmidt of w against V_0..j,
   // twice, and V_{j+1} = w / |w|.
-  template <int E>
+  template <int E, bool Many>
   cudaError_t gram_schmidt(KBuf& b, int j) {
     const int nk = j + 1;
     const int64_t dim = b.dim, ldv = b.ldv;
     const dim3 grid(b.gb), block(kGsThreads);
     for (int x = 0; x < 4; ++x) count_launch();
-    cudaError_t e = launch_after(gs_dots_kernel<E>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part);
+    cudaError_t e = launch_after(gs_dots_kernel<E, Many>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part);
     if (e == cudaSuccess)
-      e = launch_after(gs_update_kernel<E>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part, 0, b.part2, b.hdots);
+      e = launch_after(gs_update_kernel<E, Many>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part, 0, b.part2, b.hdots);
     if (e == cudaSuccess)
-      e = launch_after(gs_update_kernel<E>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part2, 1, b.part, b.gdots);
+      e = launch_after(gs_update_kernel<E, Many>, grid, block, st, b.V, ldv, nk, b.w, dim, b.part2, 1, b.part, b.gdots);
     if (e == cudaSuccess)
-      e = launch_after(gs_scale_kernel<E>, grid, block, st, b.V + (int64_t)nk * ldv, b.w, dim, b.part, j, b.hdots, b.gdots,
+      e = launch_after(gs_scale_kernel<E, Many>, grid, block, st, b.V + (int64_t)nk * ldv, b.w, dim, b.part, j, b.hdots, b.gdots,
                        b.alpha, b.beta);
     return e;
   }
@@ -1325,8 +1330,10 @@ struct Dmrg {
         matvecs++;
         if (e != cudaSuccess) break;
         e = timed(2, 16.0 * dim * (j + 1) * 4, [&] {
-          return b.ge == 1 ? gram_schmidt<1>(b, j) : b.ge == 2 ? gram_schmidt<2>(b, j)
-                 : b.ge == 4 ? gram_schmidt<4>(b, j) : gram_schmidt<8>(b, j);
+          if (b.ge == 1) return gram_schmidt<1, false>(b, j);
+          if (b.ge == 2) return gram_schmidt<2, false>(b, j);
+          if (b.ge == 4) return gram_schmidt<4, false>(b, j);
+          return (int64_t)b.gb * kGsThreads * 8 < dim ? gram_schmidt<8, true>(b, j) : gram_schmidt<8, false>(b, j);
         });
       }
       return e;
@@ -1539,8 +1546,8 @@ struct Dmrg {
       sm[k] = right_moving ? E.cols : E.rows;
       sn[k] = right_moving ? E.rows : E.cols;
     }
-    // a step has few sectors: when one CTA each would leave most SMs idle, the sectors from
-    // min(m, n) >= 48 run on 8-CTA clusters instead
+    // a step has few sectors: when one CTA each would leave most SMs idle, the sectors of the FP64 sweeps from
+    // min(m, n) >= 48 run on 8-CTA clusters instead, and cluster fronts take 8 CTAs
     const bool spread = ns * 8 <= 152;
     SvdScratchLayout JL;
     if (!svd_layout(ns, sm.data(), sn.data(), JL, spread ? 48 : -1)) return fail(MPS_EINVAL, "DMRG SVD layout");
