@@ -65,9 +65,15 @@ typedef struct mps_s* mps_t;
  * SVD, truncation and renormalisation are FP64 in all modes and follow the same
  * rules (the reduced modes only round the GEMM inputs); the observable error of
  * each mode against the FP64 result is stated with its tests.  A bounded-wait
- * expiry inside a tensor-core GEMM
+ * expiry inside a tensor-core GEMM or a sector SVD
  * is reported as MPS_ETIMEOUT by the update call that launched it, or, for the
  * reassembly product, by the next update call on the same handle or executor.
+ * Which to take: MPS_FP64.  Its handles refine their sector SVDs on the tensor cores
+ * (mps_svd_mixed_min_k), which the reduced modes do not, because their rounding sees the phases of the
+ * singular vectors; the SVD is 87-99% of the time, so FP64 is the faster mode too: updates/s of Bose-Hubbard layers
+ * at L = 64, chi = 512 237 against 93 in TF32 and BF16x3, at L = 128, chi = 2048 12.8 against 3.35 in TF32.  The reduced
+ * modes are faster where few updates of chi = 2048 have the GPU to themselves (one: 185 against 432 ms, on teams of
+ * CTAs).
  */
 #define MPS_FP64   0
 #define MPS_TF32   1
@@ -321,8 +327,8 @@ MPS_API int mps_set_site(mps_t h, int site, int n_blocks, const int32_t* lcharge
 
 /*
  * mps_last_update_stats - diagnostics of the last update on h: counts of sectors,
- * (l,m,r) triples, Jacobi sweeps (max over sectors), ties resolved at the chi cut,
- * and the pre-renormalisation norm |S_all| and kept norm |S_kept|.
+ * (l,m,r) triples, refinement steps or FP64 Jacobi sweeps of a sector's SVD (the largest of the
+ * d_status values of mps_svd_sectors), ties resolved at the chi cut, and the pre-renormalisation norm |S_all| and kept norm |S_kept|.
  * Any pointer may be NULL.  Diagnostics; no counterpart in the paper.
  */
 MPS_API int mps_last_update_stats(mps_t h, int* n_sectors, int* n_triples, int* max_sweeps,
@@ -471,8 +477,9 @@ MPS_API int mps_autotune_force(int candidate);
 MPS_API int mps_autotune_min_flops(double flops);
 
 /*
- * mps_last_batch_sweeps - Jacobi sweeps of the last update call on h over all of its
- * sectors: sector count, summed sweeps and the largest sweep count (any may be NULL).
+ * mps_last_batch_sweeps - refinement steps and FP64 Jacobi sweeps of the last update call on h
+ * over all of its sectors: sector count, their sum and the largest of one sector (any may be
+ * NULL); mps_last_batch_paths tells how many sectors counted which.
  * Diagnostics of the per-sector SVDs of Sec. II; no counterpart in the paper.
  */
 MPS_API int mps_last_batch_sweeps(mps_t h, int* n_sectors, int64_t* sweeps_sum, int* sweeps_max);
@@ -678,8 +685,9 @@ MPS_API int mps_gate_layout(int d, int zn, int ncomp, const int32_t* phys_charge
                             int* n_blocks, int64_t* length);
 
 /*
- * mps_svd_sectors - the batched per-sector SVD kernel alone, on device memory
- * (one-sided Jacobi in FP64; Sec. II: the local update needs one SVD per charge block).
+ * mps_svd_sectors - the batched per-sector SVD alone, on device memory, to FP64 accuracy
+ * (QR and FP32 one-sided Jacobi finished by FP64-accurate products, or by FP64 sweeps where those do not
+ * settle; Sec. II: the local update needs one SVD per charge block).
  * For each sector k it decomposes M_k = diag(rowscale_k) A_k, A_k being the
  * m_k x n_k row-major complex128 matrix at d_mats + mat_off[k] (in complex
  * numbers), rowscale_k the m_k doubles at d_rowscale + row_off[k] (NULL = 1):
@@ -749,9 +757,10 @@ MPS_API int mps_svd_mixed_min_k(int min_k);
  * FP32 sweeps minimise the time; the FP64 sweeps finish either way); MPS_EINVAL outside.  Tuning;
  * no counterpart in the paper. */
 MPS_API int mps_svd_mixed_sweeps(int max_sweeps);
-/* mps_svd_cluster_min_k - sectors with min(m, n) >= min_k run on the cluster SVD kernels even when
+/* mps_svd_cluster_min_k - sectors of the FP64 sweeps (TF32 and BF16x3 handles, keep_phases, and every handle
+ * with mps_svd_mixed_min_k(0)) with min(m, n) >= min_k run on the cluster SVD kernels even when
  * they fit in one CTA's shared memory (spreading a batch of few sectors over more SMs); 0 (the
- * default): only sectors that do not fit.  A process setting read when mps_svd_sectors or an
+ * default): only sectors that do not fit.  Refined sectors choose for themselves from 25 columns.  A process setting read when mps_svd_sectors or an
  * update call lays out its scratch; mps_dmrg picks its own threshold per step.  MPS_EINVAL for
  * 0 < min_k < 16 or min_k < 0.  Tuning; no counterpart in the paper. */
 MPS_API int mps_svd_cluster_min_k(int min_k);
@@ -769,7 +778,9 @@ MPS_API int mps_svd_cluster_min_k(int min_k);
  *   array of MPS_NOALLOC_SCRATCH_BYTES bytes that every GPU which loads the
  *   library holds until the process exits.
  *   Limit: mps_svd_work_bytes() of the batch must not exceed
- *   MPS_NOALLOC_SCRATCH_BYTES; larger batches are rejected with MPS_ENOMEM before
+ *   MPS_NOALLOC_SCRATCH_BYTES.  A batch beyond it whose
+ *   mps_svd_path_work_bytes(..., keep_phases = 1) fits runs the FP64 sweeps, which need less scratch and
+ *   more time; larger ones are rejected with MPS_ENOMEM before
  *   anything runs (split the batch, or use mps_svd_sectors).
  *   The first call on a device looks up the array's device address with that
  *   device current; make that first call before any stream capture.
