@@ -938,6 +938,7 @@ struct JacobiBlocks32 {
   }
 };
 struct NoJacobi32 {};
+struct FrontStart {};      // no FP32 sweeps: a refined sector's front has run them
 
 // S.vd holds ns columns V of K (ld K), unitary to about 1e-5: one Cholesky QR makes V unitary (V^dag V = U^dag U,
 // V <- V U^-1), and S.a1 (column c at S.a1 + c * jld) becomes J V in its first ns columns, zero in the rest.  Every
@@ -1627,8 +1628,10 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   double2* W = w.W;
   // A sector whose refinement did not settle (large groups of close values) goes on from the front's J and rotations: no
   // second QR, no second FP32 sweeps.  300 x 300 with its values in equal pairs: 147 -> 78 ms.
+  // Compiled for the kernel that follows the refinement alone: in the others the branch cost QR and sweeps (one update
+  // at chi = 2048 in TF32 on a team: 166 ms without, 186 with it).
   bool resume = false;
-  if constexpr (std::is_same<J32, JacobiBlocks32>::value) resume = S.F && __ldcg(S.rstate + 1) >= kLeftAt;
+  if constexpr (std::is_same<J32, FrontStart>::value) resume = __ldcg(S.rstate + 1) >= kLeftAt;
   if (resume) {
     const double up = S.rfloor2[1];      // J is scaled
     for (int64_t e = tid_all; e < (int64_t)K * n; e += threads_all) {
@@ -1951,10 +1954,12 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   const double floor2 = fmax(frel * frel * fro2, S.floor_abs * S.floor_abs);
   bool converged = false;
   int Kj = K;                    // columns the FP64 sweeps rotate
-  if constexpr (std::is_same<J32, JacobiBlocks32>::value) {
-    if (resume || (S.f32 && K >= 2)) {       // the FP64 sweeps start from J V, V the rotations of FP32 sweeps
+  bool start = resume;
+  if constexpr (std::is_same<J32, JacobiBlocks32>::value) start = S.f32 && K >= 2;
+  if constexpr (!std::is_same<J32, NoJacobi32>::value) {
+    if (start) {       // the FP64 sweeps start from J V, V the rotations of FP32 sweeps
       int ns = K;
-      if (resume) {
+      if constexpr (std::is_same<J32, FrontStart>::value) {
         ns = __ldcg(S.rstate);
         for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all)
           Mem::st(S.vd + e, make_double2((double)S.V32[e].x, (double)S.V32[e].y));
@@ -2069,7 +2074,6 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
   }
   if (tid_all == 0) {
     *S.status = converged ? sweep : -1;
-    const bool start = std::is_same<J32, JacobiBlocks32>::value && (resume || (S.f32 && K >= 2));
     if (S.path) *S.path = MPS_SVD_SWEEPS | (start ? MPS_SVD_FP32_START : 0) | Sync::kPath | Jacobi::kPath;
   }
 }
@@ -2677,8 +2681,9 @@ __global__ void __launch_bounds__(kSvdThreads) jacobi_cluster_kernel(const SvdSe
   svd_sector<L2Mem>(S, cluster_work(S), rank, cluster, ClusterSync{}, max_sweeps, JacobiRoundRobin<L2Mem>{});
 }
 
-// The block-Jacobi SVD of one sector by nctas CTAs in the ordering of a cluster of cl0.
-template <class Sync>
+// The block-Jacobi SVD of one sector by nctas CTAs in the ordering of a cluster of cl0; Refined: a sector that has
+// passed through a front and the refinement.
+template <bool Refined, class Sync>
 __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* smem, int rank, int nctas, int cl0,
                                            Sync sync, int max_sweeps, int stall) {
   const int K = min(S.m, S.n);
@@ -2690,6 +2695,10 @@ __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* sm
   jb.bsmax = (K + 2 * cl0 * jb.g - 1) / (2 * cl0 * jb.g);
   jb.sm = reinterpret_cast<double2*>(smem);
   jb.smn = reinterpret_cast<double*>(smem + 16LL * 2 * jb.gs * jb.bsmax * (S.wide ? K : S.n));
+  if constexpr (Refined) {
+    svd_sector<L2Mem>(S, cluster_work(S), rank, nctas, sync, max_sweeps, jb, FrontStart{});
+    return;
+  }
   // the FP32 sweeps of a mixed-precision sector stage columns of jlen + K <= 2 jlen FP32
   // complex values in the same area
   JacobiBlocks32 j32;
@@ -2703,12 +2712,13 @@ __device__ __forceinline__ void svd_blocks(const SvdSector& S, unsigned char* sm
   svd_sector<L2Mem>(S, cluster_work(S), rank, nctas, sync, max_sweeps, jb, j32);
 }
 
+template <bool Refined>
 __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(const SvdSector* __restrict__ secs,
                                                                                 int cluster, int max_sweeps, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SvdSector S = secs[blockIdx.x / cluster];
-  if (S.F && S.rstate[1] == 0 && S.rstate[2] > 0) return;   // settled by the refinement
-  svd_blocks(S, smem_raw, (int)cluster_rank(), cluster, cluster, ClusterSync{}, max_sweeps, stall);
+  if (Refined && S.rstate[1] == 0 && S.rstate[2] > 0) return;   // settled by the refinement
+  svd_blocks<Refined>(S, smem_raw, (int)cluster_rank(), cluster, cluster, ClusterSync{}, max_sweeps, stall);
 }
 
 // The same for batches with few large sectors: one cooperative launch, in which a sector has a team
@@ -2725,7 +2735,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const Svd
   const SvdSector S = secs[k];
   __shared__ unsigned s_target;
   if (threadIdx.x == 0) s_target = 0;
-  svd_blocks(S, smem_raw, (int)blockIdx.x - S.team_first, S.team_size, S.team_cl0,
+  svd_blocks<false>(S, smem_raw, (int)blockIdx.x - S.team_first, S.team_size, S.team_cl0,
              TeamSync{S.teambar, S.status, (unsigned)S.team_size, &s_target}, max_sweeps, stall);
 }
 
@@ -2795,7 +2805,10 @@ cudaError_t set_attrs(int* big_out) {
     e = cudaFuncSetAttribute(svd_small_kernel<kFrontThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kFrontSmemMax);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(jacobi_cluster_block_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kBlockSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(jacobi_cluster_block_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kBlockSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemMax);
@@ -2806,7 +2819,9 @@ cudaError_t set_attrs(int* big_out) {
   int big = 8;
   if (cudaFuncSetAttribute(jacobi_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
           cudaSuccess &&
-      cudaFuncSetAttribute(jacobi_cluster_block_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+      cudaFuncSetAttribute(jacobi_cluster_block_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+          cudaSuccess &&
+      cudaFuncSetAttribute(jacobi_cluster_block_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
           cudaSuccess &&
       cudaFuncSetAttribute(svd_front_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
@@ -2821,7 +2836,7 @@ cudaError_t set_attrs(int* big_out) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, jacobi_cluster_block_kernel, &cfg) == cudaSuccess && n >= 4) big = 16;
+    if (cudaOccupancyMaxActiveClusters(&n, jacobi_cluster_block_kernel<false>, &cfg) == cudaSuccess && n >= 4) big = 16;
   }
   cudaGetLastError();
   g_big_cluster[dev] = big;
@@ -2891,7 +2906,8 @@ cudaError_t launch_group(const SvdSector* d_secs, const SvdGroup& g, int max_swe
   cfg.numAttrs = 1;
   if (g.kind == kSvdTeam) return launch_teams(d, g, max_sweeps, st);
   if (g.kind == kSvdRefine && !fallback) return cudaLaunchKernelEx(&cfg, svd_front_kernel, d, g.cl, max_sweeps, svd_stall());
-  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel, d, cl, max_sweeps, svd_stall());
+  if (g.kind == kSvdRefine) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel<true>, d, cl, max_sweeps, svd_stall());
+  if (g.kind != kSvdCluster) return cudaLaunchKernelEx(&cfg, jacobi_cluster_block_kernel<false>, d, cl, max_sweeps, svd_stall());
   return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel, d, g.cl, max_sweeps);
 }
 
