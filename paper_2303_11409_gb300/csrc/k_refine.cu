@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
   __shared__ float s_d[kOzN];      // second-order part of W's diagonal
   const SvdSector S = secs[blockIdx.y];
   if (skip(S)) return;
+  const float2* E = S.E();
   const int K = min(S.m, S.n), n = S.n, ns = ns_of(S);
   const int ct = (ns + kOzN - 1) / kOzN, rtA = (n + kOzM - 1) / kOzM, rtV = step == 0 ? 0 : (K + kOzM - 1) / kOzM;
   const int tile = blockIdx.x;
@@ -315,7 +316,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
           const int e = max((int)((__double_as_longlong(w.x) >> 52) & 0x7ff), (int)((__double_as_longlong(w.y) >> 52) & 0x7ff));
           if (e) cs.top = max(cs.top, e - 1022 + S.cexp[k]);
         } else {
-          const float2 w = S.E[(int64_t)(c0 + c) * K + k];
+          const float2 w = E[(int64_t)(c0 + c) * K + k];
           const int d = ec - S.cexp[k];      // E_kc = w 2^d
           cs.add(w.x, w.y, d, onV ? d + S.vexp[k] : 0, k == c0 + c);
         }
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_update_kernel(const SvdS
       if (step == 0) {
         vd[a] = in ? S.V0[(int64_t)(c0 + r) * K + k] : make_double2(0.0, 0.0);
       } else {
-        vf[a] = in ? S.E[(int64_t)(c0 + r) * K + k] : make_float2(0.f, 0.f);
+        vf[a] = in ? E[(int64_t)(c0 + r) * K + k] : make_float2(0.f, 0.f);
         if (in && k == c0 + r) vf[a].x += s_d[r];
       }
     }
@@ -389,6 +390,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSec
   __shared__ int s_ep[kOzM], s_eq[kOzN], s_vp[kOzM], s_vq[kOzN];
   const SvdSector S = secs[blockIdx.y];
   if (skip(S)) return;
+  float2* E = S.E();
   const int K = min(S.m, S.n), n = S.n, ns = ns_of(S);
   const int ct = (ns + kOzN - 1) / kOzN, rt = (ns + kOzM - 1) / kOzM;
   if ((int)blockIdx.x >= ct * rt) return;
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSec
       const int p = p0 + wr * 16 + g + ((x >> 1) << 3), q = q0 + wc * 16 + h * 8 + 2 * qq + (x & 1);
       if (p >= ns || q >= ns || p > q) continue;
       if (p == q) {
-        S.E[(int64_t)q * K + p] = make_float2(0.5f * Rr[h][x], 0.f);
+        E[(int64_t)q * K + p] = make_float2(0.5f * Rr[h][x], 0.f);
         worst = fmaxf(worst, fabsf(Rr[h][x]));
         continue;
       }
@@ -455,8 +457,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) refine_gram_kernel(const SvdSec
         eqp = P.qp;
         worst = fmaxf(worst, P.size);
       }
-      S.E[(int64_t)q * K + p] = epq;
-      S.E[(int64_t)p * K + q] = eqp;
+      E[(int64_t)q * K + p] = epq;
+      E[(int64_t)p * K + q] = eqp;
     }
   for (int o = 16; o; o >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, o));
   if (lane == 0 && worst > 0.f) atomicMax(S.rstate + 4 + it, __float_as_int(worst));

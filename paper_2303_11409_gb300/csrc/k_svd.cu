@@ -1612,7 +1612,8 @@ __device__ void svd_front(const SvdSector& S, const Work& w, int rank, int nctas
     S.V0[e] = make_double2((double)__ldcg(v), (double)__ldcg(v + 2));
   }
   sync();      // F is read
-  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) S.V32[e] = make_float2((float)S.V0[e].x, (float)S.V0[e].y);
+  float2* V32 = S.V32();
+  for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all) V32[e] = make_float2((float)S.V0[e].x, (float)S.V0[e].y);
 }
 
 template <class Mem, class Sync, class Jacobi, class J32 = NoJacobi32>
@@ -1961,8 +1962,9 @@ __device__ void svd_sector(const SvdSector& S, const Work& w, int rank, int ncta
       int ns = K;
       if constexpr (std::is_same<J32, FrontStart>::value) {
         ns = __ldcg(S.rstate);
+        const float2* V32 = S.V32();
         for (int64_t e = tid_all; e < (int64_t)K * ns; e += threads_all)
-          Mem::st(S.vd + e, make_double2((double)S.V32[e].x, (double)S.V32[e].y));
+          Mem::st(S.vd + e, make_double2((double)V32[e].x, (double)V32[e].y));
         sync();
         orthonormal_start(S, w, J, jlen, jld, K, ns, rank, nctas, sync, max_sweeps);
       } else if (!mixed_precondition(S, w, J, jlen, jld, K, rank, nctas, sync, floor2, max_sweeps, j32, &ns)) {
@@ -2498,10 +2500,11 @@ __global__ void __launch_bounds__(Threads, 1) svd_small_kernel(const SvdSector* 
     __syncthreads();
     const int ns = s_ns;
     if (!full) {
+      float2* V32 = S.V32();
       for (int e = tid; e < K * ns; e += blockDim.x) {
         const float2 v = row32(F + sel[e / K] * L.fld, vr + e % K);
         S.V0[e] = make_double2((double)v.x, (double)v.y);
-        S.V32[e] = v;
+        V32[e] = v;
       }
       for (int j = tid; j < n; j += blockDim.x) S.order[j] = perm[j];
       if (tid == 0) {
@@ -3318,8 +3321,6 @@ void svd_fill_scratch(SvdSector& S, const SvdScratchLayout& L, int k, char* base
     S.nrm32 = reinterpret_cast<float*>(p);         p += 4 * K;
     S.sel = reinterpret_cast<int*>(p);             p += 4 * (K + 1);
     S.F = reinterpret_cast<float2*>(base + ((p - base + 255) & ~int64_t(255)));
-    S.E = S.F;
-    S.V32 = S.F + K * K;
     // for the FP64 sweeps that go on from J and V32 (copied to work and vd first): J's space holds the Gram matrix; J V is in
     // A1's, or in F's where a wide sector has Q2's product in A1's (R2 is in V1's)
     S.vd = S.V0;

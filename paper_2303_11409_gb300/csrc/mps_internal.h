@@ -246,8 +246,6 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   float2* F;                  // the Jacobi matrix in FP32 stacked on V (identity), (jlen + K, even) x K
   double2 *J, *A0, *A1;       // n x K column-major: R^dag, and J V of even / odd refinement steps (A0 overlays work)
   double2 *V0, *V1;           // K x K: the rotations of even / odd steps
-  float2* E;                  // K x K: the scaled correction of a step (overlays F)
-  float2* V32;                // K x K: the kept columns' rotations as the FP32 sweeps left them (F's second half)
   double* rnorm;              // K squared column norms of the current A
   double* rfloor2;            // [0] the floor in the scale of J, [1] the power of two that undoes that scale
   int *cexp, *vexp;           // K scale exponents of the columns of J or A, and of V
@@ -256,6 +254,13 @@ struct SvdSector {            // one Theta(c): M = diag(rowscale) * Theta, m x n
   unsigned* teambar;          // barrier of the sector's team (nullptr: no teams in this batch)
   int team_first, team_size;  // the team's CTAs in its launch
   int team_cl0;               // the cluster size whose block ordering the team keeps
+  // over F once its sweeps are done, K x K each: the scaled correction of a step, and the kept columns' rotations as the
+  // FP32 sweeps left them
+  __host__ __device__ float2* E() const { return F; }
+  __host__ __device__ float2* V32() const {
+    const int64_t K = m < n ? m : n;
+    return F + K * K;
+  }
 };
 
 // Scratch layout of a batch of sector SVDs (cluster-mode sectors only need global scratch).
