@@ -72,7 +72,7 @@ typedef struct mps_s* mps_t;
  * (mps_svd_mixed_min_k), which the reduced modes do not, because their rounding sees the phases of the
  * singular vectors; the SVD is 87-99% of the time, so FP64 is the faster mode too: updates/s of Bose-Hubbard layers
  * at L = 64, chi = 512 237 against 93 in TF32 and BF16x3, at L = 128, chi = 2048 12.8 against 3.35 in TF32.  The reduced
- * modes are faster where few updates of chi = 2048 have the GPU to themselves (one: 185 against 432 ms, on teams of
+ * modes are faster where few updates of chi = 2048 have the GPU to themselves (one: 166 against 432 ms, on teams of
  * CTAs).
  */
 #define MPS_FP64   0

@@ -2728,7 +2728,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_cluster_block_kernel(
 // of S.team_size CTAs (those from S.team_first) instead of a cluster of at most 8.  The block ordering and
 // every sum stay those of the cluster, so the results are the same bits; only more SMs share a
 // round's block pairs, a column's trailing update and the products.  A chi = 2048 update whose 796 x 796
-// sector kept 8 SMs busy for 1.23 s takes 165 ms (a team of 104), three updates at chi = 1024 297 -> 125 ms;
+// sector kept 8 SMs busy for 1.23 s takes 166 ms (a team of 104), three updates at chi = 1024 297 -> 126 ms;
 // there the FP64 pipes of the whole chip are the bound.
 __global__ void __launch_bounds__(kBlockThreads, 2) jacobi_team_kernel(const SvdSector* __restrict__ secs, int count,
                                                                        int max_sweeps, int stall) {
